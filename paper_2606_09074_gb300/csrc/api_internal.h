@@ -242,6 +242,7 @@ struct ScenePlan {
 
 struct SceneScratch {
     CamRec *cams;
+    CamExt *ext;  // one per view scored
     PrimRec *recs;
     float2 *partials;  // per feature-pass block, float-float sums
     SceneConsts *consts;
@@ -277,7 +278,7 @@ inline ScenePlan plan_scene(int64_t n, int V, int max_views = 0, int vpp = kView
 inline size_t scene_bytes(const ScenePlan &pl)
 {
     const size_t n = (size_t)pl.n, cells = (size_t)order_keys(pl.bits);
-    return carve_size({sizeof(CamRec) * (size_t)pl.V, sizeof(PrimRec) * n, sizeof(float2) * kFeatSums * 1024,
+    return carve_size({sizeof(CamRec) * (size_t)pl.V, sizeof(CamExt) * (size_t)pl.V, sizeof(PrimRec) * n, sizeof(float2) * kFeatSums * 1024,
                        sizeof(SceneConsts), sizeof(SceneStats), sizeof(uint2) * n,
                        sizeof(unsigned) * (cells + 64), sizeof(unsigned) * cells,
                        sizeof(unsigned) * (cells / kScanCells), sizeof(uint32_t) * n,
@@ -291,6 +292,7 @@ inline SceneScratch carve_scene(Carver &cv, const ScenePlan &pl)
     const int cells = order_keys(pl.bits);
     SceneScratch x;
     x.cams = cv.take<CamRec>(pl.V);
+    x.ext = cv.take<CamExt>(pl.V);
     x.recs = cv.take<PrimRec>(n);
     x.partials = cv.take<float2>(kFeatSums * 1024);
     x.consts = cv.take<SceneConsts>(1);
@@ -323,6 +325,7 @@ inline refine_status enqueue_prep(refine_ctx *c, L &&run, const refine_scene *sc
     tail.V = pl.V;
     tail.vstride = pl.vstride;
     tail.cam_out = x.cams;
+    tail.ext_out = proj_mode(p.flags) == kProjFullJ ? x.ext : nullptr;
     tail.p = p;
     tail.cell_bits = pl.bits;
     tail.consts = x.consts;
@@ -353,6 +356,7 @@ inline ScoreLaunch make_score_launch(const refine_scene *sc, const ScenePlan &pl
     a.perm = x.perm;
     a.n = pl.n;
     a.cams = x.cams + v0;
+    a.ext = proj_mode(p.flags) == kProjFullJ ? x.ext + v0 : nullptr;
     a.vcount = pl.V - v0 < pl.vpp ? pl.V - v0 : pl.vpp;
     a.first = v0 == 0;
     a.last = v0 + a.vcount >= pl.V;
@@ -400,7 +404,7 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, need_dev != nullptr, c->d_status, s))) return st;
     for (int v0 = 0; v0 < pl.V; v0 += pl.vpp) {
         ScoreLaunch a = make_score_launch(sc, pl, x, p, v0, scores, view_sum, need_dev != nullptr, c->d_status);
-        a.grid = score_grid(c->num_sms, pl.n, a.vcount, c->shape);
+        a.grid = score_grid(c->num_sms, pl.n, a.vcount, a.flags, c->shape);
         a.tiles_taken = x.tiles;
         const cudaError_t e = cudaMemsetAsync(x.tiles, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");

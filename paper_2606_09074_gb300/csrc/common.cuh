@@ -20,23 +20,30 @@ __device__ __forceinline__ void set_status(int *status, int code)
     atomicCAS(status, 0, code);  // the first error wins
 }
 
-// Derived camera record (144 bytes).  With the intrinsic matrix K and the
+// Derived camera record (80 bytes).  With the intrinsic matrix K and the
 // world-to-camera rotation rows R0, R1, R2 (Eq. 13), each row a linear form
 // (a, a0) evaluated as a . mu + a0:
 //   U = P0 mu + p0, V = P1 mu + p1, z = R2 mu + t2   (P = K W, p = K t),
 //   pixel (u, v) = (U / z, V / z).
+// 80 bytes is 20 words: the 16-byte loads of 8 lanes reading 8 consecutive
+// records meet no bank conflict, and a block of 512 views fits four times in
+// an SM's shared memory.
 struct __align__(16) CamRec {
     float4 r0;   // U:        (fx R0 + cx R2, fx t0 + cx t2)
     float4 r1;   // V:        (fy R1 + cy R2, fy t1 + cy t2)
     float4 r2;   // z:        (R2, t2)
     float4 lim;  // (width, height, znear, zfar)
-    float4 k;    // (fx^2, fy^2, cx, cy)
-    float4 uw;   // U - w z:  (P0 - w R2, p0 - w t2)
-    float4 vh;   // V - h z:  (P1 - h R2, p1 - h t2)
-    float4 tx;   // fx x:     (fx R0, fx t0)
-    float4 ty;   // fy y:     (fy R1, fy t1)
+    float4 k;    // (Ex, Ey: edge norms of the footprint bound; tile slack per unit of |mu|_1, and its constant)
 };
-static_assert(sizeof(CamRec) == 144, "camera record layout");
+static_assert(sizeof(CamRec) == 80, "camera record layout");
+
+// What REFINE_FLAG_FULL_JACOBIAN needs of a camera besides (48 bytes).
+struct __align__(16) CamExt {
+    float4 tx;  // fx x:     (fx R0, fx t0)
+    float4 ty;  // fy y:     (fy R1, fy t1)
+    float4 f;   // (fx^2, fy^2, 0, 0)
+};
+static_assert(sizeof(CamExt) == 48, "camera extension layout");
 
 // Per-scene constants produced by the content-feature pass (Eq. 18-19) and
 // the quantisation of the processing-order grid.
@@ -270,6 +277,14 @@ __device__ __forceinline__ float rcp_approx_ftz(float x)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Square root on the MUFU pipe (max relative error 2^-22); subnormals flush.
+__device__ __forceinline__ float sqrt_approx_ftz(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 

@@ -10,8 +10,8 @@
 
 namespace refine {
 
-// Cameras processed per score launch at most (144 bytes each in shared
-// memory).  A larger view set is split into passes (camera blocks) of
+// Cameras processed per score launch at most (80 bytes each in shared
+// memory, 128 with REFINE_FLAG_FULL_JACOBIAN).  A larger view set is split into passes (camera blocks) of
 // ScoreShape::views_per_pass views, a multiple of 32; a primitive's running
 // Kahan pair (sum, compensation) is carried from pass to pass, so its sum
 // is the same whatever the block size.
@@ -109,11 +109,24 @@ struct __align__(16) PrimRec {
 };
 static_assert(sizeof(PrimRec) == 64, "primitive record layout");
 
+// Projection mode of a set of flags (the weight of a visible pair).
+enum { kProjEq17 = 0, kProjNone = 1, kProjFullJ = 2 };
+__host__ __device__ inline int proj_mode(int flags)
+{
+    return (flags & REFINE_FLAG_NO_PROJ) ? kProjNone : (flags & REFINE_FLAG_FULL_JACOBIAN) ? kProjFullJ : kProjEq17;
+}
+// Shared memory of a camera block.
+__host__ __device__ inline size_t cams_smem(int vcount, int flags)
+{
+    return (size_t)vcount * (sizeof(CamRec) + (proj_mode(flags) == kProjFullJ ? sizeof(CamExt) : 0));
+}
+
 struct ScoreLaunch {
     const PrimRec *recs;        // records in scene order
     int64_t n;
     const uint32_t *perm;       // processing order (a permutation of 0..n-1)
     const CamRec *cams;         // this pass's cameras (device, 16-byte aligned)
+    const CamExt *ext;          // their extensions (FULL_JACOBIAN, else NULL)
     int vcount;                 // cameras in this pass
     int first, last;            // first / last pass of the view set
     float eta;
@@ -138,6 +151,7 @@ struct FeatureTail {
     const refine_camera *cams;
     int V, vstride;
     CamRec *cam_out;
+    CamExt *ext_out;  // NULL unless FULL_JACOBIAN
     refine_params p;
     int cell_bits;
     SceneConsts *consts;
@@ -156,7 +170,7 @@ cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n,
                                 const unsigned *off_local, const unsigned *bsum, uint32_t *perm,
                                 int num_sms, cudaStream_t s);
 cudaError_t launch_score(const ScoreLaunch &a, const ScoreShape &sh, cudaStream_t s);
-int score_grid(int num_sms, int64_t n, int vcount, const ScoreShape &sh);
+int score_grid(int num_sms, int64_t n, int vcount, int flags, const ScoreShape &sh);
 
 // FP32 FMA throughput probe (refine_fma_rate): FLOPs of one launch of
 // `iters` steps on `num_sms` SMs, and the launch itself (sink: one float,
@@ -181,8 +195,9 @@ struct BatchLaunch {
     int *status;
     int rounds;                      // warp tiles per warp in an item (batch_tile)
 };
-int score_batch_grid(int num_sms, int max_vcount, const ScoreShape &sh);
-cudaError_t launch_score_batch(const BatchLaunch &b, int max_vcount, int grid, const ScoreShape &sh, cudaStream_t s);
+// smem: the largest camera block among the scenes (cams_smem).
+int score_batch_grid(int num_sms, size_t smem, const ScoreShape &sh);
+cudaError_t launch_score_batch(const BatchLaunch &b, size_t smem, int grid, const ScoreShape &sh, cudaStream_t s);
 
 // ------------------------------------------------------------- select
 struct SelState {

@@ -3,16 +3,20 @@
 // importance kernel (Eq. 7, Eq. 20).
 #include <math.h>
 
+#include <float.h>
+
 #include "internal.h"
 
 namespace refine {
+
+constexpr float kTileSlack = 7.62939453125e-06f;  // 2^-17, see classify
 
 // ---------------------------------------------------------------------
 // Camera preparation: refine_camera -> CamRec (P = K W and p = K t formed
 // in double and rounded once), with validation.
 // ---------------------------------------------------------------------
 __device__ void prep_camera(const refine_camera *__restrict__ cams, int v, int vstride, CamRec *__restrict__ out,
-                            int *status)
+                            CamExt *__restrict__ ext, int *status)
 {
     refine_camera c = cams[(int64_t)v * vstride];
     bool ok = isfinite(c.fx) && isfinite(c.fy) && isfinite(c.cx) && isfinite(c.cy) &&
@@ -24,12 +28,10 @@ __device__ void prep_camera(const refine_camera *__restrict__ cams, int v, int v
     if (!ok) {
         set_status(status, kEinval);
         r.r0 = make_float4(0.f, 0.f, 0.f, 0.f);
-        r.r1 = r.r0;
-        r.r2 = r.r0;
+        r.r1 = r.r2 = r.k = r.r0;
         r.lim = make_float4(0.f, 0.f, 1.f, 0.f);  // znear > zfar: never visible
-        r.k = r.r0;
-        r.uw = r.vh = r.tx = r.ty = r.r0;
         out[v] = r;
+        if (ext) ext[v] = CamExt{r.r0, r.r0, r.r0};
         return;
     }
     double fx = c.fx, fy = c.fy, cx = c.cx, cy = c.cy;
@@ -38,16 +40,40 @@ __device__ void prep_camera(const refine_camera *__restrict__ cams, int v, int v
     r.r1 = make_float4((float)(fy * c.R[3] + cy * c.R[6]), (float)(fy * c.R[4] + cy * c.R[7]),
                        (float)(fy * c.R[5] + cy * c.R[8]), (float)(fy * c.t[1] + cy * c.t[2]));
     r.r2 = make_float4(c.R[6], c.R[7], c.R[8], c.t[2]);
-    r.lim = make_float4((float)c.width, (float)c.height, c.znear, c.zfar);
-    r.k = make_float4((float)(fx * fx), (float)(fy * fy), c.cx, c.cy);
-    const double w = c.width, h = c.height;
-    r.uw = make_float4((float)(fx * c.R[0] + (cx - w) * c.R[6]), (float)(fx * c.R[1] + (cx - w) * c.R[7]),
-                       (float)(fx * c.R[2] + (cx - w) * c.R[8]), (float)(fx * c.t[0] + (cx - w) * c.t[2]));
-    r.vh = make_float4((float)(fy * c.R[3] + (cy - h) * c.R[6]), (float)(fy * c.R[4] + (cy - h) * c.R[7]),
-                       (float)(fy * c.R[5] + (cy - h) * c.R[8]), (float)(fy * c.t[1] + (cy - h) * c.t[2]));
-    r.tx = make_float4((float)(fx * c.R[0]), (float)(fx * c.R[1]), (float)(fx * c.R[2]), (float)(fx * c.t[0]));
-    r.ty = make_float4((float)(fy * c.R[3]), (float)(fy * c.R[4]), (float)(fy * c.R[5]), (float)(fy * c.t[1]));
+    const float w = (float)c.width, h = (float)c.height;
+    r.lim = make_float4(w, h, c.znear, c.zfar);
+    // The edge norms Ex, Ey of the footprint bound (classify), rounded up;
+    // the bound needs orthonormal rows of R (to well within the 2^-11 that the
+    // primitives' s3 carries), so other cameras get none (every open pair
+    // runs the exact test).
+    float dot[6];
+    for (int i = 0, k = 0; i < 3; ++i)
+        for (int j = i; j < 3; ++j, ++k) {
+            const float *a = c.R + 3 * i, *b = c.R + 3 * j;
+            dot[k] = fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2])) - (i == j ? 1.f : 0.f);
+        }
+    bool ortho = true;
+    for (int k = 0; k < 6; ++k) ortho = ortho && fabsf(dot[k]) <= 1.220703125e-4f;  // 2^-13
+    const float ex = fmaxf(fabsf(c.cx), fabsf(w - c.cx)), ey = fmaxf(fabsf(c.cy), fabsf(h - c.cy));
+    const float Ex = sqrtf(fmaf(c.fx, c.fx, ex * ex)) * 1.00001f, Ey = sqrtf(fmaf(c.fy, c.fy, ey * ey)) * 1.00001f;
+    // tile slack of the forms U, V, U - w z, V - h z (classify)
+    float ca = 0.f, c0 = 0.f;
+    for (const float4 &q : {r.r0, r.r1}) {
+        ca = fmaxf(ca, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
+        c0 = fmaxf(c0, fabsf(q.w));
+    }
+    const float wh = fmaxf(w, h);
+    ca = fmaxf(ca, wh * fmaxf(fabsf(r.r2.x), fmaxf(fabsf(r.r2.y), fabsf(r.r2.z))));
+    c0 = fmaxf(c0, wh * fabsf(r.r2.w));
+    r.k = make_float4(ortho ? Ex : FLT_MAX, ortho ? Ey : FLT_MAX, 2.f * kTileSlack * ca, 2.f * kTileSlack * c0);
     out[v] = r;
+    if (ext) {
+        CamExt e;
+        e.tx = make_float4((float)(fx * c.R[0]), (float)(fx * c.R[1]), (float)(fx * c.R[2]), (float)(fx * c.t[0]));
+        e.ty = make_float4((float)(fy * c.R[3]), (float)(fy * c.R[4]), (float)(fy * c.R[5]), (float)(fy * c.t[1]));
+        e.f = make_float4((float)(fx * fx), (float)(fy * fy), 0.f, 0.f);
+        ext[v] = e;
+    }
 }
 
 // Eq. (features) -> Eq. 18 -> Eq. 19 in double, by one block (every thread
@@ -157,7 +183,7 @@ __global__ void __launch_bounds__(kFeatThreads, 4) k_features(const float *__res
 {
     for (int64_t v = blockIdx.x + (int64_t)gridDim.x * threadIdx.x; v < tail.V;
          v += (int64_t)gridDim.x * blockDim.x)
-        prep_camera(tail.cams, (int)v, tail.vstride, tail.cam_out, status);
+        prep_camera(tail.cams, (int)v, tail.vstride, tail.cam_out, tail.ext_out, status);
 
     FeatSums acc;
 #pragma unroll
@@ -475,20 +501,26 @@ cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n, const unsigned *of
 struct PairIn {
     float mx, my, mz;
     float L[9];
-    float b2;  // 9 s_max^2 (1 + 2^-10)
+    float s3;  // 3 s_max (1 + 2^-11), the square root of the record's footprint bound factor
 };
 
 struct __align__(16) TileBox {
     float cx, cy, cz;  // centre of the box of the tile's centres
     float hx, hy, hz;  // half extents
-    float mx, my, mz;  // |centre| + half extent (magnitude bound)
-    float b2;          // max over the tile of 9 s_max^2 (1 + 2^-10)
-    float pad[2];
+    float l1;          // sum over the axes of |centre| + half extent (magnitude bound)
+    float s3;          // max over the tile of PairIn::s3
 };
 
-// The tile box lives in the warp's shared-memory slot while its views are
-// scored and is read back for each classification, so that it holds no
-// registers across the view loop (the loads are volatile: never hoisted).
+// A warp's shared-memory slot.  The tile box lives there while the tile's
+// views are scored and is read back for each classification, so that it
+// holds no registers across the view loop (the loads are volatile: never
+// hoisted); k holds the footprint reach (classify) of the 32 views being
+// scored, one per classifying lane.
+struct __align__(16) WarpSlot {
+    TileBox box;
+    float2 k[32];
+};
+
 __device__ __forceinline__ TileBox load_box(const TileBox *s)
 {
     TileBox t;
@@ -496,25 +528,20 @@ __device__ __forceinline__ TileBox load_box(const TileBox *s)
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(t.cx), "=f"(t.cy), "=f"(t.cz), "=f"(t.hx) : "r"(a));
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(t.hy), "=f"(t.hz), "=f"(t.mx), "=f"(t.my) : "r"(a + 16));
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(t.mz), "=f"(t.b2) : "r"(a + 32));
+                 : "=f"(t.hy), "=f"(t.hz), "=f"(t.l1), "=f"(t.s3) : "r"(a + 16));
     return t;
 }
-
-constexpr float kTileSlack = 6.103515625e-05f;  // 2^-14
 
 struct Range {
     float lo, hi;
 };
 
-// [lo, hi] of a . mu + a0 over the tile box, widened by the slack.
-__device__ __forceinline__ Range form_range(const float4 &a, const TileBox &t)
+// [lo, hi] of a . mu + a0 over the tile box, widened by the slack sl.
+__device__ __forceinline__ Range form_range(const float4 &a, const TileBox &t, float sl)
 {
     const float mid = fmaf(a.x, t.cx, fmaf(a.y, t.cy, fmaf(a.z, t.cz, a.w)));
-    const float rad = fmaf(fabsf(a.x), t.hx, fmaf(fabsf(a.y), t.hy, fabsf(a.z) * t.hz));
-    const float mag = fmaf(fabsf(a.x), t.mx, fmaf(fabsf(a.y), t.my, fmaf(fabsf(a.z), t.mz, fabsf(a.w))));
-    const float sl = kTileSlack * mag;
-    return {mid - rad - sl, mid + rad + sl};
+    const float rad = fmaf(fabsf(a.x), t.hx, fmaf(fabsf(a.y), t.hy, fmaf(fabsf(a.z), t.hz, sl)));
+    return {mid - rad, mid + rad};
 }
 
 // Class of one view for one tile: kClsMixed, kClsIn or kClsOut in the low two
@@ -522,76 +549,55 @@ __device__ __forceinline__ Range form_range(const float4 &a, const TileBox &t)
 // (kAxX: 0 < u < w, kAxY: 0 < v < h, kAxZ: znear < z < zfar) above them.  An
 // axis that is not flagged holds for every centre of the tile, with the same
 // float32 slack as the IN class, so a pair's test on it needs no evaluation.
+//
+// The slack of a range is at least 8 times the float32 rounding of its form
+// evaluated pair by pair plus that of the range itself (together under 14 x
+// 2^-24 of the sum of the terms' magnitudes, counted operation by operation).
+// One slack serves U, V, U - w z and V - h z of a camera: 2^-16 times (its
+// largest coefficient or w |R2| x the tile's l1 + its largest constant or w
+// |t2|), twice the largest magnitude at 2^-17.
+//
+// The footprint bound.  The exact test passes an extent only if du^2 <= 9
+// s_max^2 (fx^2 + (u - cx)^2), as |g0|^2 = fx^2 (x^2 + z^2).  Outside the image
+// by du = max(-U, U - w z) > 0, |u - cx| <= e + du / z with e the larger
+// distance of an edge from cx, so with E = sqrt(fx^2 + e^2)
+//   du <= 3 s_max (E + du / z),  i.e.  du (z - s3) <= s3 E z,  s3 = 3 s_max,
+// and over a box with z >= z_lo: du <= s3 K, K = min(E z_lo / (z_lo - max s3)
+// (if z_lo > max s3), E + max du / z_lo).  *reach (MIXED with the depth range
+// closed) is (Kx, Ky), infinite (nothing is excluded) where a square of the
+// exact test could overflow or underflow.
 enum { kClsMixed = 0, kClsIn = 1, kClsOut = 2 };
 enum { kAxX = 4, kAxY = 8, kAxZ = 16 };
 
-__device__ __forceinline__ int classify(const CamRec &c, const TileBox &t)
+__device__ __forceinline__ float4 edge_form(const float4 &a, const float4 &c2, float w)
 {
-    const Range z = form_range(c.r2, t);
-    if (z.hi < c.lim.z || z.lo > c.lim.w) return kClsOut;
-    const Range U = form_range(c.r0, t), V = form_range(c.r1, t);
-    const Range UW = form_range(c.uw, t), VH = form_range(c.vh, t);
-    const bool zin = z.lo > c.lim.z && z.hi < c.lim.w;
+    return make_float4(fmaf(-w, c2.x, a.x), fmaf(-w, c2.y, a.y), fmaf(-w, c2.z, a.z), fmaf(-w, c2.w, a.w));
+}
+
+__device__ __forceinline__ int classify(const CamRec &c, const TileBox &t, float2 *reach)
+{
+    const float4 c2 = c.r2, lim = c.lim;
+    const float zmax = fmaxf(fabsf(c2.x), fmaxf(fabsf(c2.y), fabsf(c2.z)));
+    const Range z = form_range(c2, t, kTileSlack * fmaf(zmax, t.l1, fabsf(c2.w)));
+    if (z.hi < lim.z || z.lo > lim.w) return kClsOut;
+    const float4 k = c.k, c0 = c.r0, c1 = c.r1;
+    const float sl = fmaf(k.z, t.l1, k.w);
+    const Range U = form_range(c0, t, sl), V = form_range(c1, t, sl);
+    const Range UW = form_range(edge_form(c0, c2, lim.x), t, sl), VH = form_range(edge_form(c1, c2, lim.y), t, sl);
+    const bool zin = z.lo > lim.z && z.hi < lim.w;
     const bool xin = U.lo > 0.f && UW.hi < 0.f, yin = V.lo > 0.f && VH.hi < 0.f;
     if (zin && xin && yin) return kClsIn;
     const int mixed = kClsMixed | (xin ? 0 : kAxX) | (yin ? 0 : kAxY) | (zin ? 0 : kAxZ);
-    if (!(z.lo > 0.f)) return mixed;
-    // outside an edge by more than the footprint bound (times z^2)
-    const Range TX = form_range(c.tx, t), TY = form_range(c.ty, t);
-    const float tx2 = fmaxf(TX.lo * TX.lo, TX.hi * TX.hi), ty2 = fmaxf(TY.lo * TY.lo, TY.hi * TY.hi);
-    // per pair the bound reads (d z)^2 > b2 (fx^2 z^2 + tx^2), i.e. d^2 > b2 (fx^2 + (tx / z)^2): over
-    // the box d >= d_lo and z >= z_lo > 0, so (d_lo z_lo)^2 > b2 (fx^2 z_lo^2 + max tx^2) suffices
-    const float zz = z.lo * z.lo;
-    const float bx = t.b2 * fmaf(c.k.x, zz, tx2) * 1.00390625f;  // (1 + 2^-8)
-    const float by = t.b2 * fmaf(c.k.y, zz, ty2) * 1.00390625f;
-    const float dl = fmaxf(-U.hi, UW.lo) * z.lo;  // > 0 when the box is left or right of the image
-    const float dt = fmaxf(-V.hi, VH.lo) * z.lo;
-    if ((dl > 0.f && dl * dl > bx) || (dt > 0.f && dt * dt > by)) return kClsOut;
+    const float dx = fmaxf(-U.lo, UW.hi), dy = fmaxf(-V.lo, VH.hi);  // largest du, dv of the box
+    const float zs = z.lo - t.s3;
+    const float iz = rcp_approx_ftz(z.lo), q = zs > 0.f ? z.lo * rcp_approx_ftz(zs) : INFINITY;
+    const bool safe = z.lo > 1e-15f && fmaxf(dx, dy) * z.hi < 1e18f;
+    const float kx = safe ? fminf(k.x * q, fmaf(fmaxf(dx, 0.f), iz, k.x)) * 1.00390625f : INFINITY;
+    const float ky = safe ? fminf(k.y * q, fmaf(fmaxf(dy, 0.f), iz, k.y)) * 1.00390625f : INFINITY;
+    *reach = make_float2(kx, ky);
+    // the whole box beyond an edge by more than the reach of its largest primitive
+    if (fmaxf(-U.hi, UW.lo) > t.s3 * kx || fmaxf(-V.hi, VH.lo) > t.s3 * ky) return kClsOut;
     return mixed;
-}
-
-template <bool DET>
-__device__ __forceinline__ bool exact_box(const float4 &c0, const float4 &c1, const float4 &c2, float U, float V,
-                                          float z, float ex2, float ey2, const PairIn &p)
-{
-    const float g0x = fmaf(-U, c2.x, z * c0.x), g0y = fmaf(-U, c2.y, z * c0.y), g0z = fmaf(-U, c2.z, z * c0.z);
-    const float g1x = fmaf(-V, c2.x, z * c1.x), g1y = fmaf(-V, c2.y, z * c1.y), g1z = fmaf(-V, c2.z, z * c1.z);
-    const float a0 = fmaf(p.L[0], g0x, fmaf(p.L[1], g0y, p.L[2] * g0z));
-    const float a1 = fmaf(p.L[3], g0x, fmaf(p.L[4], g0y, p.L[5] * g0z));
-    const float a2 = fmaf(p.L[6], g0x, fmaf(p.L[7], g0y, p.L[8] * g0z));
-    const float b0 = fmaf(p.L[0], g1x, fmaf(p.L[1], g1y, p.L[2] * g1z));
-    const float b1 = fmaf(p.L[3], g1x, fmaf(p.L[4], g1y, p.L[5] * g1z));
-    const float b2 = fmaf(p.L[6], g1x, fmaf(p.L[7], g1y, p.L[8] * g1z));
-    const float Qx = fmaf(a0, a0, fmaf(a1, a1, a2 * a2));
-    const float Qy = fmaf(b0, b0, fmaf(b1, b1, b2 * b2));
-    bool ok = (ex2 <= Qx) & (ey2 <= Qy);
-    if (DET) {
-        const float x0 = a1 * b2 - a2 * b1, x1 = a2 * b0 - a0 * b2, x2 = a0 * b1 - a1 * b0;
-        ok = ok & ((x0 != 0.f) | (x1 != 0.f) | (x2 != 0.f));
-    }
-    return ok;
-}
-
-struct PairGeom {
-    float U, V, z, ex2, ey2;
-    bool inz, inside;
-};
-
-__device__ __forceinline__ PairGeom pair_geom(const float4 &c0, const float4 &c1, const float4 &c2, const float4 &lim,
-                                              const PairIn &p)
-{
-    PairGeom r;
-    r.U = fmaf(c0.x, p.mx, fmaf(c0.y, p.my, fmaf(c0.z, p.mz, c0.w)));
-    r.V = fmaf(c1.x, p.mx, fmaf(c1.y, p.my, fmaf(c1.z, p.mz, c1.w)));
-    r.z = fmaf(c2.x, p.mx, fmaf(c2.y, p.my, fmaf(c2.z, p.mz, c2.w)));
-    const float du = fmaxf(-r.U, fmaf(-lim.x, r.z, r.U));
-    const float dv = fmaxf(-r.V, fmaf(-lim.y, r.z, r.V));
-    r.inz = (r.z > lim.z) & (r.z < lim.w);
-    r.inside = r.inz & (du <= 0.f) & (dv <= 0.f);
-    const float ex = fmaxf(du, 0.f) * r.z, ey = fmaxf(dv, 0.f) * r.z;
-    r.ex2 = ex * ex;
-    r.ey2 = ey * ey;
-    return r;
 }
 
 // Projection term of a visible (primitive, view) pair.  PM (projection
@@ -600,16 +606,14 @@ __device__ __forceinline__ PairGeom pair_geom(const float4 &c0, const float4 &c1
 // fy^2)/z^2 + ((fx x)^2 + (fy y)^2)/z^4, with fx x and fy y from the camera's
 // fx R0 and fy R1 rows (the same arithmetic on every path, so the weight does
 // not depend on the tile's classification).
-enum { kProjEq17 = 0, kProjNone = 1, kProjFullJ = 2 };
-
 template <int PM>
-__device__ __forceinline__ float weight(const CamRec &c, float z, float eta, float mx, float my, float mz)
+__device__ __forceinline__ float weight(const CamExt *e, float z, float eta, float mx, float my, float mz)
 {
     if (PM == kProjNone) return 1.f;
     // z^2 + eta >= eta >= 2^-126 (checked on the host), so the operand is
     // never subnormal; weights below 2^-126 (z beyond 9.2e18) flush to zero
     if (PM == kProjEq17) return rcp_approx_ftz(fmaf(z, z, eta));
-    const float4 tx = c.tx, ty = c.ty, k = c.k;
+    const float4 tx = e->tx, ty = e->ty, k = e->f;
     const float fxx = fmaf(tx.x, mx, fmaf(tx.y, my, fmaf(tx.z, mz, tx.w)));
     const float fyy = fmaf(ty.x, mx, fmaf(ty.y, my, fmaf(ty.z, mz, ty.w)));
     // explicit rounding intrinsics: never contracted into a neighbouring
@@ -618,176 +622,154 @@ __device__ __forceinline__ float weight(const CamRec &c, float z, float eta, flo
     return __fmul_rn(fmaf(fmaf(fxx, fxx, __fmul_rn(fyy, fyy)), iz2, __fadd_rn(k.x, k.y)), iz2);
 }
 
-__host__ __device__ inline int proj_mode(int flags)
-{
-    return (flags & REFINE_FLAG_NO_PROJ) ? kProjNone : (flags & REFINE_FLAG_FULL_JACOBIAN) ? kProjFullJ : kProjEq17;
-}
-
-template <int PM, bool DET, bool COUNT, int GPT>
-__device__ __forceinline__ void mixed_view(const CamRec &c, float eta, const PairIn (&p)[GPT],
-                                           const bool (&valid)[GPT], float (&part)[GPT],
-                                           unsigned long long (&cnt)[kCountSlots])
+// A view of a tile that holds an underflowed scale: every pair in the depth
+// range runs the whole test, the determinant included.
+template <int PM, bool COUNT, int GPT>
+__device__ __forceinline__ void mixed_view_det(const CamRec &c, const CamExt *e, float eta, const PairIn (&p)[GPT],
+                                               const bool (&valid)[GPT], float (&part)[GPT],
+                                               unsigned long long (&cnt)[kCountSlots])
 {
     const float4 c0 = c.r0, c1 = c.r1, c2 = c.r2, lim = c.lim;
-    PairGeom q[GPT];
-    bool vis[GPT], out = false;
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
-        q[g] = pair_geom(c0, c1, c2, lim, p[g]);
-        vis[g] = q[g].inside;
-        out |= q[g].inz & !q[g].inside;
+        const float U = fmaf(c0.x, p[g].mx, fmaf(c0.y, p[g].my, fmaf(c0.z, p[g].mz, c0.w)));
+        const float V = fmaf(c1.x, p[g].mx, fmaf(c1.y, p[g].my, fmaf(c1.z, p[g].mz, c1.w)));
+        const float z = fmaf(c2.x, p[g].mx, fmaf(c2.y, p[g].my, fmaf(c2.z, p[g].mz, c2.w)));
+        const float du = fmaxf(-U, fmaf(-lim.x, z, U)), dv = fmaxf(-V, fmaf(-lim.y, z, V));
+        const bool inz = (z > lim.z) & (z < lim.w);
+        const float ex = fmaxf(du, 0.f) * z, ey = fmaxf(dv, 0.f) * z;
+        const float ex2 = ex * ex, ey2 = ey * ey;
+        const float g0x = fmaf(-U, c2.x, z * c0.x), g0y = fmaf(-U, c2.y, z * c0.y), g0z = fmaf(-U, c2.z, z * c0.z);
+        const float g1x = fmaf(-V, c2.x, z * c1.x), g1y = fmaf(-V, c2.y, z * c1.y), g1z = fmaf(-V, c2.z, z * c1.z);
+        const float a0 = fmaf(p[g].L[0], g0x, fmaf(p[g].L[1], g0y, p[g].L[2] * g0z));
+        const float a1 = fmaf(p[g].L[3], g0x, fmaf(p[g].L[4], g0y, p[g].L[5] * g0z));
+        const float a2 = fmaf(p[g].L[6], g0x, fmaf(p[g].L[7], g0y, p[g].L[8] * g0z));
+        const float b0 = fmaf(p[g].L[0], g1x, fmaf(p[g].L[1], g1y, p[g].L[2] * g1z));
+        const float b1 = fmaf(p[g].L[3], g1x, fmaf(p[g].L[4], g1y, p[g].L[5] * g1z));
+        const float b2 = fmaf(p[g].L[6], g1x, fmaf(p[g].L[7], g1y, p[g].L[8] * g1z));
+        const float Qx = fmaf(a0, a0, fmaf(a1, a1, a2 * a2));
+        const float Qy = fmaf(b0, b0, fmaf(b1, b1, b2 * b2));
+        const float x0 = a1 * b2 - a2 * b1, x1 = a2 * b0 - a0 * b2, x2 = a0 * b1 - a1 * b0;
+        const bool vis = inz & (ex2 <= Qx) & (ey2 <= Qy) & ((x0 != 0.f) | (x1 != 0.f) | (x2 != 0.f));
+        part[g] += vis ? weight<PM>(e, z, eta, p[g].mx, p[g].my, p[g].mz) : 0.f;
         if (COUNT && valid[g]) {
+            const bool o = inz & !((du <= 0.f) & (dv <= 0.f));
             cnt[kCntMixedPairs] += 1;
             cnt[kCntOpenX] += 1;
             cnt[kCntOpenY] += 1;
             cnt[kCntOpenZ] += 1;
+            cnt[kCntBoundPairs] += o ? 1 : 0;
+            cnt[kCntBoundX] += o ? 1 : 0;
+            cnt[kCntBoundY] += o ? 1 : 0;
+            cnt[kCntExactPairs] += inz ? 1 : 0;
+            cnt[kCntExactX] += inz ? 1 : 0;
+            cnt[kCntExactY] += inz ? 1 : 0;
+            cnt[kCntVisMixed] += vis ? 1 : 0;
         }
+        if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 2;
     }
-    if (DET || __any_sync(0xffffffffu, out)) {
-        const float4 k = c.k;
-        bool nearq = false, nq[GPT];
-#pragma unroll
-        for (int g = 0; g < GPT; ++g) {
-            const float tx = fmaf(-k.z, q[g].z, q[g].U), ty = fmaf(-k.w, q[g].z, q[g].V);
-            const float zz = q[g].z * q[g].z;
-            const bool o = q[g].inz & !q[g].inside;
-            nq[g] = o & (q[g].ex2 <= p[g].b2 * fmaf(k.x, zz, tx * tx)) & (q[g].ey2 <= p[g].b2 * fmaf(k.y, zz, ty * ty));
-            nearq |= nq[g];
-            if (COUNT && valid[g]) {
-                cnt[kCntBoundPairs] += o ? 1 : 0;
-                cnt[kCntBoundX] += o ? 1 : 0;
-                cnt[kCntBoundY] += o ? 1 : 0;
-                cnt[kCntExactPairs] += nq[g] ? 1 : 0;
-                // the determinant path evaluates both extents of every pair
-                cnt[kCntExactX] += q[g].inz ? 1 : 0;
-                cnt[kCntExactY] += q[g].inz ? 1 : 0;
-            }
-        }
-        if (DET || __any_sync(0xffffffffu, nearq)) {
-#pragma unroll
-            for (int g = 0; g < GPT; ++g)
-                vis[g] = q[g].inz & exact_box<DET>(c0, c1, c2, q[g].U, q[g].V, q[g].z, q[g].ex2, q[g].ey2, p[g]);
-            if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 2 * GPT;
-        }
-    }
-#pragma unroll
-    for (int g = 0; g < GPT; ++g) {
-        part[g] += vis[g] ? weight<PM>(c, q[g].z, eta, p[g].mx, p[g].my, p[g].mz) : 0.f;
-        if (COUNT) cnt[kCntVisMixed] += (valid[g] && vis[g]) ? 1 : 0;
-    }
+}
+
+// One extent of the exact footprint test: |L g|^2 with g = z r - W c2 (r the
+// camera row of U or V, W its value).
+__device__ __forceinline__ float extent2(const float4 &r, const float4 &c2, float W, float z, const PairIn &p)
+{
+    const float gx = fmaf(-W, c2.x, z * r.x), gy = fmaf(-W, c2.y, z * r.y), gz = fmaf(-W, c2.z, z * r.z);
+    const float a0 = fmaf(p.L[0], gx, fmaf(p.L[1], gy, p.L[2] * gz));
+    const float a1 = fmaf(p.L[3], gx, fmaf(p.L[4], gy, p.L[5] * gz));
+    const float a2 = fmaf(p.L[6], gx, fmaf(p.L[7], gy, p.L[8] * gz));
+    return fmaf(a0, a0, fmaf(a1, a1, a2 * a2));
 }
 
 // A MIXED view of a tile without underflowed scales, evaluated only on the
 // axes its classification left open (NX: 0 < u < w, NY: 0 < v < h, NZ: the
 // depth range); an axis that holds for every centre of the tile contributes
 // d = 0 to the box test, which it then passes for every Sigma2D, so leaving
-// it out changes no decision.  The stages are those of the full test, with
-// the same expressions (so the same float32 roundings): the centre test; for
-// centres outside, the footprint bound; and the exact footprint test, entered
-// per primitive slot g and per axis only when some lane of the warp needs it
-// (a lane whose bound test failed, or whose centre lies within that axis's
-// interval, passes or fails it without evaluation).
+// it out changes no decision.  First the centre test and, for centres
+// outside, a footprint bound; then the exact footprint test, entered per
+// primitive slot g and per axis only when some lane of the warp needs it (a
+// lane whose bound failed, or whose centre lies within that axis's interval,
+// fails or passes it without evaluation).
+//
+// The bound (classify) with the depth range closed: du <= s3 Kx, the tile's
+// reach, one multiply-add and one compare a pair (the 1e-15 covers a square
+// that would underflow in the exact test); with the depth range open a pair
+// forms its own, du (z - s3) <= s3 E z.  Both exclude only pairs that the exact
+// test fails.
 template <int PM, bool COUNT, int GPT, bool NX, bool NY, bool NZ>
-__device__ __forceinline__ void mixed_view_ax(const CamRec &c, float eta, const PairIn (&p)[GPT],
-                                              const bool (&valid)[GPT], float (&part)[GPT],
-                                              unsigned long long (&cnt)[kCountSlots])
+__device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, const float2 &reach, float eta, const PairIn (&p)[GPT],
+                                           const bool (&valid)[GPT], float (&part)[GPT],
+                                           unsigned long long (&cnt)[kCountSlots])
 {
     const float4 c2 = c.r2, lim = c.lim;
+    const float2 K = NZ ? make_float2(0.f, 0.f) : reach;
     float z[GPT], U[GPT], V[GPT], du[GPT], dv[GPT];
-    bool vis[GPT], o[GPT], anyo = false;
+    bool vis[GPT], nq[GPT];
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
         z[g] = fmaf(c2.x, p[g].mx, fmaf(c2.y, p[g].my, fmaf(c2.z, p[g].mz, c2.w)));
-        bool inside = NZ ? (z[g] > lim.z) & (z[g] < lim.w) : true;
-        const bool inz = inside;
+        const bool inz = NZ ? (z[g] > lim.z) & (z[g] < lim.w) : true;
+        bool inside = inz, reaches = inz;
         if (NX) {
             const float4 c0 = c.r0;
             U[g] = fmaf(c0.x, p[g].mx, fmaf(c0.y, p[g].my, fmaf(c0.z, p[g].mz, c0.w)));
             du[g] = fmaxf(-U[g], fmaf(-lim.x, z[g], U[g]));
             inside &= du[g] <= 0.f;
+            if (!NZ) reaches &= du[g] <= fmaf(p[g].s3, K.x, 1e-15f);
         }
         if (NY) {
             const float4 c1 = c.r1;
             V[g] = fmaf(c1.x, p[g].mx, fmaf(c1.y, p[g].my, fmaf(c1.z, p[g].mz, c1.w)));
             dv[g] = fmaxf(-V[g], fmaf(-lim.y, z[g], V[g]));
             inside &= dv[g] <= 0.f;
+            if (!NZ) reaches &= dv[g] <= fmaf(p[g].s3, K.y, 1e-15f);
+        }
+        if (NZ) {
+            const float4 k = c.k;
+            const float zs = z[g] - p[g].s3, t = p[g].s3 * z[g] * 1.00390625f;
+            reaches &= (du[g] * zs <= k.x * t) & (dv[g] * zs <= k.y * t);
         }
         vis[g] = inside;
-        o[g] = inz & !inside;
-        anyo |= o[g];
+        nq[g] = reaches & !inside;
         if (COUNT && valid[g]) {
+            const bool o = inz & !inside;
             cnt[kCntMixedPairs] += 1;
             cnt[kCntOpenX] += NX ? 1 : 0;
             cnt[kCntOpenY] += NY ? 1 : 0;
             cnt[kCntOpenZ] += NZ ? 1 : 0;
-        }
-    }
-    if (__any_sync(0xffffffffu, anyo)) {
-        const float4 k = c.k;
-        float ex2[GPT], ey2[GPT];
-        bool nq[GPT];
-#pragma unroll
-        for (int g = 0; g < GPT; ++g) {
-            const float zz = z[g] * z[g];
-            bool ok = o[g];
-            if (NX) {
-                const float ex = fmaxf(du[g], 0.f) * z[g];
-                ex2[g] = ex * ex;
-                const float tx = fmaf(-k.z, z[g], U[g]);
-                ok &= ex2[g] <= p[g].b2 * fmaf(k.x, zz, tx * tx);
-            }
-            if (NY) {
-                const float ey = fmaxf(dv[g], 0.f) * z[g];
-                ey2[g] = ey * ey;
-                const float ty = fmaf(-k.w, z[g], V[g]);
-                ok &= ey2[g] <= p[g].b2 * fmaf(k.y, zz, ty * ty);
-            }
-            nq[g] = ok;
-            if (COUNT && valid[g]) {
-                cnt[kCntBoundPairs] += o[g] ? 1 : 0;
-                cnt[kCntBoundX] += (NX && o[g]) ? 1 : 0;
-                cnt[kCntBoundY] += (NY && o[g]) ? 1 : 0;
-                cnt[kCntExactPairs] += nq[g] ? 1 : 0;
-                cnt[kCntExactX] += (NX && nq[g] && ex2[g] > 0.f) ? 1 : 0;
-                cnt[kCntExactY] += (NY && nq[g] && ey2[g] > 0.f) ? 1 : 0;
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < GPT; ++g) {
-            bool xt = true, yt = true;
-            if (NX && __any_sync(0xffffffffu, nq[g] & (ex2[g] > 0.f))) {
-                const float4 c0 = c.r0;
-                const float gx = fmaf(-U[g], c2.x, z[g] * c0.x), gy = fmaf(-U[g], c2.y, z[g] * c0.y),
-                            gz = fmaf(-U[g], c2.z, z[g] * c0.z);
-                const float a0 = fmaf(p[g].L[0], gx, fmaf(p[g].L[1], gy, p[g].L[2] * gz));
-                const float a1 = fmaf(p[g].L[3], gx, fmaf(p[g].L[4], gy, p[g].L[5] * gz));
-                const float a2 = fmaf(p[g].L[6], gx, fmaf(p[g].L[7], gy, p[g].L[8] * gz));
-                xt = ex2[g] <= fmaf(a0, a0, fmaf(a1, a1, a2 * a2));
-                if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 1;
-            }
-            if (NY && __any_sync(0xffffffffu, nq[g] & (ey2[g] > 0.f))) {
-                const float4 c1 = c.r1;
-                const float gx = fmaf(-V[g], c2.x, z[g] * c1.x), gy = fmaf(-V[g], c2.y, z[g] * c1.y),
-                            gz = fmaf(-V[g], c2.z, z[g] * c1.z);
-                const float b0 = fmaf(p[g].L[0], gx, fmaf(p[g].L[1], gy, p[g].L[2] * gz));
-                const float b1 = fmaf(p[g].L[3], gx, fmaf(p[g].L[4], gy, p[g].L[5] * gz));
-                const float b2 = fmaf(p[g].L[6], gx, fmaf(p[g].L[7], gy, p[g].L[8] * gz));
-                yt = ey2[g] <= fmaf(b0, b0, fmaf(b1, b1, b2 * b2));
-                if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 1;
-            }
-            vis[g] |= nq[g] & xt & yt;
+            cnt[kCntBoundPairs] += o ? 1 : 0;
+            cnt[kCntBoundX] += (NX && o) ? 1 : 0;
+            cnt[kCntBoundY] += (NY && o) ? 1 : 0;
+            cnt[kCntExactPairs] += nq[g] ? 1 : 0;
+            cnt[kCntExactX] += (NX && nq[g] && du[g] > 0.f) ? 1 : 0;
+            cnt[kCntExactY] += (NY && nq[g] && dv[g] > 0.f) ? 1 : 0;
         }
     }
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
-        part[g] += vis[g] ? weight<PM>(c, z[g], eta, p[g].mx, p[g].my, p[g].mz) : 0.f;
+        bool ok = nq[g];
+        if (NX && __any_sync(0xffffffffu, nq[g] & (du[g] > 0.f))) {
+            const float ex = fmaxf(du[g], 0.f) * z[g];
+            ok &= ex * ex <= extent2(c.r0, c2, U[g], z[g], p[g]);
+            if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 1;
+        }
+        if (NY && __any_sync(0xffffffffu, nq[g] & (dv[g] > 0.f))) {
+            const float ey = fmaxf(dv[g], 0.f) * z[g];
+            ok &= ey * ey <= extent2(c.r1, c2, V[g], z[g], p[g]);
+            if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 1;
+        }
+        vis[g] |= ok;
+    }
+#pragma unroll
+    for (int g = 0; g < GPT; ++g) {
+        part[g] += vis[g] ? weight<PM>(e, z[g], eta, p[g].mx, p[g].my, p[g].mz) : 0.f;
         if (COUNT) cnt[kCntVisMixed] += (valid[g] && vis[g]) ? 1 : 0;
     }
 }
 
 template <int PM, bool DET, bool COUNT, int GPT>
-__device__ __forceinline__ void view_loop(const CamRec *cs, int vcount, float eta, const PairIn (&p)[GPT],
-                                          const bool (&valid)[GPT], const TileBox *tbs,
+__device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, int vcount, float eta, const PairIn (&p)[GPT],
+                                          const bool (&valid)[GPT], WarpSlot *slot,
                                           float (&acc)[GPT], float (&comp)[GPT],
                                           unsigned long long (&cnt)[kCountSlots])
 {
@@ -800,8 +782,12 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, int vcount, float et
         const unsigned vmask = nv == 32 ? 0xffffffffu : ((1u << nv) - 1u);
         unsigned in_m = 0u, out_m = 0u, ux_m = 0u, uy_m = 0u, uz_m = 0u;
         if (!DET) {
-            const TileBox tb = load_box(tbs);
-            const int cls = lane < nv ? classify(cs[vb + lane], tb) : (kAxX | kAxY | kAxZ);
+            const TileBox tb = load_box(&slot->box);
+            float2 reach = make_float2(0.f, 0.f);
+            const int cls = lane < nv ? classify(cs[vb + lane], tb, &reach) : (kAxX | kAxY | kAxZ);
+            __syncwarp();  // every lane is done with the reaches of the views before
+            slot->k[lane] = reach;
+            __syncwarp();
             in_m = __ballot_sync(0xffffffffu, (cls & 3) == kClsIn);
             out_m = __ballot_sync(0xffffffffu, (cls & 3) == kClsOut);
             ux_m = __ballot_sync(0xffffffffu, (cls & kAxX) != 0);
@@ -822,25 +808,27 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, int vcount, float et
                 const int b = __ffs(todo) - 1;
                 todo &= todo - 1u;
                 const CamRec &c = cs[vb + b];
+                const CamExt *ext = PM == kProjFullJ ? ce + vb + b : nullptr;
                 if ((in_m >> b) & 1u) {
                     const float4 c2 = c.r2;
 #pragma unroll
                     for (int g = 0; g < GPT; ++g) {
                         const float z = fmaf(c2.x, p[g].mx, fmaf(c2.y, p[g].my, fmaf(c2.z, p[g].mz, c2.w)));
-                        part[g] += weight<PM>(c, z, eta, p[g].mx, p[g].my, p[g].mz);
+                        part[g] += weight<PM>(ext, z, eta, p[g].mx, p[g].my, p[g].mz);
                     }
                 } else if (DET) {
-                    mixed_view<PM, true, COUNT, GPT>(c, eta, p, valid, part, cnt);
+                    mixed_view_det<PM, COUNT, GPT>(c, ext, eta, p, valid, part, cnt);
                 } else {
                     const unsigned bit = 1u << b;
+                    const float2 &reach = slot->k[b];
                     if (uz_m & bit)
-                        mixed_view_ax<PM, COUNT, GPT, true, true, true>(c, eta, p, valid, part, cnt);
+                        mixed_view<PM, COUNT, GPT, true, true, true>(c, ext, reach, eta, p, valid, part, cnt);
                     else if (ux_m & uy_m & bit)
-                        mixed_view_ax<PM, COUNT, GPT, true, true, false>(c, eta, p, valid, part, cnt);
+                        mixed_view<PM, COUNT, GPT, true, true, false>(c, ext, reach, eta, p, valid, part, cnt);
                     else if (ux_m & bit)
-                        mixed_view_ax<PM, COUNT, GPT, true, false, false>(c, eta, p, valid, part, cnt);
+                        mixed_view<PM, COUNT, GPT, true, false, false>(c, ext, reach, eta, p, valid, part, cnt);
                     else
-                        mixed_view_ax<PM, COUNT, GPT, false, true, false>(c, eta, p, valid, part, cnt);
+                        mixed_view<PM, COUNT, GPT, false, true, false>(c, ext, reach, eta, p, valid, part, cnt);
                 }
             }
             // Kahan-compensated sum of the 32-view partial sums
@@ -855,18 +843,20 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, int vcount, float et
     }
 }
 
+// Smallest and largest value of the warp (one instruction each on sm_103a;
+// a NaN is passed over).
 __device__ __forceinline__ float warp_min(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 __device__ __forceinline__ float warp_max(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 __device__ __forceinline__ void prefetch_l2(const void *p)
@@ -881,11 +871,11 @@ __device__ __forceinline__ void fence_proxy_async_shared()
 
 // Scores one warp tile: the 32 * GPT primitives of the processing order
 // starting at `base`; `next_base` (or -1) is the tile this warp takes next,
-// whose primitives are pulled towards L2 meanwhile.  `tbs` is the warp's
-// shared-memory slot for the tile box.
+// whose primitives are pulled towards L2 meanwhile.  `slot` is the warp's
+// shared-memory slot.
 template <int PM, bool COUNT, int GPT>
-__device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *cs, const SceneConsts &sc,
-                                           int64_t base, int64_t next_base, TileBox *tbs,
+__device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *cs, const CamExt *ce, const SceneConsts &sc,
+                                           int64_t base, int64_t next_base, WarpSlot *slot,
                                            unsigned long long (&cnt)[kCountSlots])
 {
     const int lane = threadIdx.x & 31;
@@ -900,7 +890,7 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
     float acc[GPT], comp[GPT];
     bool valid[GPT];
     bool degen = false;
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY}, b2 = 0.f;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY}, s3 = 0.f;
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
         const int64_t j = base + g * 32 + lane;
@@ -918,7 +908,8 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
                 comp[g] = run.y;
             }
         }
-        p[g].mx = ra.x; p[g].my = ra.y; p[g].mz = ra.z; p[g].b2 = ra.w;
+        p[g].mx = ra.x; p[g].my = ra.y; p[g].mz = ra.z;
+        p[g].s3 = fmaxf(sqrt_approx_ftz(fabsf(ra.w)), 1e-30f);
         p[g].L[0] = rb.x; p[g].L[1] = rb.y; p[g].L[2] = rb.z; p[g].L[3] = rb.w;
         p[g].L[4] = rc.x; p[g].L[5] = rc.y; p[g].L[6] = rc.z; p[g].L[7] = rc.w;
         p[g].L[8] = rd.x;
@@ -927,7 +918,7 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
             lo[0] = fminf(lo[0], p[g].mx); hi[0] = fmaxf(hi[0], p[g].mx);
             lo[1] = fminf(lo[1], p[g].my); hi[1] = fmaxf(hi[1], p[g].my);
             lo[2] = fminf(lo[2], p[g].mz); hi[2] = fmaxf(hi[2], p[g].mz);
-            b2 = fmaxf(b2, p[g].b2);
+            s3 = fmaxf(s3, p[g].s3);
         }
     }
     if (!__any_sync(0xffffffffu, valid[0])) return;  // warp past the end
@@ -935,27 +926,24 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
     {
         const float l0 = warp_min(lo[0]), l1 = warp_min(lo[1]), l2 = warp_min(lo[2]);
         const float h0 = warp_max(hi[0]), h1 = warp_max(hi[1]), h2 = warp_max(hi[2]);
-        const float tb2 = warp_max(b2);
+        const float ts3 = warp_max(s3);
         __syncwarp();  // every lane is done with the previous tile's box
         if (lane == 0) {
             TileBox tb;
-            tb.b2 = tb2;
+            tb.s3 = ts3;
             tb.cx = 0.5f * (l0 + h0); tb.hx = 0.5f * (h0 - l0);
             tb.cy = 0.5f * (l1 + h1); tb.hy = 0.5f * (h1 - l1);
             tb.cz = 0.5f * (l2 + h2); tb.hz = 0.5f * (h2 - l2);
-            tb.mx = fabsf(tb.cx) + tb.hx;
-            tb.my = fabsf(tb.cy) + tb.hy;
-            tb.mz = fabsf(tb.cz) + tb.hz;
-            tb.pad[0] = tb.pad[1] = 0.f;
-            *tbs = tb;
+            tb.l1 = (fabsf(tb.cx) + tb.hx) + (fabsf(tb.cy) + tb.hy) + (fabsf(tb.cz) + tb.hz);
+            slot->box = tb;
         }
         __syncwarp();
     }
 
     if (__any_sync(0xffffffffu, degen))
-        view_loop<PM, true, COUNT, GPT>(cs, a.vcount, a.eta, p, valid, tbs, acc, comp, cnt);
+        view_loop<PM, true, COUNT, GPT>(cs, ce, a.vcount, a.eta, p, valid, slot, acc, comp, cnt);
     else
-        view_loop<PM, false, COUNT, GPT>(cs, a.vcount, a.eta, p, valid, tbs, acc, comp, cnt);
+        view_loop<PM, false, COUNT, GPT>(cs, ce, a.vcount, a.eta, p, valid, slot, acc, comp, cnt);
 
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
@@ -974,14 +962,34 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
     }
 }
 
-// A camera block may be staged by one bulk copy chain only if its source is
-// 16-byte aligned and it fits the launch's dynamic shared memory.
-__device__ __forceinline__ int cams_stageable(const CamRec *cams, int vcount)
+// A camera block may be staged by bulk copies only if its sources are 16-byte
+// aligned and it fits the launch's dynamic shared memory.
+__device__ __forceinline__ int cams_stageable(const ScoreLaunch &a)
 {
     uint32_t dyn;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-    return vcount >= 1 && (reinterpret_cast<uintptr_t>(cams) & 15u) == 0 &&
-           (uint64_t)vcount * sizeof(CamRec) <= (uint64_t)dyn;
+    const bool full_j = proj_mode(a.flags) == kProjFullJ;
+    return a.vcount >= 1 && (reinterpret_cast<uintptr_t>(a.cams) & 15u) == 0 &&
+           (!full_j || (a.ext != nullptr && (reinterpret_cast<uintptr_t>(a.ext) & 15u) == 0)) &&
+           (uint64_t)cams_smem(a.vcount, a.flags) <= (uint64_t)dyn;
+}
+
+__device__ __forceinline__ void bulk_g2s_chunks(unsigned char *dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    for (uint32_t off = 0; off < bytes; off += 16384u) {
+        const uint32_t len = bytes - off < 16384u ? bytes - off : 16384u;
+        bulk_g2s(dst + off, static_cast<const unsigned char *>(src) + off, len, bar);
+    }
+}
+
+// The camera records of a pass, then (FULL_JACOBIAN) their extensions.
+__device__ __forceinline__ void stage_cams(const ScoreLaunch &a, unsigned char *smem, uint64_t *bar)
+{
+    const uint32_t bytes = (uint32_t)a.vcount * (uint32_t)sizeof(CamRec);
+    mbar_expect_tx(bar, (uint32_t)cams_smem(a.vcount, a.flags));
+    bulk_g2s_chunks(smem, a.cams, bytes, bar);
+    if (proj_mode(a.flags) == kProjFullJ)
+        bulk_g2s_chunks(smem + bytes, a.ext, (uint32_t)a.vcount * (uint32_t)sizeof(CamExt), bar);
 }
 
 template <int PM, bool COUNT, int GPT>
@@ -989,21 +997,17 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ TileBox s_box[kScoreThreads / 32];
+    __shared__ WarpSlot s_slot[kScoreThreads / 32];
     CamRec *cs = reinterpret_cast<CamRec *>(smem_raw);
 
     // Stage this pass's cameras once per CTA (TMA bulk copy, mbarrier).
     __shared__ int s_ok;
-    const uint32_t bytes = (uint32_t)a.vcount * (uint32_t)sizeof(CamRec);
+    const CamExt *ce = reinterpret_cast<const CamExt *>(smem_raw + (size_t)a.vcount * sizeof(CamRec));
     if (threadIdx.x == 0) {
-        s_ok = cams_stageable(a.cams, a.vcount) && a.tiles_taken != nullptr;
+        s_ok = cams_stageable(a) && a.tiles_taken != nullptr;
         if (s_ok) {
             mbar_init(&bar, 1);
-            mbar_expect_tx(&bar, bytes);
-            for (uint32_t off = 0; off < bytes; off += 16384u) {
-                const uint32_t len = bytes - off < 16384u ? bytes - off : 16384u;
-                bulk_g2s(smem_raw + off, reinterpret_cast<const unsigned char *>(a.cams) + off, len, &bar);
-            }
+            stage_cams(a, smem_raw, &bar);
         } else {
             set_status(a.status, kEinval);
         }
@@ -1034,8 +1038,8 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
         int nxt = 0;
         if (lane == 0) nxt = (int)min((unsigned long long)ntiles, atomicAdd(a.tiles_taken, 1ull));
         nxt = __shfl_sync(0xffffffffu, nxt, 0);
-        score_tile<PM, COUNT, GPT>(a, cs, sc, (int64_t)cur * (32 * GPT),
-                                   nxt < ntiles ? (int64_t)nxt * (32 * GPT) : -1, &s_box[threadIdx.x >> 5], cnt);
+        score_tile<PM, COUNT, GPT>(a, cs, ce, sc, (int64_t)cur * (32 * GPT),
+                                   nxt < ntiles ? (int64_t)nxt * (32 * GPT) : -1, &s_slot[threadIdx.x >> 5], cnt);
         cur = nxt;
     }
     if (COUNT) {
@@ -1062,7 +1066,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_scene, s_ok, s_wt;
     __shared__ long long s_base;
-    __shared__ TileBox s_box[THREADS / 32];
+    __shared__ WarpSlot s_slot[THREADS / 32];
     CamRec *cs = reinterpret_cast<CamRec *>(smem_raw);
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
@@ -1096,15 +1100,10 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
         const ScoreLaunch &a = b.scenes[sidx];
         if (sidx != cur) {
             if (threadIdx.x == 0) {
-                s_ok = cams_stageable(a.cams, a.vcount);
+                s_ok = cams_stageable(a);
                 if (s_ok) {
                     fence_proxy_async_shared();
-                    const uint32_t bytes = (uint32_t)a.vcount * (uint32_t)sizeof(CamRec);
-                    mbar_expect_tx(&bar, bytes);
-                    for (uint32_t off = 0; off < bytes; off += 16384u) {
-                        const uint32_t len = bytes - off < 16384u ? bytes - off : 16384u;
-                        bulk_g2s(smem_raw + off, reinterpret_cast<const unsigned char *>(a.cams) + off, len, &bar);
-                    }
+                    stage_cams(a, smem_raw, &bar);
                 } else {
                     set_status(a.status, kEinval);
                 }
@@ -1127,6 +1126,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
         }
         const SceneConsts sc = *a.consts;
         const int pm = proj_mode(a.flags);
+        const CamExt *ce = reinterpret_cast<const CamExt *>(smem_raw + (size_t)a.vcount * sizeof(CamRec));
         // the item's warp tiles go to whichever warp of the CTA is free
         const int wtiles = (int)((min(tile, a.n - base) + 32 * GPT - 1) / (32 * GPT));
         for (;;) {
@@ -1136,11 +1136,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
             if (t >= wtiles) break;
             const int64_t wbase = base + (int64_t)t * (32 * GPT);
             if (pm == kProjEq17)
-                score_tile<kProjEq17, false, GPT>(a, cs, sc, wbase, -1, &s_box[threadIdx.x >> 5], cnt);
+                score_tile<kProjEq17, false, GPT>(a, cs, ce, sc, wbase, -1, &s_slot[threadIdx.x >> 5], cnt);
             else if (pm == kProjNone)
-                score_tile<kProjNone, false, GPT>(a, cs, sc, wbase, -1, &s_box[threadIdx.x >> 5], cnt);
+                score_tile<kProjNone, false, GPT>(a, cs, ce, sc, wbase, -1, &s_slot[threadIdx.x >> 5], cnt);
             else
-                score_tile<kProjFullJ, false, GPT>(a, cs, sc, wbase, -1, &s_box[threadIdx.x >> 5], cnt);
+                score_tile<kProjFullJ, false, GPT>(a, cs, ce, sc, wbase, -1, &s_slot[threadIdx.x >> 5], cnt);
         }
         __syncthreads();  // the cameras, s_scene and s_wt are free again
     }
@@ -1204,12 +1204,12 @@ bool shape_valid(const ScoreShape &sh)
            sh.views_per_pass >= 32 && sh.views_per_pass <= kViewsPerPass && sh.views_per_pass % 32 == 0;
 }
 
-int score_grid(int num_sms, int64_t n, int vcount, const ScoreShape &sh)
+int score_grid(int num_sms, int64_t n, int vcount, int flags, const ScoreShape &sh)
 {
     // Persistent grid: as many CTAs as fit per SM, capped by the tile count.
     int per_sm = 0;
-    const size_t smem = (size_t)vcount * sizeof(CamRec);
-    const void *fn = pick_score(kProjEq17, false, sh.gpt);
+    const size_t smem = cams_smem(vcount, flags);
+    const void *fn = pick_score(proj_mode(flags), false, sh.gpt);
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kScoreThreads, smem) != cudaSuccess ||
         per_sm < 1) {
@@ -1227,7 +1227,7 @@ int score_grid(int num_sms, int64_t n, int vcount, const ScoreShape &sh)
 cudaError_t launch_score(const ScoreLaunch &a, const ScoreShape &sh, cudaStream_t s)
 {
     const void *fn = pick_score(proj_mode(a.flags), a.need != nullptr, sh.gpt);
-    const size_t smem = (size_t)a.vcount * sizeof(CamRec);
+    const size_t smem = cams_smem(a.vcount, a.flags);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1246,10 +1246,9 @@ static const void *batch_fn(const ScoreShape &sh)
                        : reinterpret_cast<const void *>(&k_score_batch<2, 256>);
 }
 
-int score_batch_grid(int num_sms, int max_vcount, const ScoreShape &sh)
+int score_batch_grid(int num_sms, size_t smem, const ScoreShape &sh)
 {
     const void *fn = batch_fn(sh);
-    const size_t smem = (size_t)max_vcount * sizeof(CamRec);
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sh.threads, smem) != cudaSuccess || per_sm < 1) {
@@ -1260,10 +1259,9 @@ int score_batch_grid(int num_sms, int max_vcount, const ScoreShape &sh)
     return num_sms * per_sm;
 }
 
-cudaError_t launch_score_batch(const BatchLaunch &b, int max_vcount, int grid, const ScoreShape &sh, cudaStream_t s)
+cudaError_t launch_score_batch(const BatchLaunch &b, size_t smem, int grid, const ScoreShape &sh, cudaStream_t s)
 {
     const void *fn = batch_fn(sh);
-    const size_t smem = (size_t)max_vcount * sizeof(CamRec);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -316,16 +316,16 @@ cudaEvent_t issue_scoring(refine_queue *q, std::vector<QJob *> &round)
     }
     refine_status st = REFINE_OK;
     if (!live.empty()) {
-        int max_v = 0;
+        size_t smem = 0;
         std::vector<int64_t> ns;
         for (size_t i = 0; i < live.size(); ++i) {
             QJob *j = live[i];
             R.h_launch[i] = make_score_launch(&j->scene, j->plan, j->sx, j->params, 0, j->scores, nullptr, false,
                                               j->status);
-            max_v = std::max(max_v, R.h_launch[i].vcount);
+            smem = std::max(smem, cams_smem(R.h_launch[i].vcount, j->params.flags));
             ns.push_back(j->req.n);
         }
-        const int full_grid = score_batch_grid(q->pc.num_sms, max_v, q->shape);
+        const int full_grid = score_batch_grid(q->pc.num_sms, smem, q->shape);
         const int rounds = batch_rounds(q->shape, ns.data(), (int)ns.size(), full_grid);
         const long long tile = batch_tile(q->shape, rounds);
         R.h_tb[0] = 0;
@@ -350,7 +350,7 @@ cudaEvent_t issue_scoring(refine_queue *q, std::vector<QJob *> &round)
             bl.rounds = rounds;
             int grid = full_grid;
             if (grid > bl.total_tiles) grid = (int)bl.total_tiles;
-            e = launch_score_batch(bl, max_v, grid, q->shape, m);
+            e = launch_score_batch(bl, smem, grid, q->shape, m);
             if (e == cudaSuccess) q->launches.fetch_add(1, std::memory_order_relaxed);
         }
         // Further camera blocks of requests with more views than one block:
@@ -360,7 +360,7 @@ cudaEvent_t issue_scoring(refine_queue *q, std::vector<QJob *> &round)
             for (int v0 = j->plan.vpp; v0 < j->plan.V && e == cudaSuccess; v0 += j->plan.vpp) {
                 ScoreLaunch a = make_score_launch(&j->scene, j->plan, j->sx, j->params, v0, j->scores, nullptr, false,
                                                   j->status);
-                a.grid = score_grid(q->pc.num_sms, j->plan.n, a.vcount, q->shape);
+                a.grid = score_grid(q->pc.num_sms, j->plan.n, a.vcount, a.flags, q->shape);
                 a.tiles_taken = j->sx.tiles;
                 e = cudaMemsetAsync(j->sx.tiles, 0, sizeof(unsigned long long), m);
                 if (e == cudaSuccess) e = launch_score(a, q->shape, m);

@@ -369,7 +369,7 @@ struct refine_batch {
         unsigned long long *d_counter = nullptr;
         std::vector<int> jobs;                 // the scenes taking part
         long long total_tiles = 0;
-        int max_v = 0;                         // largest camera block of the level
+        size_t smem = 0;                       // largest camera block of the level, in bytes
         int grid = 1;
         int rounds = kBatchRounds;             // item size (batch_rounds)
     };
@@ -426,7 +426,7 @@ refine_status batch_record(refine_batch *b)
         bl.counter = lv.d_counter;
         bl.status = c->d_status;
         bl.rounds = lv.rounds;
-        e = launch_score_batch(bl, lv.max_v, lv.grid, b->shape, m);
+        e = launch_score_batch(bl, lv.smem, lv.grid, b->shape, m);
         if (e == cudaSuccess) ++launches;
     }
     if (e == cudaSuccess && !st) e = cudaEventRecord(fork2, m);
@@ -471,7 +471,7 @@ cudaError_t set_level_tiles(refine_batch *b, refine_batch::Level &lv, const Scor
 {
     std::vector<int64_t> ns;
     for (int j : lv.jobs) ns.push_back(b->jobs[j].scene.n);
-    const int full_grid = score_batch_grid(b->ctx->num_sms, lv.max_v, sh);
+    const int full_grid = score_batch_grid(b->ctx->num_sms, lv.smem, sh);
     lv.rounds = batch_rounds(sh, ns.data(), (int)ns.size(), full_grid);
     const long long tile = batch_tile(sh, lv.rounds);
     std::vector<long long> tb(lv.jobs.size() + 1, 0);
@@ -577,7 +577,7 @@ refine_status refine_batch_create(refine_ctx *c, const refine_job *jobs, int32_t
             hl.push_back(make_score_launch(&jobs[j].scene, b->plans[j], b->sx[j], p, v0, jobs[j].scores_dev, nullptr,
                                            false, c->d_status));
             lv.jobs.push_back(j);
-            lv.max_v = std::max(lv.max_v, hl.back().vcount);
+            lv.smem = std::max(lv.smem, cams_smem(hl.back().vcount, p.flags));
         }
         e = cudaMemcpy(lv.d_launch, hl.data(), sizeof(ScoreLaunch) * hl.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = set_level_tiles(b, lv, b->shape, nullptr);
@@ -761,7 +761,7 @@ refine_status refine_autotune(refine_ctx *c, const refine_job *jobs, int32_t n_j
                             bl.status = c->d_status;
                             bl.rounds = lv.rounds;
                             e = cudaMemsetAsync(lv.d_counter, 0, sizeof(unsigned long long), m);
-                            if (e == cudaSuccess) e = launch_score_batch(bl, lv.max_v, lv.grid, sh, m);
+                            if (e == cudaSuccess) e = launch_score_batch(bl, lv.smem, lv.grid, sh, m);
                         }
                     }
                     if (e == cudaSuccess) e = cudaEventRecord(e1, m);
