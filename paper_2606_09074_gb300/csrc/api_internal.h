@@ -369,6 +369,9 @@ inline ScoreLaunch make_score_launch(const refine_scene *sc, const ScenePlan &pl
     a.view_sum = view_sum;
     a.need = count ? x.need : nullptr;
     a.tiles_taken = nullptr;
+    a.split_tiles = 0;
+    a.parts = nullptr;
+    a.parts_done = nullptr;
     a.status = status;
     a.grid = 0;
     return a;
@@ -395,20 +398,34 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     refine_status st = check_score_args(c, sc, cams, V, p, scores);
     if (st || sc->n == 0) return st;
     const ScenePlan pl = plan_scene(sc->n, V, p.max_views, c->shape.views_per_pass);
-    if ((st = ensure(c, c->score, scene_bytes(pl)))) return st;
+    // every pass but the last is like the first; the split scratch serves all
+    const bool count = need_dev != nullptr;  // the counting kernel scores whole tiles of the shape
+    const int vfirst = std::min(pl.V, pl.vpp), vlast = pl.V - (pl.passes - 1) * pl.vpp;
+    const ScorePlan sp0 = score_plan(c->num_sms, pl.n, vfirst, p.flags, !count, c->shape);
+    const ScorePlan sp1 = pl.multipass ? score_plan(c->num_sms, pl.n, vlast, p.flags, !count, c->shape) : sp0;
+    const size_t parts = std::max(split_part_floats(sp0, vfirst), split_part_floats(sp1, vlast));
+    const size_t taken = sizeof(unsigned long long) +
+                         sizeof(unsigned) * (size_t)std::max(sp0.split_tiles, sp1.split_tiles);
+    if ((st = ensure(c, c->score, scene_bytes(pl) + carve_size({sizeof(float) * parts, taken})))) return st;
     Carver cv(c->score.p);
     const SceneScratch x = carve_scene(cv, pl);
+    float *part_sums = cv.take<float>(parts);
+    char *counters = cv.take<char>(taken);  // the item counter, then a count per split tile
     if (stats_dev) *stats_dev = x.stats;
     if (need_dev) *need_dev = x.need;
     auto run = [&](int cls, auto &&f) { return launch(c, cls, s, f); };
-    if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, need_dev != nullptr, c->d_status, s))) return st;
+    if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, count, c->d_status, s))) return st;
     for (int v0 = 0; v0 < pl.V; v0 += pl.vpp) {
-        ScoreLaunch a = make_score_launch(sc, pl, x, p, v0, scores, view_sum, need_dev != nullptr, c->d_status);
-        a.grid = score_grid(c->num_sms, pl.n, a.vcount, a.flags, c->shape);
-        a.tiles_taken = x.tiles;
-        const cudaError_t e = cudaMemsetAsync(x.tiles, 0, sizeof(unsigned long long), s);
+        ScoreLaunch a = make_score_launch(sc, pl, x, p, v0, scores, view_sum, count, c->d_status);
+        const ScorePlan &sp = a.last ? sp1 : sp0;
+        a.grid = sp.grid;
+        a.tiles_taken = reinterpret_cast<unsigned long long *>(counters);
+        a.split_tiles = sp.split_tiles;
+        a.parts = part_sums;
+        a.parts_done = reinterpret_cast<unsigned *>(counters + sizeof(unsigned long long));
+        const cudaError_t e = cudaMemsetAsync(counters, 0, taken, s);
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
-        if ((st = launch(c, K_SCORE, s, [&] { return launch_score(a, c->shape, s); }))) return st;
+        if ((st = launch(c, K_SCORE, s, [&] { return launch_score(a, sp.gpt, s); }))) return st;
     }
     return REFINE_OK;
 }

@@ -139,9 +139,23 @@ struct ScoreLaunch {
     unsigned long long *need;   // optional diagnostic counters (kCountSlots), see k_score
     unsigned long long *tiles_taken;  // k_score: warp-tile counter, zero before the launch (required;
                                       // k_score_batch takes its items from BatchLaunch::counter)
+    int split_tiles;            // k_score: tiles taken in items of kSplitViews views (score_plan)
+    float *parts;               //   their block sums, [split_tiles][blocks of the pass][tile]
+    unsigned *parts_done;       //   items finished per split tile, zero before the launch
     int *status;
     int grid;                   // CTAs (persistent)
 };
+
+constexpr int kSplitViews = 64;  // views per item of a split tile, a multiple of 32
+// How k_score runs a pass (score_plan): CTAs, primitives per thread, and the
+// tiles at the end of the launch whose views are split into items.
+struct ScorePlan {
+    int grid = 1, gpt = 2, split_tiles = 0;
+};
+inline size_t split_part_floats(const ScorePlan &pl, int vcount)
+{
+    return (size_t)pl.split_tiles * ((vcount + 31) / 32) * 32 * pl.gpt;
+}
 
 // What the feature pass forms besides the primitive records: the camera
 // records of views 0, vstride, 2 vstride, ... (V of them, spread over its
@@ -169,8 +183,9 @@ cudaError_t launch_cell_scan(unsigned *counts, unsigned *off_local, unsigned *bs
 cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n,
                                 const unsigned *off_local, const unsigned *bsum, uint32_t *perm,
                                 int num_sms, cudaStream_t s);
-cudaError_t launch_score(const ScoreLaunch &a, const ScoreShape &sh, cudaStream_t s);
-int score_grid(int num_sms, int64_t n, int vcount, int flags, const ScoreShape &sh);
+cudaError_t launch_score(const ScoreLaunch &a, int gpt, cudaStream_t s);
+// split: tiles may be split (the caller provides parts and parts_done).
+ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, const ScoreShape &sh);
 
 // FP32 FMA throughput probe (refine_fma_rate): FLOPs of one launch of
 // `iters` steps on `num_sms` SMs, and the launch itself (sink: one float,

@@ -767,18 +767,31 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
     }
 }
 
-template <int PM, bool DET, bool COUNT, int GPT>
-__device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, int vcount, float eta, const PairIn (&p)[GPT],
-                                          const bool (&valid)[GPT], WarpSlot *slot,
-                                          float (&acc)[GPT], float (&comp)[GPT],
+// Kahan-compensated sum of the 32-view block sums.
+__device__ __forceinline__ void kahan_add(float &acc, float &comp, float x)
+{
+    const float y = x - comp;
+    const float t = acc + y;
+    comp = (t - acc) - y;
+    acc = t;
+}
+
+// Views [v0, vend) of the pass (v0 a multiple of 32) for one tile: added to
+// (acc, comp), or with pp their block sums stored at pp.  take_next() runs
+// once, before the last block.
+template <int PM, bool DET, bool COUNT, int GPT, typename F>
+__device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, int v0, int vend, float *pp, float eta,
+                                          const PairIn (&p)[GPT], const bool (&valid)[GPT], WarpSlot *slot,
+                                          float (&acc)[GPT], float (&comp)[GPT], F &&take_next,
                                           unsigned long long (&cnt)[kCountSlots])
 {
     const int lane = threadIdx.x & 31;
     int nvalid = 0;
 #pragma unroll
     for (int g = 0; g < GPT; ++g) nvalid += __popc(__ballot_sync(0xffffffffu, valid[g]));
-    for (int vb = 0; vb < vcount; vb += 32) {
-        const int nv = min(32, vcount - vb);
+    for (int vb = v0; vb < vend; vb += 32) {
+        const int nv = min(32, vend - vb);
+        if (vb + 32 >= vend) take_next();
         const unsigned vmask = nv == 32 ? 0xffffffffu : ((1u << nv) - 1u);
         unsigned in_m = 0u, out_m = 0u, ux_m = 0u, uy_m = 0u, uz_m = 0u;
         if (!DET) {
@@ -831,13 +844,12 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, in
                         mixed_view<PM, COUNT, GPT, false, true, false>(c, ext, reach, eta, p, valid, part, cnt);
                 }
             }
-            // Kahan-compensated sum of the 32-view partial sums
+            if (pp) {  // a part of the tile's views: its block sums are added by the tile's last item
 #pragma unroll
-            for (int g = 0; g < GPT; ++g) {
-                const float y = part[g] - comp[g];
-                const float t = acc[g] + y;
-                comp[g] = (t - acc[g]) - y;
-                acc[g] = t;
+                for (int g = 0; g < GPT; ++g) pp[(vb >> 5) * (32 * GPT) + g * 32 + lane] = part[g];
+            } else {
+#pragma unroll
+                for (int g = 0; g < GPT; ++g) kahan_add(acc[g], comp[g], part[g]);
             }
         }
     }
@@ -870,22 +882,27 @@ __device__ __forceinline__ void fence_proxy_async_shared()
 }
 
 // Scores one warp tile: the 32 * GPT primitives of the processing order
-// starting at `base`; `next_base` (or -1) is the tile this warp takes next,
-// whose primitives are pulled towards L2 meanwhile.  `slot` is the warp's
-// shared-memory slot.
-template <int PM, bool COUNT, int GPT>
+// starting at `base`; `take_next` runs before the last block of views (the
+// warp draws its next item there).  `slot` is the warp's shared-memory slot.
+//
+// With `tp.parts` the item is only the views [tp.v0, tp.vend) of the tile: it
+// stores their 32-view block sums, and whichever of the tile's tp.items items
+// ends last (tp.done counts them, no waiting) adds the block sums of the pass
+// in view order and finishes the tile, so the sum has the same bits as a
+// whole tile's.
+struct TilePart {
+    int v0, vend;
+    float *parts;    // the tile's block sums, [blocks of the pass][32 * GPT], or NULL for a whole tile
+    unsigned *done;  // the tile's count of finished items, zero before the launch
+    int items;
+};
+
+template <int PM, bool COUNT, int GPT, typename F>
 __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *cs, const CamExt *ce, const SceneConsts &sc,
-                                           int64_t base, int64_t next_base, WarpSlot *slot,
+                                           int64_t base, const TilePart &tp, WarpSlot *slot, F &&take_next,
                                            unsigned long long (&cnt)[kCountSlots])
 {
     const int lane = threadIdx.x & 31;
-    if (next_base >= 0) {
-#pragma unroll
-        for (int g = 0; g < GPT; ++g) {
-            const int64_t j = next_base + g * 32 + lane;
-            if (j < a.n) prefetch_l2(a.recs + __ldg(a.perm + j));
-        }
-    }
     PairIn p[GPT];
     float acc[GPT], comp[GPT];
     bool valid[GPT];
@@ -941,9 +958,21 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
     }
 
     if (__any_sync(0xffffffffu, degen))
-        view_loop<PM, true, COUNT, GPT>(cs, ce, a.vcount, a.eta, p, valid, slot, acc, comp, cnt);
+        view_loop<PM, true, COUNT, GPT>(cs, ce, tp.v0, tp.vend, tp.parts, a.eta, p, valid, slot, acc, comp, take_next, cnt);
     else
-        view_loop<PM, false, COUNT, GPT>(cs, ce, a.vcount, a.eta, p, valid, slot, acc, comp, cnt);
+        view_loop<PM, false, COUNT, GPT>(cs, ce, tp.v0, tp.vend, tp.parts, a.eta, p, valid, slot, acc, comp, take_next, cnt);
+
+    if (tp.parts) {
+        __threadfence();
+        __syncwarp();
+        unsigned before = 0;
+        if (lane == 0) before = atomicAdd(tp.done, 1u);
+        if (__shfl_sync(0xffffffffu, before, 0) != (unsigned)(tp.items - 1)) return;
+        __threadfence();
+        for (int b = 0; b < (a.vcount + 31) >> 5; ++b)
+#pragma unroll
+            for (int g = 0; g < GPT; ++g) kahan_add(acc[g], comp[g], __ldcg(tp.parts + b * (32 * GPT) + g * 32 + lane));
+    }
 
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
@@ -1024,22 +1053,47 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
 #pragma unroll
     for (int k = 0; k < kCountSlots; ++k) cnt[k] = 0;
     const SceneConsts sc = *a.consts;
-    // Every warp takes its own tiles of 32 * GPT primitives from a counter,
-    // one ahead (the records of the next are pulled towards L2 while the
-    // current one is scored): warps that draw cheap tiles take more of them,
-    // and no warp waits for the others of its CTA.  Tile indices stay below
-    // 2^31 (n <= INT32_MAX).
+    // Every warp takes its own items from a counter: warps that draw cheap
+    // tiles take more of them, and no warp waits for the others of its CTA.  A
+    // warp draws its next item before the last block of views of the current
+    // one (drawn any earlier, it could hold a whole tile back while the others
+    // run out of work) and pulls that tile's records towards L2.  Tiles of
+    // 32 * GPT primitives are taken from the end of the processing order, where
+    // the large primitives are (the tiles with the most pairs to decide); the
+    // last a.split_tiles tiles taken are split into items of kSplitViews
+    // views.  Item indices stay below 2^31 (n <= INT32_MAX, and only a wave's
+    // worth of tiles is split).
     const int lane = threadIdx.x & 31;
     const int ntiles = (int)((a.n + 32 * GPT - 1) / (32 * GPT));
-    int cur = 0;
-    if (lane == 0) cur = (int)min((unsigned long long)ntiles, atomicAdd(a.tiles_taken, 1ull));
-    cur = __shfl_sync(0xffffffffu, cur, 0);
-    while (cur < ntiles) {
+    const int whole = ntiles - a.split_tiles;
+    const int per = a.split_tiles > 0 ? (a.vcount + kSplitViews - 1) / kSplitViews : 1;
+    const int items = whole + a.split_tiles * per;
+    auto draw = [&]() {
+        int i = 0;
+        if (lane == 0) i = (int)min((unsigned long long)items, atomicAdd(a.tiles_taken, 1ull));
+        return __shfl_sync(0xffffffffu, i, 0);
+    };
+    auto tile_of = [&](int i) { return ntiles - 1 - (i < whole ? i : whole + (i - whole) / per); };
+    for (int cur = draw(); cur < items;) {
+        const int tile = tile_of(cur);
+        TilePart tp = {0, a.vcount, nullptr, nullptr, 1};
+        if (cur >= whole) {  // here tile = ntiles - 1 - whole - (cur - whole) / per, in [0, split_tiles)
+            const int k = (cur - whole) % per, blocks = (a.vcount + 31) >> 5;
+            tp = {k * kSplitViews, min(a.vcount, (k + 1) * kSplitViews),
+                  a.parts + (size_t)tile * blocks * (32 * GPT), a.parts_done + tile, per};
+        }
         int nxt = 0;
-        if (lane == 0) nxt = (int)min((unsigned long long)ntiles, atomicAdd(a.tiles_taken, 1ull));
-        nxt = __shfl_sync(0xffffffffu, nxt, 0);
-        score_tile<PM, COUNT, GPT>(a, cs, ce, sc, (int64_t)cur * (32 * GPT),
-                                   nxt < ntiles ? (int64_t)nxt * (32 * GPT) : -1, &s_slot[threadIdx.x >> 5], cnt);
+        auto take_next = [&]() {
+            nxt = draw();
+            if (nxt >= items || tile_of(nxt) == tile) return;
+#pragma unroll
+            for (int g = 0; g < GPT; ++g) {
+                const int64_t j = (int64_t)tile_of(nxt) * (32 * GPT) + g * 32 + lane;
+                if (j < a.n) prefetch_l2(a.recs + __ldg(a.perm + j));
+            }
+        };
+        score_tile<PM, COUNT, GPT>(a, cs, ce, sc, (int64_t)tile * (32 * GPT), tp, &s_slot[threadIdx.x >> 5], take_next,
+                                   cnt);
         cur = nxt;
     }
     if (COUNT) {
@@ -1135,12 +1189,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
             t = __shfl_sync(0xffffffffu, t, 0);
             if (t >= wtiles) break;
             const int64_t wbase = base + (int64_t)t * (32 * GPT);
+            const TilePart tp = {0, a.vcount, nullptr, nullptr, 1};
             if (pm == kProjEq17)
-                score_tile<kProjEq17, false, GPT>(a, cs, ce, sc, wbase, -1, &s_slot[threadIdx.x >> 5], cnt);
+                score_tile<kProjEq17, false, GPT>(a, cs, ce, sc, wbase, tp, &s_slot[threadIdx.x >> 5], [] {}, cnt);
             else if (pm == kProjNone)
-                score_tile<kProjNone, false, GPT>(a, cs, ce, sc, wbase, -1, &s_slot[threadIdx.x >> 5], cnt);
+                score_tile<kProjNone, false, GPT>(a, cs, ce, sc, wbase, tp, &s_slot[threadIdx.x >> 5], [] {}, cnt);
             else
-                score_tile<kProjFullJ, false, GPT>(a, cs, ce, sc, wbase, -1, &s_slot[threadIdx.x >> 5], cnt);
+                score_tile<kProjFullJ, false, GPT>(a, cs, ce, sc, wbase, tp, &s_slot[threadIdx.x >> 5], [] {}, cnt);
         }
         __syncthreads();  // the cameras, s_scene and s_wt are free again
     }
@@ -1204,29 +1259,55 @@ bool shape_valid(const ScoreShape &sh)
            sh.views_per_pass >= 32 && sh.views_per_pass <= kViewsPerPass && sh.views_per_pass % 32 == 0;
 }
 
-int score_grid(int num_sms, int64_t n, int vcount, int flags, const ScoreShape &sh)
+// Persistent grid: as many CTAs as fit per SM, capped by the items.
+//
+// Split tiles.  A tile's views are one serial chain of a few tens of
+// microseconds, so a launch of whole tiles ends on a ragged last wave, and one
+// with fewer tiles than warp slots leaves the others idle.  The last wave of
+// tiles (all of them, when there are no more) is therefore split into items of
+// kSplitViews = 64 views, which costs a reload of the records per item and 4
+// bytes per primitive and 32 views.  Measured (k_score, whole tiles against
+// the split, each with the late draw of the next item): 1M x 150 (3.2 waves of
+// tiles) 189 -> 156 us, 3.5M x 250 (11 waves) 660 -> 615 us, 150k x 1100 (half
+// a wave) 610 -> 288 us.  Items of 32 views: 160, 625 and 307 us; of 96: 159,
+// 616 and 293 us.  Two waves split instead of one cost 2-5 us, half a wave 0-6.
+// Views of one or two blocks are not split: 77k x 61 takes 28.6 us whole and
+// 32 us in single blocks.
+// When all the blocks of 64-primitive tiles fill less than two waves, tiles of
+// 32 primitives are taken (more instructions per pair but twice the warps).
+ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, const ScoreShape &sh)
 {
-    // Persistent grid: as many CTAs as fit per SM, capped by the tile count.
-    int per_sm = 0;
+    ScorePlan pl;
     const size_t smem = cams_smem(vcount, flags);
-    const void *fn = pick_score(proj_mode(flags), false, sh.gpt);
+    const int64_t blocks = (vcount + 31) / 32;
+    pl.gpt = sh.gpt;
+    int per_sm = 0;
+    const void *fn = pick_score(proj_mode(flags), false, pl.gpt);
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kScoreThreads, smem) != cudaSuccess ||
         per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
     }
-    const int64_t tile = (int64_t)kScoreThreads * sh.gpt;
-    const int64_t tiles = (n + tile - 1) / tile;
+    constexpr int kWarps = kScoreThreads / 32;
+    const int64_t slots = (int64_t)num_sms * per_sm * kWarps;
+    if (split && pl.gpt == 2 && (n + 63) / 64 * blocks < 2 * slots) pl.gpt = 1;
+    const int64_t tiles = (n + 32 * pl.gpt - 1) / (32 * pl.gpt);
+    int64_t items = tiles;
+    if (split && vcount > kSplitViews) {
+        pl.split_tiles = (int)(tiles < slots ? tiles : slots);
+        items += pl.split_tiles * (int64_t)((vcount - 1) / kSplitViews);
+    }
     int64_t g = (int64_t)num_sms * per_sm;
-    if (g > tiles) g = tiles;
+    if (g > (items + kWarps - 1) / kWarps) g = (items + kWarps - 1) / kWarps;
     if (g < 1) g = 1;
-    return (int)g;
+    pl.grid = (int)g;
+    return pl;
 }
 
-cudaError_t launch_score(const ScoreLaunch &a, const ScoreShape &sh, cudaStream_t s)
+cudaError_t launch_score(const ScoreLaunch &a, int gpt, cudaStream_t s)
 {
-    const void *fn = pick_score(proj_mode(a.flags), a.need != nullptr, sh.gpt);
+    const void *fn = pick_score(proj_mode(a.flags), a.need != nullptr, gpt);
     const size_t smem = cams_smem(a.vcount, a.flags);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

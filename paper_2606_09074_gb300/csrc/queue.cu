@@ -360,10 +360,11 @@ cudaEvent_t issue_scoring(refine_queue *q, std::vector<QJob *> &round)
             for (int v0 = j->plan.vpp; v0 < j->plan.V && e == cudaSuccess; v0 += j->plan.vpp) {
                 ScoreLaunch a = make_score_launch(&j->scene, j->plan, j->sx, j->params, v0, j->scores, nullptr, false,
                                                   j->status);
-                a.grid = score_grid(q->pc.num_sms, j->plan.n, a.vcount, a.flags, q->shape);
+                const ScorePlan sp = score_plan(q->pc.num_sms, j->plan.n, a.vcount, a.flags, false, q->shape);
+                a.grid = sp.grid;
                 a.tiles_taken = j->sx.tiles;
                 e = cudaMemsetAsync(j->sx.tiles, 0, sizeof(unsigned long long), m);
-                if (e == cudaSuccess) e = launch_score(a, q->shape, m);
+                if (e == cudaSuccess) e = launch_score(a, sp.gpt, m);
                 if (e == cudaSuccess) q->launches.fetch_add(1, std::memory_order_relaxed);
             }
         }

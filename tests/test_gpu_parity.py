@@ -524,3 +524,26 @@ def test_timing_modes(torch, rb, ctx):
     kt = ctx.kernel_times()
     assert {"features", "score", "select_mask"} <= set(kt) and all(v["ms"] > 0 for v in kt.values())
     assert rb.refine_ctx_set_timing(ctx.handle, 3) == rb.REFINE_EINVAL
+
+
+@pytest.mark.parametrize("n,v,flags", [(63, 65, 0), (64, 96, 0), (65, 129, 0), (3000, 64, 0), (3000, 65, 0), (40_001, 577, 0),
+                                       (40_001, 130, 1 << 4), (320_000, 66, 0)])
+def test_split_tiles_same_bits(torch, rb, ctx, n, v, flags):
+    """Tiles whose views are split into items (the plain call) against whole
+    tiles (the counting call, which splits none): the same bits, for view
+    counts about the item and block sizes, one and two passes, more tiles
+    than one wave, a tile holding an underflowed scale, and repeated calls."""
+    w = synth.random_scene(seed=n + v, n=n, v=v, means="core_shell")
+    w.scene.attr[0, n // 2] = -200.0
+    if flags:
+        w.cams["znear"] = 1.0
+    pos, attr, cams = upload(torch, rb, w.scene, w.cams)
+    p = rb.default_params(flags=rb.FLAG_NORM_ATTR | flags)
+    whole, _ = ctx.score(pos, attr, cams, params=p, stats=True)
+    for _ in range(2):
+        vs = torch.empty(n, dtype=torch.float32, device=pos.device)
+        split = ctx.score(pos, attr, cams, params=p, view_sum=vs)
+        assert torch.equal(split.view(torch.int32), whole.view(torch.int32))
+    if n <= 3000:
+        ref = oracle.score(w.scene.params_f64(), w.cams, oracle_params_from(p, rb))
+        assert_score_parity(split.cpu().numpy(), vs.cpu().numpy(), ref)
