@@ -55,7 +55,7 @@ inline int batch_rounds(const ScoreShape &sh, const int64_t *n, int k, int grid)
 constexpr int kFeatThreads = 256;
 
 // Spatial cells for the processing order of k_score: a 2^b x 2^b x 2^b grid
-// over the scene's mean +- 3 sigma box, numbered in Morton order, with b the
+// over the scene's mean +- 3 sigma box, numbered along a Hilbert curve, with b the
 // largest value in [kMinCellBits, kMaxCellBits] that leaves ~0.5 primitives
 // per cell or more (cell_bits_for).  Fine cells keep the counting sort's
 // atomics spread out: dense scenes put hundreds of centres in one coarse
@@ -70,11 +70,15 @@ inline int cell_bits_for(int64_t n)
     while (b < kMaxCellBits && (int64_t(1) << (3 * (b + 1))) <= n * 2) ++b;
     return b;
 }
-inline int cell_count(int bits) { return 1 << (3 * bits); }
-// Keys of the processing order: the cell, plus cell_count(bits) for the
-// primitives with large scales (ln s_max > SceneConsts::big_ls), which
-// thereby follow all the others.
-inline int order_keys(int bits) { return 2 * cell_count(bits); }
+// Keys of the processing order: the cell, then, for the primitives with large
+// scales (ln s_max > SceneConsts::big_ls), which thereby follow all the others,
+// 2^(3b) plus a cell of a grid half as fine; rounded up to whole blocks of the
+// cell scan.
+inline int order_keys(int bits)
+{
+    const int keys = (1 << (3 * bits)) + (1 << (3 * (bits - 1)));
+    return (keys + kScanCells - 1) / kScanCells * kScanCells;
+}
 constexpr double kSizeSplitSd = 1.28;
 
 // Diagnostic counters of k_score (written only when ScoreLaunch::need is set).
