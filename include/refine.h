@@ -364,7 +364,8 @@ refine_status refine_ctx_set_shape(refine_ctx *ctx, const refine_shape *shape);
  *     slot stream;
  *   - the scorer batches continuously: as soon as the previous batched
  *     launch has ended, ONE persistent launch scores every request whose
- *     preparation has ended (those requests form a round; a request with
+ *     preparation has ended, or whose copy has ended if it is no larger
+ *     than the oldest of them (those requests form a round; a request with
  *     more views than the camera block has its further blocks scored right
  *     after it, in order, on the same stream); selection and compaction
  *     then run on the requests' slot streams and the copies back on one

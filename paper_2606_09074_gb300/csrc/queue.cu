@@ -9,7 +9,7 @@
 //                preparation on the request's slot stream.
 //   scorer       continuous batching: as soon as the previous batched launch
 //                has ended, takes every request whose preparation has ended
-//                and scores them with ONE k_score_batch launch on the score
+//                (or is about to) and scores them with ONE k_score_batch launch on the score
 //                stream (its round); per request on its slot stream again the
 //                selection and the compaction, the copies back on the queue's
 //                one output-copy stream (asynchronous when the host buffers
@@ -246,7 +246,7 @@ refine_status issue_prep(refine_queue *q, QJob *j)
     if (e == cudaSuccess) e = cudaMemsetAsync(j->status, 0, sizeof(int), s);
     if (e != cudaSuccess) return cuda_fail(c, e, "queue: input copy");
     auto run = [q, c](int cls, auto &&f) { return counted_run(q, c, cls, f); };
-    refine_status st = enqueue_prep(c, run, &j->scene, j->cams, j->plan, j->sx, j->params, false, j->status, s);
+    refine_status st = enqueue_prep(c, run, &j->scene, j->cams, j->plan, j->sx, j->params, false, nullptr, 0, j->status, s);
     if (st) return st;
     e = cudaEventRecord(q->prepped[j->slot], s);
     j->prepped = e == cudaSuccess;
@@ -431,18 +431,23 @@ void dispatcher_main(refine_queue *q)
 }
 
 // Continuous batching: each batched launch scores every request whose
-// preparation has ended by the time the previous launch has ended.
+// preparation has ended by the time the previous launch has ended, and every
+// one that is no larger than the oldest and whose copy has ended (its
+// preparation, a few tens of microseconds, is waited for on the score
+// stream: one launch for both costs less than one each).
 void scorer_main(refine_queue *q)
 {
     cudaSetDevice(q->pc.device);
     cudaEvent_t last = nullptr;  // the previous batched launch's completion
     for (;;) {
         QJob *head = nullptr;
+        int64_t head_n = 0;
         {
             std::unique_lock<std::mutex> lk(q->mu);
             q->cv_score.wait(lk, [q] { return !q->prepping.empty() || q->dispatcher_done; });
             if (q->prepping.empty()) break;  // the dispatcher has stopped and nothing is left
             head = q->prepping.front();
+            head_n = head->req.n;
         }
         // outside the lock: the oldest waiting request's preparation, then the
         // previous launch (the requests prepared meanwhile join this one)
@@ -455,7 +460,8 @@ void scorer_main(refine_queue *q)
             for (auto it = q->prepping.begin(); it != q->prepping.end();) {
                 QJob *j = *it;
                 const bool done = j->host_status || !j->prepped ||
-                                  cudaEventQuery(q->prepped[j->slot]) != cudaErrorNotReady;
+                                  cudaEventQuery(q->prepped[j->slot]) != cudaErrorNotReady ||
+                                  (j->req.n <= head_n && cudaEventQuery(q->copied[j->slot]) != cudaErrorNotReady);
                 if (done) {
                     ready.push_back(j);
                     it = q->prepping.erase(it);
