@@ -143,6 +143,7 @@ struct refine_queue {
     std::condition_variable cv_dispatch, cv_score, cv_complete, cv_poll;
     std::deque<QJob *> pending;
     std::deque<QJob *> prepping;  // admitted and issued, waiting for a batched score launch
+    int64_t issuing_n = 0;          // primitives of the request that the dispatcher is issuing, 0 = none
     std::list<QJob *> inflight;
     std::unordered_map<uint64_t, refine_result> results;
     std::unordered_set<uint64_t> live;  // submitted, not yet returned by refine_queue_poll
@@ -414,13 +415,16 @@ void dispatcher_main(refine_queue *q)
                 admitted.push_back(j);
             }
             q->peak = std::max(q->peak, q->used);
+            q->issuing_n = admitted.front()->req.n;
         }
         // copies and preparation of each request, at once, in admission order
-        for (QJob *j : admitted) {
+        for (size_t k = 0; k < admitted.size(); ++k) {
+            QJob *j = admitted[k];
             const double t_issue = now_ms(q->t0);
             j->host_status = issue_prep(q, j);
             std::lock_guard<std::mutex> lk(q->mu);
             q->prepping.push_back(j);
+            q->issuing_n = k + 1 < admitted.size() ? admitted[k + 1]->req.n : 0;
             q->dispatch_ms += now_ms(q->t0) - t_issue;
             q->cv_score.notify_one();
         }
@@ -435,6 +439,8 @@ void dispatcher_main(refine_queue *q)
 // one that is no larger than the oldest and whose copy has ended (its
 // preparation, a few tens of microseconds, is waited for on the score
 // stream: one launch for both costs less than one each).
+constexpr int64_t kJoinFraction = 64;
+
 void scorer_main(refine_queue *q)
 {
     cudaSetDevice(q->pc.device);
@@ -456,7 +462,11 @@ void scorer_main(refine_queue *q)
         cudaGetLastError();
         std::vector<QJob *> ready;
         {
-            std::lock_guard<std::mutex> lk(q->mu);
+            std::unique_lock<std::mutex> lk(q->mu);
+            // a request of a small fraction of the oldest's size that is being
+            // issued right now joins as well, within a short bound
+            q->cv_score.wait_for(lk, std::chrono::microseconds(200),
+                                 [&] { return q->issuing_n == 0 || q->issuing_n > head_n / kJoinFraction; });
             for (auto it = q->prepping.begin(); it != q->prepping.end();) {
                 QJob *j = *it;
                 const bool done = j->host_status || !j->prepped ||
