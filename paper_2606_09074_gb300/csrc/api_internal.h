@@ -22,8 +22,8 @@ using namespace refine;
 namespace refine_api {
 
 enum KClass {
-    K_FEATURES = 0,
-    K_CELLS,
+    K_PREPARE = 0,
+    K_FEATURES,
     K_CELL_SCAN,
     K_CELL_SCATTER,
     K_SCORE,
@@ -37,8 +37,7 @@ enum KClass {
     K_FMA_PROBE,
     K_NCLASS
 };
-const char *const kClassName[K_NCLASS] = {"features",
-                                          "cells",         "cell_scan",    "cell_scatter",
+const char *const kClassName[K_NCLASS] = {"prepare",       "features",      "cell_scan",    "cell_scatter",
                                           "score",         "select_pass",  "select_ties",
                                           "select_mask",   "mask_fill",    "compact_count",
                                           "compact_scatter", "selftest",   "fma_probe"};
@@ -246,10 +245,11 @@ struct SceneScratch {
     PrimRec *recs;
     float2 *partials;  // per feature-pass block, float-float sums
     SceneConsts *consts;
+    OrderGrid *grid;
     SceneStats *stats;
     uint2 *cell;  // (cell, slot within the cell) of every primitive
-    unsigned *counts;  // order_keys(bits) + 64 words; the two after the keys count the finished blocks of
-                       // the cell scan and of the feature pass
+    unsigned *counts;  // order_keys(bits) + 64 words; the one after the keys counts the finished blocks of
+                       // the cell scan
     unsigned *off_local;
     unsigned *bsum;
     uint32_t *perm;
@@ -278,8 +278,9 @@ inline ScenePlan plan_scene(int64_t n, int V, int max_views = 0, int vpp = kView
 inline size_t scene_bytes(const ScenePlan &pl)
 {
     const size_t n = (size_t)pl.n, cells = (size_t)order_keys(pl.bits);
-    return carve_size({sizeof(CamRec) * (size_t)pl.V, sizeof(CamExt) * (size_t)pl.V, sizeof(PrimRec) * n, sizeof(float2) * kFeatSums * 1024,
-                       sizeof(SceneConsts), sizeof(SceneStats), sizeof(uint2) * n,
+    return carve_size({sizeof(CamRec) * (size_t)pl.V, sizeof(CamExt) * (size_t)pl.V, sizeof(PrimRec) * n,
+                       sizeof(float2) * kFeatSums * 1024,
+                       sizeof(SceneConsts), sizeof(OrderGrid), sizeof(SceneStats), sizeof(uint2) * n,
                        sizeof(unsigned) * (cells + 64), sizeof(unsigned) * cells,
                        sizeof(unsigned) * (cells / kScanCells), sizeof(uint32_t) * n,
                        kCountSlots * sizeof(unsigned long long), sizeof(unsigned long long),
@@ -296,6 +297,7 @@ inline SceneScratch carve_scene(Carver &cv, const ScenePlan &pl)
     x.recs = cv.take<PrimRec>(n);
     x.partials = cv.take<float2>(kFeatSums * 1024);
     x.consts = cv.take<SceneConsts>(1);
+    x.grid = cv.take<OrderGrid>(1);
     x.stats = cv.take<SceneStats>(1);
     x.cell = cv.take<uint2>(n);
     x.counts = cv.take<unsigned>(cells + 64);
@@ -308,44 +310,65 @@ inline SceneScratch carve_scene(Carver &cv, const ScenePlan &pl)
     return x;
 }
 
-// Camera records, content features and lambda, processing order.
+// Camera records, content features and lambda, processing order.  `more`:
+// more_bytes (a multiple of 16) that the first kernel clears besides.
 template <typename L>
 inline refine_status enqueue_prep(refine_ctx *c, L &&run, const refine_scene *sc, const refine_camera *cams,
                            const ScenePlan &pl, const SceneScratch &x, const refine_params &p, bool count,
-                           int *status, cudaStream_t s)
+                           void *more, size_t more_bytes, int *status, cudaStream_t s)
 {
     const int64_t n = pl.n;
     const int cells = order_keys(pl.bits);
-    cudaError_t e = cudaMemsetAsync(x.counts, 0, sizeof(unsigned) * (cells + 64), s);
-    if (e == cudaSuccess && count) e = cudaMemsetAsync(x.need, 0, kCountSlots * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
+    if (count) {
+        const cudaError_t e = cudaMemsetAsync(x.need, 0, kCountSlots * sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
+    }
+    PrepLaunch pre;
+    pre.cams = cams;
+    pre.V = pl.V;
+    pre.vstride = pl.vstride;
+    pre.cam_out = x.cams;
+    pre.ext_out = proj_mode(p.flags) == kProjFullJ ? x.ext : nullptr;
+    pre.cell_bits = pl.bits;
+    pre.grid = x.grid;
+    pre.zero = reinterpret_cast<uint4 *>(x.counts);
+    pre.zero4 = (cells + 64) / 4;
+    pre.more = static_cast<uint4 *>(more);
+    pre.more4 = (int64_t)(more_bytes / 16);
+    pre.status = status;
     refine_status st;
-    FeatureTail tail;
-    tail.cams = cams;
-    tail.V = pl.V;
-    tail.vstride = pl.vstride;
-    tail.cam_out = x.cams;
-    tail.ext_out = proj_mode(p.flags) == kProjFullJ ? x.ext : nullptr;
-    tail.p = p;
-    tail.cell_bits = pl.bits;
-    tail.consts = x.consts;
-    tail.stats = x.stats;
-    tail.done = x.counts + cells + 1;  // zeroed with the counts above
-    if ((st = run(K_FEATURES, [&] {
-             return launch_features(sc->pos, sc->attr, sc->dtype, sc->row_stride, n, p.eta, p.luma, x.recs,
-                                    x.partials, status, tail, s);
+    if ((st = run(K_PREPARE, [&] {
+             return launch_prepare(sc->pos, sc->attr, sc->dtype, sc->row_stride, n, pre, c->num_sms, s);
          })))
         return st;
-    if ((st = run(K_CELLS, [&] {
-             return launch_cells(sc->pos, sc->attr, sc->dtype, sc->row_stride, n, pl.bits, x.consts, x.cell,
-                                 x.counts, c->num_sms, s);
-         })))
-        return st;
+    FeatureLaunch f;
+    f.pos = sc->pos;
+    f.attr = sc->attr;
+    f.stride = sc->row_stride;
+    f.n = n;
+    f.eta = p.eta;
+    f.luma = p.luma;
+    f.recs = x.recs;
+    f.partials = x.partials;
+    f.grid = x.grid;
+    f.cell_bits = pl.bits;
+    f.cell = x.cell;
+    f.counts = x.counts;
+    f.status = status;
+    if ((st = run(K_FEATURES, [&] { return launch_features(f, sc->dtype, c->num_sms, s); }))) return st;
     if ((st = run(K_CELL_SCAN,
                   [&] { return launch_cell_scan(x.counts, x.off_local, x.bsum, x.counts + cells, pl.bits, s); })))
         return st;
-    return run(K_CELL_SCATTER,
-               [&] { return launch_cell_scatter(x.cell, n, x.off_local, x.bsum, x.perm, c->num_sms, s); });
+    SceneTail tail;
+    tail.partials = x.partials;
+    tail.nblocks = pl.nb;
+    tail.n = n;
+    tail.p = p;
+    tail.consts = x.consts;
+    tail.stats = x.stats;
+    return run(K_CELL_SCATTER, [&] {
+        return launch_cell_scatter(x.cell, n, x.off_local, x.bsum, x.perm, tail, c->num_sms, s);
+    });
 }
 
 inline ScoreLaunch make_score_launch(const refine_scene *sc, const ScenePlan &pl, const SceneScratch &x,
@@ -404,8 +427,8 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     const ScorePlan sp0 = score_plan(c->num_sms, pl.n, vfirst, p.flags, !count, c->shape);
     const ScorePlan sp1 = pl.multipass ? score_plan(c->num_sms, pl.n, vlast, p.flags, !count, c->shape) : sp0;
     const size_t parts = std::max(split_part_floats(sp0, vfirst), split_part_floats(sp1, vlast));
-    const size_t taken = sizeof(unsigned long long) +
-                         sizeof(unsigned) * (size_t)std::max(sp0.split_tiles, sp1.split_tiles);
+    const size_t counts = (size_t)std::max(sp0.split_tiles, sp1.split_tiles);
+    const size_t taken = (sizeof(unsigned long long) + sizeof(unsigned) * counts + 15) & ~size_t(15);
     if ((st = ensure(c, c->score, scene_bytes(pl) + carve_size({sizeof(float) * parts, taken})))) return st;
     Carver cv(c->score.p);
     const SceneScratch x = carve_scene(cv, pl);
@@ -414,7 +437,7 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     if (stats_dev) *stats_dev = x.stats;
     if (need_dev) *need_dev = x.need;
     auto run = [&](int cls, auto &&f) { return launch(c, cls, s, f); };
-    if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, count, c->d_status, s))) return st;
+    if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, count, counters, taken, c->d_status, s))) return st;
     for (int v0 = 0; v0 < pl.V; v0 += pl.vpp) {
         ScoreLaunch a = make_score_launch(sc, pl, x, p, v0, scores, view_sum, count, c->d_status);
         const ScorePlan &sp = a.last ? sp1 : sp0;
@@ -423,7 +446,7 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
         a.split_tiles = sp.split_tiles;
         a.parts = part_sums;
         a.parts_done = reinterpret_cast<unsigned *>(counters + sizeof(unsigned long long));
-        const cudaError_t e = cudaMemsetAsync(counters, 0, taken, s);
+        const cudaError_t e = v0 > 0 ? cudaMemsetAsync(counters, 0, taken, s) : cudaSuccess;  // first: k_prepare
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
         if ((st = launch(c, K_SCORE, s, [&] { return launch_score(a, sp.gpt, s); }))) return st;
     }

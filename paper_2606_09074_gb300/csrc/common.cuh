@@ -45,14 +45,19 @@ struct __align__(16) CamExt {
 };
 static_assert(sizeof(CamExt) == 48, "camera extension layout");
 
-// Per-scene constants produced by the content-feature pass (Eq. 18-19) and
-// the quantisation of the processing-order grid.
+// Slack of the tile classification's ranges (classify, kernels_score.cu).
+constexpr float kTileSlack = 7.62939453125e-06f;  // 2^-17
+
+// Per-scene constants of Eq. 18-19.
 struct SceneConsts {
     float kappa[3];   // lambda^k / mean(m^k)  (or lambda^k without NORM_ATTR)
+};
+
+// Quantisation of the processing-order grid.
+struct OrderGrid {
     float lo[3];      // grid origin (mean - 3 sigma per axis)
     float qscale[3];  // cells per unit length per axis
     float big_ls;     // ln s_max above which a primitive is ordered with the large ones
-    float pad[2];
 };
 
 // Scene statistics (host-visible copy of refine_scene_stats).
@@ -64,9 +69,8 @@ struct SceneStats {
 };
 
 // Number of float sums the content-feature pass reduces per block:
-// y, y^2, a(1-a), gem ratio, m_gem, m_col, m_opa, mu (3), mu^2 (3), and
-// ln s_max with its square (for the size split of the processing order).
-constexpr int kFeatSums = 15;
+// y, y^2, a(1-a), gem ratio, m_gem, m_col, m_opa.
+constexpr int kFeatSums = 7;
 
 // Float-float numbers: an unevaluated sum hi + lo of two floats, added on
 // the FP32 pipes (the FP64 rate of this part is 1/64 of the FP32 rate).
@@ -92,48 +96,31 @@ __device__ __forceinline__ FF ff_add(FF a, FF b)
 // The value as a double (exact: hi and lo do not overlap).
 __device__ __forceinline__ double ff_to_double(FF a) { return (double)a.hi + (double)a.lo; }
 
-// Per-thread content-feature sums (kFeatSums of them) and a non-finite trap.
-struct FeatSums {
-    float s[kFeatSums];
-    float bad;  // accumulates x * 0, which is NaN iff some x was not finite
-};
-
-// Activation of one primitive (Eq. 1) and its feature terms (the readings R1,
-// R3: y = C0 (l . dc) is the luma minus its constant offset 0.5 sum(l);
-// gem = max(s) / (min(s) + eta); m_gem = product of the two largest scales;
-// m_col = |SH|_2; m_opa = alpha).  Adds to the thirteen sums and returns the
-// primitive's record (layout: PrimRec in internal.h).  *zero_q is set for a
-// zero quaternion (then R = I).
-__device__ __forceinline__ void primitive_record(FeatSums &acc, float mx, float my, float mz, float ls0, float ls1,
-                                                 float ls2, float qw, float qx, float qy, float qz, float logit,
-                                                 float dc0, float dc1, float dc2, float sumsq, float eta, float l0,
-                                                 float l1, float l2, float4 &ra, float4 &rb, float4 &rc, float4 &rd,
-                                                 bool &zero_q)
+// The luma of the SH DC colour minus its constant offset 0.5 sum(l) (reading
+// R3): y = C0 (l . dc).
+__device__ __forceinline__ float luma_term(float l0, float l1, float l2, float dc0, float dc1, float dc2)
 {
     constexpr float kC0 = 0.28209479177387814f;  // 1 / (2 sqrt(pi))
+    return __fmul_rn(kC0, fmaf(l0, dc0, fmaf(l1, dc1, l2 * dc2)));
+}
+
+// Activation of one primitive (Eq. 1) and its feature terms (reading R1):
+// gem = max(s) / (min(s) + eta); m_gem = product of the two largest scales;
+// m_col = |SH|_2; m_opa = alpha.  Returns the primitive's record (layout:
+// PrimRec in internal.h; d = (L8, alpha, m_gem, m_col)), the scale ratio gem,
+// and bad + x * 0 over its inputs, which is NaN iff some input was not finite.
+// *zero_q is set for a zero quaternion (then R = I).
+__device__ __forceinline__ float primitive_record(float bad, float mx, float my, float mz, float ls0, float ls1, float ls2,
+                                                  float qw, float qx, float qy, float qz, float logit, float sumsq, float eta,
+                                                  float4 &ra, float4 &rb, float4 &rc, float4 &rd, float &gem, bool &zero_q)
+{
     const float e0 = expf(ls0), e1 = expf(ls1), e2 = expf(ls2);
     const float alpha = 1.f / (1.f + expf(-logit));
-    const float y = kC0 * fmaf(l0, dc0, fmaf(l1, dc1, l2 * dc2));
     const float smax = fmaxf(e0, fmaxf(e1, e2)), smin = fminf(e0, fminf(e1, e2));
     const float mg = fmaxf(fmaxf(e0 * e1, e0 * e2), e1 * e2);
     const float mc = sqrtf(sumsq);
-    acc.s[0] += y;
-    acc.s[1] = fmaf(y, y, acc.s[1]);
-    acc.s[2] = fmaf(alpha, 1.f - alpha, acc.s[2]);
-    acc.s[3] += smax / (smin + eta);
-    acc.s[4] += mg;
-    acc.s[5] += mc;
-    acc.s[6] += alpha;
-    acc.s[7] += mx;
-    acc.s[8] += my;
-    acc.s[9] += mz;
-    acc.s[10] = fmaf(mx, mx, acc.s[10]);
-    acc.s[11] = fmaf(my, my, acc.s[11]);
-    acc.s[12] = fmaf(mz, mz, acc.s[12]);
-    const float lsmax = fmaxf(ls0, fmaxf(ls1, ls2));
-    acc.s[13] += lsmax;
-    acc.s[14] = fmaf(lsmax, lsmax, acc.s[14]);
-    acc.bad = fmaf(mx + my + mz + ls0 + ls1 + ls2 + qw + qx + qy + qz + logit + sumsq, 0.f, acc.bad);
+    gem = smax / (smin + eta);
+    bad = fmaf(mx + my + mz + ls0 + ls1 + ls2 + qw + qx + qy + qz + logit + sumsq, 0.f, bad);
 
     const float qn2 = fmaf(qw, qw, fmaf(qx, qx, fmaf(qy, qy, qz * qz)));
     if (!(qn2 > 0.f)) {
@@ -154,6 +141,7 @@ __device__ __forceinline__ void primitive_record(FeatSums &acc, float mx, float 
     rc = make_float4(s1 * (1.f - 2.f * (qx * qx + qz * qz)), s1 * (2.f * (qy * qz + qw * qx)),
                      s2 * (2.f * (qx * qz + qw * qy)), s2 * (2.f * (qy * qz - qw * qx)));
     rd = make_float4(s2 * (1.f - 2.f * (qx * qx + qy * qy)), alpha, mg, mc);
+    return bad;
 }
 
 // ------------------------------------------------------ row layouts

@@ -52,7 +52,6 @@ inline int batch_rounds(const ScoreShape &sh, const int64_t *n, int k, int grid)
     }
     return 1;
 }
-constexpr int kFeatThreads = 256;
 
 // Spatial cells for the processing order of k_score: a 2^b x 2^b x 2^b grid
 // over the scene's mean +- 3 sigma box, numbered along a Hilbert curve, with b the
@@ -71,7 +70,7 @@ inline int cell_bits_for(int64_t n)
     return b;
 }
 // Keys of the processing order: the cell, then, for the primitives with large
-// scales (ln s_max > SceneConsts::big_ls), which thereby follow all the others,
+// scales (ln s_max > OrderGrid::big_ls), which thereby follow all the others,
 // 2^(3b) plus a cell of a grid half as fine; rounded up to whole blocks of the
 // cell scan.
 inline int order_keys(int bits)
@@ -79,7 +78,7 @@ inline int order_keys(int bits)
     const int keys = (1 << (3 * bits)) + (1 << (3 * (bits - 1)));
     return (keys + kScanCells - 1) / kScanCells * kScanCells;
 }
-constexpr double kSizeSplitSd = 1.28;
+constexpr float kSizeSplitSd = 1.28f;
 
 // Diagnostic counters of k_score (written only when ScoreLaunch::need is set).
 enum {
@@ -161,32 +160,53 @@ inline size_t split_part_floats(const ScorePlan &pl, int vcount)
     return (size_t)pl.split_tiles * ((vcount + 31) / 32) * 32 * pl.gpt;
 }
 
-// What the feature pass forms besides the primitive records: the camera
-// records of views 0, vstride, 2 vstride, ... (V of them, spread over its
-// blocks) and, in its last block, the scene constants (Eq. 18-19, the
-// processing-order grid and size split).
-struct FeatureTail {
+// First kernel of a scene: the processing-order grid, the camera records of
+// views 0, vstride, 2 vstride, ... (V of them), and two ranges to clear.
+struct PrepLaunch {
     const refine_camera *cams;
     int V, vstride;
     CamRec *cam_out;
     CamExt *ext_out;  // NULL unless FULL_JACOBIAN
-    refine_params p;
     int cell_bits;
-    SceneConsts *consts;
-    SceneStats *stats;
-    unsigned *done;  // count of finished blocks, zero before the launch
+    OrderGrid *grid;
+    uint4 *zero, *more;  // 16-byte words to clear
+    int64_t zero4, more4;
+    int *status;
+};
+cudaError_t launch_prepare(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n, const PrepLaunch &a,
+                           int num_sms, cudaStream_t s);
+
+struct FeatureLaunch {
+    const float *pos;
+    const void *attr;
+    int64_t stride, n;
+    float eta;
+    const float *luma;  // host
+    PrimRec *recs;
+    float2 *partials;   // per block, float-float sums
+    const OrderGrid *grid;
+    int cell_bits;
+    uint2 *cell;        // (key, slot) of every primitive
+    unsigned *counts;   // per key, zero before the launch
+    int *status;
 };
 int feature_blocks(int64_t n);
-cudaError_t launch_features(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n,
-                            float eta, const float luma[3], PrimRec *recs, float2 *partials, int *status,
-                            const FeatureTail &tail, cudaStream_t s);
-cudaError_t launch_cells(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n, int cell_bits,
-                         const SceneConsts *consts, uint2 *cell, unsigned *counts, int num_sms, cudaStream_t s);
+cudaError_t launch_features(const FeatureLaunch &f, int dtype, int num_sms, cudaStream_t s);
+
+// What the cell scatter's first block forms from the feature pass's block sums.
+struct SceneTail {
+    const float2 *partials;
+    int nblocks;
+    int64_t n;
+    refine_params p;
+    SceneConsts *consts;
+    SceneStats *stats;
+};
 cudaError_t launch_cell_scan(unsigned *counts, unsigned *off_local, unsigned *bsum, unsigned *done, int cell_bits,
                              cudaStream_t s);
 cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n,
                                 const unsigned *off_local, const unsigned *bsum, uint32_t *perm,
-                                int num_sms, cudaStream_t s);
+                                const SceneTail &tail, int num_sms, cudaStream_t s);
 cudaError_t launch_score(const ScoreLaunch &a, int gpt, cudaStream_t s);
 // split: tiles may be split (the caller provides parts and parts_done).
 ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, const ScoreShape &sh);

@@ -1,526 +1,9 @@
-// Scoring kernels: camera preparation, the content-feature pass (Eq.
-// (features), Eq. 18-19), the spatial processing order, and the N x V
-// importance kernel (Eq. 7, Eq. 20).
+// The N x V importance kernel (Eq. 7, Eq. 20), plain and batched.
 #include <math.h>
-
-#include <float.h>
 
 #include "internal.h"
 
 namespace refine {
-
-constexpr float kTileSlack = 7.62939453125e-06f;  // 2^-17, see classify
-
-// ---------------------------------------------------------------------
-// Camera preparation: refine_camera -> CamRec (P = K W and p = K t formed
-// in double and rounded once), with validation.
-// ---------------------------------------------------------------------
-__device__ void prep_camera(const refine_camera *__restrict__ cams, int v, int vstride, CamRec *__restrict__ out,
-                            CamExt *__restrict__ ext, int *status)
-{
-    refine_camera c = cams[(int64_t)v * vstride];
-    bool ok = isfinite(c.fx) && isfinite(c.fy) && isfinite(c.cx) && isfinite(c.cy) &&
-              isfinite(c.znear) && isfinite(c.zfar) && c.fx > 0.f && c.fy > 0.f &&
-              c.width >= 1 && c.height >= 1 && c.znear > 0.f && c.zfar > c.znear;
-    for (int k = 0; k < 9; ++k) ok = ok && isfinite(c.R[k]);
-    for (int k = 0; k < 3; ++k) ok = ok && isfinite(c.t[k]);
-    CamRec r;
-    if (!ok) {
-        set_status(status, kEinval);
-        r.r0 = make_float4(0.f, 0.f, 0.f, 0.f);
-        r.r1 = r.r2 = r.k = r.r0;
-        r.lim = make_float4(0.f, 0.f, 1.f, 0.f);  // znear > zfar: never visible
-        out[v] = r;
-        if (ext) ext[v] = CamExt{r.r0, r.r0, r.r0};
-        return;
-    }
-    double fx = c.fx, fy = c.fy, cx = c.cx, cy = c.cy;
-    r.r0 = make_float4((float)(fx * c.R[0] + cx * c.R[6]), (float)(fx * c.R[1] + cx * c.R[7]),
-                       (float)(fx * c.R[2] + cx * c.R[8]), (float)(fx * c.t[0] + cx * c.t[2]));
-    r.r1 = make_float4((float)(fy * c.R[3] + cy * c.R[6]), (float)(fy * c.R[4] + cy * c.R[7]),
-                       (float)(fy * c.R[5] + cy * c.R[8]), (float)(fy * c.t[1] + cy * c.t[2]));
-    r.r2 = make_float4(c.R[6], c.R[7], c.R[8], c.t[2]);
-    const float w = (float)c.width, h = (float)c.height;
-    r.lim = make_float4(w, h, c.znear, c.zfar);
-    // The edge norms Ex, Ey of the footprint bound (classify), rounded up;
-    // the bound needs orthonormal rows of R (to well within the 2^-11 that the
-    // primitives' s3 carries), so other cameras get none (every open pair
-    // runs the exact test).
-    float dot[6];
-    for (int i = 0, k = 0; i < 3; ++i)
-        for (int j = i; j < 3; ++j, ++k) {
-            const float *a = c.R + 3 * i, *b = c.R + 3 * j;
-            dot[k] = fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2])) - (i == j ? 1.f : 0.f);
-        }
-    bool ortho = true;
-    for (int k = 0; k < 6; ++k) ortho = ortho && fabsf(dot[k]) <= 1.220703125e-4f;  // 2^-13
-    const float ex = fmaxf(fabsf(c.cx), fabsf(w - c.cx)), ey = fmaxf(fabsf(c.cy), fabsf(h - c.cy));
-    const float Ex = sqrtf(fmaf(c.fx, c.fx, ex * ex)) * 1.00001f, Ey = sqrtf(fmaf(c.fy, c.fy, ey * ey)) * 1.00001f;
-    // tile slack of the forms U, V, U - w z, V - h z (classify)
-    float ca = 0.f, c0 = 0.f;
-    for (const float4 &q : {r.r0, r.r1}) {
-        ca = fmaxf(ca, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
-        c0 = fmaxf(c0, fabsf(q.w));
-    }
-    const float wh = fmaxf(w, h);
-    ca = fmaxf(ca, wh * fmaxf(fabsf(r.r2.x), fmaxf(fabsf(r.r2.y), fabsf(r.r2.z))));
-    c0 = fmaxf(c0, wh * fabsf(r.r2.w));
-    r.k = make_float4(ortho ? Ex : FLT_MAX, ortho ? Ey : FLT_MAX, 2.f * kTileSlack * ca, 2.f * kTileSlack * c0);
-    out[v] = r;
-    if (ext) {
-        CamExt e;
-        e.tx = make_float4((float)(fx * c.R[0]), (float)(fx * c.R[1]), (float)(fx * c.R[2]), (float)(fx * c.t[0]));
-        e.ty = make_float4((float)(fy * c.R[3]), (float)(fy * c.R[4]), (float)(fy * c.R[5]), (float)(fy * c.t[1]));
-        e.f = make_float4((float)(fx * fx), (float)(fy * fy), 0.f, 0.f);
-        ext[v] = e;
-    }
-}
-
-// Eq. (features) -> Eq. 18 -> Eq. 19 in double, by one block (every thread
-// calls it); also the grid box (mean +- 3 sigma of the means) and the size
-// split of the processing order.
-__device__ void finalize_features(const float2 *partials, int nblocks, int64_t n, const refine_params &p,
-                                  int cell_bits, SceneConsts *consts, SceneStats *stats)
-{
-    // each sum k is reduced by one warp over the block partials in a fixed
-    // order (lane-strided, then a shuffle tree) in float-float, whichever
-    // warp it is, and converted to double once
-    __shared__ double red[kFeatSums][1];
-    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int k = threadIdx.x >> 5; k < kFeatSums; k += nwarps) {
-        FF v = {0.f, 0.f};
-#pragma unroll 4
-        for (int b = lane; b < nblocks; b += 32) {
-            const float2 q = __ldcg(partials + (int64_t)b * kFeatSums + k);
-            v = ff_add(v, FF{q.x, q.y});
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            v = ff_add(v, FF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
-        if (lane == 0) red[k][0] = ff_to_double(v);
-    }
-    __syncthreads();
-    // The scalar tail in double, spread over three threads: thread t forms
-    // lambda~ of attribute t (Eq. 18), then its lambda, kappa (Eq. 19) and
-    // the grid box along axis t, each by the same expression as a one-thread
-    // evaluation would use.
-    __shared__ double lam_t[3];
-    const int t = threadIdx.x;
-    const double N = (double)n;
-    if (t < 3) {
-        double lt;
-        if (t == 0) {
-            lt = log(red[3][0] / N + (double)p.eta) / p.e_ln_gem;
-        } else if (t == 1) {
-            const double ybar = red[0][0] / N;
-            double fc = red[1][0] / N - ybar * ybar;
-            if (fc < 0.0) fc = 0.0;
-            lt = fc / p.e_col;
-            if (stats) stats->F_col = fc;
-        } else {
-            lt = (red[2][0] / N) / p.e_opa;
-        }
-        if (!(lt > 0.0)) lt = 0.0;
-        lam_t[t] = lt;
-    }
-    __syncthreads();
-    if (t >= 3) return;  // no barrier follows
-    const double tot = (lam_t[0] + lam_t[1]) + lam_t[2];
-    const double lambda = ((p.flags & REFINE_FLAG_EQUAL_LAMBDA) || tot == 0.0) ? 1.0 / 3.0 : lam_t[t] / tot;
-    const double mean_m = red[4 + t][0] / N;
-    double kap = lambda;
-    if (p.flags & REFINE_FLAG_NORM_ATTR) kap = mean_m > 0.0 ? lambda / mean_m : 0.0;
-    consts->kappa[t] = (float)kap;
-    const double mean = red[7 + t][0] / N;
-    const double var = red[10 + t][0] / N - mean * mean;
-    const double sd = var > 0.0 ? sqrt(var) : 0.0;
-    consts->lo[t] = (float)(mean - 3.0 * sd);
-    consts->qscale[t] = sd > 0.0 && isfinite(sd) ? (float)((1 << cell_bits) / (6.0 * sd)) : 0.f;
-    if (t < 2) consts->pad[t] = 0.f;
-    if (t == 0) {
-        // The primitives whose ln s_max lies above its scene mean + 1.28 sd
-        // (the largest ~10 % for a normal spread) are ordered after all the
-        // others, so that the tiles of the rest carry small footprint bounds.
-        const double ml = red[13][0] / N, vl = red[14][0] / N - ml * ml;
-        const double big = ml + kSizeSplitSd * (vl > 0.0 ? sqrt(vl) : 0.0);
-        consts->big_ls = isfinite(big) ? (float)big : INFINITY;
-    }
-    if (stats) {
-        stats->lambda_t[t] = lam_t[t];
-        stats->lambda[t] = lambda;
-        stats->mean_m[t] = mean_m;
-        if (t == 0) {
-            stats->F_opa = red[2][0] / N;
-            stats->F_gem = red[3][0] / N;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------
-// Content features.  One primitive per thread: its 59 attribute rows are
-// read with coalesced loads (all in flight at once), its record and its
-// feature terms formed (primitive_record), fifteen sums per thread kept in
-// float and reduced per block in a fixed float-float order.  The camera
-// records (prep_camera, in double) are spread over the blocks, one camera
-// per thread, blocks first, before the primitives.  The block that
-// finishes last (a count of finished blocks, no waiting) then forms the
-// scene constants from all blocks' sums (finalize_features), which saves
-// two small launches per scene.
-// ---------------------------------------------------------------------
-constexpr int kFeatRedLanes = 16;                                 // threads per sum in the block reduction
-constexpr int kFeatRedRow = kFeatThreads + kFeatRedLanes;         // padded row: two sums of a warp hit
-                                                                  // different banks
-static_assert(kFeatSums * kFeatRedLanes <= kFeatThreads, "one reduction thread per (sum, lane)");
-static_assert(kFeatThreads % kFeatRedLanes == 0, "whole columns per reduction lane");
-
-template <int DT>
-__global__ void __launch_bounds__(kFeatThreads, 4) k_features(const float *__restrict__ pos,
-                                                           AttrRows<DT> attr, int64_t S, int64_t n,
-                                                           float eta, float l0, float l1, float l2,
-                                                           PrimRec *__restrict__ recs,
-                                                           float2 *__restrict__ partials, int *status,
-                                                           FeatureTail tail)
-{
-    for (int64_t v = blockIdx.x + (int64_t)gridDim.x * threadIdx.x; v < tail.V;
-         v += (int64_t)gridDim.x * blockDim.x)
-        prep_camera(tail.cams, (int)v, tail.vstride, tail.cam_out, tail.ext_out, status);
-
-    FeatSums acc;
-#pragma unroll
-    for (int k = 0; k < kFeatSums; ++k) acc.s[k] = 0.f;
-    acc.bad = 0.f;
-    bool zero_q = false;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        float sq = 0.f;
-#pragma unroll
-        for (int r = 8; r < 56; ++r) {
-            const float x = attr.ld(r, i);
-            sq = fmaf(x, x, sq);
-        }
-        float4 ra, rb, rc, rd;
-        primitive_record(acc, __ldg(pos + i), __ldg(pos + S + i), __ldg(pos + 2 * S + i), attr.ld(0, i),
-                         attr.ld(1, i), attr.ld(2, i), attr.ld(3, i), attr.ld(4, i), attr.ld(5, i), attr.ld(6, i),
-                         attr.ld(7, i), attr.ld(8, i), attr.ld(9, i), attr.ld(10, i), sq, eta, l0, l1, l2, ra, rb,
-                         rc, rd, zero_q);
-        PrimRec *r = recs + i;
-        r->a = ra; r->b = rb; r->c = rc; r->d = rd;
-    }
-    if (!isfinite(acc.bad)) set_status(status, kEnonfinite);
-    if (zero_q) set_status(status, kEinval);
-
-    // Block sums in float-float: thread (k, j) adds the values of threads
-    // j, j + 16, j + 32, ... of sum k in that order, then the 16 lanes of
-    // sum k meet in a shuffle tree (xor 8, 4, 2, 1).
-    __shared__ float red[kFeatSums * kFeatRedRow];
-#pragma unroll
-    for (int k = 0; k < kFeatSums; ++k) red[k * kFeatRedRow + threadIdx.x] = acc.s[k];
-    __syncthreads();
-    if (threadIdx.x < kFeatSums * kFeatRedLanes) {
-        const int k = threadIdx.x / kFeatRedLanes, j = threadIdx.x % kFeatRedLanes;
-        const float *col = red + k * kFeatRedRow + j;
-        FF v = {col[0], 0.f};
-#pragma unroll
-        for (int t = kFeatRedLanes; t < kFeatThreads; t += kFeatRedLanes) v = ff_add(v, FF{col[t], 0.f});
-        // lanes of other sums in the same warp run the same tree on their own
-        // 16-lane groups (xor below 16 stays within a group); the last warp
-        // may hold reduction threads in its low lanes only
-        constexpr int kRedThreads = kFeatSums * kFeatRedLanes;
-        const unsigned grp = (int)(threadIdx.x | 31u) < kRedThreads ? 0xffffffffu : (1u << (kRedThreads & 31)) - 1u;
-#pragma unroll
-        for (int o = kFeatRedLanes / 2; o > 0; o >>= 1)
-            v = ff_add(v, FF{__shfl_xor_sync(grp, v.hi, o), __shfl_xor_sync(grp, v.lo, o)});
-        if (j == 0) partials[(int64_t)blockIdx.x * kFeatSums + k] = make_float2(v.hi, v.lo);
-    }
-
-    // the last block to finish: scene constants
-    __shared__ bool s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(tail.done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    finalize_features(partials, gridDim.x, n, tail.p, tail.cell_bits, tail.consts, tail.stats);
-}
-
-// A single wave on a 152-SM part (4 CTAs of 256 threads per SM); the grid
-// depends only on n, so the per-block sums, and the scene constants, do too.
-int feature_blocks(int64_t n)
-{
-    int64_t b = (n + (int64_t)kFeatThreads * 8 - 1) / ((int64_t)kFeatThreads * 8);
-    if (b < 1) b = 1;
-    if (b > 608) b = 608;
-    return (int)b;
-}
-
-cudaError_t launch_features(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n,
-                            float eta, const float luma[3], PrimRec *recs, float2 *partials, int *status,
-                            const FeatureTail &tail, cudaStream_t s)
-{
-    const int nb = feature_blocks(n);
-    if (dtype == REFINE_BF16)
-        k_features<REFINE_BF16><<<nb, kFeatThreads, 0, s>>>(pos, AttrRows<REFINE_BF16>(attr, stride), stride, n, eta,
-                                                            luma[0], luma[1], luma[2], recs, partials, status, tail);
-    else if (dtype == REFINE_BF16S)
-        k_features<REFINE_BF16S><<<nb, kFeatThreads, 0, s>>>(pos, AttrRows<REFINE_BF16S>(attr, stride), stride, n,
-                                                             eta, luma[0], luma[1], luma[2], recs, partials, status,
-                                                             tail);
-    else
-        k_features<REFINE_F32><<<nb, kFeatThreads, 0, s>>>(pos, AttrRows<REFINE_F32>(attr, stride), stride, n, eta,
-                                                           luma[0], luma[1], luma[2], recs, partials, status, tail);
-    return cudaGetLastError();
-}
-
-
-// ---------------------------------------------------------------------
-// Processing order.  Primitives are sorted by their cell in a 2^b x 2^b x
-// 2^b grid over the mean +- 3 sigma box of the centres, cells numbered along
-// a Hilbert curve (a counting sort: count, scan, scatter), so that the 32
-// lanes of a warp hold nearby primitives and tend to take the same side of
-// each view's frustum edges.  The primitives with the largest scales (ln
-// s_max above SceneConsts::big_ls) come after all the others, in cells of
-// their own, twice as wide (they are about a tenth), so that a tile's
-// footprint bound (set by its largest s_max) is not set by a few large
-// primitives among small ones.  The order only affects speed: every
-// primitive's score is computed by one thread with the views in a fixed
-// order, whatever its position, so the sort need not be stable (the
-// count atomics order the primitives of a cell arbitrarily).  Each
-// thread keeps kSortU primitives in flight.
-//
-// Hilbert, not Morton order: neighbours along the curve are neighbours in
-// space, so the boxes of 64 consecutive primitives are smaller.  MIXED pairs
-// fall from 22.3 to 19.2 % (3.5M x 250 core-shell), 32.9 to 28.5 % (1M x
-// 150) and 51.3 to 43.7 % (150k x 1100).  Finer grids (2^8, 2^10 per axis) and
-// equal-mass cells gave no better tiles in a simulation.
-// ---------------------------------------------------------------------
-constexpr int kSortU = 4;
-
-// Hilbert curve as a state machine (Hamilton's formulation: a state is the
-// entry corner e and the axis d of a cube; octant o of the cube is its w-th
-// along the curve): two levels per step.
-struct HilbertTable {
-    uint16_t t[24 * 64];  // [state][octant of level 1 << 3 | octant of level 2] -> next state << 6 | w1 << 3 | w2
-};
-
-constexpr HilbertTable make_hilbert_table()
-{
-    HilbertTable r{};
-    int w1[24][8] = {}, nx[24][8] = {};
-    for (int e = 0; e < 8; ++e)
-        for (int d = 0; d < 3; ++d)
-            for (int o = 0; o < 8; ++o) {
-                const int k = (d + 1) % 3, x = o ^ e;
-                const int l = ((x >> k) | (x << (3 - k))) & 7;  // rotate right by d + 1
-                const int w = l ^ (l >> 1) ^ (l >> 2);          // inverse Gray code
-                const int p = w == 0 ? 0 : 2 * ((w - 1) / 2);
-                const int g = p ^ (p >> 1);  // entry corner of the w-th octant
-                int dir = 0;
-                if (w > 0)
-                    for (int i = w % 2 == 0 ? w - 1 : w; i & 1; i >>= 1) ++dir;
-                w1[e * 3 + d][o] = w;
-                nx[e * 3 + d][o] = (e ^ (((g << k) | (g >> (3 - k))) & 7)) * 3 + (d + dir % 3 + 1) % 3;
-            }
-    for (int s = 0; s < 24; ++s)
-        for (int a = 0; a < 8; ++a)
-            for (int b = 0; b < 8; ++b)
-                r.t[s * 64 + a * 8 + b] = (uint16_t)(nx[nx[s][a]][b] << 6 | w1[s][a] << 3 | w1[nx[s][a]][b]);
-    return r;
-}
-
-__device__ const HilbertTable kHilbert = make_hilbert_table();
-
-__device__ __forceinline__ void load_hilbert(uint16_t *smem)
-{
-    for (int k = threadIdx.x; k < 24 * 32; k += blockDim.x)
-        reinterpret_cast<uint32_t *>(smem)[k] = __ldg(reinterpret_cast<const uint32_t *>(kHilbert.t) + k);
-}
-
-// Index of the cell (x, y, z), each below 2^8, along the curve.  Leading zero
-// levels contribute zero digits, so it is below 2^(3b) for coordinates below
-// 2^b (the orientation of the curve then depends on b, which does not matter).
-__device__ __forceinline__ uint32_t hilbert_index(const uint16_t *t, uint32_t x, uint32_t y, uint32_t z)
-{
-    uint32_t h = 0, state = 0;
-#pragma unroll
-    for (int k = 6; k >= 0; k -= 2) {
-        const uint32_t a = (x >> k) & 3u, b = (y >> k) & 3u, c = (z >> k) & 3u;  // two levels
-        const uint32_t o = ((a >> 1) | (b & 2u) | ((c & 2u) << 1)) << 3 | (a & 1u) | ((b & 1u) << 1) | ((c & 1u) << 2);
-        const uint32_t e = t[state * 64 + o];
-        h = h << 6 | (e & 63u);
-        state = e >> 6;
-    }
-    return h;
-}
-
-__device__ __forceinline__ uint32_t quantise(float x, float lo, float qs, float top)
-{
-    return (uint32_t)fminf(fmaxf((x - lo) * qs, 0.f), top);
-}
-
-// Key of a primitive: its cell, the large primitives (ls > big_ls) in cells
-// twice as wide after all the others.
-__device__ __forceinline__ uint32_t order_key(const uint16_t *hilbert, const SceneConsts &c, int cell_bits, float x, float y,
-                                              float z, float ls)
-{
-    const float top = (float)((1 << cell_bits) - 1);
-    const int big = ls > c.big_ls ? 1 : 0;
-    const uint32_t h = hilbert_index(hilbert, quantise(x, c.lo[0], c.qscale[0], top) >> big,
-                                     quantise(y, c.lo[1], c.qscale[1], top) >> big,
-                                     quantise(z, c.lo[2], c.qscale[2], top) >> big);
-    return h + (big ? 1u << (3 * cell_bits) : 0u);
-}
-
-template <int DT>
-__global__ void k_cells(const float *__restrict__ pos, AttrRows<DT> attr, int64_t stride, int64_t n,
-                        int cell_bits, const SceneConsts *__restrict__ consts, uint2 *__restrict__ cell,
-                        unsigned *__restrict__ counts)
-{
-    __shared__ __align__(4) uint16_t hilbert[24 * 64];
-    load_hilbert(hilbert);
-    __syncthreads();
-    const SceneConsts c = *consts;
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kSortU * step) {
-        float x[kSortU], y[kSortU], z[kSortU], ls[kSortU];
-#pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
-            const int64_t j = i + u * step;
-            const bool ok = j < n;
-            x[u] = ok ? __ldg(pos + j) : 0.f;
-            y[u] = ok ? __ldg(pos + stride + j) : 0.f;
-            z[u] = ok ? __ldg(pos + 2 * stride + j) : 0.f;
-            ls[u] = ok ? fmaxf(attr.ld(0, j), fmaxf(attr.ld(1, j), attr.ld(2, j))) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
-            const int64_t j = i + u * step;
-            if (j >= n) break;
-            const uint32_t id = order_key(hilbert, c, cell_bits, x[u], y[u], z[u], ls[u]);
-            cell[j] = make_uint2(id, atomicAdd(&counts[id], 1u));  // the key and the slot in it
-        }
-    }
-}
-
-static int sort_grid(int num_sms, int64_t n)
-{
-    int64_t g = (n + 255) / 256;
-    if (g > (int64_t)num_sms * 8) g = (int64_t)num_sms * 8;
-    if (g < 1) g = 1;
-    return (int)g;
-}
-
-cudaError_t launch_cells(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n, int cell_bits,
-                         const SceneConsts *consts, uint2 *cell, unsigned *counts, int num_sms, cudaStream_t s)
-{
-    const int g = sort_grid(num_sms, n);
-    if (dtype == REFINE_BF16)
-        k_cells<REFINE_BF16><<<g, 256, 0, s>>>(pos, AttrRows<REFINE_BF16>(attr, stride), stride, n, cell_bits, consts,
-                                               cell, counts);
-    else if (dtype == REFINE_BF16S)
-        k_cells<REFINE_BF16S><<<g, 256, 0, s>>>(pos, AttrRows<REFINE_BF16S>(attr, stride), stride, n, cell_bits,
-                                                consts, cell, counts);
-    else
-        k_cells<REFINE_F32><<<g, 256, 0, s>>>(pos, AttrRows<REFINE_F32>(attr, stride), stride, n, cell_bits, consts,
-                                              cell, counts);
-    return cudaGetLastError();
-}
-
-// Exclusive scan of the cell counts: local offsets within blocks of
-// kScanCells cells (4 consecutive cells per thread, one 16-byte load), then
-// the last block turns the block totals into block offsets, so cell c
-// starts at bsum[c / kScanCells] + off_local[c].
-__device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *wsum)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned s = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned x = __shfl_up_sync(0xffffffffu, s, o);
-        if (lane >= o) s += x;
-    }
-    if (lane == 31) wsum[warp] = s;
-    __syncthreads();
-    if (warp == 0) {
-        unsigned w = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned x = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += x;
-        }
-        wsum[lane] = w;
-    }
-    __syncthreads();
-    const unsigned r = s - v + (warp > 0 ? wsum[warp - 1] : 0u);
-    __syncthreads();
-    return r;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_cell_scan(const unsigned *__restrict__ counts,
-                                                            unsigned *__restrict__ off_local,
-                                                            unsigned *bsum, unsigned *done)
-{
-    __shared__ unsigned wsum[32];
-    __shared__ unsigned is_last, carry;
-    const int nblocks = gridDim.x;
-    const int64_t c4 = (int64_t)blockIdx.x * kScanThreads + threadIdx.x;  // 4 cells from 4 * c4
-    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(counts) + c4);
-    const unsigned tot = v.x + v.y + v.z + v.w;
-    const unsigned ex = block_excl_scan(tot, wsum);
-    reinterpret_cast<uint4 *>(off_local)[c4] = make_uint4(ex, ex + v.x, ex + v.x + v.y, ex + v.x + v.y + v.z);
-    if (threadIdx.x == kScanThreads - 1) bsum[blockIdx.x] = ex + tot;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(done, 1u) == gridDim.x - 1);
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    if (threadIdx.x == 0) carry = 0u;
-    __syncthreads();
-    for (int b0 = 0; b0 < nblocks; b0 += kScanThreads) {
-        const int bi = b0 + threadIdx.x;
-        const unsigned b = bi < nblocks ? __ldcg(bsum + bi) : 0u;
-        const unsigned bex = block_excl_scan(b, wsum) + carry;
-        __syncthreads();
-        if (bi < nblocks) bsum[bi] = bex;
-        if (threadIdx.x == kScanThreads - 1) carry = bex + b;
-        __syncthreads();
-    }
-}
-
-cudaError_t launch_cell_scan(unsigned *counts, unsigned *off_local, unsigned *bsum, unsigned *done, int cell_bits,
-                             cudaStream_t s)
-{
-    k_cell_scan<<<order_keys(cell_bits) / kScanCells, kScanThreads, 0, s>>>(counts, off_local, bsum, done);
-    return cudaGetLastError();
-}
-
-// Primitive j goes to the start of its cell (block offset + offset within
-// the block) plus the slot that its count atomic returned in k_cells.
-__global__ void k_cell_scatter(const uint2 *__restrict__ cell, int64_t n, const unsigned *__restrict__ off_local,
-                               const unsigned *__restrict__ boff, uint32_t *__restrict__ perm)
-{
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kSortU * step) {
-        uint2 c[kSortU];
-#pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
-            const int64_t j = i + u * step;
-            c[u] = j < n ? __ldg(cell + j) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
-            const int64_t j = i + u * step;
-            if (j < n) perm[__ldg(boff + c[u].x / kScanCells) + __ldg(off_local + c[u].x) + c[u].y] = (uint32_t)j;
-        }
-    }
-}
-
-cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n, const unsigned *off_local, const unsigned *bsum,
-                                uint32_t *perm, int num_sms, cudaStream_t s)
-{
-    k_cell_scatter<<<sort_grid(num_sms, n), 256, 0, s>>>(cell, n, off_local, bsum, perm);
-    return cudaGetLastError();
-}
 
 // ---------------------------------------------------------------------
 // The N x V importance kernel.

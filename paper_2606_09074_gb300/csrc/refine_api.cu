@@ -412,7 +412,7 @@ refine_status batch_record(refine_batch *b)
         e = cudaStreamWaitEvent(ls, fork, 0);
         for (int j = l; j < S && e == cudaSuccess && !st; j += L)
             st = enqueue_prep(c, counted(ls), &b->jobs[j].scene, b->jobs[j].cams_dev, b->plans[j], b->sx[j],
-                              b->params, false, c->d_status, ls);
+                              b->params, false, nullptr, 0, c->d_status, ls);
         if (e == cudaSuccess && !st) e = cudaEventRecord(b->events[1 + l], ls);
     }
     for (int l = 0; l < L && e == cudaSuccess && !st; ++l) e = cudaStreamWaitEvent(m, b->events[1 + l], 0);
@@ -735,7 +735,7 @@ refine_status refine_autotune(refine_ctx *c, const refine_job *jobs, int32_t n_j
         const int S = (int)b->jobs.size();
         for (int j = 0; j < S && !st; ++j)
             st = enqueue_prep(c, run, &b->jobs[j].scene, b->jobs[j].cams_dev, b->plans[j], b->sx[j], b->params, false,
-                              c->d_status, m);
+                              nullptr, 0, c->d_status, m);
         for (int gpt : {2, 1})
             for (int threads : {256, 128})
                 for (int cap : {0, threads == 256 ? 2 : 4}) {
