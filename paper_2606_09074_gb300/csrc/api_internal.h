@@ -470,18 +470,26 @@ inline refine_status enqueue_select(refine_ctx *c, L &&run, const float *scores,
     Carver cv(scratch);
     SelState *ss = cv.take<SelState>(1);
     unsigned *seg = cv.take<unsigned>((n + kTieSeg - 1) / kTieSeg);
+    refine_status st;
+    if (n <= kSelClusterMax) {
+        if ((st = run(K_SEL_MASK, [&] {
+                 return launch_select_cluster(scores, n, (uint32_t)n_keep, ss, mask, status, s);
+             })))
+            return st;
+        *kstar_dev = &ss->kstar;
+        return REFINE_OK;
+    }
     cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(SelState), s);
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
     const bool vec = aligned16(scores);
     const int grid = select_grid(c->num_sms, n);
-    refine_status st;
     for (int pass = 0; pass < 3; ++pass)
         if ((st = run(K_SEL_PASS, [&] {
                  return launch_select_pass(pass, scores, n, (uint32_t)n_keep, ss, vec, grid, status, s);
              })))
             return st;
     if ((st = run(K_SEL_TIES, [&] { return launch_select_ties(scores, n, ss, seg, grid, s); }))) return st;
-    if ((st = run(K_SEL_MASK, [&] { return launch_select_mask(scores, n, ss, mask, grid, s); }))) return st;
+    if ((st = run(K_SEL_MASK, [&] { return launch_select_mask(scores, n, ss, mask, c->num_sms, s); }))) return st;
     *kstar_dev = &ss->kstar;
     return REFINE_OK;
 }

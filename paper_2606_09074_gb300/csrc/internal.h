@@ -244,13 +244,17 @@ struct SelState {
     unsigned int done;
     unsigned int prefix;
     unsigned int remaining;
-    unsigned int count_gt;
     unsigned int kstar;
-    unsigned int cnt_eq;
     unsigned int need_ties;
-    unsigned int pad;
+    unsigned int pad[3];
     long long idx_cut;
 };
+// Up to this many scores the selection is one cluster launch
+// (launch_select_cluster, which needs nothing cleared and only kstar of the
+// state); above it, the passes below.
+constexpr int64_t kSelClusterMax = 8 * 32 * 1024;
+cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_keep, SelState *st, uint32_t *mask,
+                                  int *status, cudaStream_t s);
 constexpr int kTieSeg = 4096;
 int select_grid(int num_sms, int64_t n);
 cudaError_t launch_select_pass(int pass, const float *scores, int64_t n, uint32_t n_keep,
@@ -258,7 +262,7 @@ cudaError_t launch_select_pass(int pass, const float *scores, int64_t n, uint32_
 cudaError_t launch_select_ties(const float *scores, int64_t n, SelState *st, unsigned *seg_cnt,
                                int grid, cudaStream_t s);
 cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *st, uint32_t *mask,
-                               int grid, cudaStream_t s);
+                               int num_sms, cudaStream_t s);
 cudaError_t launch_mask_fill(uint32_t *mask, int64_t n, cudaStream_t s);
 
 // ------------------------------------------------------------- compact

@@ -1,8 +1,12 @@
 // Ratio pruning (Sec. 3.3): radix select of the n_keep-th largest score with
 // an index tie-break, keep-mask construction, and stable compaction.
+#include <cooperative_groups.h>
+
 #include "internal.h"
 
 namespace refine {
+
+namespace cg = cooperative_groups;
 
 // Radix digits from the most significant end: 11, 11 and 10 bits.
 __host__ __device__ constexpr int pass_shift(int p) { return p == 0 ? 21 : (p == 1 ? 10 : 0); }
@@ -66,8 +70,32 @@ __device__ unsigned long long block_prefix_sum(unsigned long long v, unsigned lo
     return r;
 }
 
+// Adds one count for digit d of the lanes with `match` to the histogram.
+// Shared-memory atomics take equal addresses of a warp one by one, which is
+// cheap for a few, so only the commonest case of many is grouped: the lanes
+// that share the first matching lane's digit (zeros, and the few exponents
+// that most scores have) go in one add.  Every lane of the warp calls it.
+__device__ __forceinline__ void hist_add(unsigned *h, unsigned d, bool match)
+{
+    const unsigned any = __ballot_sync(0xffffffffu, match);
+    if (!any) return;
+    const int lead = __ffs(any) - 1;
+    const unsigned d0 = __shfl_sync(0xffffffffu, d, lead);
+    const unsigned same = __ballot_sync(0xffffffffu, match && d == d0);
+    if ((int)(threadIdx.x & 31) == lead)
+        atomicAdd(&h[d0], (unsigned)__popc(same));
+    else if (match && d != d0)
+        atomicAdd(&h[d], 1u);
+}
+
 // One histogram pass over the keys that match the digits decided so far.
 // The last CTA to finish chooses the digit of the n_keep-th largest key.
+// The scores are in L2 after the score kernel; what counts is loads in flight
+// (kSelU 16-byte loads a thread) and the histogram adds: 53 against 60 us a
+// selection of 3.5M scores, 36 against 40 us of 1M, with one load a thread and
+// every digit grouped by a match of the whole warp.
+constexpr int kSelU = 4;
+
 template <int PASS, bool VEC>
 __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__restrict__ scores, int64_t n,
                                                              uint32_t n_keep, SelState *st, int *status)
@@ -81,17 +109,11 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
     const unsigned int prefix = PASS == 0 ? 0u : st->prefix;
     bool bad = false;
     // Every lane of a warp runs the same iterations (warp-uniform bounds), so
-    // the full-mask match below sees a converged warp; `valid` masks lanes.
+    // the full-mask votes see a converged warp; `valid` masks lanes.
     auto add = [&](float f, bool valid) {
-        bad |= valid && isnan(f);
+        if (PASS == 0) bad |= valid && isnan(f);
         const uint32_t k = score_key(f);
-        const bool match = valid && (PASS == 0 ? true : ((k >> (SHIFT + WIDTH)) == prefix));
-        // after the first pass few keys still match the digits decided so
-        // far: a warp with none skips the grouping
-        if (PASS > 0 && !__any_sync(0xffffffffu, match)) return;
-        const unsigned int d = (k >> SHIFT) & (NB - 1);
-        const unsigned int grp = __match_any_sync(0xffffffffu, match ? d : 0xffffffffu);
-        if (match && (__ffs(grp) - 1) == (int)(threadIdx.x & 31)) atomicAdd(&h[d], __popc(grp));
+        hist_add(h, (k >> SHIFT) & (NB - 1), valid && (PASS == 0 ? true : ((k >> (SHIFT + WIDTH)) == prefix)));
     };
     const int lane = threadIdx.x & 31;
     const int64_t wbase = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
@@ -100,11 +122,19 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
     if (VEC) {
         const int64_t n4 = n / 4;
         const float4 *s4 = reinterpret_cast<const float4 *>(scores);
-        for (int64_t i0 = wbase; i0 < n4; i0 += nthr) {
-            const int64_t i = i0 + lane;
-            const bool valid = i < n4;
-            const float4 q = valid ? __ldg(s4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-            add(q.x, valid); add(q.y, valid); add(q.z, valid); add(q.w, valid);
+        for (int64_t i0 = wbase; i0 < n4; i0 += kSelU * nthr) {
+            float4 q[kSelU];
+#pragma unroll
+            for (int u = 0; u < kSelU; ++u) {
+                const int64_t i = i0 + u * nthr + lane;
+                q[u] = i < n4 ? __ldg(s4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < kSelU; ++u) {
+                if (i0 + u * nthr >= n4) break;  // uniform in the warp
+                const bool valid = i0 + u * nthr + lane < n4;
+                add(q[u].x, valid); add(q[u].y, valid); add(q[u].z, valid); add(q[u].w, valid);
+            }
         }
         done_to = n4 * 4;
     }
@@ -129,7 +159,7 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
     unsigned int cnt[PER], loc = 0;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        cnt[k] = atomicAdd(&st->hist[threadIdx.x * PER + k], 0u);  // coherent read
+        cnt[k] = __ldcg(&st->hist[threadIdx.x * PER + k]);  // from L2, where the atomics were
         loc += cnt[k];
     }
     const unsigned int remaining = PASS == 0 ? n_keep : st->remaining;
@@ -141,12 +171,10 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
             if (above + cnt[k] >= remaining) {
                 const unsigned int digit = threadIdx.x * PER + k;
                 const unsigned int rem = remaining - above;
-                st->count_gt = (PASS == 0 ? 0u : st->count_gt) + above;
                 st->remaining = rem;
                 st->prefix = (prefix << WIDTH) | digit;
                 if (PASS == 2) {
                     st->kstar = (prefix << WIDTH) | digit;
-                    st->cnt_eq = cnt[k];
                     st->need_ties = cnt[k] > rem ? 1u : 0u;
                     st->idx_cut = n;  // refined by k_select_ties when needed
                 }
@@ -273,7 +301,7 @@ cudaError_t launch_select_ties(const float *scores, int64_t n, SelState *st, uns
 
 // Keep mask: a warp builds kMaskWords consecutive 32-element words per
 // step, their loads issued together.
-constexpr int kMaskWords = 4;
+constexpr int kMaskWords = 8;
 
 __global__ void k_select_mask(const float *__restrict__ scores, int64_t n, const SelState *st,
                               uint32_t *__restrict__ mask)
@@ -303,10 +331,188 @@ __global__ void k_select_mask(const float *__restrict__ scores, int64_t n, const
 }
 
 cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *st, uint32_t *mask,
-                               int grid, cudaStream_t s)
+                               int num_sms, cudaStream_t s)
 {
-    k_select_mask<<<grid, 256, 0, s>>>(scores, n, st, mask);
+    // one step of every warp, up to 8 CTAs of 8 warps per SM
+    int64_t g = ((n + 31) / 32 + 8 * kMaskWords - 1) / (8 * kMaskWords);
+    if (g > (int64_t)num_sms * 8) g = (int64_t)num_sms * 8;
+    if (g < 1) g = 1;
+    k_select_mask<<<(int)g, 256, 0, s>>>(scores, n, st, mask);
     return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------
+// The whole selection in one launch of one thread-block cluster, for up to
+// kSelClusterMax scores: CTA r holds the keys of its range in shared memory,
+// so the scores are read once.  Three digits as above: each CTA counts its
+// keys, the cluster meets at its (hardware) barrier, and every CTA adds all
+// histograms through distributed shared memory and picks the same digit.
+// Among keys equal to k* the first in index order are kept: the CTAs exchange
+// their counts of them and each cuts its own range.  Then each writes the mask
+// words of its range.
+//
+// What it saves is launches: six stream operations become one.  The cluster
+// has 1, 2, 4 or 8 CTAs, about 12k keys each before the next size is taken.
+// Per selection, against the five kernels and a memset of the other form (a
+// chain of latencies, 33 us whatever the size): 1k scores 7.3, 10k 12.4, 50k
+// 16.5, 100k 20.6, 200k 27.6, 300k 34.9, 393k 41.1 us, hence the limit.
+// ---------------------------------------------------------------------
+constexpr int kClThreads = 1024;
+constexpr int kClKeys = 32 * 1024;  // keys of a CTA at most (128 KB)
+constexpr int kClMaxCtas = 8;
+constexpr int kClLoads = 6;         // loads in flight per thread
+static_assert(kSelClusterMax == (int64_t)kClKeys * kClMaxCtas, "cluster selection limit");
+
+__global__ void __launch_bounds__(kClThreads) k_select_cluster(const float *__restrict__ scores, int n, int per,
+                                                               uint32_t n_keep, SelState *st, uint32_t *__restrict__ mask,
+                                                               int *status)
+{
+    extern __shared__ uint32_t keys[];
+    __shared__ unsigned hist[3][2048];
+    __shared__ unsigned wsum[kClThreads / 32];
+    __shared__ unsigned pick[3], equal;
+    cg::cluster_group cl = cg::this_cluster();
+    const int ctas = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i0 = rank * per, m = max(0, min(per, n - i0));  // per is a multiple of 32
+    for (int b = threadIdx.x; b < 3 * 2048; b += kClThreads) (&hist[0][0])[b] = 0u;
+    __syncthreads();
+    bool bad = false;
+    for (int j0 = warp * 32; j0 < m; j0 += kClLoads * kClThreads) {
+        float f[kClLoads];
+#pragma unroll
+        for (int u = 0; u < kClLoads; ++u) {
+            const int j = j0 + u * kClThreads + lane;
+            f[u] = j < m ? __ldg(scores + i0 + j) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kClLoads; ++u) {
+            const int j = j0 + u * kClThreads + lane;
+            if (j - lane >= m) break;  // uniform in the warp
+            bad |= isnan(f[u]);
+            const uint32_t k = score_key(f[u]);
+            if (j < m) keys[j] = k;
+            hist_add(hist[0], k >> pass_shift(0), j < m);
+        }
+    }
+    if (bad) set_status(status, kEnonfinite);
+    unsigned prefix = 0u, remaining = n_keep, count = 0u;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        if (p > 0) {
+            __syncthreads();
+            for (int j0 = warp * 32; j0 < m; j0 += kClThreads) {
+                const int j = j0 + lane;
+                const uint32_t k = j < m ? keys[j] : 0u;
+                hist_add(hist[p], (k >> pass_shift(p)) & ((1u << pass_width(p)) - 1u),
+                         j < m && (k >> (pass_shift(p) + pass_width(p))) == prefix);
+            }
+        }
+        cl.sync();
+        // thread t owns bins 2t and 2t + 1; suffix sums over the block
+        uint2 c = make_uint2(0u, 0u);
+        for (int r = 0; r < ctas; ++r) {
+            const uint2 q = *reinterpret_cast<const uint2 *>(cl.map_shared_rank(&hist[p][2 * threadIdx.x], r));
+            c.x += q.x;
+            c.y += q.y;
+        }
+        unsigned s = c.x + c.y;
+        const unsigned own = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned x = __shfl_down_sync(0xffffffffu, s, o);
+            if (lane + o < 32) s += x;
+        }
+        if (lane == 0) wsum[warp] = s;
+        __syncthreads();
+        unsigned w = lane > warp ? wsum[lane] : 0u;  // the warps above
+        w = __reduce_add_sync(0xffffffffu, w);
+        const unsigned excl = s - own + w;  // keys in bins above mine
+        if (excl < remaining && remaining <= excl + own) {
+            const bool hi = excl + c.y >= remaining;
+            const unsigned above = hi ? excl : excl + c.y;
+            pick[0] = 2u * threadIdx.x + (hi ? 1u : 0u);
+            pick[1] = remaining - above;
+            pick[2] = hi ? c.y : c.x;
+        }
+        __syncthreads();
+        prefix = (prefix << pass_width(p)) | pick[0];
+        remaining = pick[1];
+        count = pick[2];
+        __syncthreads();
+    }
+    const uint32_t kstar = prefix;
+    int cut = m;  // keys equal to k* are kept below this position of the range
+    if (count > remaining) {  // the same in every CTA
+        // each thread counts a run of positions of the range
+        const int run = (m + kClThreads - 1) / kClThreads;
+        const int a = min(m, (int)threadIdx.x * run), b = min(m, a + run);
+        unsigned e = 0u;
+        for (int j = a; j < b; ++j) e += keys[j] == kstar;
+        unsigned s = e;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned x = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += x;
+        }
+        if (lane == 31) wsum[warp] = s;
+        __syncthreads();
+        const unsigned below = __reduce_add_sync(0xffffffffu, lane < warp ? wsum[lane] : 0u);
+        const unsigned before_me = below + s - e;
+        if (threadIdx.x == kClThreads - 1) equal = below + s;
+        if (threadIdx.x == 0) pick[0] = (unsigned)m;
+        cl.sync();
+        unsigned before = 0u;
+        for (int r = 0; r < rank; ++r) before += *cl.map_shared_rank(&equal, r);
+        // position after the last kept one of this range (m when all are kept)
+        const unsigned left = remaining > before ? remaining - before : 0u;
+        if (left == 0u) {
+            if (threadIdx.x == 0) pick[0] = 0u;
+        } else if (before_me < left && left <= before_me + e) {
+            unsigned seen = before_me;
+            for (int j = a; j < b; ++j)
+                if (keys[j] == kstar && ++seen == left) {
+                    pick[0] = (unsigned)(j + 1);
+                    break;
+                }
+        }
+        __syncthreads();
+        cut = (int)pick[0];
+    }
+    for (int j0 = warp * 32; j0 < m; j0 += kClThreads) {
+        const int j = j0 + lane;
+        const uint32_t k = j < m ? keys[j] : 0u;
+        const uint32_t word = __ballot_sync(0xffffffffu, j < m && (k > kstar || (k == kstar && j < cut)));
+        if (lane == 0) mask[(i0 + j0) >> 5] = word;
+    }
+    if (rank == 0 && threadIdx.x == 0) st->kstar = kstar;
+    cl.sync();  // no CTA leaves while another may read its shared memory
+}
+
+cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_keep, SelState *st, uint32_t *mask,
+                                  int *status, cudaStream_t s)
+{
+    int ctas = 1;
+    while (ctas < kClMaxCtas && n > (int64_t)12 * 1024 * ctas) ctas *= 2;
+    const int per = (int)(((n + ctas - 1) / ctas + 31) / 32 * 32);
+    const size_t smem = sizeof(uint32_t) * (size_t)per;
+    if (smem + 3 * 2048 * sizeof(unsigned) + 1024 > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_select_cluster),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_select_cluster, scores, (int)n, per, n_keep, st, mask, status);
 }
 
 __global__ void k_mask_fill(uint32_t *mask, int64_t n)

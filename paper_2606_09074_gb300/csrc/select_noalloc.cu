@@ -103,12 +103,15 @@ extern "C" refine_status refine_select_noalloc(const float *scores_dev, int64_t 
     // The previous call's state is still in the array: clear what the
     // kernels expect to start at zero (selection state and status word).
     e = cudaMemsetAsync(scr, 0, offsetof(NoallocScratch, seg), s);
+    const bool one = n <= kSelClusterMax;
+    if (one && e == cudaSuccess)
+        e = launch_select_cluster(scores_dev, n, (uint32_t)n_keep, &scr->state, keep_mask_dev, &scr->status, s);
     const bool vec = (reinterpret_cast<uintptr_t>(scores_dev) & 15u) == 0;
     const int grid = select_grid(num_sms, n);
-    for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass)
+    for (int pass = 0; pass < 3 && !one && e == cudaSuccess; ++pass)
         e = launch_select_pass(pass, scores_dev, n, (uint32_t)n_keep, &scr->state, vec, grid, &scr->status, s);
-    if (e == cudaSuccess) e = launch_select_ties(scores_dev, n, &scr->state, scr->seg, grid, s);
-    if (e == cudaSuccess) e = launch_select_mask(scores_dev, n, &scr->state, keep_mask_dev, grid, s);
+    if (!one && e == cudaSuccess) e = launch_select_ties(scores_dev, n, &scr->state, scr->seg, grid, s);
+    if (!one && e == cudaSuccess) e = launch_select_mask(scores_dev, n, &scr->state, keep_mask_dev, num_sms, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         put_err(errbuf, errlen, cudaGetErrorString(e));

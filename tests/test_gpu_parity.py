@@ -547,3 +547,39 @@ def test_split_tiles_same_bits(torch, rb, ctx, n, v, flags):
     if n <= 3000:
         ref = oracle.score(w.scene.params_f64(), w.cams, oracle_params_from(p, rb))
         assert_score_parity(split.cpu().numpy(), vs.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 12_288, 12_289, 24_577, 49_152, 49_153, 98_305, 262_144, 262_145])
+def test_select_cluster_edges(torch, rb, ctx, n):
+    """Sizes about the cluster selection's CTA counts, range ends and limit,
+    with ties that span CTAs, all scores equal, and an unaligned score
+    pointer: bit-exact against the oracle."""
+    rng = np.random.default_rng(n)
+    for s in (rng.random(n), rng.integers(0, 3, n) / 4.0, np.full(n, -2.5), np.sort(rng.random(n))[::-1]):
+        s = np.ascontiguousarray(s, dtype=np.float32)
+        for ratio in (0.1, 0.5, 0.9999):
+            check_select_exact(torch, ctx, s, ratio)
+    t = torch.from_numpy(np.concatenate([[9.0], s]).astype(np.float32)).cuda()[1:]
+    mask, thr, nk = ctx.select(t, 0.66)
+    m_ref, thr_ref, nk_ref = oracle.select(s.astype(np.float64), 0.66)
+    assert nk == nk_ref and thr == np.float32(thr_ref)
+    assert np.array_equal(mask.cpu().numpy().view(np.uint32)[: (n + 31) // 32], m_ref)
+
+
+@pytest.mark.parametrize("n", [255, 256, 257, 1_048_575, 1_048_577, 4_194_304, 4_194_305])
+def test_compact_count_sizes(torch, rb, ctx, n):
+    """Kept counts and offsets about the segment and step limits of the counting
+    kernel, checked through the indices (the attribute rows are zeros)."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    keep = torch.rand(n, generator=g, device="cuda") < 0.03
+    words = (n + 31) // 32
+    bits = torch.zeros(words * 32, dtype=torch.int64, device="cuda")
+    bits[:n] = keep
+    w = (bits.view(words, 32) << torch.arange(32, device="cuda")).sum(1)
+    mask = w.to(torch.int32) if n % 2 else torch.cat([w[:1], w]).to(torch.int32)[1:]  # both alignments
+    pos = torch.arange(n, device="cuda", dtype=torch.float32).repeat(3, 1)
+    attr = torch.zeros((56, n), device="cuda", dtype=torch.bfloat16)
+    want = torch.nonzero(keep).flatten().to(torch.int32)
+    op, oa, idx, cnt = ctx.compact(pos, attr, mask, want.numel(), return_count=True)
+    assert cnt == want.numel() and torch.equal(idx, want) and torch.equal(op[2], pos[2][want.long()])
+    ctx.check()
