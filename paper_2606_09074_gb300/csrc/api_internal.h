@@ -542,19 +542,25 @@ inline refine_status enqueue_compact(refine_ctx *c, L &&run, const refine_scene 
     CmpState *cs = cv.take<CmpState>(1);
     unsigned *seg_cnt = cv.take<unsigned>(nseg);
     unsigned long long *seg_off = cv.take<unsigned long long>(nseg);
-    cudaError_t e = cudaMemsetAsync(cs, 0, sizeof(CmpState), s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
-    int64_t cgrid = (nseg + 1023) / 1024;
-    if (cgrid > c->num_sms) cgrid = c->num_sms;
-    if (cgrid < 1) cgrid = 1;
     refine_status st;
-    if ((st = run(K_CMP_COUNT, [&] {
-             return launch_compact_count(mask, n, seg_cnt, seg_off, cs, out_stride, (int)cgrid, status, s);
-         })))
-        return st;
-    const CmpShape sshape = compact_shape(c->num_sms, n, in->dtype);
+    CmpOffsets off{0, nullptr, nullptr, seg_off, cs};
+    if (cmp_blocks(n) <= kCmpMaxBlocks) {
+        // the offsets within blocks in place of the counts, the blocks' totals in place of the offsets
+        unsigned *totals = reinterpret_cast<unsigned *>(seg_off);
+        off = CmpOffsets{cmp_blocks(n), seg_cnt, totals, nullptr, cs};
+        if ((st = run(K_CMP_COUNT, [&] { return launch_compact_local(mask, n, seg_cnt, totals, s); }))) return st;
+    } else {
+        const cudaError_t e = cudaMemsetAsync(cs, 0, sizeof(CmpState), s);
+        if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
+        int64_t cgrid = (nseg + 1023) / 1024;
+        if (cgrid > c->num_sms) cgrid = c->num_sms;
+        if ((st = run(K_CMP_COUNT, [&] {
+                 return launch_compact_count(mask, n, seg_cnt, seg_off, cs, out_stride, (int)cgrid, status, s);
+             })))
+            return st;
+    }
     if ((st = run(K_CMP_SCATTER, [&] {
-             return launch_compact_scatter(*in, mask, seg_off, cs, out_pos, out_attr, out_stride, idx, sshape, s);
+             return launch_compact_scatter(*in, mask, off, out_pos, out_attr, out_stride, idx, c->num_sms, status, s);
          })))
         return st;
     *total_dev = &cs->total;

@@ -271,17 +271,24 @@ struct CmpState {
     unsigned int ok;
     long long total;
 };
-constexpr int kCmpSeg = 256;  // elements per compaction segment (8 mask words)
+constexpr int kCmpSeg = 256;        // elements per compaction segment (8 mask words)
+constexpr int kCmpBlockSegs = 256;  // segments per block of launch_compact_local (65,536 elements)
+constexpr int kCmpMaxBlocks = 256;  // its blocks at most (16.8M elements)
+inline int cmp_blocks(int64_t n) { return (int)((n + (int64_t)kCmpSeg * kCmpBlockSegs - 1) / (kCmpSeg * kCmpBlockSegs)); }
+// Where the segments' kept elements go: offsets within blocks and the blocks'
+// totals (blocks > 0), or offsets in the whole output.
+struct CmpOffsets {
+    int blocks;
+    const unsigned *local, *totals;
+    const unsigned long long *global;
+    CmpState *state;
+};
+cudaError_t launch_compact_local(const uint32_t *mask, int64_t n, unsigned *local, unsigned *totals, cudaStream_t s);
 cudaError_t launch_compact_count(const uint32_t *mask, int64_t n, unsigned *seg_cnt,
                                  unsigned long long *seg_off, CmpState *cs, int64_t out_stride,
                                  int grid, int *status, cudaStream_t s);
-struct CmpShape {
-    int grid;  // CTAs of the scatter
-    bool seg;  // k_compact_seg (a warp per segment) rather than k_compact_warp (a warp per mask word)
-};
-CmpShape compact_shape(int num_sms, int64_t n, int dtype);
-cudaError_t launch_compact_scatter(const refine_scene &in, const uint32_t *mask, const unsigned long long *seg_off,
-                                   const CmpState *cs, float *out_pos, void *out_attr, int64_t out_stride,
-                                   int32_t *out_idx, CmpShape shape, cudaStream_t s);
+cudaError_t launch_compact_scatter(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
+                                   void *out_attr, int64_t out_stride, int32_t *out_idx, int num_sms, int *status,
+                                   cudaStream_t s);
 
 }  // namespace refine

@@ -426,11 +426,6 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-__device__ __forceinline__ void fence_proxy_async_shared()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 // Scores one warp tile: the 32 * GPT primitives of the processing order
 // starting at `base`; `take_next` runs before the last block of views (the
 // warp draws its next item there).  `slot` is the warp's shared-memory slot.

@@ -537,10 +537,63 @@ cudaError_t launch_mask_fill(uint32_t *mask, int64_t n, cudaStream_t s)
 
 // ---------------------------------------------------------------------
 // Compaction, pass 1.  Segment s covers elements [s*kCmpSeg, (s+1)*kCmpSeg)
-// (8 mask words).  Kept elements are counted per segment and the last CTA
-// turns the counts into exclusive offsets; the scatter of every row is
-// k_compact_warp or k_compact_seg.
+// (8 mask words).
+//
+// Up to kCmpMaxBlocks blocks of kCmpBlockSegs segments (k_compact_local): a
+// block counts its segments and leaves their offsets within it and its total;
+// every CTA of the scatter adds up the totals.  No CTA waits for the others
+// and nothing needs clearing: 6 against 18 us (3.5M) and 10 us (1M).
+// Larger scenes (k_compact_count): the last CTA turns all the counts into
+// offsets.
 // ---------------------------------------------------------------------
+__global__ void __launch_bounds__(kCmpBlockSegs) k_compact_local(const uint32_t *__restrict__ mask, int64_t n,
+                                                                 unsigned *__restrict__ local,
+                                                                 unsigned *__restrict__ totals)
+{
+    constexpr int kWords = kCmpSeg / 32;
+    static_assert(kWords == 8, "a segment is two 16-byte loads");
+    __shared__ unsigned wsum[kCmpBlockSegs / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t sg = (int64_t)blockIdx.x * kCmpBlockSegs + threadIdx.x, nseg = (n + kCmpSeg - 1) / kCmpSeg;
+    const int64_t words = (n + 31) / 32;
+    unsigned c = 0u;
+    if ((sg + 1) * kCmpSeg <= n && (reinterpret_cast<uintptr_t>(mask) & 15u) == 0) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(mask) + 2 * sg);
+        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(mask) + 2 * sg + 1);
+        c = __popc(a.x) + __popc(a.y) + __popc(a.z) + __popc(a.w) + __popc(b.x) + __popc(b.y) + __popc(b.z) + __popc(b.w);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kWords; ++k) {
+            const int64_t w = sg * kWords + k;
+            if (w < words) {
+                uint32_t word = __ldg(mask + w);
+                const int64_t valid = n - w * 32;  // bits past n do not count
+                if (valid < 32) word &= (1u << valid) - 1u;
+                c += __popc(word);
+            }
+        }
+    }
+    unsigned s = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned x = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += x;
+    }
+    if (lane == 31) wsum[warp] = s;
+    __syncthreads();
+    unsigned below = 0u;
+#pragma unroll
+    for (int w = 0; w < kCmpBlockSegs / 32; ++w) below += w < warp ? wsum[w] : 0u;
+    if (sg < nseg) local[sg] = below + s - c;
+    if (threadIdx.x == kCmpBlockSegs - 1) totals[blockIdx.x] = below + s;
+}
+
+cudaError_t launch_compact_local(const uint32_t *mask, int64_t n, unsigned *local, unsigned *totals, cudaStream_t s)
+{
+    k_compact_local<<<cmp_blocks(n), kCmpBlockSegs, 0, s>>>(mask, n, local, totals);
+    return cudaGetLastError();
+}
+
 constexpr int kCmpThreads = 1024;
 
 __global__ void __launch_bounds__(kCmpThreads) k_compact_count(const uint32_t *__restrict__ mask, int64_t n,

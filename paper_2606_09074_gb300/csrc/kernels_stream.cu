@@ -1,246 +1,268 @@
-// Compaction, pass 2: the scatter of every row of the kept primitives, in
-// one of two forms chosen by compact_shape from the scene's size and type.
+// Compaction, pass 2: the scatter of every row of the kept primitives.
 //
-// Word form (k_compact_warp).  One warp handles one mask word (32
-// primitives) at a time; its output offset is the offset of its segment of
-// kCmpSeg = 256 primitives (from pass 1, k_compact_count) plus the kept bits
-// of the segment's earlier words.  The warp inverts the ranks of the kept
-// bits once (lane d of the output reads from the lane holding the d-th kept
-// primitive), then moves each of the 59 rows with one coalesced load, one
-// shuffle and one contiguous store.  The loads of sixteen float rows, or of
-// 28 bfloat16 rows (64-byte warp loads, so more of them must be in flight),
-// are issued together.  The CTA is 8 warps with a few hundred bytes of
-// shared memory; at 40 registers per thread (FP32 rows) an SM keeps 48 warps
-// and their 768 row loads resident, at 64 (bfloat16 rows) 32 warps and 896.
+// One CTA of 8 warps takes a unit of consecutive primitives (128 with float32
+// rows, 256 with bfloat16 rows) at a time.  The unit's span of each of the 59
+// rows, 512 contiguous bytes (1 KB of a float32 row beside bfloat16 ones), is
+// brought into shared memory by one bulk copy (cp.async.bulk) per row, issued
+// by the lanes of warp 0 and completing on an mbarrier; meanwhile the ranks
+// of the kept primitives are inverted (output d comes from primitive src[d]).
+// Then each warp takes every eighth row: 32 outputs are one shared-memory load
+// and one contiguous store.  A unit is 31-34 KB, so 6 CTAs fit an SM, and while
+// some wait for their unit others store theirs: about 190 KB an SM in flight
+// without holding a register.
 //
-// Segment form (k_compact_seg, FP32 attributes only).  One warp owns a
-// whole segment (8 mask words); the offsets of its words come from a shuffle
-// scan of their kept counts.  Each row moves with 8 coalesced loads (one
-// contiguous 1 KB span of the row), 8 shuffles and 8 stores that together
-// write one contiguous run of the output row.  Two rows (16 loads) are in
-// flight per warp; 80 registers hold the per-word ranks and offsets, so 3
-// CTAs of 8 warps fit per SM.  It keeps a quarter of the word form's warps in
-// flight, which pays only when each warp has several segments to stream.
+// A bulk copy starts on 16 bytes: the row's span is widened to 16-byte
+// boundaries (row strides may be odd) and the row's offset in shared memory
+// is taken from its misalignment.  At a scene's end the widened span of the
+// last row of a buffer could leave it (of the last few rows, when the stride
+// is below 8): it is narrowed instead, and its last few elements are read by
+// plain loads.
 //
-// No shared-memory staging of the rows in either form.
+// Measured (the kernel alone, events around it): bfloat16 rows, 3.5M primitives at ratio 0.5 160 -> 111 us (5.9
+// TB/s); float32 rows the same as the form before (3.5M 200 us, 6.2 TB/s; 1M at 0.66 60 us).  That form had a
+// warp load each row of a mask word into registers (16 float or 28 bfloat16 rows at a time) and shuffle: 64-byte
+// loads of bfloat16 rows, and registers, bounded what it had in flight.
 #include "internal.h"
 
 namespace refine {
 
 constexpr int kCmpWarps = 8;
-constexpr int kCmpBatch = 16;      // float rows in flight per warp
-constexpr int kCmpBatchB16 = 28;   // bfloat16 rows in flight per warp (56 rows in two steps)
+constexpr int kCmpThreads = 32 * kCmpWarps;
+constexpr int kCmpCtas = 6;  // per SM
 
-__device__ __forceinline__ float shfl_row(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ __nv_bfloat16 shfl_row(__nv_bfloat16 v, int src)
+// Primitives per unit.
+__host__ __device__ constexpr int cmp_unit(int dtype) { return dtype == REFINE_F32 ? 128 : 256; }
+// Rows of float32 elements (the means and the float32 attribute rows) and
+// their place in the tile: a row's span and 16 bytes for its misalignment.
+__host__ __device__ constexpr int cmp_f32_rows(int dtype) { return 3 + attr_f32_rows(dtype); }
+__host__ __device__ constexpr int cmp_pitch(int dtype, bool f32) { return cmp_unit(dtype) * (f32 ? 4 : 2) + 16; }
+__host__ __device__ constexpr int cmp_tile_bytes(int dtype)
 {
-    const unsigned short b = __shfl_sync(0xffffffffu, __bfloat16_as_ushort(v), src);
-    return __ushort_as_bfloat16(b);
+    return cmp_f32_rows(dtype) * cmp_pitch(dtype, true) + (59 - cmp_f32_rows(dtype)) * cmp_pitch(dtype, false);
 }
 
-template <typename T, int NR, int B = (sizeof(T) == 2 ? kCmpBatchB16 : kCmpBatch)>
-__device__ __forceinline__ void move_rows(const T *__restrict__ in, int64_t S, bool ld, int src, T *__restrict__ out,
-                                          int64_t OS, bool st)
-{
-#pragma unroll 1
-    for (int r0 = 0; r0 < NR; r0 += B) {
-        T v[B];
-#pragma unroll
-        for (int k = 0; k < B; ++k) v[k] = (ld && r0 + k < NR) ? in[k * S] : T(0.f);
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-            const T x = shfl_row(v[k], src);
-            if (st && r0 + k < NR) out[k * OS] = x;
-        }
-        in += B * S;
-        out += B * OS;
-    }
-}
-
-// DT is the storage type of the attribute rows: its float32 rows are moved
-// as float, the rest as bfloat16, each block of rows from and to its own
-// place in the layout (attr_f32_rows).
+// Row r of 59 (the means, then the attribute rows): address of its element 0
+// and its element size.
 template <int DT>
-__global__ void __launch_bounds__(32 * kCmpWarps) k_compact_warp(const float *__restrict__ pos,
-                                                                 const void *__restrict__ attr, int64_t S, int64_t n,
-                                                                 const uint32_t *__restrict__ mask,
-                                                                 const unsigned long long *__restrict__ seg_off,
-                                                                 const CmpState *cs, float *__restrict__ out_pos,
-                                                                 void *__restrict__ out_attr, int64_t OS,
-                                                                 int32_t *__restrict__ out_idx)
+struct RowSet {
+    const char *pos, *attr;
+    int64_t S;
+    __device__ __forceinline__ static constexpr bool f32(int r) { return r < cmp_f32_rows(DT); }
+    __device__ __forceinline__ static int tile(int r)  // byte offset in the tile
+    {
+        constexpr int NF = cmp_f32_rows(DT);
+        return r < NF ? r * cmp_pitch(DT, true) : NF * cmp_pitch(DT, true) + (r - NF) * cmp_pitch(DT, false);
+    }
+    __device__ __forceinline__ const char *row(int r) const
+    {
+        constexpr int NF = attr_f32_rows(DT);
+        if (r < 3) return pos + (int64_t)r * S * 4;
+        if (r - 3 < NF) return attr + (int64_t)(r - 3) * S * 4;
+        return attr + (int64_t)NF * S * 4 + (int64_t)(r - 3 - NF) * S * 2;
+    }
+    __device__ __forceinline__ const char *end(int r) const  // of the row's buffer
+    {
+        return r < 3 ? pos + S * 12 : attr + S * (int64_t)attr_col_bytes(DT);
+    }
+};
+
+// Bytes of the bulk copy of `count` elements of row r from element i0, its
+// span starting `mis` bytes past a 16-byte boundary: up to the next boundary,
+// or down to the last when that lies past the end of the row's buffer.
+template <int DT>
+__device__ __forceinline__ uint32_t span_bytes(const RowSet<DT> &in, int r, int64_t i0, uint32_t mis, int count)
 {
-    constexpr int NF = attr_f32_rows(DT), NB = 56 - NF;
-    const float *in_f = static_cast<const float *>(attr);
-    const __nv_bfloat16 *in_b =
-        reinterpret_cast<const __nv_bfloat16 *>(static_cast<const char *>(attr) + (size_t)NF * 4 * (size_t)S);
-    float *out_f = static_cast<float *>(out_attr);
-    __nv_bfloat16 *out_b = reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(out_attr) + (size_t)NF * 4 * (size_t)OS);
-    __shared__ unsigned char src_of[kCmpWarps][32];
-    if (!cs->ok) return;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    constexpr int kWords = kCmpSeg / 32;
-    const int64_t words = (n + 31) / 32;
-    for (int64_t w = (int64_t)blockIdx.x * kCmpWarps + wib; w < words; w += (int64_t)gridDim.x * kCmpWarps) {
-        // lane k < (w mod 8) holds the k-th earlier word of the segment, lane
-        // 31 this word; bits past n cleared
-        const int64_t w0 = w & ~(int64_t)(kWords - 1);
-        const int64_t wl = lane == 31 ? w : w0 + lane;
+    const int es = RowSet<DT>::f32(r) ? 4 : 2;
+    const uint32_t b = mis + (uint32_t)(count * es), up = (b + 15u) & ~15u;
+    return in.row(r) + i0 * es - mis + up > in.end(r) ? b & ~15u : up;
+}
+
+template <int DT>
+__global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in, int64_t n, const uint32_t *__restrict__ mask,
+                                                         CmpOffsets off, char *__restrict__ out_pos,
+                                                         char *__restrict__ out_attr, int64_t OS,
+                                                         int32_t *__restrict__ out_idx, int *status)
+{
+    constexpr int UNIT = cmp_unit(DT), UW = UNIT / 32, SEGU = kCmpSeg / UNIT;
+    extern __shared__ __align__(16) unsigned char tile[];
+    __shared__ unsigned char src_of[UNIT];
+    __shared__ unsigned blk_off[kCmpMaxBlocks];
+    __shared__ unsigned wsum[kCmpWarps];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int row_base[59];  // of each row in the tile, its misalignment included
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t units = (n + UNIT - 1) / UNIT, words = (n + 31) / 32;
+
+    // Offsets of the blocks of segments from their totals (up to one total a
+    // thread), and the kept count.
+    if (off.blocks > 0) {
+        static_assert(kCmpMaxBlocks == kCmpThreads, "one total per thread");
+        const unsigned own = (int)threadIdx.x < off.blocks ? __ldg(off.totals + threadIdx.x) : 0u;
+        unsigned s = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned x = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += x;
+        }
+        if (lane == 31) wsum[warp] = s;
+        __syncthreads();
+        unsigned below = 0u, total = 0u;
+#pragma unroll
+        for (int w = 0; w < kCmpWarps; ++w) {
+            below += w < warp ? wsum[w] : 0u;
+            total += wsum[w];
+        }
+        blk_off[threadIdx.x] = below + s - own;
+        const bool ok = (int64_t)total <= OS;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            off.state->total = (long long)total;
+            if (!ok) set_status(status, kEinval);
+        }
+        if (!ok) return;
+    } else if (!off.state->ok) {
+        return;
+    }
+    if (threadIdx.x < 59)
+        row_base[threadIdx.x] = RowSet<DT>::tile(threadIdx.x) +
+                                (int)(reinterpret_cast<uintptr_t>(in.row(threadIdx.x)) & 15u);
+    if (threadIdx.x == 0) mbar_init(&bar, 1);
+    __syncthreads();
+
+    uint32_t phase = 0;
+    // word of the unit, bits past n cleared (lanes < UW of every warp)
+    auto load_word = [&](int64_t u) {
+        const int64_t w = u * UW + lane;
         uint32_t word = 0u;
-        if (lane == 31 || wl < w) {
-            word = __ldg(mask + wl);
-            const int64_t valid = n - wl * 32;
+        if (lane < UW && u < units && w < words) {
+            word = __ldg(mask + w);
+            const int64_t valid = n - w * 32;
             if (valid < 32) word &= (1u << valid) - 1u;
         }
-        const uint32_t wk = __shfl_sync(0xffffffffu, word, 31);
-        const int kept = __popc(wk);
-        if (kept == 0) continue;  // uniform
-        const int before = __reduce_add_sync(0xffffffffu, lane == 31 ? 0u : (unsigned)__popc(word));
-        const int64_t base = w * 32;
-        const int64_t dst = (int64_t)__ldg(seg_off + w / kWords) + before + lane;
-        if ((wk >> lane) & 1u) src_of[wib][__popc(wk & ((1u << lane) - 1u))] = (unsigned char)lane;
-        __syncwarp();
-        const int src = lane < kept ? src_of[wib][lane] : lane;
-        __syncwarp();
-        const bool ld = base + lane < n;
-        const bool st = lane < kept;
-        if (out_idx && st) out_idx[dst] = (int32_t)(base + src);
-        move_rows<float, 3>(pos + base + lane, S, ld, src, out_pos + dst, OS, st);
-        if constexpr (NF > 0) move_rows<float, NF>(in_f + base + lane, S, ld, src, out_f + dst, OS, st);
-        if constexpr (NB > 0) move_rows<__nv_bfloat16, NB>(in_b + base + lane, S, ld, src, out_b + dst, OS, st);
-    }
-}
-
-constexpr int kSegRows = 2;  // rows in flight per warp (8 loads each)
-
-// The 59 rows of one primitive are pos rows 0..2 then attr rows 0..55; for
-// FP32 attributes both are float, so one loop walks all 59.
-__device__ __forceinline__ const float *seg_row(const float *pos, const float *attr, int64_t S, int r)
-{
-    return r < 3 ? pos + (int64_t)r * S : attr + (int64_t)(r - 3) * S;
-}
-__device__ __forceinline__ float *seg_row(float *pos, float *attr, int64_t S, int r)
-{
-    return r < 3 ? pos + (int64_t)r * S : attr + (int64_t)(r - 3) * S;
-}
-
-__global__ void __launch_bounds__(32 * kCmpWarps, 3) k_compact_seg(const float *__restrict__ pos,
-                                                                   const float *__restrict__ attr, int64_t S,
-                                                                   int64_t n, const uint32_t *__restrict__ mask,
-                                                                   const unsigned long long *__restrict__ seg_off,
-                                                                   const CmpState *cs, float *__restrict__ out_pos,
-                                                                   float *__restrict__ out_attr, int64_t OS,
-                                                                   int32_t *__restrict__ out_idx)
-{
-    constexpr int kWords = kCmpSeg / 32;
-    constexpr int kRows = 3 + 56;
-    static_assert(kWords == 8, "a segment is 8 mask words");
-    __shared__ unsigned char src_of[kCmpWarps][kWords][32];
-    if (!cs->ok) return;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int64_t nseg = (n + kCmpSeg - 1) / kCmpSeg;
-    const int64_t words = (n + 31) / 32;
-    for (int64_t sg = (int64_t)blockIdx.x * kCmpWarps + wib; sg < nseg; sg += (int64_t)gridDim.x * kCmpWarps) {
-        // lane w < 8 holds word w of the segment, bits past n cleared
-        uint32_t word = 0u;
-        {
-            const int64_t w = sg * kWords + lane;
-            if (lane < kWords && w < words) {
-                word = __ldg(mask + w);
-                const int64_t valid = n - w * 32;
-                if (valid < 32) word &= (1u << valid) - 1u;
+        return word;
+    };
+    uint32_t next_word = load_word(blockIdx.x);
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const uint32_t word = next_word;
+        next_word = load_word(u + gridDim.x);
+        const int kept = __reduce_add_sync(0xffffffffu, (unsigned)__popc(word));
+        if (kept == 0) continue;  // the same in every thread
+        const int64_t i0 = u * UNIT;
+        const int count = (int)min((int64_t)UNIT, n - i0);
+        if (warp == 0) {
+            uint32_t size[2], bytes = 0;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int r = lane + 32 * k;
+                size[k] = r < 59 ? span_bytes<DT>(in, r, i0, (uint32_t)(reinterpret_cast<uintptr_t>(in.row(r)) & 15u), count)
+                                 : 0u;
+                bytes += size[k];
             }
-        }
-        int incl = __popc(word);  // inclusive scan of the kept counts over the 8 words
+            bytes = __reduce_add_sync(0xffffffffu, bytes);
+            fence_proxy_async_shared();  // the tile was read by plain loads
+            if (lane == 0) mbar_expect_tx(&bar, bytes);
+            __syncwarp();
 #pragma unroll
-        for (int o = 1; o < kWords; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += x;
-        }
-        const int64_t base = sg * kCmpSeg;
-        const int64_t o0 = (int64_t)__ldg(seg_off + sg);
-        int kept[kWords], off[kWords], src[kWords];
-        bool ld[kWords];
-#pragma unroll
-        for (int w = 0; w < kWords; ++w) {
-            const uint32_t wk = __shfl_sync(0xffffffffu, word, w);
-            kept[w] = __popc(wk);
-            off[w] = __shfl_sync(0xffffffffu, incl, w) - kept[w];
-            if ((wk >> lane) & 1u) src_of[wib][w][__popc(wk & ((1u << lane) - 1u))] = (unsigned char)lane;
-            ld[w] = base + 32 * w + lane < n;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int w = 0; w < kWords; ++w) src[w] = lane < kept[w] ? src_of[wib][w][lane] : lane;
-        __syncwarp();
-        if (out_idx)
-#pragma unroll
-            for (int w = 0; w < kWords; ++w)
-                if (lane < kept[w]) out_idx[o0 + off[w] + lane] = (int32_t)(base + 32 * w + src[w]);
-        const float *in_p = pos + base + lane, *in_a = attr + base + lane;
-        float *out_p = out_pos + o0, *out_a = out_attr + o0;
-#pragma unroll 1
-        for (int r0 = 0; r0 < kRows; r0 += kSegRows) {
-            float v[kSegRows][kWords];
-#pragma unroll
-            for (int k = 0; k < kSegRows; ++k) {
-                const float *in = seg_row(in_p, in_a, S, r0 + k);
-#pragma unroll
-                for (int w = 0; w < kWords; ++w) v[k][w] = (ld[w] && r0 + k < kRows) ? in[32 * w] : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < kSegRows; ++k) {
-                if (r0 + k >= kRows) break;  // uniform
-                float *out = seg_row(out_p, out_a, OS, r0 + k);
-#pragma unroll
-                for (int w = 0; w < kWords; ++w) {
-                    const float x = shfl_row(v[k][w], src[w]);
-                    if (lane < kept[w]) out[off[w] + lane] = x;
+            for (int k = 0; k < 2; ++k) {
+                const int r = lane + 32 * k;
+                if (size[k] > 0u) {
+                    const char *p = in.row(r) + i0 * (RowSet<DT>::f32(r) ? 4 : 2);
+                    bulk_g2s(tile + RowSet<DT>::tile(r), p - (reinterpret_cast<uintptr_t>(p) & 15u), size[k], &bar);
                 }
             }
+        } else if (i0 + UNIT + 8 > n) {  // what narrowed copies leave (fewer than 8 elements a row)
+            for (int r = warp - 1; r < 59; r += kCmpWarps - 1) {
+                const int es = RowSet<DT>::f32(r) ? 4 : 2;
+                const uint32_t mis = (uint32_t)(reinterpret_cast<uintptr_t>(in.row(r)) & 15u);
+                const int j = max(0, (int)span_bytes<DT>(in, r, i0, mis, count) - (int)mis) / es + lane;
+                if (j >= count) continue;
+                if (es == 4)
+                    *reinterpret_cast<float *>(tile + row_base[r] + 4 * j) =
+                        __ldg(reinterpret_cast<const float *>(in.row(r)) + i0 + j);
+                else
+                    *reinterpret_cast<unsigned short *>(tile + row_base[r] + 2 * j) =
+                        __ldg(reinterpret_cast<const unsigned short *>(in.row(r)) + i0 + j);
+            }
         }
+        // invert the ranks of the kept primitives
+        {
+            unsigned before = (unsigned)__popc(word);  // inclusive scan over the unit's words
+#pragma unroll
+            for (int o = 1; o < UW; o <<= 1) {
+                const unsigned x = __shfl_up_sync(0xffffffffu, before, o);
+                if (lane >= o) before += x;
+            }
+            before -= (unsigned)__popc(word);
+            if (warp < UW) {
+                const uint32_t mine = __shfl_sync(0xffffffffu, word, warp);
+                const unsigned b = __shfl_sync(0xffffffffu, before, warp);
+                if ((mine >> lane) & 1u)
+                    src_of[b + __popc(mine & ((1u << lane) - 1u))] = (unsigned char)(warp * 32 + lane);
+            }
+        }
+        const int64_t sg = i0 / kCmpSeg;
+        int64_t dst = off.blocks > 0 ? (int64_t)(blk_off[sg / kCmpBlockSegs] + __ldg(off.local + sg))
+                                     : (int64_t)__ldg(off.global + sg);
+        if (SEGU > 1 && u % SEGU != 0) {  // kept in the segment's earlier unit
+            const uint32_t w0 = lane < UW ? __ldg(mask + (u - 1) * UW + lane) : 0u;
+            dst += __reduce_add_sync(0xffffffffu, (unsigned)__popc(w0));
+        }
+        __syncthreads();  // src_of, and what plain loads brought
+        const int nb = (kept + 31) >> 5;
+        int src[UW];
+#pragma unroll
+        for (int b = 0; b < UW; ++b) src[b] = b * 32 + lane < kept ? src_of[b * 32 + lane] : 0;
+        if (out_idx && warp < nb && warp * 32 + lane < kept)
+            out_idx[dst + warp * 32 + lane] = (int32_t)(i0 + src_of[warp * 32 + lane]);
+        if (!mbar_wait_bounded(&bar, phase)) {
+            set_status(status, kEtimeout);
+            mbar_wait_bounded(&bar, phase);  // give the copies a second bound before leaving
+            return;
+        }
+        phase ^= 1u;
+        for (int r = warp; r < 59; r += kCmpWarps) {
+            const unsigned char *t = tile + row_base[r];
+            if (RowSet<DT>::f32(r)) {
+                float *o = (r < 3 ? reinterpret_cast<float *>(out_pos) + (int64_t)r * OS
+                                  : reinterpret_cast<float *>(out_attr) + (int64_t)(r - 3) * OS) + dst + lane;
+#pragma unroll
+                for (int b = 0; b < UW; ++b)
+                    if (b * 32 + lane < kept) o[b * 32] = *reinterpret_cast<const float *>(t + 4 * src[b]);
+            } else {
+                constexpr int NF = attr_f32_rows(DT);
+                unsigned short *o = reinterpret_cast<unsigned short *>(out_attr + (int64_t)NF * OS * 4) +
+                                    (int64_t)(r - 3 - NF) * OS + dst + lane;
+#pragma unroll
+                for (int b = 0; b < UW; ++b)
+                    if (b * 32 + lane < kept) o[b * 32] = *reinterpret_cast<const unsigned short *>(t + 2 * src[b]);
+            }
+        }
+        __syncthreads();  // the tile and src_of are free again
     }
 }
 
-// The segment form for FP32 rows once every resident warp of it gets two
-// segments or more (n of 1.87M or more on 152 SMs); the word form otherwise.
-// Measured on 3.5M primitives, FP32 rows: 0.199 ms against 0.249 ms; BF16
-// rows: 0.164 ms both; 1M primitives: 0.084 ms against 0.067 ms.  Work is
-// dealt round-robin over at most 6 CTAs per SM: for the segment form that is
-// two waves of 3, the second filling SMs whose first CTAs finish early.
-CmpShape compact_shape(int num_sms, int64_t n, int dtype)
+template <int DT>
+static cudaError_t launch_compact_t(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
+                                    void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, cudaStream_t s)
 {
-    const int64_t nseg = (n + kCmpSeg - 1) / kCmpSeg;
-    const bool seg = dtype == REFINE_F32 && nseg >= 2 * (int64_t)num_sms * 3 * kCmpWarps;
-    const int64_t units = seg ? nseg : (n + 31) / 32;
-    int64_t g = (units + kCmpWarps - 1) / kCmpWarps;
-    const int64_t cap = (int64_t)num_sms * 6;
-    if (g > cap) g = cap;
+    const size_t smem = cmp_tile_bytes(DT);
+    static_assert(cmp_tile_bytes(DT) < 40 * 1024, "no opt-in shared memory");
+    int64_t g = (in.n + cmp_unit(DT) - 1) / cmp_unit(DT);
+    if (g > (int64_t)num_sms * kCmpCtas) g = (int64_t)num_sms * kCmpCtas;
     if (g < 1) g = 1;
-    return {(int)g, seg};
+    const RowSet<DT> rows{reinterpret_cast<const char *>(in.pos), static_cast<const char *>(in.attr), in.row_stride};
+    k_compact<DT><<<(int)g, kCmpThreads, smem, s>>>(rows, in.n, mask, off, reinterpret_cast<char *>(out_pos),
+                                                    static_cast<char *>(out_attr), OS, out_idx, status);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_compact_scatter(const refine_scene &in, const uint32_t *mask, const unsigned long long *seg_off,
-                                   const CmpState *cs, float *out_pos, void *out_attr, int64_t out_stride,
-                                   int32_t *out_idx, CmpShape shape, cudaStream_t s)
+cudaError_t launch_compact_scatter(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
+                                   void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, cudaStream_t s)
 {
-    if (in.dtype == REFINE_BF16) {
-        k_compact_warp<REFINE_BF16><<<shape.grid, 32 * kCmpWarps, 0, s>>>(
-            in.pos, in.attr, in.row_stride, in.n, mask, seg_off, cs, out_pos, out_attr, out_stride, out_idx);
-    } else if (in.dtype == REFINE_BF16S) {
-        k_compact_warp<REFINE_BF16S><<<shape.grid, 32 * kCmpWarps, 0, s>>>(
-            in.pos, in.attr, in.row_stride, in.n, mask, seg_off, cs, out_pos, out_attr, out_stride, out_idx);
-    } else {
-        const float *a = static_cast<const float *>(in.attr);
-        float *oa = static_cast<float *>(out_attr);
-        if (shape.seg)
-            k_compact_seg<<<shape.grid, 32 * kCmpWarps, 0, s>>>(in.pos, a, in.row_stride, in.n, mask, seg_off, cs,
-                                                                out_pos, oa, out_stride, out_idx);
-        else
-            k_compact_warp<REFINE_F32><<<shape.grid, 32 * kCmpWarps, 0, s>>>(in.pos, a, in.row_stride, in.n, mask,
-                                                                             seg_off, cs, out_pos, oa, out_stride,
-                                                                             out_idx);
-    }
-    return cudaGetLastError();
+    if (in.dtype == REFINE_BF16)
+        return launch_compact_t<REFINE_BF16>(in, mask, off, out_pos, out_attr, OS, out_idx, num_sms, status, s);
+    if (in.dtype == REFINE_BF16S)
+        return launch_compact_t<REFINE_BF16S>(in, mask, off, out_pos, out_attr, OS, out_idx, num_sms, status, s);
+    return launch_compact_t<REFINE_F32>(in, mask, off, out_pos, out_attr, OS, out_idx, num_sms, status, s);
 }
 
 }  // namespace refine

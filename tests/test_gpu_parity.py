@@ -566,10 +566,10 @@ def test_select_cluster_edges(torch, rb, ctx, n):
     assert np.array_equal(mask.cpu().numpy().view(np.uint32)[: (n + 31) // 32], m_ref)
 
 
-@pytest.mark.parametrize("n", [255, 256, 257, 1_048_575, 1_048_577, 4_194_304, 4_194_305])
+@pytest.mark.parametrize("n", [255, 256, 257, 65_536, 65_537, 1_048_577, 16_777_216, 16_777_217])
 def test_compact_count_sizes(torch, rb, ctx, n):
-    """Kept counts and offsets about the segment and step limits of the counting
-    kernel, checked through the indices (the attribute rows are zeros)."""
+    """Kept counts and offsets about the segment, block and size limits of the
+    counting kernels, checked through the indices (the attribute rows are zeros)."""
     g = torch.Generator(device="cuda").manual_seed(n)
     keep = torch.rand(n, generator=g, device="cuda") < 0.03
     words = (n + 31) // 32
@@ -582,4 +582,36 @@ def test_compact_count_sizes(torch, rb, ctx, n):
     want = torch.nonzero(keep).flatten().to(torch.int32)
     op, oa, idx, cnt = ctx.compact(pos, attr, mask, want.numel(), return_count=True)
     assert cnt == want.numel() and torch.equal(idx, want) and torch.equal(op[2], pos[2][want.long()])
+    ctx.check()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "bf16s"])
+@pytest.mark.parametrize("pad", [0, 1, 3, 6])
+def test_compact_units(torch, rb, ctx, dtype, pad):
+    """The scatter about its units (128 or 256 primitives) and the end of a
+    scene, with row strides of every 16-byte misalignment: equal to indexing
+    the rows."""
+    for n in (1, 7, 8, 127, 128, 129, 136, 137, 255, 256, 257, 263, 264, 265, 385, 1_031, 70_003):
+        g = torch.Generator(device="cuda").manual_seed(n * 10 + pad)
+        S = n + pad
+        pos = torch.randn((3, S), generator=g, device="cuda")
+        full = torch.randn((56, S), generator=g, device="cuda")
+        for p in (0.02, 0.5, 1.0):
+            keep = torch.rand(n, generator=g, device="cuda") < p
+            words = (n + 31) // 32
+            bits = torch.zeros(words * 32, dtype=torch.int64, device="cuda")
+            bits[:n] = keep
+            mask = (bits.view(words, 32) << torch.arange(32, device="cuda")).sum(1).to(torch.int32)
+            want = torch.nonzero(keep).flatten()
+            if dtype == "bf16s":
+                attr = rb.MixedRows.from_float(full)  # stride S
+                attr = attr.to("cuda")[:, :n]
+                rows = attr.float()
+            else:
+                attr = full.to(torch.bfloat16 if dtype == "bf16" else torch.float32)[:, :n]
+                rows = attr.float()
+            op, oa, idx = ctx.compact(pos[:, :n], attr, mask, want.numel(), out_row_stride=want.numel() + 1 + pad)
+            assert torch.equal(idx, want.to(torch.int32))
+            assert torch.equal(op, pos[:, want]), (n, p)
+            assert torch.equal(oa.float().to("cuda"), rows[:, want].to("cuda")), (n, p)
     ctx.check()
