@@ -315,12 +315,12 @@ inline SceneScratch carve_scene(Carver &cv, const ScenePlan &pl)
 template <typename L>
 inline refine_status enqueue_prep(refine_ctx *c, L &&run, const refine_scene *sc, const refine_camera *cams,
                            const ScenePlan &pl, const SceneScratch &x, const refine_params &p, bool count,
-                           void *more, size_t more_bytes, int *status, cudaStream_t s)
+                           void *more, size_t more_bytes, int *status, const Chain &s)
 {
     const int64_t n = pl.n;
     const int cells = order_keys(pl.bits);
     if (count) {
-        const cudaError_t e = cudaMemsetAsync(x.need, 0, kCountSlots * sizeof(unsigned long long), s);
+        const cudaError_t e = cudaMemsetAsync(x.need, 0, kCountSlots * sizeof(unsigned long long), s.s);
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
     }
     PrepLaunch pre;
@@ -337,8 +337,12 @@ inline refine_status enqueue_prep(refine_ctx *c, L &&run, const refine_scene *sc
     pre.more4 = (int64_t)(more_bytes / 16);
     pre.status = status;
     refine_status st;
+    // Not chained: its launch leaves the SMs idle for a moment, in which the
+    // feature pass's large L1 takes the place of the shared memory that a
+    // compaction just before had (chained, 1.75M primitives took 481 us a pass,
+    // 374 us so: the loads in flight had no room).
     if ((st = run(K_PREPARE, [&] {
-             return launch_prepare(sc->pos, sc->attr, sc->dtype, sc->row_stride, n, pre, c->num_sms, s);
+             return launch_prepare(sc->pos, sc->attr, sc->dtype, sc->row_stride, n, pre, c->num_sms, s.s);
          })))
         return st;
     FeatureLaunch f;
@@ -437,7 +441,7 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     if (stats_dev) *stats_dev = x.stats;
     if (need_dev) *need_dev = x.need;
     auto run = [&](int cls, auto &&f) { return launch(c, cls, s, f); };
-    if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, count, counters, taken, c->d_status, s))) return st;
+    if ((st = enqueue_prep(c, run, sc, cams, pl, x, p, count, counters, taken, c->d_status, Chain(s, true)))) return st;
     for (int v0 = 0; v0 < pl.V; v0 += pl.vpp) {
         ScoreLaunch a = make_score_launch(sc, pl, x, p, v0, scores, view_sum, count, c->d_status);
         const ScorePlan &sp = a.last ? sp1 : sp0;
@@ -448,7 +452,7 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
         a.parts_done = reinterpret_cast<unsigned *>(counters + sizeof(unsigned long long));
         const cudaError_t e = v0 > 0 ? cudaMemsetAsync(counters, 0, taken, s) : cudaSuccess;  // first: k_prepare
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
-        if ((st = launch(c, K_SCORE, s, [&] { return launch_score(a, sp.gpt, s); }))) return st;
+        if ((st = launch(c, K_SCORE, s, [&] { return launch_score(a, sp.gpt, Chain(s, true)); }))) return st;
     }
     return REFINE_OK;
 }
@@ -462,7 +466,7 @@ inline size_t select_bytes(int64_t n)
 // Radix select into the given state; *kstar_dev is NULL when nothing is pruned.
 template <typename L>
 inline refine_status enqueue_select(refine_ctx *c, L &&run, const float *scores, int64_t n, int64_t n_keep,
-                             uint32_t *mask, void *scratch, unsigned int **kstar_dev, int *status, cudaStream_t s)
+                             uint32_t *mask, void *scratch, unsigned int **kstar_dev, int *status, const Chain &s)
 {
     *kstar_dev = nullptr;
     if (n == 0) return REFINE_OK;
@@ -479,7 +483,7 @@ inline refine_status enqueue_select(refine_ctx *c, L &&run, const float *scores,
         *kstar_dev = &ss->kstar;
         return REFINE_OK;
     }
-    cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(SelState), s);
+    cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(SelState), s.s);
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
     const bool vec = aligned16(scores);
     const int grid = select_grid(c->num_sms, n);
@@ -506,7 +510,7 @@ inline refine_status select_impl(refine_ctx *c, const float *scores, int64_t n, 
     refine_status st;
     if ((st = ensure(c, c->select, select_bytes(n)))) return st;
     auto run = [&](int cls, auto &&f) { return launch(c, cls, s, f); };
-    return enqueue_select(c, run, scores, n, *n_keep, mask, c->select.p, kstar_dev, c->d_status, s);
+    return enqueue_select(c, run, scores, n, *n_keep, mask, c->select.p, kstar_dev, c->d_status, Chain(s, true));
 }
 
 inline refine_status read_threshold(refine_ctx *c, unsigned int *kstar_dev, float *thr, cudaStream_t s)
@@ -534,7 +538,7 @@ inline size_t compact_bytes(int64_t n)
 template <typename L>
 inline refine_status enqueue_compact(refine_ctx *c, L &&run, const refine_scene *in, const uint32_t *mask, float *out_pos,
                               void *out_attr, int64_t out_stride, int32_t *idx, void *scratch, long long **total_dev,
-                              int *status, cudaStream_t s)
+                              int *status, const Chain &s)
 {
     const int64_t n = in->n;
     const int64_t nseg = (n + kCmpSeg - 1) / kCmpSeg;
@@ -550,7 +554,7 @@ inline refine_status enqueue_compact(refine_ctx *c, L &&run, const refine_scene 
         off = CmpOffsets{cmp_blocks(n), seg_cnt, totals, nullptr, cs};
         if ((st = run(K_CMP_COUNT, [&] { return launch_compact_local(mask, n, seg_cnt, totals, s); }))) return st;
     } else {
-        const cudaError_t e = cudaMemsetAsync(cs, 0, sizeof(CmpState), s);
+        const cudaError_t e = cudaMemsetAsync(cs, 0, sizeof(CmpState), s.s);
         if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemsetAsync");
         int64_t cgrid = (nseg + 1023) / 1024;
         if (cgrid > c->num_sms) cgrid = c->num_sms;
@@ -580,7 +584,7 @@ inline refine_status compact_impl(refine_ctx *c, const refine_scene *in, const u
     if ((st = ensure(c, c->compact, compact_bytes(in->n)))) return st;
     auto run = [&](int cls, auto &&f) { return launch(c, cls, s, f); };
     return enqueue_compact(c, run, in, mask, out_pos, out_attr, out_stride, idx, c->compact.p, total_dev,
-                           c->d_status, s);
+                           c->d_status, Chain(s, true));
 }
 
 }  // namespace refine_api

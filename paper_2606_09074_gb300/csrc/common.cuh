@@ -255,6 +255,29 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return true;
 }
 
+// Programmatic dependent launch.  A kernel of a chain (Chain, internal.h) may
+// start while the one before it ends; it calls pdl_wait first, which returns
+// when every earlier kernel of the stream has ended and its writes are
+// visible, then lets the next one start its launch.  It returns a zero that
+// the compiler does not know: pointers offset by it (after) cannot be
+// read before the wait, whatever the loads' cache path.  That is for what the
+// kernel just before wrote, or a kernel of the caller's; anything older was
+// complete when that kernel went on from its own wait.  (An offset pointer is
+// no longer uniform: offset for all 59 rows, the feature pass took a third
+// longer.)
+__device__ __forceinline__ int64_t pdl_wait()
+{
+    int64_t zero;
+    asm volatile("griddepcontrol.wait;\n\tmov.b64 %0, 0;" : "=l"(zero)::"memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    return zero;
+}
+template <typename P>
+__device__ __forceinline__ void after(int64_t zero, P &p)
+{
+    p = p + zero;
+}
+
 // Fast reciprocal on the MUFU pipe (max error 1 ulp).
 __device__ __forceinline__ float rcp_approx(float x)
 {

@@ -10,6 +10,35 @@
 
 namespace refine {
 
+// Where a launcher puts its kernel: a stream, and whether the kernel may start
+// its launch while the kernel before it in the stream ends (programmatic
+// dependent launch; every kernel launched so waits for the earlier ones with
+// pdl_wait before it touches memory).  The plain calls chain their kernels: a
+// selection of 1.75M scores takes 29 instead of 43 us, a pass over 1M x 150
+// 313 instead of 342 us.  The batch and the queue do not: kernels that wait on
+// one stream would hold the SMs that another stream's could use.
+struct Chain {
+    cudaStream_t s;
+    bool on = false;
+    Chain(cudaStream_t stream) : s(stream) {}
+    Chain(cudaStream_t stream, bool chained) : s(stream), on(chained) {}
+};
+template <typename... K, typename... A>
+cudaError_t launch_chained(void (*k)(K...), int grid, int threads, size_t smem, const Chain &c, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = c.on ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<K>(args)...);
+}
+
 // Cameras processed per score launch at most (80 bytes each in shared
 // memory, 128 with REFINE_FLAG_FULL_JACOBIAN).  A larger view set is split into passes (camera blocks) of
 // ScoreShape::views_per_pass views, a multiple of 32; a primitive's running
@@ -174,7 +203,7 @@ struct PrepLaunch {
     int *status;
 };
 cudaError_t launch_prepare(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n, const PrepLaunch &a,
-                           int num_sms, cudaStream_t s);
+                           int num_sms, const Chain &s);
 
 struct FeatureLaunch {
     const float *pos;
@@ -191,7 +220,7 @@ struct FeatureLaunch {
     int *status;
 };
 int feature_blocks(int64_t n);
-cudaError_t launch_features(const FeatureLaunch &f, int dtype, int num_sms, cudaStream_t s);
+cudaError_t launch_features(const FeatureLaunch &f, int dtype, int num_sms, const Chain &s);
 
 // What the cell scatter's first block forms from the feature pass's block sums.
 struct SceneTail {
@@ -203,11 +232,11 @@ struct SceneTail {
     SceneStats *stats;
 };
 cudaError_t launch_cell_scan(unsigned *counts, unsigned *off_local, unsigned *bsum, unsigned *done, int cell_bits,
-                             cudaStream_t s);
+                             const Chain &s);
 cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n,
                                 const unsigned *off_local, const unsigned *bsum, uint32_t *perm,
-                                const SceneTail &tail, int num_sms, cudaStream_t s);
-cudaError_t launch_score(const ScoreLaunch &a, int gpt, cudaStream_t s);
+                                const SceneTail &tail, int num_sms, const Chain &s);
+cudaError_t launch_score(const ScoreLaunch &a, int gpt, const Chain &s);
 // split: tiles may be split (the caller provides parts and parts_done).
 ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, const ScoreShape &sh);
 
@@ -254,16 +283,16 @@ struct SelState {
 // state); above it, the passes below.
 constexpr int64_t kSelClusterMax = 8 * 32 * 1024;
 cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_keep, SelState *st, uint32_t *mask,
-                                  int *status, cudaStream_t s);
+                                  int *status, const Chain &s);
 constexpr int kTieSeg = 4096;
 int select_grid(int num_sms, int64_t n);
 cudaError_t launch_select_pass(int pass, const float *scores, int64_t n, uint32_t n_keep,
-                               SelState *st, bool vec, int grid, int *status, cudaStream_t s);
+                               SelState *st, bool vec, int grid, int *status, const Chain &s);
 cudaError_t launch_select_ties(const float *scores, int64_t n, SelState *st, unsigned *seg_cnt,
-                               int grid, cudaStream_t s);
+                               int grid, const Chain &s);
 cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *st, uint32_t *mask,
-                               int num_sms, cudaStream_t s);
-cudaError_t launch_mask_fill(uint32_t *mask, int64_t n, cudaStream_t s);
+                               int num_sms, const Chain &s);
+cudaError_t launch_mask_fill(uint32_t *mask, int64_t n, const Chain &s);
 
 // ------------------------------------------------------------- compact
 struct CmpState {
@@ -283,12 +312,12 @@ struct CmpOffsets {
     const unsigned long long *global;
     CmpState *state;
 };
-cudaError_t launch_compact_local(const uint32_t *mask, int64_t n, unsigned *local, unsigned *totals, cudaStream_t s);
+cudaError_t launch_compact_local(const uint32_t *mask, int64_t n, unsigned *local, unsigned *totals, const Chain &s);
 cudaError_t launch_compact_count(const uint32_t *mask, int64_t n, unsigned *seg_cnt,
                                  unsigned long long *seg_off, CmpState *cs, int64_t out_stride,
-                                 int grid, int *status, cudaStream_t s);
+                                 int grid, int *status, const Chain &s);
 cudaError_t launch_compact_scatter(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
                                    void *out_attr, int64_t out_stride, int32_t *out_idx, int num_sms, int *status,
-                                   cudaStream_t s);
+                                   const Chain &s);
 
 }  // namespace refine

@@ -185,6 +185,7 @@ template <int DT>
 __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restrict__ pos, AttrRows<DT> attr, int64_t S,
                                                           int64_t n, PrepLaunch a)
 {
+    pdl_wait();  // never chained itself; lets the next kernel's launch begin
     if (blockIdx.x > 0) {
         const int64_t b = blockIdx.x - 1, nb = gridDim.x - 1;
         for (int64_t v = b + nb * threadIdx.x; v < a.V; v += nb * kPrepThreads)
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
 }
 
 cudaError_t launch_prepare(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n, const PrepLaunch &a,
-                           int num_sms, cudaStream_t s)
+                           int num_sms, const Chain &s)
 {
     // 4 stores of 16 bytes a thread, at most 64 cameras a block
     int64_t g = (a.zero4 + a.more4 + 4 * kPrepThreads - 1) / (4 * kPrepThreads);
@@ -251,12 +252,13 @@ cudaError_t launch_prepare(const float *pos, const void *attr, int dtype, int64_
     if (g < 1) g = 1;
     const int grid = (int)g + 1;
     if (dtype == REFINE_BF16)
-        k_prepare<REFINE_BF16><<<grid, kPrepThreads, 0, s>>>(pos, AttrRows<REFINE_BF16>(attr, stride), stride, n, a);
-    else if (dtype == REFINE_BF16S)
-        k_prepare<REFINE_BF16S><<<grid, kPrepThreads, 0, s>>>(pos, AttrRows<REFINE_BF16S>(attr, stride), stride, n, a);
-    else
-        k_prepare<REFINE_F32><<<grid, kPrepThreads, 0, s>>>(pos, AttrRows<REFINE_F32>(attr, stride), stride, n, a);
-    return cudaGetLastError();
+        return launch_chained(k_prepare<REFINE_BF16>, grid, kPrepThreads, 0, s, pos, AttrRows<REFINE_BF16>(attr, stride),
+                              stride, n, a);
+    if (dtype == REFINE_BF16S)
+        return launch_chained(k_prepare<REFINE_BF16S>, grid, kPrepThreads, 0, s, pos,
+                              AttrRows<REFINE_BF16S>(attr, stride), stride, n, a);
+    return launch_chained(k_prepare<REFINE_F32>, grid, kPrepThreads, 0, s, pos, AttrRows<REFINE_F32>(attr, stride), stride,
+                          n, a);
 }
 
 // ---------------------------------------------------------------------
@@ -295,6 +297,7 @@ struct FeatureArgs {
     uint2 *cell;
     unsigned *counts;
     int *status;
+
 };
 
 // Block sums in float-float: thread (k, j) adds the values of threads
@@ -355,6 +358,7 @@ __device__ __forceinline__ FeatTerms feature_one(const FeatureArgs<DT> &f, const
 template <int DT>
 __global__ void __launch_bounds__(kFeatCol, 4) k_features(FeatureArgs<DT> f)
 {
+    after(pdl_wait(), f.grid);  // the rows are older than the kernel before this one
     __shared__ float red[kFeatSums * kFeatRedRow];
     __shared__ __align__(4) uint16_t hilbert[24 * 64];
     load_hilbert(hilbert);
@@ -402,6 +406,7 @@ constexpr int kFeatSmallThreads = 1024;
 template <int DT>
 __global__ void __launch_bounds__(kFeatSmallThreads, 1) k_features_small(FeatureArgs<DT> f)
 {
+    after(pdl_wait(), f.grid);  // the rows are older than the kernel before this one
     constexpr int kGroups = kFeatSmallThreads / kFeatCol;
     __shared__ float val[5][kFeatCols][kFeatCol];  // y, alpha, gem, m_gem, m_col
     __shared__ __align__(4) uint16_t hilbert[24 * 64];
@@ -475,26 +480,21 @@ int feature_blocks(int64_t n)
 }
 
 template <int DT>
-static void launch_features_t(const FeatureLaunch &l, int num_sms, cudaStream_t s)
+static cudaError_t launch_features_t(const FeatureLaunch &l, int num_sms, const Chain &s)
 {
     FeatureArgs<DT> f{l.pos, AttrRows<DT>(l.attr, l.stride), l.stride, l.n, l.eta, l.luma[0], l.luma[1], l.luma[2], l.recs,
                       l.partials, l.grid, l.cell_bits, l.cell, l.counts, l.status};
     const int nb = feature_blocks(l.n);
     if (nb <= num_sms && l.n <= (int64_t)nb * kFeatCol * kFeatCols)
-        k_features_small<DT><<<nb, kFeatSmallThreads, 0, s>>>(f);
-    else
-        k_features<DT><<<nb, kFeatCol, 0, s>>>(f);
+        return launch_chained(k_features_small<DT>, nb, kFeatSmallThreads, 0, s, f);
+    return launch_chained(k_features<DT>, nb, kFeatCol, 0, s, f);
 }
 
-cudaError_t launch_features(const FeatureLaunch &f, int dtype, int num_sms, cudaStream_t s)
+cudaError_t launch_features(const FeatureLaunch &f, int dtype, int num_sms, const Chain &s)
 {
-    if (dtype == REFINE_BF16)
-        launch_features_t<REFINE_BF16>(f, num_sms, s);
-    else if (dtype == REFINE_BF16S)
-        launch_features_t<REFINE_BF16S>(f, num_sms, s);
-    else
-        launch_features_t<REFINE_F32>(f, num_sms, s);
-    return cudaGetLastError();
+    if (dtype == REFINE_BF16) return launch_features_t<REFINE_BF16>(f, num_sms, s);
+    if (dtype == REFINE_BF16S) return launch_features_t<REFINE_BF16S>(f, num_sms, s);
+    return launch_features_t<REFINE_F32>(f, num_sms, s);
 }
 
 // Eq. (features) -> Eq. 18 -> Eq. 19 in double, by one block (every thread
@@ -590,6 +590,7 @@ __global__ void __launch_bounds__(kScanThreads) k_cell_scan(const unsigned *__re
                                                             unsigned *__restrict__ off_local,
                                                             unsigned *bsum, unsigned *done)
 {
+    after(pdl_wait(), counts);
     const int nblocks = gridDim.x;
     __shared__ unsigned wsum[32];
     __shared__ unsigned is_last, carry;
@@ -619,10 +620,9 @@ __global__ void __launch_bounds__(kScanThreads) k_cell_scan(const unsigned *__re
 }
 
 cudaError_t launch_cell_scan(unsigned *counts, unsigned *off_local, unsigned *bsum, unsigned *done, int cell_bits,
-                             cudaStream_t s)
+                             const Chain &s)
 {
-    k_cell_scan<<<order_keys(cell_bits) / kScanCells, kScanThreads, 0, s>>>(counts, off_local, bsum, done);
-    return cudaGetLastError();
+    return launch_chained(k_cell_scan, order_keys(cell_bits) / kScanCells, kScanThreads, 0, s, counts, off_local, bsum, done);
 }
 
 constexpr int kSortU = 4;  // primitives in flight per thread
@@ -645,6 +645,9 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const uint2 *__restrict__ 
                                                       const unsigned *__restrict__ boff, uint32_t *__restrict__ perm,
                                                       SceneTail tail)
 {
+    const int64_t zero = pdl_wait();
+    after(zero, off_local);  // (the rest is older than the kernel before this one)
+    after(zero, boff);
     if (blockIdx.x == 0) {
         finalize_features(tail);
         return;
@@ -666,10 +669,9 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const uint2 *__restrict__ 
 }
 
 cudaError_t launch_cell_scatter(const uint2 *cell, int64_t n, const unsigned *off_local, const unsigned *bsum,
-                                uint32_t *perm, const SceneTail &tail, int num_sms, cudaStream_t s)
+                                uint32_t *perm, const SceneTail &tail, int num_sms, const Chain &s)
 {
-    k_cell_scatter<<<sort_grid(num_sms, n) + 1, 256, 0, s>>>(cell, n, off_local, bsum, perm, tail);
-    return cudaGetLastError();
+    return launch_chained(k_cell_scatter, sort_grid(num_sms, n) + 1, 256, 0, s, cell, n, off_local, bsum, perm, tail);
 }
 
 }  // namespace refine

@@ -569,6 +569,9 @@ __device__ __forceinline__ void stage_cams(const ScoreLaunch &a, unsigned char *
 template <int PM, bool COUNT, int GPT>
 __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLaunch a)
 {
+    const int64_t zero = pdl_wait();
+    after(zero, a.perm);  // (the records are older than the kernel before this one)
+    after(zero, a.consts);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ WarpSlot s_slot[kScoreThreads / 32];
@@ -773,27 +776,29 @@ cudaError_t launch_wait_selftest(const void *src, uint32_t bytes, uint32_t missi
     return cudaGetLastError();
 }
 
+using ScoreFn = void (*)(ScoreLaunch);
+
 template <int PM, bool COUNT, int GPT>
-static const void *score_fn()
+static ScoreFn score_fn()
 {
-    return reinterpret_cast<const void *>(&k_score<PM, COUNT, GPT>);
+    return &k_score<PM, COUNT, GPT>;
 }
 
 template <int PM, int GPT>
-static const void *pick_score_pg(bool count)
+static ScoreFn pick_score_pg(bool count)
 {
     return count ? score_fn<PM, true, GPT>() : score_fn<PM, false, GPT>();
 }
 
 template <int GPT>
-static const void *pick_score_g(int pm, bool count)
+static ScoreFn pick_score_g(int pm, bool count)
 {
     if (pm == kProjNone) return pick_score_pg<kProjNone, GPT>(count);
     if (pm == kProjFullJ) return pick_score_pg<kProjFullJ, GPT>(count);
     return pick_score_pg<kProjEq17, GPT>(count);
 }
 
-static const void *pick_score(int pm, bool count, int gpt)
+static ScoreFn pick_score(int pm, bool count, int gpt)
 {
     return gpt == 1 ? pick_score_g<1>(pm, count) : pick_score_g<2>(pm, count);
 }
@@ -827,7 +832,7 @@ ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, 
     const int64_t blocks = (vcount + 31) / 32;
     pl.gpt = sh.gpt;
     int per_sm = 0;
-    const void *fn = pick_score(proj_mode(flags), false, pl.gpt);
+    const ScoreFn fn = pick_score(proj_mode(flags), false, pl.gpt);
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kScoreThreads, smem) != cudaSuccess ||
         per_sm < 1) {
@@ -850,17 +855,15 @@ ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, 
     return pl;
 }
 
-cudaError_t launch_score(const ScoreLaunch &a, int gpt, cudaStream_t s)
+cudaError_t launch_score(const ScoreLaunch &a, int gpt, const Chain &s)
 {
-    const void *fn = pick_score(proj_mode(a.flags), a.need != nullptr, gpt);
+    const ScoreFn fn = pick_score(proj_mode(a.flags), a.need != nullptr, gpt);
     const size_t smem = cams_smem(a.vcount, a.flags);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    ScoreLaunch arg = a;
-    void *args[] = {&arg};
-    return cudaLaunchKernel(fn, dim3(a.grid), dim3(kScoreThreads), args, smem, s);
+    return launch_chained(fn, a.grid, kScoreThreads, smem, s, a);
 }
 
 static const void *batch_fn(const ScoreShape &sh)

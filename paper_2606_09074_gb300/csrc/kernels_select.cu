@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(kSelThreads) k_select_pass(const float *__rest
     __shared__ unsigned int wsum[32];
     __shared__ unsigned int is_last;
     for (int b = threadIdx.x; b < NB; b += blockDim.x) h[b] = 0u;
+    after(pdl_wait(), scores);
     __syncthreads();
     const unsigned int prefix = PASS == 0 ? 0u : st->prefix;
     bool bad = false;
@@ -199,17 +200,14 @@ int select_grid(int num_sms, int64_t n)
 
 template <int PASS>
 static cudaError_t launch_pass_t(const float *scores, int64_t n, uint32_t n_keep, SelState *st,
-                                 bool vec, int grid, int *status, cudaStream_t s)
+                                 bool vec, int grid, int *status, const Chain &s)
 {
-    if (vec)
-        k_select_pass<PASS, true><<<grid, kSelThreads, 0, s>>>(scores, n, n_keep, st, status);
-    else
-        k_select_pass<PASS, false><<<grid, kSelThreads, 0, s>>>(scores, n, n_keep, st, status);
-    return cudaGetLastError();
+    if (vec) return launch_chained(k_select_pass<PASS, true>, grid, kSelThreads, 0, s, scores, n, n_keep, st, status);
+    return launch_chained(k_select_pass<PASS, false>, grid, kSelThreads, 0, s, scores, n, n_keep, st, status);
 }
 
 cudaError_t launch_select_pass(int pass, const float *scores, int64_t n, uint32_t n_keep,
-                               SelState *st, bool vec, int grid, int *status, cudaStream_t s)
+                               SelState *st, bool vec, int grid, int *status, const Chain &s)
 {
     if (pass == 0) return launch_pass_t<0>(scores, n, n_keep, st, vec, grid, status, s);
     if (pass == 1) return launch_pass_t<1>(scores, n, n_keep, st, vec, grid, status, s);
@@ -222,6 +220,7 @@ cudaError_t launch_select_pass(int pass, const float *scores, int64_t n, uint32_
 __global__ void __launch_bounds__(kSelThreads) k_select_ties(const float *__restrict__ scores, int64_t n,
                                                              SelState *st, unsigned *seg_cnt)
 {
+    after(pdl_wait(), scores);
     if (!st->need_ties) return;
     __shared__ unsigned long long wsum[32];
     __shared__ unsigned int is_last;
@@ -293,10 +292,9 @@ __global__ void __launch_bounds__(kSelThreads) k_select_ties(const float *__rest
 }
 
 cudaError_t launch_select_ties(const float *scores, int64_t n, SelState *st, unsigned *seg_cnt,
-                               int grid, cudaStream_t s)
+                               int grid, const Chain &s)
 {
-    k_select_ties<<<grid, kSelThreads, 0, s>>>(scores, n, st, seg_cnt);
-    return cudaGetLastError();
+    return launch_chained(k_select_ties, grid, kSelThreads, 0, s, scores, n, st, seg_cnt);
 }
 
 // Keep mask: a warp builds kMaskWords consecutive 32-element words per
@@ -306,6 +304,9 @@ constexpr int kMaskWords = 8;
 __global__ void k_select_mask(const float *__restrict__ scores, int64_t n, const SelState *st,
                               uint32_t *__restrict__ mask)
 {
+    const int64_t zero = pdl_wait();
+    after(zero, scores);
+    after(zero, st);
     const uint32_t kstar = st->kstar;
     const long long cut = st->idx_cut;
     const int64_t words = (n + 31) / 32;
@@ -331,14 +332,13 @@ __global__ void k_select_mask(const float *__restrict__ scores, int64_t n, const
 }
 
 cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *st, uint32_t *mask,
-                               int num_sms, cudaStream_t s)
+                               int num_sms, const Chain &s)
 {
     // one step of every warp, up to 8 CTAs of 8 warps per SM
     int64_t g = ((n + 31) / 32 + 8 * kMaskWords - 1) / (8 * kMaskWords);
     if (g > (int64_t)num_sms * 8) g = (int64_t)num_sms * 8;
     if (g < 1) g = 1;
-    k_select_mask<<<(int)g, 256, 0, s>>>(scores, n, st, mask);
-    return cudaGetLastError();
+    return launch_chained(k_select_mask, (int)g, 256, 0, s, scores, n, st, mask);
 }
 
 // ---------------------------------------------------------------------
@@ -376,6 +376,7 @@ __global__ void __launch_bounds__(kClThreads) k_select_cluster(const float *__re
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = rank * per, m = max(0, min(per, n - i0));  // per is a multiple of 32
     for (int b = threadIdx.x; b < 3 * 2048; b += kClThreads) (&hist[0][0])[b] = 0u;
+    after(pdl_wait(), scores);
     __syncthreads();
     bool bad = false;
     for (int j0 = warp * 32; j0 < m; j0 += kClLoads * kClThreads) {
@@ -490,7 +491,7 @@ __global__ void __launch_bounds__(kClThreads) k_select_cluster(const float *__re
 }
 
 cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_keep, SelState *st, uint32_t *mask,
-                                  int *status, cudaStream_t s)
+                                  int *status, const Chain &s)
 {
     int ctas = 1;
     while (ctas < kClMaxCtas && n > (int64_t)12 * 1024 * ctas) ctas *= 2;
@@ -505,18 +506,21 @@ cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_kee
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kClThreads);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)ctas;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.stream = s.s;
+    cudaLaunchAttribute at[2]{};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = s.on ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, k_select_cluster, scores, (int)n, per, n_keep, st, mask, status);
 }
 
 __global__ void k_mask_fill(uint32_t *mask, int64_t n)
 {
+    after(pdl_wait(), mask);
     const int64_t words = (n + 31) / 32;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
          w += (int64_t)gridDim.x * blockDim.x) {
@@ -525,14 +529,13 @@ __global__ void k_mask_fill(uint32_t *mask, int64_t n)
     }
 }
 
-cudaError_t launch_mask_fill(uint32_t *mask, int64_t n, cudaStream_t s)
+cudaError_t launch_mask_fill(uint32_t *mask, int64_t n, const Chain &s)
 {
     int64_t words = (n + 31) / 32;
     int grid = (int)((words + 255) / 256);
     if (grid > 1024) grid = 1024;
     if (grid < 1) grid = 1;
-    k_mask_fill<<<grid, 256, 0, s>>>(mask, n);
-    return cudaGetLastError();
+    return launch_chained(k_mask_fill, grid, 256, 0, s, mask, n);
 }
 
 // ---------------------------------------------------------------------
@@ -553,6 +556,7 @@ __global__ void __launch_bounds__(kCmpBlockSegs) k_compact_local(const uint32_t 
     constexpr int kWords = kCmpSeg / 32;
     static_assert(kWords == 8, "a segment is two 16-byte loads");
     __shared__ unsigned wsum[kCmpBlockSegs / 32];
+    after(pdl_wait(), mask);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t sg = (int64_t)blockIdx.x * kCmpBlockSegs + threadIdx.x, nseg = (n + kCmpSeg - 1) / kCmpSeg;
     const int64_t words = (n + 31) / 32;
@@ -588,10 +592,9 @@ __global__ void __launch_bounds__(kCmpBlockSegs) k_compact_local(const uint32_t 
     if (threadIdx.x == kCmpBlockSegs - 1) totals[blockIdx.x] = below + s;
 }
 
-cudaError_t launch_compact_local(const uint32_t *mask, int64_t n, unsigned *local, unsigned *totals, cudaStream_t s)
+cudaError_t launch_compact_local(const uint32_t *mask, int64_t n, unsigned *local, unsigned *totals, const Chain &s)
 {
-    k_compact_local<<<cmp_blocks(n), kCmpBlockSegs, 0, s>>>(mask, n, local, totals);
-    return cudaGetLastError();
+    return launch_chained(k_compact_local, cmp_blocks(n), kCmpBlockSegs, 0, s, mask, n, local, totals);
 }
 
 constexpr int kCmpThreads = 1024;
@@ -602,6 +605,7 @@ __global__ void __launch_bounds__(kCmpThreads) k_compact_count(const uint32_t *_
 {
     __shared__ unsigned long long wsum[32];
     __shared__ unsigned int is_last;
+    after(pdl_wait(), mask);
     const int64_t words = (n + 31) / 32;
     const int64_t nseg = (n + kCmpSeg - 1) / kCmpSeg;
     constexpr int kWords = kCmpSeg / 32;
@@ -662,10 +666,9 @@ __global__ void __launch_bounds__(kCmpThreads) k_compact_count(const uint32_t *_
 
 cudaError_t launch_compact_count(const uint32_t *mask, int64_t n, unsigned *seg_cnt,
                                  unsigned long long *seg_off, CmpState *cs, int64_t out_stride,
-                                 int grid, int *status, cudaStream_t s)
+                                 int grid, int *status, const Chain &s)
 {
-    k_compact_count<<<grid, kCmpThreads, 0, s>>>(mask, n, seg_cnt, seg_off, cs, out_stride, status);
-    return cudaGetLastError();
+    return launch_chained(k_compact_count, grid, kCmpThreads, 0, s, mask, n, seg_cnt, seg_off, cs, out_stride, status);
 }
 
 }  // namespace refine

@@ -92,6 +92,10 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in
     __shared__ int row_base[59];  // of each row in the tile, its misalignment included
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t units = (n + UNIT - 1) / UNIT, words = (n + 31) / 32;
+    const int64_t zero = pdl_wait();
+    after(zero, off.local);  // (the rows and the mask are older than the kernel before this one)
+    after(zero, off.totals);
+    after(zero, off.global);
 
     // Offsets of the blocks of segments from their totals (up to one total a
     // thread), and the kept count.
@@ -242,7 +246,7 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in
 
 template <int DT>
 static cudaError_t launch_compact_t(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
-                                    void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, cudaStream_t s)
+                                    void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, const Chain &s)
 {
     const size_t smem = cmp_tile_bytes(DT);
     static_assert(cmp_tile_bytes(DT) < 40 * 1024, "no opt-in shared memory");
@@ -250,13 +254,12 @@ static cudaError_t launch_compact_t(const refine_scene &in, const uint32_t *mask
     if (g > (int64_t)num_sms * kCmpCtas) g = (int64_t)num_sms * kCmpCtas;
     if (g < 1) g = 1;
     const RowSet<DT> rows{reinterpret_cast<const char *>(in.pos), static_cast<const char *>(in.attr), in.row_stride};
-    k_compact<DT><<<(int)g, kCmpThreads, smem, s>>>(rows, in.n, mask, off, reinterpret_cast<char *>(out_pos),
-                                                    static_cast<char *>(out_attr), OS, out_idx, status);
-    return cudaGetLastError();
+    return launch_chained(k_compact<DT>, (int)g, kCmpThreads, smem, s, rows, in.n, mask, off,
+                          reinterpret_cast<char *>(out_pos), static_cast<char *>(out_attr), OS, out_idx, status);
 }
 
 cudaError_t launch_compact_scatter(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
-                                   void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, cudaStream_t s)
+                                   void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, const Chain &s)
 {
     if (in.dtype == REFINE_BF16)
         return launch_compact_t<REFINE_BF16>(in, mask, off, out_pos, out_attr, OS, out_idx, num_sms, status, s);

@@ -615,3 +615,49 @@ def test_compact_units(torch, rb, ctx, dtype, pad):
             assert torch.equal(op, pos[:, want]), (n, p)
             assert torch.equal(oa.float().to("cuda"), rows[:, want].to("cuda")), (n, p)
     ctx.check()
+
+
+@pytest.mark.parametrize("n,v,dtype", [(900, 5, "f32"), (20_001, 33, "bf16"), (300_007, 70, "bf16s"), (270_000, 20, "f32")])
+def test_chained_calls_same_bits(torch, rb, ctx, n, v, dtype):
+    """The plain calls, whose kernels overlap their launches, one after another
+    on two scenes in turn without a wait in between, and captured in a graph:
+    the same bits as the batched form, whose kernels do not."""
+    scenes, want = [], []
+    for k in range(2):
+        w = synth.random_scene(seed=n + k, n=n - 7 * k, v=v, means="core_shell")
+        sc = w.scene if dtype == "f32" else (w.scene.to_bf16() if dtype == "bf16" else w.scene.to_bf16s())
+        pos, attr, cams = upload(torch, rb, sc, w.cams)
+        scenes.append((pos, attr, cams))
+        b = rb.Batch(ctx, [{"pos": pos, "attr": attr, "cams": cams, "ratio": 0.6}])
+        b.run()
+        b.results()
+        want.append({x: (y if isinstance(y, int) else y.float().cpu() if x == "out_attr" else y.clone())
+                     for x, y in b.outputs[0].items()})
+        b.close()
+
+    def one(k):
+        pos, attr, cams = scenes[k]
+        s = ctx.score(pos, attr, cams)
+        mask, _, nk = ctx.select(s, 0.6, threshold=False)
+        return (s, mask) + ctx.compact(pos, attr, mask, nk)
+
+    def same(k, got):
+        s, mask, op, oa, idx = got
+        return (torch.equal(s, want[k]["scores"]) and torch.equal(mask, want[k]["mask"]) and torch.equal(op, want[k]["out_pos"])
+                and torch.equal(oa.float().cpu(), want[k]["out_attr"]) and torch.equal(idx, want[k]["idx"]))
+    got = [(i % 2, one(i % 2)) for i in range(24)]
+    torch.cuda.synchronize()
+    assert all(same(k, g) for k, g in got)
+    ctx.check()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        one(0), one(1)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            held = [one(0), one(1)]
+        for _ in range(3):
+            graph.replay()
+        stream.synchronize()
+        assert all(same(k, held[k]) for k in range(2))
+        ctx.check()
