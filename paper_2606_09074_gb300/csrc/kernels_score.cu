@@ -48,6 +48,10 @@ namespace refine {
 // depend on the tile it is in and its rounding error does not grow with V.
 // The epilogue forms D_i = alpha_i S_i / |V| * sum_k lambda^k G~_i^k (Eq. 7).
 // ---------------------------------------------------------------------
+// Floor of PairIn::s3: with it, and E > 1e-3 and z > 1e-6 (classify), s3 K is
+// above every du whose (du z)^2 underflows, which the exact test would pass.
+constexpr float kMinS3 = 1e-12f;
+
 struct PairIn {
     float mx, my, mz;
     float L[9];
@@ -65,10 +69,12 @@ struct __align__(16) TileBox {
 // views are scored and is read back for each classification, so that it
 // holds no registers across the view loop (the loads are volatile: never
 // hoisted); k holds the footprint reach (classify) of the 32 views being
-// scored, one per classifying lane.
+// scored, one per classifying lane; run holds every lane's running (sum,
+// compensation) of its primitives, touched once in 32 views.
 struct __align__(16) WarpSlot {
     TileBox box;
     float2 k[32];
+    float2 run[2][32];
 };
 
 __device__ __forceinline__ TileBox load_box(const TileBox *s)
@@ -141,7 +147,7 @@ __device__ __forceinline__ int classify(const CamRec &c, const TileBox &t, float
     const float dx = fmaxf(-U.lo, UW.hi), dy = fmaxf(-V.lo, VH.hi);  // largest du, dv of the box
     const float zs = z.lo - t.s3;
     const float iz = rcp_approx_ftz(z.lo), q = zs > 0.f ? z.lo * rcp_approx_ftz(zs) : INFINITY;
-    const bool safe = z.lo > 1e-15f && fmaxf(dx, dy) * z.hi < 1e18f;
+    const bool safe = z.lo > 1e-6f && fminf(k.x, k.y) > 1e-3f && fmaxf(dx, dy) * z.hi < 1e18f;
     const float kx = safe ? fminf(k.x * q, fmaf(fmaxf(dx, 0.f), iz, k.x)) * 1.00390625f : INFINITY;
     const float ky = safe ? fminf(k.y * q, fmaf(fmaxf(dy, 0.f), iz, k.y)) * 1.00390625f : INFINITY;
     *reach = make_float2(kx, ky);
@@ -242,8 +248,7 @@ __device__ __forceinline__ float extent2(const float4 &r, const float4 &c2, floa
 // fails or passes it without evaluation).
 //
 // The bound (classify) with the depth range closed: du <= s3 Kx, the tile's
-// reach, one multiply-add and one compare a pair (the 1e-15 covers a square
-// that would underflow in the exact test); with the depth range open a pair
+// reach, one multiply and one compare a pair; with the depth range open a pair
 // forms its own, du (z - s3) <= s3 E z.  Both exclude only pairs that the exact
 // test fails.
 template <int PM, bool COUNT, int GPT, bool NX, bool NY, bool NZ>
@@ -265,14 +270,14 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
             U[g] = fmaf(c0.x, p[g].mx, fmaf(c0.y, p[g].my, fmaf(c0.z, p[g].mz, c0.w)));
             du[g] = fmaxf(-U[g], fmaf(-lim.x, z[g], U[g]));
             inside &= du[g] <= 0.f;
-            if (!NZ) reaches &= du[g] <= fmaf(p[g].s3, K.x, 1e-15f);
+            if (!NZ) reaches &= du[g] <= p[g].s3 * K.x;
         }
         if (NY) {
             const float4 c1 = c.r1;
             V[g] = fmaf(c1.x, p[g].mx, fmaf(c1.y, p[g].my, fmaf(c1.z, p[g].mz, c1.w)));
             dv[g] = fmaxf(-V[g], fmaf(-lim.y, z[g], V[g]));
             inside &= dv[g] <= 0.f;
-            if (!NZ) reaches &= dv[g] <= fmaf(p[g].s3, K.y, 1e-15f);
+            if (!NZ) reaches &= dv[g] <= p[g].s3 * K.y;
         }
         if (NZ) {
             const float4 k = c.k;
@@ -280,7 +285,7 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
             reaches &= (du[g] * zs <= k.x * t) & (dv[g] * zs <= k.y * t);
         }
         vis[g] = inside;
-        nq[g] = reaches & !inside;
+        nq[g] = !inside & reaches;
         if (COUNT && valid[g]) {
             const bool o = inz & !inside;
             cnt[kCntMixedPairs] += 1;
@@ -295,16 +300,18 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
             cnt[kCntExactY] += (NY && nq[g] && dv[g] > 0.f) ? 1 : 0;
         }
     }
+    // with one axis open, a centre outside is outside on that axis
+    constexpr bool kOne = NX != NY;
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
         bool ok = nq[g];
-        if (NX && __any_sync(0xffffffffu, nq[g] & (du[g] > 0.f))) {
-            const float ex = fmaxf(du[g], 0.f) * z[g];
+        if (NX && __any_sync(0xffffffffu, kOne ? nq[g] : nq[g] & (du[g] > 0.f))) {
+            const float ex = (kOne ? du[g] : fmaxf(du[g], 0.f)) * z[g];
             ok &= ex * ex <= extent2(c.r0, c2, U[g], z[g], p[g]);
             if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 1;
         }
-        if (NY && __any_sync(0xffffffffu, nq[g] & (dv[g] > 0.f))) {
-            const float ey = fmaxf(dv[g], 0.f) * z[g];
+        if (NY && __any_sync(0xffffffffu, kOne ? nq[g] : nq[g] & (dv[g] > 0.f))) {
+            const float ey = (kOne ? dv[g] : fmaxf(dv[g], 0.f)) * z[g];
             ok &= ey * ey <= extent2(c.r1, c2, V[g], z[g], p[g]);
             if (COUNT && (threadIdx.x & 31) == 0) cnt[kCntExactWarpAxes] += 1;
         }
@@ -318,21 +325,20 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
 }
 
 // Kahan-compensated sum of the 32-view block sums.
-__device__ __forceinline__ void kahan_add(float &acc, float &comp, float x)
+__device__ __forceinline__ void kahan_add(float2 &run, float x)
 {
-    const float y = x - comp;
-    const float t = acc + y;
-    comp = (t - acc) - y;
-    acc = t;
+    const float2 r = run;
+    const float y = x - r.y;
+    const float t = r.x + y;
+    run = make_float2(t, (t - r.x) - y);
 }
 
 // Views [v0, vend) of the pass (v0 a multiple of 32) for one tile: added to
-// (acc, comp), or with pp their block sums stored at pp.  take_next() runs
+// the slot's running sums, or with pp their block sums stored at pp.  take_next() runs
 // once, before the last block.
 template <int PM, bool DET, bool COUNT, int GPT, typename F>
 __device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, int v0, int vend, float *pp, float eta,
-                                          const PairIn (&p)[GPT], const bool (&valid)[GPT], WarpSlot *slot,
-                                          float (&acc)[GPT], float (&comp)[GPT], F &&take_next,
+                                          const PairIn (&p)[GPT], const bool (&valid)[GPT], WarpSlot *slot, F &&take_next,
                                           unsigned long long (&cnt)[kCountSlots])
 {
     const int lane = threadIdx.x & 31;
@@ -366,13 +372,16 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, in
             float part[GPT];
 #pragma unroll
             for (int g = 0; g < GPT; ++g) part[g] = 0.f;
+            // the single open axes first among the MIXED views: most of them
+            const unsigned x_m = ux_m & ~uy_m & ~uz_m, y_m = uy_m & ~ux_m & ~uz_m;
             unsigned todo = vmask & ~out_m;
             while (todo) {
-                const int b = __ffs(todo) - 1;
-                todo &= todo - 1u;
+                const unsigned bit = todo & (0u - todo);
+                const int b = 31 - __clz(bit);
+                todo ^= bit;
                 const CamRec &c = cs[vb + b];
                 const CamExt *ext = PM == kProjFullJ ? ce + vb + b : nullptr;
-                if ((in_m >> b) & 1u) {
+                if (in_m & bit) {
                     const float4 c2 = c.r2;
 #pragma unroll
                     for (int g = 0; g < GPT; ++g) {
@@ -382,16 +391,15 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, in
                 } else if (DET) {
                     mixed_view_det<PM, COUNT, GPT>(c, ext, eta, p, valid, part, cnt);
                 } else {
-                    const unsigned bit = 1u << b;
                     const float2 &reach = slot->k[b];
-                    if (uz_m & bit)
-                        mixed_view<PM, COUNT, GPT, true, true, true>(c, ext, reach, eta, p, valid, part, cnt);
-                    else if (ux_m & uy_m & bit)
-                        mixed_view<PM, COUNT, GPT, true, true, false>(c, ext, reach, eta, p, valid, part, cnt);
-                    else if (ux_m & bit)
-                        mixed_view<PM, COUNT, GPT, true, false, false>(c, ext, reach, eta, p, valid, part, cnt);
-                    else
+                    if (y_m & bit)
                         mixed_view<PM, COUNT, GPT, false, true, false>(c, ext, reach, eta, p, valid, part, cnt);
+                    else if (x_m & bit)
+                        mixed_view<PM, COUNT, GPT, true, false, false>(c, ext, reach, eta, p, valid, part, cnt);
+                    else if (uz_m & bit)
+                        mixed_view<PM, COUNT, GPT, true, true, true>(c, ext, reach, eta, p, valid, part, cnt);
+                    else
+                        mixed_view<PM, COUNT, GPT, true, true, false>(c, ext, reach, eta, p, valid, part, cnt);
                 }
             }
             if (pp) {  // a part of the tile's views: its block sums are added by the tile's last item
@@ -399,7 +407,7 @@ __device__ __forceinline__ void view_loop(const CamRec *cs, const CamExt *ce, in
                 for (int g = 0; g < GPT; ++g) pp[(vb >> 5) * (32 * GPT) + g * 32 + lane] = part[g];
             } else {
 #pragma unroll
-                for (int g = 0; g < GPT; ++g) kahan_add(acc[g], comp[g], part[g]);
+                for (int g = 0; g < GPT; ++g) kahan_add(slot->run[g][lane], part[g]);
             }
         }
     }
@@ -449,7 +457,6 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
 {
     const int lane = threadIdx.x & 31;
     PairIn p[GPT];
-    float acc[GPT], comp[GPT];
     bool valid[GPT];
     bool degen = false;
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY}, s3 = 0.f;
@@ -457,21 +464,17 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
     for (int g = 0; g < GPT; ++g) {
         const int64_t j = base + g * 32 + lane;
         float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra, rc = ra, rd = ra;
-        acc[g] = 0.f;
-        comp[g] = 0.f;
+        float2 run = make_float2(0.f, 0.f);
         valid[g] = j < a.n;
         if (valid[g]) {
             const int64_t i = __ldg(a.perm + j);
             const PrimRec *r = a.recs + i;
             ra = __ldg(&r->a); rb = __ldg(&r->b); rc = __ldg(&r->c); rd = __ldg(&r->d);
-            if (!a.first) {
-                const float2 run = a.running[i];
-                acc[g] = run.x;
-                comp[g] = run.y;
-            }
+            if (!a.first) run = a.running[i];
         }
+        slot->run[g][lane] = run;  // read and written by this lane only
         p[g].mx = ra.x; p[g].my = ra.y; p[g].mz = ra.z;
-        p[g].s3 = fmaxf(sqrt_approx_ftz(fabsf(ra.w)), 1e-30f);
+        p[g].s3 = fmaxf(sqrt_approx_ftz(fabsf(ra.w)), kMinS3);
         p[g].L[0] = rb.x; p[g].L[1] = rb.y; p[g].L[2] = rb.z; p[g].L[3] = rb.w;
         p[g].L[4] = rc.x; p[g].L[5] = rc.y; p[g].L[6] = rc.z; p[g].L[7] = rc.w;
         p[g].L[8] = rd.x;
@@ -503,9 +506,9 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
     }
 
     if (__any_sync(0xffffffffu, degen))
-        view_loop<PM, true, COUNT, GPT>(cs, ce, tp.v0, tp.vend, tp.parts, a.eta, p, valid, slot, acc, comp, take_next, cnt);
+        view_loop<PM, true, COUNT, GPT>(cs, ce, tp.v0, tp.vend, tp.parts, a.eta, p, valid, slot, take_next, cnt);
     else
-        view_loop<PM, false, COUNT, GPT>(cs, ce, tp.v0, tp.vend, tp.parts, a.eta, p, valid, slot, acc, comp, take_next, cnt);
+        view_loop<PM, false, COUNT, GPT>(cs, ce, tp.v0, tp.vend, tp.parts, a.eta, p, valid, slot, take_next, cnt);
 
     if (tp.parts) {
         __threadfence();
@@ -516,18 +519,19 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
         __threadfence();
         for (int b = 0; b < (a.vcount + 31) >> 5; ++b)
 #pragma unroll
-            for (int g = 0; g < GPT; ++g) kahan_add(acc[g], comp[g], __ldcg(tp.parts + b * (32 * GPT) + g * 32 + lane));
+            for (int g = 0; g < GPT; ++g) kahan_add(slot->run[g][lane], __ldcg(tp.parts + b * (32 * GPT) + g * 32 + lane));
     }
 
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
         if (!valid[g]) continue;
         const int64_t i = __ldg(a.perm + base + g * 32 + lane);
+        const float2 run = slot->run[g][lane];
         if (!a.last) {
-            a.running[i] = make_float2(acc[g], comp[g]);
+            a.running[i] = run;
             continue;
         }
-        const float Ssum = acc[g] - comp[g];
+        const float Ssum = run.x - run.y;
         if (a.view_sum) a.view_sum[i] = Ssum;
         const float4 rd = __ldg(&a.recs[i].d);  // (L8, alpha, m_gem, m_col)
         const float coupled = fmaf(sc.kappa[0], rd.z, fmaf(sc.kappa[1], rd.w, sc.kappa[2] * rd.y));
@@ -612,6 +616,7 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
     // views.  Item indices stay below 2^31 (n <= INT32_MAX, and only a wave's
     // worth of tiles is split).
     const int lane = threadIdx.x & 31;
+    WarpSlot *slot = &s_slot[__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0)];  // a uniform address
     const int ntiles = (int)((a.n + 32 * GPT - 1) / (32 * GPT));
     const int whole = ntiles - a.split_tiles;
     const int per = a.split_tiles > 0 ? (a.vcount + kSplitViews - 1) / kSplitViews : 1;
@@ -640,7 +645,7 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
                 if (j < a.n) prefetch_l2(a.recs + __ldg(a.perm + j));
             }
         };
-        score_tile<PM, COUNT, GPT>(a, cs, ce, sc, (int64_t)tile * (32 * GPT), tp, &s_slot[threadIdx.x >> 5], take_next,
+        score_tile<PM, COUNT, GPT>(a, cs, ce, sc, (int64_t)tile * (32 * GPT), tp, slot, take_next,
                                    cnt);
         cur = nxt;
     }
@@ -676,6 +681,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
     int cur = -1;
     uint32_t phase = 0;
     const int lane = threadIdx.x & 31;
+    WarpSlot *slot = &s_slot[__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0)];  // a uniform address
     const int64_t tile = (int64_t)THREADS * GPT * b.rounds;  // primitives per item
     for (;;) {
         if (threadIdx.x == 0) {
@@ -739,11 +745,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLa
             const int64_t wbase = base + (int64_t)t * (32 * GPT);
             const TilePart tp = {0, a.vcount, nullptr, nullptr, 1};
             if (pm == kProjEq17)
-                score_tile<kProjEq17, false, GPT>(a, cs, ce, sc, wbase, tp, &s_slot[threadIdx.x >> 5], [] {}, cnt);
+                score_tile<kProjEq17, false, GPT>(a, cs, ce, sc, wbase, tp, slot, [] {}, cnt);
             else if (pm == kProjNone)
-                score_tile<kProjNone, false, GPT>(a, cs, ce, sc, wbase, tp, &s_slot[threadIdx.x >> 5], [] {}, cnt);
+                score_tile<kProjNone, false, GPT>(a, cs, ce, sc, wbase, tp, slot, [] {}, cnt);
             else
-                score_tile<kProjFullJ, false, GPT>(a, cs, ce, sc, wbase, tp, &s_slot[threadIdx.x >> 5], [] {}, cnt);
+                score_tile<kProjFullJ, false, GPT>(a, cs, ce, sc, wbase, tp, slot, [] {}, cnt);
         }
         __syncthreads();  // the cameras, s_scene and s_wt are free again
     }
