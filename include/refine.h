@@ -315,7 +315,7 @@ void refine_batch_destroy(refine_batch *batch);
 /* ------------------------------------------------------------ autotuner
  * Work-item shape of the score kernels.  A warp scores a tile of 32 or 64
  * consecutive primitives of the processing order against every view; the
- * batched kernel hands out CTA-sized items of such tiles, and the views are
+ * warps of the batched kernel draw such tiles scene by scene; the views are
  * taken in camera blocks (passes) of `camera_block` views.  Every
  * primitive's score is computed by one thread with the views in a fixed
  * order, whatever tile it is in, and its running Kahan pair is carried

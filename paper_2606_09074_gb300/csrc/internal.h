@@ -58,28 +58,15 @@ struct ScoreShape {
     int views_per_pass = kViewsPerPass;  // camera block: views per score pass (32..512, a multiple of 32)
 };
 bool shape_valid(const ScoreShape &sh);
-// An item of the batched kernel: `rounds` warp tiles per warp of the CTA
-// (1, 2 or 4), of one scene; the CTA's warps share them out dynamically.
-// Large items cost fewer CTA barriers and counter atomics; a launch with
-// little work takes smaller ones, so that every CTA gets several items and
-// the launch does not end on a few long ones (batch_rounds).  Warp tiles
-// stay 32 * gpt aligned within a scene either way.
-constexpr int kBatchRounds = 4;
-inline int64_t batch_tile(const ScoreShape &sh, int rounds = kBatchRounds)
+// Work of a scene in a batched launch, in (32-primitive, view) pairs.
+inline long long batch_work(int64_t n, int vcount) { return (long long)((n + 31) / 32) * vcount; }
+// CTAs of a batched launch over scenes of `tiles32` 32-primitive groups in
+// all: no more than there are tiles for their warps.
+inline int batch_grid(const ScoreShape &sh, int full_grid, long long tiles32)
 {
-    return (int64_t)sh.threads * sh.gpt * rounds;
-}
-// The largest item (4, 2 or 1 rounds) that leaves at least 4 items per CTA
-// of a grid of `grid` CTAs over scenes of n[0..k) primitives.
-inline int batch_rounds(const ScoreShape &sh, const int64_t *n, int k, int grid)
-{
-    for (int r = kBatchRounds; r > 1; r /= 2) {
-        const int64_t t = batch_tile(sh, r);
-        int64_t items = 0;
-        for (int i = 0; i < k; ++i) items += (n[i] + t - 1) / t;
-        if (items >= 4 * (int64_t)grid) return r;
-    }
-    return 1;
+    const long long per_cta = (long long)sh.gpt * (sh.threads / 32);
+    const long long g = (tiles32 + per_cta - 1) / per_cta;
+    return (int)(g < 1 ? 1 : (g < full_grid ? g : full_grid));
 }
 
 // Spatial cells for the processing order of k_score: a 2^b x 2^b x 2^b grid
@@ -169,8 +156,8 @@ struct ScoreLaunch {
     float *scores;
     float *view_sum;            // optional
     unsigned long long *need;   // optional diagnostic counters (kCountSlots), see k_score
-    unsigned long long *tiles_taken;  // k_score: warp-tile counter, zero before the launch (required;
-                                      // k_score_batch takes its items from BatchLaunch::counter)
+    unsigned long long *tiles_taken;  // k_score: item counter, zero before the launch (required;
+                                      // k_score_batch draws from BatchLaunch::next)
     int split_tiles;            // k_score: tiles taken in items of kSplitViews views (score_plan)
     float *parts;               //   their block sums, [split_tiles][blocks of the pass][tile]
     unsigned *parts_done;       //   items finished per split tile, zero before the launch
@@ -256,15 +243,14 @@ cudaError_t launch_wait_selftest(const void *src, uint32_t bytes, uint32_t missi
 // pass of at most kViewsPerPass views).
 struct BatchLaunch {
     const ScoreLaunch *scenes;       // device [n_scenes]
-    const long long *tile_begin;     // device [n_scenes + 1], first tile of each scene
+    const long long *work;           // device [n_scenes + 1], work of the scenes before each (batch_work)
     int n_scenes;
-    long long total_tiles;
-    unsigned long long *counter;     // device, zero before the launch
+    unsigned *next;                  // device [n_scenes], tiles drawn of each, zero before the launch
+    bool eq17;                       // every scene has the Eq. 17 projection mode
     int *status;
-    int rounds;                      // warp tiles per warp in an item (batch_tile)
 };
 // smem: the largest camera block among the scenes (cams_smem).
-int score_batch_grid(int num_sms, size_t smem, const ScoreShape &sh);
+int score_batch_grid(int num_sms, size_t smem, bool eq17, const ScoreShape &sh);
 cudaError_t launch_score_batch(const BatchLaunch &b, size_t smem, int grid, const ScoreShape &sh, cudaStream_t s);
 
 // ------------------------------------------------------------- select

@@ -451,7 +451,7 @@ struct TilePart {
 };
 
 template <int PM, bool COUNT, int GPT, typename F>
-__device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *cs, const CamExt *ce, const SceneConsts &sc,
+__device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *cs, const CamExt *ce,
                                            int64_t base, const TilePart &tp, WarpSlot *slot, F &&take_next,
                                            unsigned long long (&cnt)[kCountSlots])
 {
@@ -534,6 +534,7 @@ __device__ __forceinline__ void score_tile(const ScoreLaunch &a, const CamRec *c
         const float Ssum = run.x - run.y;
         if (a.view_sum) a.view_sum[i] = Ssum;
         const float4 rd = __ldg(&a.recs[i].d);  // (L8, alpha, m_gem, m_col)
+        const SceneConsts sc = *a.consts;       // read here: no registers across the views
         const float coupled = fmaf(sc.kappa[0], rd.z, fmaf(sc.kappa[1], rd.w, sc.kappa[2] * rd.y));
         const float A = ((a.flags & REFINE_FLAG_NO_VIS) ? 1.f : rd.y) * (Ssum * a.inv_views);
         a.scores[i] = A * coupled;
@@ -604,7 +605,6 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
     unsigned long long cnt[kCountSlots];
 #pragma unroll
     for (int k = 0; k < kCountSlots; ++k) cnt[k] = 0;
-    const SceneConsts sc = *a.consts;
     // Every warp takes its own items from a counter: warps that draw cheap
     // tiles take more of them, and no warp waits for the others of its CTA.  A
     // warp draws its next item before the last block of views of the current
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
                 if (j < a.n) prefetch_l2(a.recs + __ldg(a.perm + j));
             }
         };
-        score_tile<PM, COUNT, GPT>(a, cs, ce, sc, (int64_t)tile * (32 * GPT), tp, slot, take_next,
+        score_tile<PM, COUNT, GPT>(a, cs, ce, (int64_t)tile * (32 * GPT), tp, slot, take_next,
                                    cnt);
         cur = nxt;
     }
@@ -660,98 +660,132 @@ __global__ void __launch_bounds__(kScoreThreads, COUNT ? 1 : 4) k_score(ScoreLau
     }
 }
 
-// The batched form: one persistent launch over the tiles of many scenes.
-// CTAs take (scene, tile) items from an atomic counter (items are ordered
-// by scene); when a CTA moves to another scene it restages that scene's
-// cameras by TMA.  Every tile is scored by score_tile exactly as in
-// k_score, so a scene's scores are the same alone and in a batch; scenes
-// may differ in storage type (the records are float32) and in flags.
-template <int GPT, int THREADS>
+// The scene that a CTA of the batched kernel is scoring, in shared memory.
+struct __align__(8) BatchScene {
+    ScoreLaunch a;
+    unsigned *next;  // tiles drawn so far
+    unsigned tiles;
+};
+
+// The scene's tiles for the warps of the CTA: each draws its next tile from
+// the scene's counter before the last view block of the current one, as in
+// k_score.
+template <int PM, int GPT>
+__device__ __forceinline__ void score_scene(const BatchScene &sc, const CamRec *cs, WarpSlot *slot)
+{
+    const int lane = threadIdx.x & 31;
+    const ScoreLaunch &a = sc.a;
+    unsigned long long cnt[kCountSlots];  // not counted
+    auto draw = [&]() {
+        unsigned t = 0;
+        if (lane == 0) t = atomicAdd(sc.next, 1u);
+        return __shfl_sync(0xffffffffu, t, 0);
+    };
+    for (unsigned cur = draw(); cur < sc.tiles;) {
+        unsigned nxt = 0;
+        auto take_next = [&]() {
+            nxt = draw();
+            if (nxt >= sc.tiles) return;
+#pragma unroll
+            for (int g = 0; g < GPT; ++g) {
+                const int64_t j = (int64_t)(sc.tiles - 1 - nxt) * (32 * GPT) + g * 32 + lane;
+                if (j < a.n) prefetch_l2(a.recs + __ldg(a.perm + j));
+            }
+        };
+        const CamExt *ce = PM == kProjFullJ ? reinterpret_cast<const CamExt *>(cs + a.vcount) : nullptr;
+        const TilePart tp = {0, a.vcount, nullptr, nullptr, 1};
+        score_tile<PM, false, GPT>(a, cs, ce, (int64_t)(sc.tiles - 1 - cur) * (32 * GPT), tp, slot, take_next, cnt);
+        cur = nxt;
+    }
+}
+
+// The batched form: one persistent launch over the tiles of many scenes.  A
+// CTA stays with a scene, its cameras staged once by TMA, while the scene has
+// tiles left: its warps draw them one by one, with no barrier in between, and
+// the CTAs' first scenes are dealt in proportion to their work (tiles x
+// views).  Then it goes on to the next scene that has tiles left.  So a CTA
+// meets barriers a few times a launch, where items of up to 32 tiles had its
+// warps wait for the slowest at every item's end: 12 scenes of 0.09-1.9M
+// primitives (bfloat16, 81-298 views) 1.55 -> 1.36 ms a score launch.
+// Every tile is scored by score_tile exactly as in k_score, so a scene's
+// scores are the same alone and in a batch; scenes may differ in storage type
+// (the records are float32) and in flags.  PM: the projection mode when every
+// scene has the Eq. 17 one (the other two's code would cost registers), or
+// kProjAny.
+constexpr int kProjAny = -1;
+
+template <int PM, int GPT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_score_batch(BatchLaunch b)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ int s_scene, s_ok, s_wt;
-    __shared__ long long s_base;
+    __shared__ BatchScene s_sc;
+    __shared__ int s_first, s_off, s_ok;
     __shared__ WarpSlot s_slot[THREADS / 32];
     CamRec *cs = reinterpret_cast<CamRec *>(smem_raw);
-    if (threadIdx.x == 0) mbar_init(&bar, 1);
-    __syncthreads();
-    unsigned long long cnt[kCountSlots];
-    int cur = -1;
-    uint32_t phase = 0;
-    const int lane = threadIdx.x & 31;
     WarpSlot *slot = &s_slot[__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0)];  // a uniform address
-    const int64_t tile = (int64_t)THREADS * GPT * b.rounds;  // primitives per item
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        const long long at = (long long)((double)b.work[b.n_scenes] * (blockIdx.x + 0.5) / gridDim.x);
+        int lo = 0, hi = b.n_scenes - 1;  // last scene whose work begins at or before this CTA's share
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (b.work[mid] <= at) lo = mid; else hi = mid - 1;
+        }
+        s_first = lo;
+    }
+    __syncthreads();
+    int scene = s_first;
+    uint32_t phase = 0;
     for (;;) {
-        if (threadIdx.x == 0) {
-            s_wt = 0;
-            const unsigned long long item = atomicAdd(b.counter, 1ull);
-            int sidx = -1;
-            long long base = 0;
-            if ((long long)item < b.total_tiles) {
-                int lo = 0, hi = b.n_scenes - 1;  // last scene whose first tile <= item
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (b.tile_begin[mid] <= (long long)item) lo = mid; else hi = mid - 1;
-                }
-                sidx = lo;
-                base = ((long long)item - b.tile_begin[lo]) * tile;
+        // the nearest scene from here on that has tiles left
+        if (threadIdx.x == 0) s_off = b.n_scenes;
+        __syncthreads();
+        for (int k = threadIdx.x; k < b.n_scenes; k += THREADS) {
+            const int s = scene + k < b.n_scenes ? scene + k : scene + k - b.n_scenes;
+            if ((int64_t)__ldcg(b.next + s) * (32 * GPT) < b.scenes[s].n) {
+                atomicMin(&s_off, k);
+                break;
             }
-            s_scene = sidx;
-            s_base = base;
         }
         __syncthreads();
-        const int sidx = s_scene;
-        const int64_t base = s_base;
-        if (sidx < 0) break;
-        const ScoreLaunch &a = b.scenes[sidx];
-        if (sidx != cur) {
-            if (threadIdx.x == 0) {
-                s_ok = cams_stageable(a);
-                if (s_ok) {
-                    fence_proxy_async_shared();
-                    stage_cams(a, smem_raw, &bar);
-                } else {
-                    set_status(a.status, kEinval);
-                }
+        if (s_off >= b.n_scenes) break;  // every tile of every scene has been drawn
+        scene = scene + s_off < b.n_scenes ? scene + s_off : scene + s_off - b.n_scenes;
+        for (int k = threadIdx.x; k < (int)(sizeof(ScoreLaunch) / 8); k += THREADS)
+            reinterpret_cast<uint64_t *>(&s_sc.a)[k] = reinterpret_cast<const uint64_t *>(b.scenes + scene)[k];
+        __syncthreads();
+        const ScoreLaunch &a = s_sc.a;
+        if (threadIdx.x == 0) {
+            s_sc.next = b.next + scene;
+            s_sc.tiles = (unsigned)((a.n + 32 * GPT - 1) / (32 * GPT));
+            s_ok = cams_stageable(a);
+            if (s_ok) {
+                fence_proxy_async_shared();
+                stage_cams(a, smem_raw, &bar);
+            } else {
+                set_status(a.status, kEinval);
+                atomicMax(b.next + scene, 0x7fffffffu);  // the scene is left unscored
             }
-            __syncthreads();
-            if (!s_ok) {
-                cur = -1;
-                continue;  // the tile is left unscored; the loop's first barrier orders s_scene
-            }
-            if (!mbar_wait_bounded(&bar, phase)) {
-                // the item left unscored belongs to this scene: its own
-                // status word carries the error, and so does the launch's
-                set_status(a.status, kEtimeout);
-                set_status(b.status, kEtimeout);
-                mbar_wait_bounded(&bar, phase);
-                return;
-            }
-            phase ^= 1u;
-            cur = sidx;
         }
-        const SceneConsts sc = *a.consts;
-        const int pm = proj_mode(a.flags);
-        const CamExt *ce = reinterpret_cast<const CamExt *>(smem_raw + (size_t)a.vcount * sizeof(CamRec));
-        // the item's warp tiles go to whichever warp of the CTA is free
-        const int wtiles = (int)((min(tile, a.n - base) + 32 * GPT - 1) / (32 * GPT));
-        for (;;) {
-            int t = 0;
-            if (lane == 0) t = atomicAdd(&s_wt, 1);
-            t = __shfl_sync(0xffffffffu, t, 0);
-            if (t >= wtiles) break;
-            const int64_t wbase = base + (int64_t)t * (32 * GPT);
-            const TilePart tp = {0, a.vcount, nullptr, nullptr, 1};
-            if (pm == kProjEq17)
-                score_tile<kProjEq17, false, GPT>(a, cs, ce, sc, wbase, tp, slot, [] {}, cnt);
-            else if (pm == kProjNone)
-                score_tile<kProjNone, false, GPT>(a, cs, ce, sc, wbase, tp, slot, [] {}, cnt);
-            else
-                score_tile<kProjFullJ, false, GPT>(a, cs, ce, sc, wbase, tp, slot, [] {}, cnt);
+        __syncthreads();
+        if (!s_ok) continue;
+        if (!mbar_wait_bounded(&bar, phase)) {
+            // the tiles left unscored belong to this scene: its own status
+            // word carries the error, and so does the launch's
+            set_status(a.status, kEtimeout);
+            set_status(b.status, kEtimeout);
+            mbar_wait_bounded(&bar, phase);
+            return;
         }
-        __syncthreads();  // the cameras, s_scene and s_wt are free again
+        phase ^= 1u;
+        const int pm = PM == kProjAny ? proj_mode(a.flags) : PM;
+        if (pm == kProjEq17)
+            score_scene<kProjEq17, GPT>(s_sc, cs, slot);
+        else if (pm == kProjNone)
+            score_scene<kProjNone, GPT>(s_sc, cs, slot);
+        else
+            score_scene<kProjFullJ, GPT>(s_sc, cs, slot);
+        __syncthreads();  // the cameras and s_sc are free again
     }
 }
 
@@ -872,18 +906,23 @@ cudaError_t launch_score(const ScoreLaunch &a, int gpt, const Chain &s)
     return launch_chained(fn, a.grid, kScoreThreads, smem, s, a);
 }
 
-static const void *batch_fn(const ScoreShape &sh)
+using BatchFn = void (*)(BatchLaunch);
+
+template <int PM>
+static BatchFn batch_fn_pm(const ScoreShape &sh)
 {
-    if (sh.threads == 128)
-        return sh.gpt == 1 ? reinterpret_cast<const void *>(&k_score_batch<1, 128>)
-                           : reinterpret_cast<const void *>(&k_score_batch<2, 128>);
-    return sh.gpt == 1 ? reinterpret_cast<const void *>(&k_score_batch<1, 256>)
-                       : reinterpret_cast<const void *>(&k_score_batch<2, 256>);
+    if (sh.threads == 128) return sh.gpt == 1 ? &k_score_batch<PM, 1, 128> : &k_score_batch<PM, 2, 128>;
+    return sh.gpt == 1 ? &k_score_batch<PM, 1, 256> : &k_score_batch<PM, 2, 256>;
 }
 
-int score_batch_grid(int num_sms, size_t smem, const ScoreShape &sh)
+static BatchFn batch_fn(const ScoreShape &sh, bool eq17)
 {
-    const void *fn = batch_fn(sh);
+    return eq17 ? batch_fn_pm<kProjEq17>(sh) : batch_fn_pm<kProjAny>(sh);
+}
+
+int score_batch_grid(int num_sms, size_t smem, bool eq17, const ScoreShape &sh)
+{
+    const BatchFn fn = batch_fn(sh, eq17);
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sh.threads, smem) != cudaSuccess || per_sm < 1) {
@@ -896,14 +935,13 @@ int score_batch_grid(int num_sms, size_t smem, const ScoreShape &sh)
 
 cudaError_t launch_score_batch(const BatchLaunch &b, size_t smem, int grid, const ScoreShape &sh, cudaStream_t s)
 {
-    const void *fn = batch_fn(sh);
+    const BatchFn fn = batch_fn(sh, b.eq17);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    BatchLaunch arg = b;
-    void *args[] = {&arg};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(sh.threads), args, smem, s);
+    fn<<<grid, sh.threads, smem, s>>>(b);
+    return cudaGetLastError();
 }
 
 }  // namespace refine

@@ -88,10 +88,10 @@ struct QJob {
 
 struct RoundRes {  // one entry of the round ring
     ScoreLaunch *h_launch = nullptr;  // page-locked [slots]
-    long long *h_tb = nullptr;        // page-locked [slots + 1]
+    long long *h_work = nullptr;      // page-locked [slots + 1]
     ScoreLaunch *d_launch = nullptr;
-    long long *d_tb = nullptr;
-    unsigned long long *d_counter = nullptr;
+    long long *d_work = nullptr;
+    unsigned *d_next = nullptr;
     int *d_status = nullptr;
     cudaEvent_t scored = nullptr;
 };
@@ -318,40 +318,40 @@ cudaEvent_t issue_scoring(refine_queue *q, std::vector<QJob *> &round)
     refine_status st = REFINE_OK;
     if (!live.empty()) {
         size_t smem = 0;
-        std::vector<int64_t> ns;
+        long long tiles32 = 0;
+        bool eq17 = true;
+        R.h_work[0] = 0;
         for (size_t i = 0; i < live.size(); ++i) {
             QJob *j = live[i];
             R.h_launch[i] = make_score_launch(&j->scene, j->plan, j->sx, j->params, 0, j->scores, nullptr, false,
                                               j->status);
             smem = std::max(smem, cams_smem(R.h_launch[i].vcount, j->params.flags));
-            ns.push_back(j->req.n);
+            tiles32 += (j->req.n + 31) / 32;
+            eq17 = eq17 && proj_mode(j->params.flags) == kProjEq17;
+            R.h_work[i + 1] = R.h_work[i] + batch_work(j->req.n, R.h_launch[i].vcount);
         }
-        const int full_grid = score_batch_grid(q->pc.num_sms, smem, q->shape);
-        const int rounds = batch_rounds(q->shape, ns.data(), (int)ns.size(), full_grid);
-        const long long tile = batch_tile(q->shape, rounds);
-        R.h_tb[0] = 0;
-        for (size_t i = 0; i < live.size(); ++i) R.h_tb[i + 1] = R.h_tb[i] + (ns[i] + tile - 1) / tile;
+        // a round with fewer tiles than warp slots takes tiles of 32 (score_plan has the figures)
+        ScoreShape shape = q->shape;
+        if (shape.gpt == 2 && tiles32 / 2 < (long long)q->pc.num_sms * 32) shape.gpt = 1;
+        const int full_grid = score_batch_grid(q->pc.num_sms, smem, eq17, shape);
         const int k = (int)live.size();
         cudaStream_t m = q->score_stream;
         cudaError_t e = cudaMemcpyAsync(R.d_launch, R.h_launch, sizeof(ScoreLaunch) * k, cudaMemcpyHostToDevice, m);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(R.d_tb, R.h_tb, sizeof(long long) * (k + 1), cudaMemcpyHostToDevice, m);
-        if (e == cudaSuccess) e = cudaMemsetAsync(R.d_counter, 0, sizeof(unsigned long long), m);
+            e = cudaMemcpyAsync(R.d_work, R.h_work, sizeof(long long) * (k + 1), cudaMemcpyHostToDevice, m);
+        if (e == cudaSuccess) e = cudaMemsetAsync(R.d_next, 0, sizeof(unsigned) * k, m);
         if (e == cudaSuccess) e = cudaMemsetAsync(R.d_status, 0, sizeof(int), m);
         for (QJob *j : live)
             if (e == cudaSuccess) e = cudaStreamWaitEvent(m, q->prepped[j->slot], 0);
         if (e == cudaSuccess) {
             BatchLaunch bl;
             bl.scenes = R.d_launch;
-            bl.tile_begin = R.d_tb;
+            bl.work = R.d_work;
             bl.n_scenes = k;
-            bl.total_tiles = R.h_tb[k];
-            bl.counter = R.d_counter;
+            bl.next = R.d_next;
+            bl.eq17 = eq17;
             bl.status = R.d_status;
-            bl.rounds = rounds;
-            int grid = full_grid;
-            if (grid > bl.total_tiles) grid = (int)bl.total_tiles;
-            e = launch_score_batch(bl, smem, grid, q->shape, m);
+            e = launch_score_batch(bl, smem, batch_grid(shape, full_grid, tiles32), shape, m);
             if (e == cudaSuccess) q->launches.fetch_add(1, std::memory_order_relaxed);
         }
         // Further camera blocks of requests with more views than one block:
@@ -684,7 +684,7 @@ refine_status refine_queue_create(refine_ctx *c, uint64_t hbm_budget_bytes, int3
     if (e == cudaSuccess) e = cudaEventSynchronize(q->ev_ref);
     if (e == cudaSuccess) e = cudaMallocHost(&q->slot_host, sizeof(SlotHost) * max_slots);
     const size_t per_dev = carve_size({sizeof(ScoreLaunch) * (size_t)max_slots, sizeof(long long) * (max_slots + 1),
-                                       sizeof(unsigned long long), sizeof(int)});
+                                       sizeof(unsigned) * (size_t)max_slots, sizeof(int)});
     const size_t per_host = carve_size({sizeof(ScoreLaunch) * (size_t)max_slots, sizeof(long long) * (max_slots + 1)});
     if (e == cudaSuccess) e = cudaMalloc(&q->ring_dev, per_dev * max_slots);
     if (e == cudaSuccess) e = cudaMallocHost(&q->ring_host, per_host * max_slots);
@@ -693,12 +693,12 @@ refine_status refine_queue_create(refine_ctx *c, uint64_t hbm_budget_bytes, int3
         RoundRes &R = q->ring[r];
         Carver dv(static_cast<char *>(q->ring_dev) + per_dev * r);
         R.d_launch = dv.take<ScoreLaunch>(max_slots);
-        R.d_tb = dv.take<long long>(max_slots + 1);
-        R.d_counter = dv.take<unsigned long long>(1);
+        R.d_work = dv.take<long long>(max_slots + 1);
+        R.d_next = dv.take<unsigned>(max_slots);
         R.d_status = dv.take<int>(1);
         Carver hv(static_cast<char *>(q->ring_host) + per_host * r);
         R.h_launch = hv.take<ScoreLaunch>(max_slots);
-        R.h_tb = hv.take<long long>(max_slots + 1);
+        R.h_work = hv.take<long long>(max_slots + 1);
         e = cudaEventCreateWithFlags(&R.scored, cudaEventDisableTiming);
     }
     if (e != cudaSuccess) {

@@ -365,13 +365,12 @@ struct refine_batch {
     // scene's passes run in order, as refine_score runs them.
     struct Level {
         ScoreLaunch *d_launch = nullptr;       // [scenes] this pass of each scene taking part
-        long long *d_tile_begin = nullptr;     // [scenes + 1]
-        unsigned long long *d_counter = nullptr;
+        long long *d_work = nullptr;           // [scenes + 1]
+        unsigned *d_next = nullptr;            // [scenes]
         std::vector<int> jobs;                 // the scenes taking part
-        long long total_tiles = 0;
+        long long tiles32 = 0;                 // 32-primitive groups of the level
         size_t smem = 0;                       // largest camera block of the level, in bytes
         int grid = 1;
-        int rounds = kBatchRounds;             // item size (batch_rounds)
     };
     std::vector<Level> levels;
     ScoreShape shape;
@@ -405,7 +404,7 @@ refine_status batch_record(refine_batch *b)
     cudaEvent_t fork = b->events[0], fork2 = b->events[1 + L];
     e = cudaSuccess;
     for (const refine_batch::Level &lv : b->levels)
-        if (e == cudaSuccess) e = cudaMemsetAsync(lv.d_counter, 0, sizeof(unsigned long long), m);
+        if (e == cudaSuccess) e = cudaMemsetAsync(lv.d_next, 0, sizeof(unsigned) * lv.jobs.size(), m);
     if (e == cudaSuccess) e = cudaEventRecord(fork, m);
     for (int l = 0; l < L && e == cudaSuccess && !st; ++l) {
         cudaStream_t ls = b->lanes[l];
@@ -420,12 +419,11 @@ refine_status batch_record(refine_batch *b)
         if (e != cudaSuccess || st) break;
         BatchLaunch bl;
         bl.scenes = lv.d_launch;
-        bl.tile_begin = lv.d_tile_begin;
+        bl.work = lv.d_work;
         bl.n_scenes = (int)lv.jobs.size();
-        bl.total_tiles = lv.total_tiles;
-        bl.counter = lv.d_counter;
+        bl.next = lv.d_next;
+        bl.eq17 = proj_mode(b->params.flags) == kProjEq17;
         bl.status = c->d_status;
-        bl.rounds = lv.rounds;
         e = launch_score_batch(bl, lv.smem, lv.grid, b->shape, m);
         if (e == cudaSuccess) ++launches;
     }
@@ -465,24 +463,10 @@ refine_status batch_record(refine_batch *b)
     return REFINE_OK;
 }
 
-// Tile prefix of a level for the work-item size of `sh`, copied to the
-// device (on `s`, or synchronously when s is NULL), and its grid.
-cudaError_t set_level_tiles(refine_batch *b, refine_batch::Level &lv, const ScoreShape &sh, cudaStream_t s)
+// Grid of a level for the shape `sh`.
+void set_level_grid(refine_batch *b, refine_batch::Level &lv, const ScoreShape &sh)
 {
-    std::vector<int64_t> ns;
-    for (int j : lv.jobs) ns.push_back(b->jobs[j].scene.n);
-    const int full_grid = score_batch_grid(b->ctx->num_sms, lv.smem, sh);
-    lv.rounds = batch_rounds(sh, ns.data(), (int)ns.size(), full_grid);
-    const long long tile = batch_tile(sh, lv.rounds);
-    std::vector<long long> tb(lv.jobs.size() + 1, 0);
-    for (size_t k = 0; k < lv.jobs.size(); ++k) tb[k + 1] = tb[k] + (ns[k] + tile - 1) / tile;
-    lv.total_tiles = tb.back();
-    lv.grid = full_grid;
-    if (lv.grid > lv.total_tiles) lv.grid = (int)lv.total_tiles;
-    if (lv.grid < 1) lv.grid = 1;
-    const size_t bytes = sizeof(long long) * tb.size();
-    return s ? cudaMemcpyAsync(lv.d_tile_begin, tb.data(), bytes, cudaMemcpyHostToDevice, s)
-             : cudaMemcpy(lv.d_tile_begin, tb.data(), bytes, cudaMemcpyHostToDevice);
+    lv.grid = batch_grid(sh, score_batch_grid(b->ctx->num_sms, lv.smem, proj_mode(b->params.flags) == kProjEq17, sh), lv.tiles32);
 }
 
 void batch_free(refine_batch *b)
@@ -543,7 +527,7 @@ refine_status refine_batch_create(refine_ctx *c, const refine_job *jobs, int32_t
     }
     for (int lv = 0; lv < max_passes; ++lv)
         total += carve_size({sizeof(ScoreLaunch) * (size_t)S, sizeof(long long) * (size_t)(S + 1),
-                             sizeof(unsigned long long)});
+                             sizeof(unsigned) * (size_t)S});
     cudaError_t e = cudaMalloc(&b->scratch, total);
     if (e != cudaSuccess) {
         delete b;
@@ -557,8 +541,8 @@ refine_status refine_batch_create(refine_ctx *c, const refine_job *jobs, int32_t
     b->levels.resize(max_passes);
     for (refine_batch::Level &lv : b->levels) {
         lv.d_launch = cv.take<ScoreLaunch>(S);
-        lv.d_tile_begin = cv.take<long long>(S + 1);
-        lv.d_counter = cv.take<unsigned long long>(1);
+        lv.d_work = cv.take<long long>(S + 1);
+        lv.d_next = cv.take<unsigned>(S);
     }
     for (int j = 0; j < S; ++j) {
         b->sx.push_back(carve_scene(cv, b->plans[j]));
@@ -571,6 +555,7 @@ refine_status refine_batch_create(refine_ctx *c, const refine_job *jobs, int32_t
     for (int l = 0; l < max_passes && e == cudaSuccess; ++l) {
         refine_batch::Level &lv = b->levels[l];
         std::vector<ScoreLaunch> hl;
+        std::vector<long long> work(1, 0);
         for (int j = 0; j < S; ++j) {
             if (b->plans[j].passes <= l) continue;
             const int v0 = l * b->plans[j].vpp;
@@ -578,9 +563,13 @@ refine_status refine_batch_create(refine_ctx *c, const refine_job *jobs, int32_t
                                            false, c->d_status));
             lv.jobs.push_back(j);
             lv.smem = std::max(lv.smem, cams_smem(hl.back().vcount, p.flags));
+            lv.tiles32 += (jobs[j].scene.n + 31) / 32;
+            work.push_back(work.back() + batch_work(jobs[j].scene.n, hl.back().vcount));
         }
         e = cudaMemcpy(lv.d_launch, hl.data(), sizeof(ScoreLaunch) * hl.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = set_level_tiles(b, lv, b->shape, nullptr);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(lv.d_work, work.data(), sizeof(long long) * work.size(), cudaMemcpyHostToDevice);
+        set_level_grid(b, lv, b->shape);
     }
     const int L = std::min(8, S);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->main, cudaStreamNonBlocking);
@@ -745,8 +734,7 @@ refine_status refine_autotune(refine_ctx *c, const refine_job *jobs, int32_t n_j
                     sh.threads = threads;
                     sh.ctas_per_sm = cap;
                     sh.views_per_pass = vpp;
-                    for (refine_batch::Level &lv : b->levels)
-                        if (e == cudaSuccess) e = set_level_tiles(b, lv, sh, m);
+                    for (refine_batch::Level &lv : b->levels) set_level_grid(b, lv, sh);
                     // one warm-up run, then `reps` timed runs of every level's launch
                     for (int r = -1; r < reps && e == cudaSuccess; ++r) {
                         if (r == 0) e = cudaEventRecord(e0, m);
@@ -754,13 +742,12 @@ refine_status refine_autotune(refine_ctx *c, const refine_job *jobs, int32_t n_j
                             if (e != cudaSuccess) break;
                             BatchLaunch bl;
                             bl.scenes = lv.d_launch;
-                            bl.tile_begin = lv.d_tile_begin;
+                            bl.work = lv.d_work;
                             bl.n_scenes = (int)lv.jobs.size();
-                            bl.total_tiles = lv.total_tiles;
-                            bl.counter = lv.d_counter;
+                            bl.next = lv.d_next;
+                            bl.eq17 = proj_mode(b->params.flags) == kProjEq17;
                             bl.status = c->d_status;
-                            bl.rounds = lv.rounds;
-                            e = cudaMemsetAsync(lv.d_counter, 0, sizeof(unsigned long long), m);
+                            e = cudaMemsetAsync(lv.d_next, 0, sizeof(unsigned) * lv.jobs.size(), m);
                             if (e == cudaSuccess) e = launch_score_batch(bl, lv.smem, lv.grid, sh, m);
                         }
                     }
