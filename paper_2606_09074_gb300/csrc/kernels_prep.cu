@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include "internal.h"
+#include "rows.cuh"
 
 namespace refine {
 
@@ -328,32 +329,71 @@ struct FeatTerms {
     float y, gem, mg, mc, alpha;
 };
 
+// The rows of one primitive: |SH|^2 summed row by row, and the others.
+struct PrimRows {
+    float sq, x, y, z, ls0, ls1, ls2, q0, q1, q2, q3, logit, dc0, dc1, dc2;
+};
+
+template <typename L>
+__device__ __forceinline__ PrimRows read_rows(L &&ld)  // ld(r): row r of 59
+{
+    PrimRows p;
+    p.sq = 0.f;
+#pragma unroll
+    for (int r = 11; r < 59; ++r) {
+        const float x = ld(r);
+        if (r == 11) p.dc0 = x;
+        if (r == 12) p.dc1 = x;
+        if (r == 13) p.dc2 = x;
+        p.sq = fmaf(x, x, p.sq);
+    }
+    p.x = ld(0); p.y = ld(1); p.z = ld(2);
+    p.ls0 = ld(3); p.ls1 = ld(4); p.ls2 = ld(5);
+    p.q0 = ld(6); p.q1 = ld(7); p.q2 = ld(8); p.q3 = ld(9);
+    p.logit = ld(10);
+    return p;
+}
+
 template <int DT>
 __device__ __forceinline__ FeatTerms feature_one(const FeatureArgs<DT> &f, const uint16_t *hilbert, const OrderGrid &og,
-                                                 int64_t i, float &bad, bool &zero_q, uint2 &key_slot)
+                                                 int64_t i, const PrimRows &p, float &bad, bool &zero_q, uint2 &key_slot)
 {
-    float sq = 0.f;
-#pragma unroll
-    for (int r = 8; r < 56; ++r) {
-        const float x = f.attr.ld(r, i);
-        sq = fmaf(x, x, sq);
-    }
-    const float x = __ldg(f.pos + i), y = __ldg(f.pos + f.S + i), z = __ldg(f.pos + 2 * f.S + i);
-    const float ls0 = f.attr.ld(0, i), ls1 = f.attr.ld(1, i), ls2 = f.attr.ld(2, i);
     float4 ra, rb, rc, rd;
     FeatTerms t;
-    bad = primitive_record(bad, x, y, z, ls0, ls1, ls2, f.attr.ld(3, i), f.attr.ld(4, i), f.attr.ld(5, i),
-                           f.attr.ld(6, i), f.attr.ld(7, i), sq, f.eta, ra, rb, rc, rd, t.gem, zero_q);
-    t.y = luma_term(f.l0, f.l1, f.l2, f.attr.ld(8, i), f.attr.ld(9, i), f.attr.ld(10, i));
+    bad = primitive_record(bad, p.x, p.y, p.z, p.ls0, p.ls1, p.ls2, p.q0, p.q1, p.q2, p.q3, p.logit, p.sq, f.eta, ra, rb,
+                           rc, rd, t.gem, zero_q);
+    t.y = luma_term(f.l0, f.l1, f.l2, p.dc0, p.dc1, p.dc2);
     t.alpha = rd.y;
     t.mg = rd.z;
     t.mc = rd.w;
     PrimRec *r = f.recs + i;
     r->a = ra; r->b = rb; r->c = rc; r->d = rd;
-    key_slot.x = order_key(hilbert, og, f.cell_bits, x, y, z, fmaxf(ls0, fmaxf(ls1, ls2)));
+    key_slot.x = order_key(hilbert, og, f.cell_bits, p.x, p.y, p.z, fmaxf(p.ls0, fmaxf(p.ls1, p.ls2)));
     key_slot.y = atomicAdd(&f.counts[key_slot.x], 1u);  // the slot in its cell
     return t;
 }
+
+// Primitive i's rows by loads of its own (coalesced over the warp).
+template <int DT>
+__device__ __forceinline__ PrimRows load_rows(const FeatureArgs<DT> &f, int64_t i)
+{
+    return read_rows([&](int r) { return r < 3 ? __ldg(f.pos + r * f.S + i) : f.attr.ld(r - 3, i); });
+}
+
+// The sums of one thread.
+struct FeatAcc {
+    float s[kFeatSums];
+    __device__ __forceinline__ void add(const FeatTerms &t)
+    {
+        s[0] += t.y;
+        s[1] = fmaf(t.y, t.y, s[1]);
+        s[2] = fmaf(t.alpha, 1.f - t.alpha, s[2]);
+        s[3] += t.gem;
+        s[4] += t.mg;
+        s[5] += t.mc;
+        s[6] += t.alpha;
+    }
+};
 
 template <int DT>
 __global__ void __launch_bounds__(kFeatCol, 4) k_features(FeatureArgs<DT> f)
@@ -364,32 +404,98 @@ __global__ void __launch_bounds__(kFeatCol, 4) k_features(FeatureArgs<DT> f)
     load_hilbert(hilbert);
     const OrderGrid og = *f.grid;
     __syncthreads();
-    float s[kFeatSums];
-#pragma unroll
-    for (int k = 0; k < kFeatSums; ++k) s[k] = 0.f;
+    FeatAcc acc = {};
     float bad = 0.f;
     bool zero_q = false;
     uint2 ks = make_uint2(0u, 0u);
     int64_t last = -1;  // its (key, slot) is stored in the next turn
     for (int64_t i = (int64_t)blockIdx.x * kFeatCol + threadIdx.x; i < f.n; i += (int64_t)gridDim.x * kFeatCol) {
         uint2 next;
-        const FeatTerms t = feature_one<DT>(f, hilbert, og, i, bad, zero_q, next);
+        const FeatTerms t = feature_one<DT>(f, hilbert, og, i, load_rows<DT>(f, i), bad, zero_q, next);
         if (last >= 0) f.cell[last] = ks;
         ks = next;
         last = i;
-        s[0] += t.y;
-        s[1] = fmaf(t.y, t.y, s[1]);
-        s[2] = fmaf(t.alpha, 1.f - t.alpha, s[2]);
-        s[3] += t.gem;
-        s[4] += t.mg;
-        s[5] += t.mc;
-        s[6] += t.alpha;
+        acc.add(t);
     }
     if (last >= 0) f.cell[last] = ks;
     if (!isfinite(bad)) set_status(f.status, kEnonfinite);
     if (zero_q) set_status(f.status, kEinval);
 #pragma unroll
-    for (int k = 0; k < kFeatSums; ++k) red[k * kFeatRedRow + threadIdx.x] = s[k];
+    for (int k = 0; k < kFeatSums; ++k) red[k * kFeatRedRow + threadIdx.x] = acc.s[k];
+    __syncthreads();
+    feature_block_sums(red, f.partials);
+}
+
+// The same with the rows of 256 primitives at a time brought into shared
+// memory by bulk copies (RowTile), for bfloat16 rows: their 2-byte loads, 64
+// bytes a warp, leave too few bytes in flight (four CTAs' tiles are 130 KB an
+// SM).  The next tile is issued as soon as every thread has read the current
+// one, so it arrives while the records are formed.  ALIGNED: every row starts
+// on 16 bytes (the stride is a multiple of 8), so places are constants.  3.5M
+// bfloat16 primitives: 157 -> 142 us (4.6 TB/s; what is left is the latency of
+// a primitive's arithmetic at 32 warps an SM); the same with all copies issued
+// by one warp 160 us.
+template <int DT, bool ALIGNED>
+__global__ void __launch_bounds__(kFeatCol, 4) k_features_bulk(FeatureArgs<DT> f)
+{
+    using Rows = RowTile<DT, kFeatCol>;
+    extern __shared__ __align__(16) unsigned char tile[];
+    __shared__ float red[kFeatSums * kFeatRedRow];
+    __shared__ __align__(4) uint16_t hilbert[24 * 64];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int row_base[59];
+    load_hilbert(hilbert);
+    const Rows in{reinterpret_cast<const char *>(f.pos), reinterpret_cast<const char *>(f.attr.f), f.S};
+    const int t = threadIdx.x;
+    if (!ALIGNED && t < 59) row_base[t] = Rows::place(t) + (int)in.mis(t);
+    if (t == 0) mbar_init(&bar, 1);
+    after(pdl_wait(), f.grid);  // the rows are older than the kernel before this one
+    const OrderGrid og = *f.grid;
+    __syncthreads();
+    auto stage = [&](int64_t i0) {
+        const int count = (int)min((int64_t)kFeatCol, f.n - i0);
+        in.template stage<kFeatCol / 32>(tile, i0, count, &bar);
+        if (!ALIGNED && Rows::at_end(i0, f.n)) in.template rest<kFeatCol / 32>(tile, i0, count);
+    };
+    FeatAcc acc = {};
+    float bad = 0.f;
+    bool zero_q = false;
+    uint2 ks = make_uint2(0u, 0u);
+    int64_t last = -1;  // its (key, slot) is stored in the next turn
+    const int64_t step = (int64_t)gridDim.x * kFeatCol;
+    uint32_t phase = 0;
+    int64_t i0 = (int64_t)blockIdx.x * kFeatCol;
+    if (i0 < f.n) stage(i0);
+    for (; i0 < f.n; i0 += step) {
+        if (!ALIGNED && Rows::at_end(i0, f.n)) __syncthreads();  // what plain loads brought
+        if (!mbar_wait_bounded(&bar, phase)) {
+            set_status(f.status, kEtimeout);
+            mbar_wait_bounded(&bar, phase);  // give the copies a second bound before leaving
+            return;
+        }
+        phase ^= 1u;
+        const PrimRows p = read_rows([&](int r) {
+            const unsigned char *a = tile + (ALIGNED ? Rows::place(r) : row_base[r]) + Rows::size(r) * t;
+            return Rows::f32(r) ? *reinterpret_cast<const float *>(a)
+                                : __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short *>(a) << 16);
+        });
+        __syncthreads();  // the tile is free
+        if (i0 + step < f.n) stage(i0 + step);
+        const int64_t i = i0 + t;
+        if (i < f.n) {
+            uint2 next;
+            const FeatTerms v = feature_one<DT>(f, hilbert, og, i, p, bad, zero_q, next);
+            if (last >= 0) f.cell[last] = ks;
+            ks = next;
+            last = i;
+            acc.add(v);
+        }
+    }
+    if (last >= 0) f.cell[last] = ks;
+    if (!isfinite(bad)) set_status(f.status, kEnonfinite);
+    if (zero_q) set_status(f.status, kEinval);
+#pragma unroll
+    for (int k = 0; k < kFeatSums; ++k) red[k * kFeatRedRow + t] = acc.s[k];
     __syncthreads();
     feature_block_sums(red, f.partials);
 }
@@ -423,7 +529,7 @@ __global__ void __launch_bounds__(kFeatSmallThreads, 1) k_features_small(Feature
         const int c = u * kGroups + grp;
         const int64_t i = first + c * step;
         if (i < f.n) {
-            const FeatTerms v = feature_one<DT>(f, hilbert, og, i, bad, zero_q, ks[u]);
+            const FeatTerms v = feature_one<DT>(f, hilbert, og, i, load_rows<DT>(f, i), bad, zero_q, ks[u]);
             val[0][c][t] = v.y;
             val[1][c][t] = v.alpha;
             val[2][c][t] = v.gem;
@@ -487,7 +593,14 @@ static cudaError_t launch_features_t(const FeatureLaunch &l, int num_sms, const 
     const int nb = feature_blocks(l.n);
     if (nb <= num_sms && l.n <= (int64_t)nb * kFeatCol * kFeatCols)
         return launch_chained(k_features_small<DT>, nb, kFeatSmallThreads, 0, s, f);
-    return launch_chained(k_features<DT>, nb, kFeatCol, 0, s, f);
+    if constexpr (DT != REFINE_F32) {
+        const size_t smem = RowTile<DT, kFeatCol>::kBytes;
+        static_assert(RowTile<DT, kFeatCol>::kBytes + 12 * 1024 < 48 * 1024, "no opt-in shared memory");
+        if (l.stride % 8 == 0) return launch_chained(k_features_bulk<DT, true>, nb, kFeatCol, smem, s, f);
+        return launch_chained(k_features_bulk<DT, false>, nb, kFeatCol, smem, s, f);
+    } else {
+        return launch_chained(k_features<DT>, nb, kFeatCol, 0, s, f);
+    }
 }
 
 cudaError_t launch_features(const FeatureLaunch &f, int dtype, int num_sms, const Chain &s)

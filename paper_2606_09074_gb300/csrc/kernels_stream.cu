@@ -3,26 +3,22 @@
 // One CTA of 8 warps takes a unit of consecutive primitives (128 with float32
 // rows, 256 with bfloat16 rows) at a time.  The unit's span of each of the 59
 // rows, 512 contiguous bytes (1 KB of a float32 row beside bfloat16 ones), is
-// brought into shared memory by one bulk copy (cp.async.bulk) per row, issued
-// by the lanes of warp 0 and completing on an mbarrier; meanwhile the ranks
+// brought into shared memory by one bulk copy (cp.async.bulk) per row,
+// completing on an mbarrier (RowTile); meanwhile the ranks
 // of the kept primitives are inverted (output d comes from primitive src[d]).
 // Then each warp takes every eighth row: 32 outputs are one shared-memory load
 // and one contiguous store.  A unit is 31-34 KB, so 6 CTAs fit an SM, and while
 // some wait for their unit others store theirs: about 190 KB an SM in flight
 // without holding a register.
 //
-// A bulk copy starts on 16 bytes: the row's span is widened to 16-byte
-// boundaries (row strides may be odd) and the row's offset in shared memory
-// is taken from its misalignment.  At a scene's end the widened span of the
-// last row of a buffer could leave it (of the last few rows, when the stride
-// is below 8): it is narrowed instead, and its last few elements are read by
-// plain loads.
-//
-// Measured (the kernel alone, events around it): bfloat16 rows, 3.5M primitives at ratio 0.5 160 -> 111 us (5.9
-// TB/s); float32 rows the same as the form before (3.5M 200 us, 6.2 TB/s; 1M at 0.66 60 us).  That form had a
-// warp load each row of a mask word into registers (16 float or 28 bfloat16 rows at a time) and shuffle: 64-byte
-// loads of bfloat16 rows, and registers, bounded what it had in flight.
+// Measured (the kernel alone, events around it): bfloat16 rows, 3.5M
+// primitives at ratio 0.5 160 -> 107 us (6.2 TB/s); float32 rows 200 -> 199 us
+// (3.5M, 6.3 TB/s) and 60 -> 55 us (1M at 0.66), against the form before, in
+// which a warp loaded each row of a mask word into registers (16 float or 28
+// bfloat16 rows at a time) and shuffled: 64-byte loads of bfloat16 rows, and
+// registers, bounded what it had in flight.
 #include "internal.h"
+#include "rows.cuh"
 
 namespace refine {
 
@@ -32,53 +28,12 @@ constexpr int kCmpCtas = 6;  // per SM
 
 // Primitives per unit.
 __host__ __device__ constexpr int cmp_unit(int dtype) { return dtype == REFINE_F32 ? 128 : 256; }
-// Rows of float32 elements (the means and the float32 attribute rows) and
-// their place in the tile: a row's span and 16 bytes for its misalignment.
-__host__ __device__ constexpr int cmp_f32_rows(int dtype) { return 3 + attr_f32_rows(dtype); }
-__host__ __device__ constexpr int cmp_pitch(int dtype, bool f32) { return cmp_unit(dtype) * (f32 ? 4 : 2) + 16; }
-__host__ __device__ constexpr int cmp_tile_bytes(int dtype)
-{
-    return cmp_f32_rows(dtype) * cmp_pitch(dtype, true) + (59 - cmp_f32_rows(dtype)) * cmp_pitch(dtype, false);
-}
-
-// Row r of 59 (the means, then the attribute rows): address of its element 0
-// and its element size.
-template <int DT>
-struct RowSet {
-    const char *pos, *attr;
-    int64_t S;
-    __device__ __forceinline__ static constexpr bool f32(int r) { return r < cmp_f32_rows(DT); }
-    __device__ __forceinline__ static int tile(int r)  // byte offset in the tile
-    {
-        constexpr int NF = cmp_f32_rows(DT);
-        return r < NF ? r * cmp_pitch(DT, true) : NF * cmp_pitch(DT, true) + (r - NF) * cmp_pitch(DT, false);
-    }
-    __device__ __forceinline__ const char *row(int r) const
-    {
-        constexpr int NF = attr_f32_rows(DT);
-        if (r < 3) return pos + (int64_t)r * S * 4;
-        if (r - 3 < NF) return attr + (int64_t)(r - 3) * S * 4;
-        return attr + (int64_t)NF * S * 4 + (int64_t)(r - 3 - NF) * S * 2;
-    }
-    __device__ __forceinline__ const char *end(int r) const  // of the row's buffer
-    {
-        return r < 3 ? pos + S * 12 : attr + S * (int64_t)attr_col_bytes(DT);
-    }
-};
-
-// Bytes of the bulk copy of `count` elements of row r from element i0, its
-// span starting `mis` bytes past a 16-byte boundary: up to the next boundary,
-// or down to the last when that lies past the end of the row's buffer.
-template <int DT>
-__device__ __forceinline__ uint32_t span_bytes(const RowSet<DT> &in, int r, int64_t i0, uint32_t mis, int count)
-{
-    const int es = RowSet<DT>::f32(r) ? 4 : 2;
-    const uint32_t b = mis + (uint32_t)(count * es), up = (b + 15u) & ~15u;
-    return in.row(r) + i0 * es - mis + up > in.end(r) ? b & ~15u : up;
-}
 
 template <int DT>
-__global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in, int64_t n, const uint32_t *__restrict__ mask,
+using CmpRows = RowTile<DT, cmp_unit(DT)>;
+
+template <int DT>
+__global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(CmpRows<DT> in, int64_t n, const uint32_t *__restrict__ mask,
                                                          CmpOffsets off, char *__restrict__ out_pos,
                                                          char *__restrict__ out_attr, int64_t OS,
                                                          int32_t *__restrict__ out_idx, int *status)
@@ -127,8 +82,7 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in
         return;
     }
     if (threadIdx.x < 59)
-        row_base[threadIdx.x] = RowSet<DT>::tile(threadIdx.x) +
-                                (int)(reinterpret_cast<uintptr_t>(in.row(threadIdx.x)) & 15u);
+        row_base[threadIdx.x] = CmpRows<DT>::place(threadIdx.x) + (int)in.mis(threadIdx.x);
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
 
@@ -152,41 +106,8 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in
         if (kept == 0) continue;  // the same in every thread
         const int64_t i0 = u * UNIT;
         const int count = (int)min((int64_t)UNIT, n - i0);
-        if (warp == 0) {
-            uint32_t size[2], bytes = 0;
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int r = lane + 32 * k;
-                size[k] = r < 59 ? span_bytes<DT>(in, r, i0, (uint32_t)(reinterpret_cast<uintptr_t>(in.row(r)) & 15u), count)
-                                 : 0u;
-                bytes += size[k];
-            }
-            bytes = __reduce_add_sync(0xffffffffu, bytes);
-            fence_proxy_async_shared();  // the tile was read by plain loads
-            if (lane == 0) mbar_expect_tx(&bar, bytes);
-            __syncwarp();
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int r = lane + 32 * k;
-                if (size[k] > 0u) {
-                    const char *p = in.row(r) + i0 * (RowSet<DT>::f32(r) ? 4 : 2);
-                    bulk_g2s(tile + RowSet<DT>::tile(r), p - (reinterpret_cast<uintptr_t>(p) & 15u), size[k], &bar);
-                }
-            }
-        } else if (i0 + UNIT + 8 > n) {  // what narrowed copies leave (fewer than 8 elements a row)
-            for (int r = warp - 1; r < 59; r += kCmpWarps - 1) {
-                const int es = RowSet<DT>::f32(r) ? 4 : 2;
-                const uint32_t mis = (uint32_t)(reinterpret_cast<uintptr_t>(in.row(r)) & 15u);
-                const int j = max(0, (int)span_bytes<DT>(in, r, i0, mis, count) - (int)mis) / es + lane;
-                if (j >= count) continue;
-                if (es == 4)
-                    *reinterpret_cast<float *>(tile + row_base[r] + 4 * j) =
-                        __ldg(reinterpret_cast<const float *>(in.row(r)) + i0 + j);
-                else
-                    *reinterpret_cast<unsigned short *>(tile + row_base[r] + 2 * j) =
-                        __ldg(reinterpret_cast<const unsigned short *>(in.row(r)) + i0 + j);
-            }
-        }
+        in.template stage<kCmpWarps>(tile, i0, count, &bar);
+        if (in.at_end(i0, n)) in.template rest<kCmpWarps>(tile, i0, count);
         // invert the ranks of the kept primitives
         {
             unsigned before = (unsigned)__popc(word);  // inclusive scan over the unit's words
@@ -225,7 +146,7 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(RowSet<DT> in
         phase ^= 1u;
         for (int r = warp; r < 59; r += kCmpWarps) {
             const unsigned char *t = tile + row_base[r];
-            if (RowSet<DT>::f32(r)) {
+            if (CmpRows<DT>::f32(r)) {
                 float *o = (r < 3 ? reinterpret_cast<float *>(out_pos) + (int64_t)r * OS
                                   : reinterpret_cast<float *>(out_attr) + (int64_t)(r - 3) * OS) + dst + lane;
 #pragma unroll
@@ -248,12 +169,12 @@ template <int DT>
 static cudaError_t launch_compact_t(const refine_scene &in, const uint32_t *mask, const CmpOffsets &off, float *out_pos,
                                     void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, const Chain &s)
 {
-    const size_t smem = cmp_tile_bytes(DT);
-    static_assert(cmp_tile_bytes(DT) < 40 * 1024, "no opt-in shared memory");
+    const size_t smem = CmpRows<DT>::kBytes;
+    static_assert(CmpRows<DT>::kBytes < 40 * 1024, "no opt-in shared memory");
     int64_t g = (in.n + cmp_unit(DT) - 1) / cmp_unit(DT);
     if (g > (int64_t)num_sms * kCmpCtas) g = (int64_t)num_sms * kCmpCtas;
     if (g < 1) g = 1;
-    const RowSet<DT> rows{reinterpret_cast<const char *>(in.pos), static_cast<const char *>(in.attr), in.row_stride};
+    const CmpRows<DT> rows{reinterpret_cast<const char *>(in.pos), static_cast<const char *>(in.attr), in.row_stride};
     return launch_chained(k_compact<DT>, (int)g, kCmpThreads, smem, s, rows, in.n, mask, off,
                           reinterpret_cast<char *>(out_pos), static_cast<char *>(out_attr), OS, out_idx, status);
 }
