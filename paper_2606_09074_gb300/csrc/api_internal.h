@@ -428,12 +428,19 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     // every pass but the last is like the first; the split scratch serves all
     const bool count = need_dev != nullptr;  // the counting kernel scores whole tiles of the shape
     const int vfirst = std::min(pl.V, pl.vpp), vlast = pl.V - (pl.passes - 1) * pl.vpp;
-    const ScorePlan sp0 = score_plan(c->num_sms, pl.n, vfirst, p.flags, !count, c->shape);
-    const ScorePlan sp1 = pl.multipass ? score_plan(c->num_sms, pl.n, vlast, p.flags, !count, c->shape) : sp0;
-    const size_t parts = std::max(split_part_floats(sp0, vfirst), split_part_floats(sp1, vlast));
-    const size_t counts = (size_t)std::max(sp0.split_tiles, sp1.split_tiles);
-    const size_t taken = (sizeof(unsigned long long) + sizeof(unsigned) * counts + 15) & ~size_t(15);
-    if ((st = ensure(c, c->score, scene_bytes(pl) + carve_size({sizeof(float) * parts, taken})))) return st;
+    ScorePlan sp0, sp1;
+    size_t parts = 0, taken = 0;
+    auto plan = [&](bool split) {
+        sp0 = score_plan(c->num_sms, pl.n, vfirst, p.flags, split, c->shape);
+        sp1 = pl.multipass ? score_plan(c->num_sms, pl.n, vlast, p.flags, split, c->shape) : sp0;
+        parts = std::max(split_part_floats(sp0, vfirst), split_part_floats(sp1, vlast));
+        const size_t counts = (size_t)std::max(sp0.split_tiles, sp1.split_tiles);
+        taken = (sizeof(unsigned long long) + sizeof(unsigned) * counts + 15) & ~size_t(15);
+        return ensure(c, c->score, scene_bytes(pl) + carve_size({sizeof(float) * parts, taken}));
+    };
+    st = plan(!count);
+    if (st == REFINE_ENOMEM && !count) st = plan(false);  // the split's scratch (20 MB at most) is not needed
+    if (st) return st;
     Carver cv(c->score.p);
     const SceneScratch x = carve_scene(cv, pl);
     float *part_sums = cv.take<float>(parts);
@@ -475,7 +482,7 @@ inline refine_status enqueue_select(refine_ctx *c, L &&run, const float *scores,
     SelState *ss = cv.take<SelState>(1);
     unsigned *seg = cv.take<unsigned>((n + kTieSeg - 1) / kTieSeg);
     refine_status st;
-    if (n <= kSelClusterMax) {
+    if (n <= (s.on ? kSelClusterChained : kSelClusterMax)) {
         if ((st = run(K_SEL_MASK, [&] {
                  return launch_select_cluster(scores, n, (uint32_t)n_keep, ss, mask, status, s);
              })))

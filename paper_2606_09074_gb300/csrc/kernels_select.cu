@@ -352,14 +352,18 @@ cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *s
 // words of its range.
 //
 // What it saves is launches: six stream operations become one.  The cluster
-// has 1, 2, 4 or 8 CTAs, about 12k keys each before the next size is taken.
-// Per selection, against the five kernels and a memset of the other form (a
-// chain of latencies, 33 us whatever the size): 1k scores 7.3, 10k 12.4, 50k
-// 16.5, 100k 20.6, 200k 27.6, 300k 34.9, 393k 41.1 us, hence the limit.
+// has 1, 2, 4 or 8 CTAs, 6k keys each before the next size is taken (10k scores
+// take 8.0 us with 2 CTAs, 10.3 with 1, 11.4 with 8; 24k 10.1 with 4, 12.8 with
+// 2, 12.2 with 8).  Per selection 1k scores 5.1, 10k 8.0, 50k 14.3, 100k 18.0,
+// 150k 21.9, 200k 25.3 us, against the five kernels and a memset of the other
+// form, a chain of latencies that takes 20.5 us up to 200k scores when the
+// kernels are chained and 33 us when they are not: hence the limits,
+// kSelClusterChained and kSelClusterMax.
 // ---------------------------------------------------------------------
 constexpr int kClThreads = 1024;
 constexpr int kClKeys = 32 * 1024;  // keys of a CTA at most (128 KB)
 constexpr int kClMaxCtas = 8;
+constexpr int kClFill = 6 * 1024;  // keys per CTA at which a larger cluster is taken
 constexpr int kClLoads = 6;         // loads in flight per thread
 static_assert(kSelClusterMax == (int64_t)kClKeys * kClMaxCtas, "cluster selection limit");
 
@@ -494,7 +498,7 @@ cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_kee
                                   int *status, const Chain &s)
 {
     int ctas = 1;
-    while (ctas < kClMaxCtas && n > (int64_t)12 * 1024 * ctas) ctas *= 2;
+    while (ctas < kClMaxCtas && n > (int64_t)kClFill * ctas) ctas *= 2;
     const int per = (int)(((n + ctas - 1) / ctas + 31) / 32 * 32);
     const size_t smem = sizeof(uint32_t) * (size_t)per;
     if (smem + 3 * 2048 * sizeof(unsigned) + 1024 > 48 * 1024) {

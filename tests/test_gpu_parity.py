@@ -6,6 +6,7 @@ band; primitives with a borderline pair must equal the oracle's sum with
 some choice of those pairs.  Selection and compaction on identical scores
 are bit-exact.  Masks from the oracle's own scores agree except for
 primitives within 1e-5 of the threshold or with a borderline pair."""
+import ctypes
 import math
 import os
 
@@ -549,7 +550,7 @@ def test_split_tiles_same_bits(torch, rb, ctx, n, v, flags):
         assert_score_parity(split.cpu().numpy(), vs.cpu().numpy(), ref)
 
 
-@pytest.mark.parametrize("n", [1, 31, 33, 12_288, 12_289, 24_577, 49_152, 49_153, 98_305, 262_144, 262_145])
+@pytest.mark.parametrize("n", [1, 31, 33, 6_144, 6_145, 12_289, 24_577, 49_152, 49_153, 131_072, 131_073, 262_144, 262_145])
 def test_select_cluster_edges(torch, rb, ctx, n):
     """Sizes about the cluster selection's CTA counts, range ends and limit,
     with ties that span CTAs, all scores equal, and an unaligned score
@@ -564,6 +565,16 @@ def test_select_cluster_edges(torch, rb, ctx, n):
     m_ref, thr_ref, nk_ref = oracle.select(s.astype(np.float64), 0.66)
     assert nk == nk_ref and thr == np.float32(thr_ref)
     assert np.array_equal(mask.cpu().numpy().view(np.uint32)[: (n + 31) // 32], m_ref)
+    # the entry point whose kernels are not chained takes the cluster form up to its own limit
+    s = (rng.integers(0, 3, n) / 4.0).astype(np.float32)
+    t = torch.from_numpy(s).cuda()
+    m2 = torch.empty((n + 31) // 32, dtype=torch.int32, device="cuda")
+    c_thr, err = ctypes.c_float(), ctypes.create_string_buffer(64)
+    st = rb.refine_select_noalloc(t.data_ptr(), n, 0.66, m2.data_ptr(), ctypes.byref(c_thr), None, err, 64,
+                                  torch.cuda.current_stream().cuda_stream)
+    m_ref, thr_ref, _ = oracle.select(s.astype(np.float64), 0.66)
+    assert st == rb.REFINE_OK and c_thr.value == (np.float32(thr_ref) if n > 1 else -math.inf)
+    assert np.array_equal(m2.cpu().numpy().view(np.uint32), m_ref)
 
 
 @pytest.mark.parametrize("n", [255, 256, 257, 65_536, 65_537, 1_048_577, 16_777_216, 16_777_217])
@@ -661,3 +672,15 @@ def test_chained_calls_same_bits(torch, rb, ctx, n, v, dtype):
         stream.synchronize()
         assert all(same(k, held[k]) for k in range(2))
         ctx.check()
+
+
+@pytest.mark.parametrize("scale", [0.5, 1.0, 1.5])
+def test_scaled_world_to_camera(torch, rb, ctx, scale):
+    """World-to-camera rows that are not orthonormal (a scale in the extrinsics)
+    get no footprint bound: scores against the oracle, which forms J W Sigma
+    W^T J^T as it stands."""
+    w = synth.random_scene(seed=31, n=5000, v=20, means="core_shell")
+    w.cams["R"] *= np.float32(scale)
+    w.cams["t"] *= np.float32(scale)
+    s, S, _, _ = gpu_score(torch, rb, ctx, w.scene, w.cams)
+    assert_score_parity(s, S, oracle.score(w.scene.params_f64(), w.cams))
