@@ -32,16 +32,16 @@ sys.path.insert(0, ROOT)
 # (primitive, view) pair needed (the kernel's diagnostic counters say which),
 # an FMA as 2 FLOPs and a compare, max or MUFU reciprocal as 1:
 FLOP_COSTS = {
-    "tile_view": 118,     # interval classification of one view for one tile: z, U, V, U - w z,
-                          # V - h z over the tile box (22 each) and the six range tests
+    "tile_view": 112,     # interval classification of one view for one tile: z, U, V, U - w z,
+                          # V - h z over the tile box (14 each), the two edge forms (8 each), the slacks
+                          # (4), the reach (16) and the six range tests
     "in_pair": 10,        # tile entirely visible: depth z (3 FMA), z^2 + eta (FMA), reciprocal, add
     "mixed_pair": 6,      # decided pair by pair: depth z (3 FMA)
     "open_axis": 10,      # per open u or v axis: U (3 FMA), d = max(-U, U - w z) (FMA, max), compare
     "open_depth": 2,      # open depth range: two compares
     "visible_mixed": 4,   # visible pair decided one by one: z^2 + eta, reciprocal, add
-    "bound_pair": 1,      # z^2 of a centre outside the image
-    "bound_axis": 10,     # per open axis: e = max(d, 0) z, e^2, t = U - c z, t^2, f^2 z^2 + t^2,
-                          # times 9 s_max^2, compare
+    "bound_pair": 0,      # nothing per centre outside the image but the axes:
+    "bound_axis": 2,      # per open axis: 3 s_max times the tile's reach, compare
     "exact_axis": 30,     # per needed extent: g = z P - U P2 (3 MUL, 3 FMA), L g (3 MUL, 6 FMA),
                           # |L g|^2 (MUL, 2 FMA), compare
     "kahan_block": 4,     # per primitive and 32-view block: compensated add of the block sum
@@ -70,7 +70,7 @@ def workload(name: str, rank: int = 0, storage: str = "f32"):
 
 def cell_bits_for(n: int) -> int:
     """Resolution of the processing-order grid the library picks for n
-    primitives (2^(3b) Morton cells, b in 4..7, about 0.5 or more per cell)."""
+    primitives (2^(3b) cells, b in 4..7, about 0.5 or more per cell)."""
     b = 4
     while b < 7 and (1 << (3 * (b + 1))) <= 2 * n:
         b += 1
@@ -80,14 +80,14 @@ def cell_bits_for(n: int) -> int:
 def stream_bytes(n: int, n_keep: int, storage: str) -> dict:
     """Algorithmic DRAM bytes of one plain step, per kernel class: what each
     kernel must read and write at least once (row bytes by storage type;
-    the processing-order keys are cells and size classes, 2 x 8^b)."""
+    the processing-order keys are 8^b cells and 8^(b-1) wider ones)."""
     col = {"f32": 224, "bf16": 112, "bf16s": 118}[storage]  # the 56 attribute rows
-    es = 2 if storage == "bf16" else 4       # bytes of a log-scale element
     row = 12 + col                           # pos (FP32) + 56 attribute rows
-    keys = 2 * (1 << (3 * cell_bits_for(n)))
+    b = cell_bits_for(n)
+    keys = (1 << (3 * b)) + (1 << (3 * (b - 1)))
     return {
-        "features": n * row + 64 * n,        # all rows in, one 64-B record out
-        "cells": n * (12 + 3 * es) + 8 * n,  # pos and log-scales in, (cell, slot) out
+        "prepare": 4 * keys,                 # the cell counts cleared
+        "features": n * row + 72 * n,        # all rows in, a 64-B record and (cell, slot) out
         "cell_scan": 8 * keys,               # counts in, offsets out
         "cell_scatter": 16 * n,              # (cell, slot) and the cell's offset in, order out
         "score": 72 * n,                     # record and order entry in, score out
