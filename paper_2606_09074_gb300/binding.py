@@ -343,8 +343,9 @@ def _dtype_code(t) -> int:
 def make_scene(pos, attr) -> refine_scene:
     """refine_scene view of device tensors pos [3, n] float32 and attr
     [56, n] float32 / bfloat16 with a common row stride."""
-    rows, n = pos.shape
-    if rows != 3 or tuple(attr.shape) != (56, n):
+    shape, ashape = pos.shape, attr.shape
+    n = shape[1]
+    if shape[0] != 3 or ashape[0] != 56 or ashape[1] != n:
         raise ValueError("expected pos [3, n] and attr [56, n]")
     stride = pos.stride(0)
     if n and (pos.stride(1) != 1 or attr.stride(1) != 1 or stride != attr.stride(0)):
@@ -434,7 +435,7 @@ class Context:
                             C.byref(cnt) if return_count else None, _stream_handle(stream, self.device))
         _check(self.handle, rc)
         out = (_cols(out_pos, n_keep), _cols(out_attr, n_keep),
-               idx if idx is None or n_keep else idx[:0])
+               idx if idx is None or n_keep > 0 else idx[:0])
         return out + (cnt.value,) if return_count else out
 
     def prune_host(self, pos_host, attr_host, cams, ratio, params=None, want_scores=False,

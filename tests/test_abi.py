@@ -158,3 +158,17 @@ def test_mixed_rows_container_host_only():
     assert isinstance(e, b.MixedRows) and e.shape == (56, 5)
     assert b.empty_attr_like(torch.zeros(56, 3, dtype=torch.bfloat16), 4).dtype == torch.bfloat16
 
+
+
+@pytest.mark.parametrize("shape", [(3, 5), (3, 5, 1)])
+def test_make_scene_trailing_dims(shape):
+    """A block of rows may carry trailing dimensions (rows and columns are
+    its first two); wrong row counts are a ValueError."""
+    torch = pytest.importorskip("torch")
+    from paper_2606_09074_gb300 import binding as b
+    pos, attr = torch.zeros(shape), torch.zeros((56,) + shape[1:])
+    sc = b.make_scene(pos, attr)
+    assert (sc.n, sc.row_stride, sc.pos, sc.attr) == (5, 5, pos.data_ptr(), attr.data_ptr())
+    for p, a in ((pos[:2], attr), (pos, attr[:55]), (pos, attr[:, :4])):
+        with pytest.raises(ValueError):
+            b.make_scene(p, a)
