@@ -436,9 +436,11 @@ void dispatcher_main(refine_queue *q)
 
 // Continuous batching: each batched launch scores every request whose
 // preparation has ended by the time the previous launch has ended, and every
-// one that is no larger than the oldest and whose copy has ended (its
-// preparation, a few tens of microseconds, is waited for on the score
-// stream: one launch for both costs less than one each).
+// one of a small fraction of the oldest's size whose copy has ended: its
+// preparation, a few tens of microseconds, is waited for on the score stream,
+// and one launch for both costs less than one each.  With larger ones let in,
+// the GPU stood idle during their preparations: 2,000 jobs back to back 1,237
+// and 1,305 scenes/s against 1,420 and 1,461 without them.
 constexpr int64_t kJoinFraction = 64;
 
 void scorer_main(refine_queue *q)
@@ -471,7 +473,7 @@ void scorer_main(refine_queue *q)
                 QJob *j = *it;
                 const bool done = j->host_status || !j->prepped ||
                                   cudaEventQuery(q->prepped[j->slot]) != cudaErrorNotReady ||
-                                  (j->req.n <= head_n && cudaEventQuery(q->copied[j->slot]) != cudaErrorNotReady);
+                                  (j->req.n <= head_n / kJoinFraction && cudaEventQuery(q->copied[j->slot]) != cudaErrorNotReady);
                 if (done) {
                     ready.push_back(j);
                     it = q->prepping.erase(it);
