@@ -471,6 +471,9 @@ __global__ void __launch_bounds__(kFeatCol, 4) k_features_bulk(FeatureArgs<DT> f
         if (!mbar_wait_bounded(&bar, phase)) {
             set_status(f.status, kEtimeout);
             mbar_wait_bounded(&bar, phase);  // give the copies a second bound before leaving
+            // the kernels that follow index with the slots: any valid ones
+            if (last >= 0) f.cell[last] = ks;
+            for (int64_t i = i0 + t; i < f.n; i += step) f.cell[i] = make_uint2(0u, atomicAdd(&f.counts[0], 1u));
             return;
         }
         phase ^= 1u;
