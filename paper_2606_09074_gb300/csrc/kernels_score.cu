@@ -849,6 +849,21 @@ bool shape_valid(const ScoreShape &sh)
            sh.views_per_pass >= 32 && sh.views_per_pass <= kViewsPerPass && sh.views_per_pass % 32 == 0;
 }
 
+// Opt-in to the shared memory of a camera block.  A launch may take 48 KB
+// without it, static part included (kStaticBound).  The limit set is one
+// constant for every launch: the attribute belongs to the function, so a
+// smaller value set for one thread's launch would refuse another's larger one.
+constexpr size_t kStaticBound = 8 * 1024;
+static_assert(sizeof(WarpSlot) * (kScoreThreads / 32) + 1024 <= kStaticBound, "static shared memory of the score kernels");
+constexpr size_t kMaxCamsSmem = (size_t)kViewsPerPass * (sizeof(CamRec) + sizeof(CamExt));
+
+template <class Fn>
+static cudaError_t allow_cams_smem(Fn fn, size_t smem)
+{
+    if (smem + kStaticBound <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCamsSmem);
+}
+
 // Persistent grid: as many CTAs as fit per SM, capped by the items.
 //
 // Split tiles.  A tile's views are one serial chain of a few tens of
@@ -873,7 +888,7 @@ ScorePlan score_plan(int num_sms, int64_t n, int vcount, int flags, bool split, 
     pl.gpt = sh.gpt;
     int per_sm = 0;
     const ScoreFn fn = pick_score(proj_mode(flags), false, pl.gpt);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    (void)allow_cams_smem(fn, smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kScoreThreads, smem) != cudaSuccess ||
         per_sm < 1) {
         cudaGetLastError();
@@ -899,10 +914,8 @@ cudaError_t launch_score(const ScoreLaunch &a, int gpt, const Chain &s)
 {
     const ScoreFn fn = pick_score(proj_mode(a.flags), a.need != nullptr, gpt);
     const size_t smem = cams_smem(a.vcount, a.flags);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_cams_smem(fn, smem);
+    if (e != cudaSuccess) return e;
     return launch_chained(fn, a.grid, kScoreThreads, smem, s, a);
 }
 
@@ -923,7 +936,7 @@ static BatchFn batch_fn(const ScoreShape &sh, bool eq17)
 int score_batch_grid(int num_sms, size_t smem, bool eq17, const ScoreShape &sh)
 {
     const BatchFn fn = batch_fn(sh, eq17);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    (void)allow_cams_smem(fn, smem);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, sh.threads, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
@@ -936,10 +949,8 @@ int score_batch_grid(int num_sms, size_t smem, bool eq17, const ScoreShape &sh)
 cudaError_t launch_score_batch(const BatchLaunch &b, size_t smem, int grid, const ScoreShape &sh, cudaStream_t s)
 {
     const BatchFn fn = batch_fn(sh, b.eq17);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_cams_smem(fn, smem);
+    if (e != cudaSuccess) return e;
     fn<<<grid, sh.threads, smem, s>>>(b);
     return cudaGetLastError();
 }

@@ -502,8 +502,11 @@ cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_kee
     const int per = (int)(((n + ctas - 1) / ctas + 31) / 32 * 32);
     const size_t smem = sizeof(uint32_t) * (size_t)per;
     if (smem + 3 * 2048 * sizeof(unsigned) + 1024 > 48 * 1024) {
+        // one constant for every launch: a smaller value set for one thread's
+        // launch would refuse another's larger one
         const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_select_cluster),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(sizeof(uint32_t) * kClKeys));
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg{};

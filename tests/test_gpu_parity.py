@@ -684,3 +684,56 @@ def test_scaled_world_to_camera(torch, rb, ctx, scale):
     w.cams["t"] *= np.float32(scale)
     s, S, _, _ = gpu_score(torch, rb, ctx, w.scene, w.cams)
     assert_score_parity(s, S, oracle.score(w.scene.params_f64(), w.cams))
+
+
+@pytest.mark.parametrize("v", [306, 333, 335, 384, 385, 512])
+def test_camera_block_shared_memory(torch, rb, ctx, v):
+    """Camera blocks about the 48 KB of shared memory that a launch gets
+    without opting in (static part included), for Eq. 17 and for the longer
+    records of FULL_JACOBIAN: plain, counting and batched launches."""
+    w = synth.config0(seed=6, n=700)
+    cams = np.resize(w.cams, v)
+    cams["znear"] = 1.0  # (as in test_ablation_flags)
+    for flags in (rb.FLAG_NORM_ATTR, rb.FLAG_NORM_ATTR | rb.FLAG_FULL_JACOBIAN):
+        p = rb.default_params(flags=flags)
+        s, S, _, (pos, attr) = gpu_score(torch, rb, ctx, w.scene, cams, params=p)
+        assert_score_parity(s, S, oracle.score(w.scene.params_f64(), cams, oracle_params_from(p, rb)))
+        cd = rb.cameras_to_device(cams, pos.device)
+        plain = ctx.score(pos, attr, cd, params=p)
+        assert np.array_equal(plain.cpu().numpy(), s)
+        batch = rb.Batch(ctx, [{"pos": pos, "attr": attr, "cams": cd, "ratio": 0.5}], params=p)
+        batch.run()
+        batch.results()
+        assert torch.equal(batch.outputs[0]["scores"], plain)
+        batch.close()
+
+
+def test_select_threads_of_two_sizes(torch, rb):
+    """Two threads, each with a context and a stream, select from different
+    sizes at once: one's launch settings do not disturb the other's."""
+    import threading
+    failed = []
+    scores = {n: np.random.default_rng(n).random(n).astype(np.float32) for n in (50_000, 120_000)}
+    refs = {n: oracle.select(s.astype(np.float64), 0.5) for n, s in scores.items()}  # (one at a time)
+
+    def work(n):
+        try:
+            c, s = rb.Context(0), torch.cuda.Stream()
+            t = torch.from_numpy(scores[n]).cuda()
+            mask = torch.empty((n + 31) // 32, dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            for _ in range(400):
+                _, _, nk = c.select(t, 0.5, mask=mask, threshold=False, stream=s)
+            s.synchronize()
+            m_ref, _, nk_ref = refs[n]
+            assert nk == nk_ref and np.array_equal(mask.cpu().numpy().view(np.uint32), m_ref)
+            c.close()
+        except Exception as e:  # noqa: BLE001 -- reported below
+            failed.append((n, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(n,)) for n in scores]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
