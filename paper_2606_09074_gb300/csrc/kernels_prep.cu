@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(kFeatCol, 4) k_features_bulk(FeatureArgs<DT> f
     __shared__ __align__(8) uint64_t bar;
     __shared__ int row_base[59];
     load_hilbert(hilbert);
-    const Rows in{reinterpret_cast<const char *>(f.pos), reinterpret_cast<const char *>(f.attr.f), f.S};
+    const Rows in{reinterpret_cast<const char *>(f.pos), reinterpret_cast<const char *>(f.attr.f), f.S,
+                  ALIGNED ? Rows::whole_chunks(f.n) : f.n};
     const int t = threadIdx.x;
     if (!ALIGNED && t < 59) row_base[t] = Rows::place(t) + (int)in.mis(t);
     if (t == 0) mbar_init(&bar, 1);

@@ -2,9 +2,11 @@
 // 59 rows, brought by one bulk copy (cp.async.bulk) a row.  A bulk copy starts
 // on 16 bytes: the row's span is widened to 16-byte boundaries (row strides may
 // be odd) and its place in shared memory is taken from its misalignment.  At
-// a scene's end the widened span of the last row of a buffer could leave it
-// (of the last few rows, when the stride is below 8): it is narrowed instead,
-// and its last few elements are read by plain loads.
+// a scene's end the widened span of the last row of a block could pass the
+// row's last element, where the caller's memory may end (a scene may be a
+// column slice that reaches the end of its block; of the last few rows, when
+// the stride is below 8): it is narrowed instead, and its last few elements are
+// read by plain loads.
 #pragma once
 
 #include "common.cuh"
@@ -21,7 +23,7 @@ struct RowTile {
     static constexpr int kBytes = kF32 * kPitch4 + (59 - kF32) * kPitch2;
 
     const char *pos, *attr;
-    int64_t S;
+    int64_t S, n;
 
     __host__ __device__ static constexpr bool f32(int r) { return r < kF32; }
     __host__ __device__ static constexpr int size(int r) { return r < kF32 ? 4 : 2; }
@@ -29,32 +31,37 @@ struct RowTile {
     {
         return r < kF32 ? r * kPitch4 : kF32 * kPitch4 + (r - kF32) * kPitch2;
     }
-    __device__ __forceinline__ const char *row(int r) const
+    __host__ __device__ __forceinline__ const char *row(int r) const
     {
         constexpr int NF = attr_f32_rows(DT);
         if (r < 3) return pos + (int64_t)r * S * 4;
         if (r - 3 < NF) return attr + (int64_t)(r - 3) * S * 4;
         return attr + (int64_t)NF * S * 4 + (int64_t)(r - 3 - NF) * S * 2;
     }
-    __device__ __forceinline__ const char *end(int r) const  // of the row's buffer
+    __host__ __device__ __forceinline__ const char *end(int r) const  // past the last element of the row's block
     {
-        return r < 3 ? pos + S * 12 : attr + S * (int64_t)attr_col_bytes(DT);
+        return r < 3 ? pos + (2 * S + n) * 4 : row(58) + n * size(58);
     }
     // Bytes of row r past a 16-byte boundary (the same at every unit's start).
-    __device__ __forceinline__ uint32_t mis(int r) const
+    __host__ __device__ __forceinline__ uint32_t mis(int r) const
     {
         return (uint32_t)(reinterpret_cast<uintptr_t>(row(r)) & 15u);
     }
     // Bytes of the bulk copy of `count` elements of row r from element i0: up
     // to the next 16-byte boundary, or down to the last when that lies past
-    // the end of the row's buffer.
-    __device__ __forceinline__ uint32_t span(int r, int64_t i0, int count) const
+    // the end of the row's block.
+    __host__ __device__ __forceinline__ uint32_t span(int r, int64_t i0, int count) const
     {
         const uint32_t m = mis(r), b = m + (uint32_t)(count * size(r)), up = (b + 15u) & ~15u;
         return row(r) + i0 * size(r) - m + up > end(r) ? b & ~15u : up;
     }
+    // With a stride that is a multiple of 8, for n: so many elements of every
+    // row are in whole 16-byte chunks of the block that the rows are from, so
+    // copies up to them need no narrowing (a slice of the block starts on 16
+    // bytes, that is on a multiple of 8 columns when it has 2-byte rows).
+    __host__ __device__ __forceinline__ static int64_t whole_chunks(int64_t n) { return (n + 7) & ~int64_t(7); }
     // Whether some copy of the unit at i0 may be narrowed.
-    __device__ __forceinline__ static bool at_end(int64_t i0, int64_t n) { return i0 + U + 8 > n; }
+    __host__ __device__ __forceinline__ static bool at_end(int64_t i0, int64_t n) { return i0 + U + 8 > n; }
 
     // Issues the copies of the unit at i0 (a multiple of U), completing on
     // `bar`; called by every warp of a CTA of WARPS warps, after a barrier that
