@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kFeatCol, 4) k_features(FeatureArgs<DT> f)
 // a primitive's arithmetic at 32 warps an SM); the same with all copies issued
 // by one warp 160 us.
 template <int DT, bool ALIGNED>
-__global__ void __launch_bounds__(kFeatCol, 4) k_features_bulk(FeatureArgs<DT> f)
+__global__ void __launch_bounds__(kFeatCol, 4) k_features_bulk(FeatureArgs<DT> f, RowTile<DT, kFeatCol> in)
 {
     using Rows = RowTile<DT, kFeatCol>;
     extern __shared__ __align__(16) unsigned char tile[];
@@ -445,8 +445,6 @@ __global__ void __launch_bounds__(kFeatCol, 4) k_features_bulk(FeatureArgs<DT> f
     __shared__ __align__(8) uint64_t bar;
     __shared__ int row_base[59];
     load_hilbert(hilbert);
-    const Rows in{reinterpret_cast<const char *>(f.pos), reinterpret_cast<const char *>(f.attr.f), f.S,
-                  ALIGNED ? Rows::whole_chunks(f.n) : f.n};
     const int t = threadIdx.x;
     if (!ALIGNED && t < 59) row_base[t] = Rows::place(t) + (int)in.mis(t);
     if (t == 0) mbar_init(&bar, 1);
@@ -598,10 +596,13 @@ static cudaError_t launch_features_t(const FeatureLaunch &l, int num_sms, const 
     if (nb <= num_sms && l.n <= (int64_t)nb * kFeatCol * kFeatCols)
         return launch_chained(k_features_small<DT>, nb, kFeatSmallThreads, 0, s, f);
     if constexpr (DT != REFINE_F32) {
-        const size_t smem = RowTile<DT, kFeatCol>::kBytes;
-        static_assert(RowTile<DT, kFeatCol>::kBytes + 12 * 1024 < 48 * 1024, "no opt-in shared memory");
-        if (l.stride % 8 == 0) return launch_chained(k_features_bulk<DT, true>, nb, kFeatCol, smem, s, f);
-        return launch_chained(k_features_bulk<DT, false>, nb, kFeatCol, smem, s, f);
+        using Rows = RowTile<DT, kFeatCol>;
+        static_assert(Rows::kBytes + 12 * 1024 < 48 * 1024, "no opt-in shared memory");
+        if (l.stride % 8 == 0)
+            return launch_chained(k_features_bulk<DT, true>, nb, kFeatCol, Rows::kBytes, s, f,
+                                  Rows(l.pos, l.attr, l.stride, Rows::whole_chunks(l.n)));
+        return launch_chained(k_features_bulk<DT, false>, nb, kFeatCol, Rows::kBytes, s, f,
+                              Rows(l.pos, l.attr, l.stride, l.n));
     } else {
         return launch_chained(k_features<DT>, nb, kFeatCol, 0, s, f);
     }

@@ -174,7 +174,7 @@ static cudaError_t launch_compact_t(const refine_scene &in, const uint32_t *mask
     int64_t g = (in.n + cmp_unit(DT) - 1) / cmp_unit(DT);
     if (g > (int64_t)num_sms * kCmpCtas) g = (int64_t)num_sms * kCmpCtas;
     if (g < 1) g = 1;
-    const CmpRows<DT> rows{reinterpret_cast<const char *>(in.pos), static_cast<const char *>(in.attr), in.row_stride, in.n};
+    const CmpRows<DT> rows(in.pos, in.attr, in.row_stride, in.n);
     return launch_chained(k_compact<DT>, (int)g, kCmpThreads, smem, s, rows, in.n, mask, off,
                           reinterpret_cast<char *>(out_pos), static_cast<char *>(out_attr), OS, out_idx, status);
 }

@@ -23,7 +23,15 @@ struct RowTile {
     static constexpr int kBytes = kF32 * kPitch4 + (59 - kF32) * kPitch2;
 
     const char *pos, *attr;
-    int64_t S, n;
+    int64_t S;
+    const char *pos_end, *attr_end;  // past the last element of the last row of each block
+
+    // The first n columns of rows S elements apart.
+    __host__ RowTile(const void *p, const void *a, int64_t stride, int64_t n)
+        : pos(static_cast<const char *>(p)), attr(static_cast<const char *>(a)), S(stride), pos_end(row(2) + n * 4),
+          attr_end(row(58) + n * size(58))
+    {
+    }
 
     __host__ __device__ static constexpr bool f32(int r) { return r < kF32; }
     __host__ __device__ static constexpr int size(int r) { return r < kF32 ? 4 : 2; }
@@ -38,10 +46,6 @@ struct RowTile {
         if (r - 3 < NF) return attr + (int64_t)(r - 3) * S * 4;
         return attr + (int64_t)NF * S * 4 + (int64_t)(r - 3 - NF) * S * 2;
     }
-    __host__ __device__ __forceinline__ const char *end(int r) const  // past the last element of the row's block
-    {
-        return r < 3 ? pos + (2 * S + n) * 4 : row(58) + n * size(58);
-    }
     // Bytes of row r past a 16-byte boundary (the same at every unit's start).
     __host__ __device__ __forceinline__ uint32_t mis(int r) const
     {
@@ -53,7 +57,7 @@ struct RowTile {
     __host__ __device__ __forceinline__ uint32_t span(int r, int64_t i0, int count) const
     {
         const uint32_t m = mis(r), b = m + (uint32_t)(count * size(r)), up = (b + 15u) & ~15u;
-        return row(r) + i0 * size(r) - m + up > end(r) ? b & ~15u : up;
+        return row(r) + i0 * size(r) - m + up > (r < 3 ? pos_end : attr_end) ? b & ~15u : up;
     }
     // With a stride that is a multiple of 8, for n: so many elements of every
     // row are in whole 16-byte chunks of the block that the rows are from, so
