@@ -125,6 +125,13 @@ inline refine_status use_device(refine_ctx *c)
     return REFINE_OK;
 }
 
+inline bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    return st == cudaStreamCaptureStatusActive;
+}
+
 inline refine_status ensure(refine_ctx *c, Arena &a, size_t bytes)
 {
     if (bytes <= a.cap) return REFINE_OK;
@@ -430,16 +437,21 @@ inline refine_status score_impl(refine_ctx *c, const refine_scene *sc, const ref
     const int vfirst = std::min(pl.V, pl.vpp), vlast = pl.V - (pl.passes - 1) * pl.vpp;
     ScorePlan sp0, sp1;
     size_t parts = 0, taken = 0;
-    auto plan = [&](bool split) {
+    auto plan = [&](bool split) {  // the scratch it takes
         sp0 = score_plan(c->num_sms, pl.n, vfirst, p.flags, split, c->shape);
         sp1 = pl.multipass ? score_plan(c->num_sms, pl.n, vlast, p.flags, split, c->shape) : sp0;
         parts = std::max(split_part_floats(sp0, vfirst), split_part_floats(sp1, vlast));
         const size_t counts = (size_t)std::max(sp0.split_tiles, sp1.split_tiles);
         taken = (sizeof(unsigned long long) + sizeof(unsigned) * counts + 15) & ~size_t(15);
-        return ensure(c, c->score, scene_bytes(pl) + carve_size({sizeof(float) * parts, taken}));
+        return scene_bytes(pl) + carve_size({sizeof(float) * parts, taken});
     };
-    st = plan(!count);
-    if (st == REFINE_ENOMEM && !count) st = plan(false);  // the split's scratch (20 MB at most) is not needed
+    // The split's scratch (20 MB at most) is not needed: whole tiles when it
+    // does not fit, or when the scratch would have to grow for it while the
+    // stream is being captured (growing synchronises and would end the capture)
+    size_t bytes = plan(!count);
+    if (!count && bytes > c->score.cap && capturing(s)) bytes = plan(false);
+    st = ensure(c, c->score, bytes);
+    if (st == REFINE_ENOMEM && !count) st = ensure(c, c->score, plan(false));
     if (st) return st;
     Carver cv(c->score.p);
     const SceneScratch x = carve_scene(cv, pl);
