@@ -230,12 +230,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
     }
     __syncthreads();
     if (threadIdx.x < 4) {
-        const float mean = sum[k] / (float)m, var = sum[4 + k] / (float)m - mean * mean;
+        const int q = threadIdx.x;  // x, y, z, ln s_max
+        const float mean = sum[q] / (float)m, var = sum[4 + q] / (float)m - mean * mean;
         const float sd = var > 0.f ? sqrtf(var) : 0.f;
-        if (k < 3) {
-            const float base = k == 0 ? x0 : (k == 1 ? y0 : z0);
-            a.grid->lo[k] = base + (mean - 3.f * sd);
-            a.grid->qscale[k] = sd > 0.f && isfinite(sd) ? (float)(1 << a.cell_bits) / (6.f * sd) : 0.f;
+        if (q < 3) {
+            const float base = q == 0 ? x0 : (q == 1 ? y0 : z0);
+            a.grid->lo[q] = base + (mean - 3.f * sd);
+            a.grid->qscale[q] = sd > 0.f && isfinite(sd) ? (float)(1 << a.cell_bits) / (6.f * sd) : 0.f;
         } else {
             const float big = mean + kSizeSplitSd * sd;
             a.grid->big_ls = isfinite(big) ? big : INFINITY;
