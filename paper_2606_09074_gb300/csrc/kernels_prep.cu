@@ -181,6 +181,8 @@ __device__ __forceinline__ uint32_t order_key(const uint16_t *hilbert, const Ord
 // a 3.5M-primitive scene, most of it waiting for its count atomics.
 // ---------------------------------------------------------------------
 constexpr int kPrepThreads = 1024;
+constexpr float kGridFar = 6.f;  // standard deviations
+constexpr int kGridRounds = 5;
 
 template <int DT>
 __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restrict__ pos, AttrRows<DT> attr, int64_t S,
@@ -196,49 +198,72 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
         for (int64_t i = b * kPrepThreads + threadIdx.x; i < a.more4; i += nb * kPrepThreads) a.more[i] = zero;
         return;
     }
-    // sums of the offsets from primitive 0 and of their squares (a scene far
-    // from the origin keeps its digits), and of ln s_max
-    const int64_t m = n < kPrepThreads ? n : kPrepThreads;
-    const int64_t k = threadIdx.x < m ? threadIdx.x : 0;
+    // Sums of the offsets from primitive 0 and of their squares (a scene far
+    // from the origin keeps its digits), and of ln s_max.  A sample beyond
+    // kGridFar standard deviations (at most 1 in 36 can be, none in an ordinary
+    // scene) is left out and the sums are formed again about the mean found:
+    // one centre of 1M at 1,000 or 10,000 scene radii among the 1,024 made the
+    // box, and with it all cells, so much wider that a pass over 60 views took
+    // 306 or 761 us, against 155 without it and 157 so.
+    const int64_t k = threadIdx.x < n ? threadIdx.x : 0;
     const int64_t i = n <= kPrepThreads ? k : (k / 4) * (n - 4) / (kPrepThreads / 4 - 1) + k % 4;
-    const float x0 = __ldg(pos), y0 = __ldg(pos + S), z0 = __ldg(pos + 2 * S);
-    const bool in = threadIdx.x < m;
-    const float v[4] = {in ? __ldg(pos + i) - x0 : 0.f, in ? __ldg(pos + S + i) - y0 : 0.f,
-                        in ? __ldg(pos + 2 * S + i) - z0 : 0.f,
-                        in ? fmaxf(attr.ld(0, i), fmaxf(attr.ld(1, i), attr.ld(2, i))) : 0.f};
-    float s[8];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        s[q] = v[q];
-        s[4 + q] = v[q] * v[q];
-    }
+    float base[4] = {__ldg(pos), __ldg(pos + S), __ldg(pos + 2 * S), 0.f};
+    const float p[4] = {__ldg(pos + i), __ldg(pos + S + i), __ldg(pos + 2 * S + i),
+                        fmaxf(attr.ld(0, i), fmaxf(attr.ld(1, i), attr.ld(2, i)))};
+    bool use = threadIdx.x < n;
+    int m = n < kPrepThreads ? (int)n : kPrepThreads;
     __shared__ float red[8][kPrepThreads / 32];
     __shared__ float sum[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    bool again = false;
+    for (int round = 0;; ++round) {
+        float s[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+        for (int q = 0; q < 4; ++q) {
+            const float v = use ? p[q] - base[q] : 0.f;
+            s[q] = v;
+            s[4 + q] = v * v;
+        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
-        if (lane == 0) red[k][warp] = s[k];
+        for (int q = 0; q < 8; ++q) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+            if (lane == 0) red[q][warp] = s[q];
+        }
+        __syncthreads();
+        if (warp < 8) {
+            float t = red[warp][lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) sum[warp] = t;
+        }
+        __syncthreads();
+        bool far = false;
+        float mean[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            mean[q] = sum[q] / (float)m;
+            const float var = sum[4 + q] / (float)m - mean[q] * mean[q], d = (p[q] - base[q]) - mean[q];
+            far |= use & (var > 0.f) & (d * d > kGridFar * kGridFar * var);
+        }
+        const int dropped = __syncthreads_count(far);  // (every thread has read the sums)
+        if ((dropped == 0 && !again) || round == kGridRounds) break;
+        again = dropped > 0;  // and once more when none is left out any longer: about the mean of those that stay
+        use &= !far;
+        m -= dropped;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) base[q] += mean[q];
     }
-    __syncthreads();
-    if (warp < 8) {
-        float t = red[warp][lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) sum[warp] = t;
-    }
-    __syncthreads();
     if (threadIdx.x < 4) {
         const int q = threadIdx.x;  // x, y, z, ln s_max
         const float mean = sum[q] / (float)m, var = sum[4 + q] / (float)m - mean * mean;
         const float sd = var > 0.f ? sqrtf(var) : 0.f;
+        const float b = q == 0 ? base[0] : (q == 1 ? base[1] : (q == 2 ? base[2] : base[3]));
         if (q < 3) {
-            const float base = q == 0 ? x0 : (q == 1 ? y0 : z0);
-            a.grid->lo[q] = base + (mean - 3.f * sd);
+            a.grid->lo[q] = b + (mean - 3.f * sd);
             a.grid->qscale[q] = sd > 0.f && isfinite(sd) ? (float)(1 << a.cell_bits) / (6.f * sd) : 0.f;
         } else {
-            const float big = mean + kSizeSplitSd * sd;
+            const float big = b + (mean + kSizeSplitSd * sd);
             a.grid->big_ls = isfinite(big) ? big : INFINITY;
         }
     }

@@ -1,5 +1,5 @@
 """The plain calls away from ordinary scenes: more views under capture than in
-the calls before it."""
+the calls before it; a few primitives far from all others."""
 import pytest
 
 from paper_2606_09074_gb300 import synth
@@ -45,3 +45,32 @@ def test_capture_with_more_views_than_before(env, n):
         ctx.check()
     ctx.close()
     ref.close()
+
+
+@pytest.mark.parametrize("n", [900, 200_000])
+@pytest.mark.parametrize("rows,value", [("pos", 1e3), ("pos", 1e6), ("pos", -1e9), ("attr", -60.0), ("both", 0.0)])
+def test_outliers_leave_the_order_as_it_is(env, n, rows, value):
+    """A few primitives far from all others (positions) or far smaller
+    (log-scales), among those that the processing order's grid is sampled
+    from, leave the other tiles as tight as they were: the pairs decided one
+    by one grow by no more than the outliers' own tiles hold.  (Scene 'both'
+    mixes three magnitudes of positions with small scales.)"""
+    torch, rb, dev = env
+    v = 24
+    pos, attr, cams = uploaded(torch, rb, dev, synth.random_scene(seed=7, n=n, v=v, means="core_shell"))
+    ctx = rb.Context(0)
+    _, plain = ctx.score(pos, attr, cams, stats=True)
+    # the first and the last four primitives are always among the samples
+    far = [0, 1, n - 1]
+    for k, i in enumerate(far):
+        if rows == "attr":
+            attr[0:3, i] = value
+        else:
+            pos[:, i] = value if rows == "pos" else 10.0 ** (3 + 2 * k)
+        if rows == "both":
+            attr[0:3, i] = -60.0
+    _, got = ctx.score(pos, attr, cams, stats=True)
+    ctx.check()
+    ctx.close()
+    own = len(far) * 64 * v  # each outlier's tile, all pairs
+    assert got["mixed_pairs"] <= 1.02 * plain["mixed_pairs"] + own, (got["mixed_pairs"], plain["mixed_pairs"])
