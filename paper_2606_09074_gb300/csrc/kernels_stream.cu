@@ -1,22 +1,31 @@
 // Compaction, pass 2: the scatter of every row of the kept primitives.
 //
-// One CTA of 8 warps takes a unit of consecutive primitives (128 with float32
-// rows, 256 with bfloat16 rows) at a time.  The unit's span of each of the 59
-// rows, 512 contiguous bytes (1 KB of a float32 row beside bfloat16 ones), is
+// One CTA of 8 warps takes a unit of 256 consecutive primitives at a time.
+// The unit's span of each of the 59 rows, 512 or 1,024 contiguous bytes, is
 // brought into shared memory by one bulk copy (cp.async.bulk) per row,
-// completing on an mbarrier (RowTile); meanwhile the ranks
-// of the kept primitives are inverted (output d comes from primitive src[d]).
-// Then each warp takes every eighth row: 32 outputs are one shared-memory load
-// and one contiguous store.  A unit is 31-34 KB, so 6 CTAs fit an SM, and while
-// some wait for their unit others store theirs: about 190 KB an SM in flight
-// without holding a register.
+// completing on an mbarrier (RowTile); meanwhile the ranks of the kept
+// primitives are inverted (output d comes from primitive src[d]).  Then each
+// warp takes every eighth row: 32 outputs are one shared-memory load and one
+// contiguous store.  A unit is 31-34 KB with bfloat16 rows and 64 KB with
+// float32 ones, so 5 or 3 CTAs fit an SM, and while some wait for their unit
+// others store theirs: 155-190 KB an SM in flight without holding a register.
+// Of a unit with at most kCmpFew kept primitives only their own sectors are
+// read, by plain loads.
 //
-// Measured (the kernel alone, events around it): bfloat16 rows, 3.5M
-// primitives at ratio 0.5 160 -> 107 us (6.2 TB/s); float32 rows 200 -> 199 us
-// (3.5M, 6.3 TB/s) and 60 -> 55 us (1M at 0.66), against the form before, in
-// which a warp loaded each row of a mask word into registers (16 float or 28
-// bfloat16 rows at a time) and shuffled: 64-byte loads of bfloat16 rows, and
-// registers, bounded what it had in flight.
+// Measured (count and scatter, cold L2, kept at random; us at ratio 0 / 0.5 /
+// 0.9 / 0.98 / 0.995):
+//   3.5M float32   268 / 203 / 152 /  92 /  57   (units of 128, all copied whole:
+//                  282 / 219 / 174 / 166 / 104; a warp for 256 primitives, rows
+//                  through registers: 272 / 222 / 187 / 178 / 173)
+//   3.5M bfloat16  156 / 115 /  90 /  76 /  47   (all units copied whole, 6 CTAs
+//                  of 40 registers: 158 / 118 / 102 / 100 /  86; a warp for 32
+//                  primitives: 210 / 182 / 159 / 118 /  69)
+//   1M float32      84 /  66 /  55 /  37 /  23   (86 / 68 / 57 / 55 / 39 and
+//                   92 /  82 /  69 /  51 /  36)
+// Units of at most 4 kept primitives instead of 8: 3.5M float32 133 us at 0.98;
+// at most 16: 164 us at 0.9.
+#include <type_traits>
+
 #include "internal.h"
 #include "rows.cuh"
 
@@ -24,21 +33,71 @@ namespace refine {
 
 constexpr int kCmpWarps = 8;
 constexpr int kCmpThreads = 32 * kCmpWarps;
-constexpr int kCmpCtas = 6;  // per SM
-
-// Primitives per unit.
-__host__ __device__ constexpr int cmp_unit(int dtype) { return dtype == REFINE_F32 ? 128 : 256; }
-
-template <int DT>
-using CmpRows = RowTile<DT, cmp_unit(DT)>;
+constexpr int kCmpUnit = kCmpSeg;  // primitives per unit
+constexpr int kCmpFew = 8;
+// Per SM: what fits its shared memory with float32 rows, registers (48 a
+// thread) with bfloat16 ones.
+__host__ __device__ constexpr int cmp_ctas(int dtype) { return dtype == REFINE_F32 ? 3 : 5; }
 
 template <int DT>
-__global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(CmpRows<DT> in, int64_t n, const uint32_t *__restrict__ mask,
+using CmpRows = RowTile<DT, kCmpUnit>;
+
+// The rows of a unit's `kept` (at most kCmpFew) primitives by loads of their
+// own: every group of kCmpFew threads takes a row.  word: the unit's mask, a
+// word per lane.
+template <int DT>
+__device__ __forceinline__ void copy_few(const CmpRows<DT> &in, int64_t i0, uint32_t word, int kept, int64_t dst,
+                                         char *out_pos, char *out_attr, int64_t OS, int32_t *out_idx)
+{
+    constexpr int kRows = kCmpThreads / kCmpFew, kTurns = (59 + kRows - 1) / kRows, NF = attr_f32_rows(DT);
+    const int d = threadIdx.x % kCmpFew;
+    // the d-th kept primitive: its word, and its rank there
+    int left = d, rank = 0;
+    int64_t i = i0;
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int w = 0; w < kCmpUnit / 32; ++w) {
+        const uint32_t m = __shfl_sync(0xffffffffu, word, w);
+        const int c = __popc(m);
+        if (left >= 0 && left < c) {
+            mine = m;
+            rank = left;
+            i = i0 + w * 32;
+        }
+        left -= c;
+    }
+    if (d >= kept) return;
+    for (int k = 0; k < rank; ++k) mine &= mine - 1u;
+    i += __ffs(mine) - 1;
+    dst += d;
+    if (out_idx && threadIdx.x < kCmpFew) out_idx[dst] = (int32_t)i;
+    uint32_t v[kTurns];
+#pragma unroll
+    for (int k = 0; k < kTurns; ++k) {
+        const int r = threadIdx.x / kCmpFew + k * kRows;
+        if (r >= 59) continue;
+        v[k] = in.f32(r) ? __ldg(reinterpret_cast<const uint32_t *>(in.row(r)) + i)
+                         : __ldg(reinterpret_cast<const unsigned short *>(in.row(r)) + i);
+    }
+#pragma unroll
+    for (int k = 0; k < kTurns; ++k) {
+        const int r = threadIdx.x / kCmpFew + k * kRows;
+        if (r >= 59) continue;
+        if (in.f32(r))
+            *((r < 3 ? reinterpret_cast<uint32_t *>(out_pos) + r * OS
+                     : reinterpret_cast<uint32_t *>(out_attr) + (r - 3) * OS) + dst) = v[k];
+        else
+            reinterpret_cast<unsigned short *>(out_attr + NF * OS * 4)[(r - 3 - NF) * OS + dst] = (unsigned short)v[k];
+    }
+}
+
+template <int DT>
+__global__ void __launch_bounds__(kCmpThreads, cmp_ctas(DT)) k_compact(CmpRows<DT> in, int64_t n, const uint32_t *__restrict__ mask,
                                                          CmpOffsets off, char *__restrict__ out_pos,
                                                          char *__restrict__ out_attr, int64_t OS,
                                                          int32_t *__restrict__ out_idx, int *status)
 {
-    constexpr int UNIT = cmp_unit(DT), UW = UNIT / 32, SEGU = kCmpSeg / UNIT;
+    constexpr int UNIT = kCmpUnit, UW = UNIT / 32;
     extern __shared__ __align__(16) unsigned char tile[];
     __shared__ unsigned char src_of[UNIT];
     __shared__ unsigned blk_off[kCmpMaxBlocks];
@@ -98,12 +157,19 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(CmpRows<DT> i
         }
         return word;
     };
+    auto start_of = [&](int64_t u) {  // where the unit's first kept primitive goes
+        return off.blocks > 0 ? (int64_t)(blk_off[u / kCmpBlockSegs] + __ldg(off.local + u)) : (int64_t)__ldg(off.global + u);
+    };
+    bool few = false;
     uint32_t next_word = load_word(blockIdx.x);
     for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
         const uint32_t word = next_word;
         next_word = load_word(u + gridDim.x);
         const int kept = __reduce_add_sync(0xffffffffu, (unsigned)__popc(word));
-        if (kept == 0) continue;  // the same in every thread
+        if (kept <= kCmpFew) {  // the same in every thread
+            few |= kept > 0;
+            continue;
+        }
         const int64_t i0 = u * UNIT;
         const int count = (int)min((int64_t)UNIT, n - i0);
         in.template stage<kCmpWarps>(tile, i0, count, &bar);
@@ -124,13 +190,7 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(CmpRows<DT> i
                     src_of[b + __popc(mine & ((1u << lane) - 1u))] = (unsigned char)(warp * 32 + lane);
             }
         }
-        const int64_t sg = i0 / kCmpSeg;
-        int64_t dst = off.blocks > 0 ? (int64_t)(blk_off[sg / kCmpBlockSegs] + __ldg(off.local + sg))
-                                     : (int64_t)__ldg(off.global + sg);
-        if (SEGU > 1 && u % SEGU != 0) {  // kept in the segment's earlier unit
-            const uint32_t w0 = lane < UW ? __ldg(mask + (u - 1) * UW + lane) : 0u;
-            dst += __reduce_add_sync(0xffffffffu, (unsigned)__popc(w0));
-        }
+        const int64_t dst = start_of(u);
         __syncthreads();  // src_of, and what plain loads brought
         const int nb = (kept + 31) >> 5;
         int src[UW];
@@ -144,24 +204,44 @@ __global__ void __launch_bounds__(kCmpThreads, kCmpCtas) k_compact(CmpRows<DT> i
             return;
         }
         phase ^= 1u;
-        for (int r = warp; r < 59; r += kCmpWarps) {
+        // The rows of the tile to their places, 32 outputs at a time.  (Left
+        // to the compiler, whether the row loop was unrolled hung on code far
+        // from it: 158 or 184 us, 3.5M bfloat16 at ratio 0.)
+        auto put = [&](auto words, auto *out, int r) {
+            using E = std::remove_pointer_t<decltype(out)>;
             const unsigned char *t = tile + row_base[r];
-            if (CmpRows<DT>::f32(r)) {
-                float *o = (r < 3 ? reinterpret_cast<float *>(out_pos) + (int64_t)r * OS
-                                  : reinterpret_cast<float *>(out_attr) + (int64_t)(r - 3) * OS) + dst + lane;
 #pragma unroll
-                for (int b = 0; b < UW; ++b)
-                    if (b * 32 + lane < kept) o[b * 32] = *reinterpret_cast<const float *>(t + 4 * src[b]);
-            } else {
-                constexpr int NF = attr_f32_rows(DT);
-                unsigned short *o = reinterpret_cast<unsigned short *>(out_attr + (int64_t)NF * OS * 4) +
-                                    (int64_t)(r - 3 - NF) * OS + dst + lane;
-#pragma unroll
-                for (int b = 0; b < UW; ++b)
-                    if (b * 32 + lane < kept) o[b * 32] = *reinterpret_cast<const unsigned short *>(t + 2 * src[b]);
-            }
-        }
+            for (int b = 0; b < decltype(words)::value; ++b)
+                if (b * 32 + lane < kept) out[b * 32] = *reinterpret_cast<const E *>(t + sizeof(E) * src[b]);
+        };
+        constexpr int NF = CmpRows<DT>::kF32;
+        auto put_rows = [&](auto words) {
+#pragma unroll 2
+            for (int r = warp; r < NF; r += kCmpWarps)
+                put(words, (r < 3 ? reinterpret_cast<float *>(out_pos) + r * OS
+                                  : reinterpret_cast<float *>(out_attr) + (r - 3) * OS) + dst + lane, r);
+            unsigned short *out2 = reinterpret_cast<unsigned short *>(out_attr + (NF - 3) * OS * 4) + dst + lane;
+#pragma unroll 7
+            for (int r = NF + warp; r < 59; r += kCmpWarps) put(words, out2 + (r - NF) * OS, r);
+        };
+        if (kept <= 32)
+            put_rows(std::integral_constant<int, 1>());
+        else
+            put_rows(std::integral_constant<int, UW>());
         __syncthreads();  // the tile and src_of are free again
+    }
+    if (!few) return;
+
+    // The units with few kept primitives, in a loop of their own: within the
+    // other it took registers from it.  No barrier: the warps go through them
+    // on their own.
+    next_word = load_word(blockIdx.x);
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const uint32_t word = next_word;
+        next_word = load_word(u + gridDim.x);
+        const int kept = __reduce_add_sync(0xffffffffu, (unsigned)__popc(word));
+        if (kept == 0 || kept > kCmpFew) continue;
+        copy_few<DT>(in, u * UNIT, word, kept, start_of(u), out_pos, out_attr, OS, out_idx);
     }
 }
 
@@ -170,9 +250,12 @@ static cudaError_t launch_compact_t(const refine_scene &in, const uint32_t *mask
                                     void *out_attr, int64_t OS, int32_t *out_idx, int num_sms, int *status, const Chain &s)
 {
     const size_t smem = CmpRows<DT>::kBytes;
-    static_assert(CmpRows<DT>::kBytes < 40 * 1024, "no opt-in shared memory");
-    int64_t g = (in.n + cmp_unit(DT) - 1) / cmp_unit(DT);
-    if (g > (int64_t)num_sms * kCmpCtas) g = (int64_t)num_sms * kCmpCtas;
+    if (smem + 4 * 1024 > 48 * 1024) {  // static part included; one constant for every launch
+        const cudaError_t e = cudaFuncSetAttribute(k_compact<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    int64_t g = (in.n + kCmpUnit - 1) / kCmpUnit;
+    if (g > (int64_t)num_sms * cmp_ctas(DT)) g = (int64_t)num_sms * cmp_ctas(DT);
     if (g < 1) g = 1;
     const CmpRows<DT> rows(in.pos, in.attr, in.row_stride, in.n);
     return launch_chained(k_compact<DT>, (int)g, kCmpThreads, smem, s, rows, in.n, mask, off,

@@ -66,3 +66,38 @@ def test_large_row_layouts(env, dtype, over):
         op, oa, oi = ctx.compact(p, a, mask, nk)
         assert torch.equal(op, kept[0]) and torch.equal(oa.float(), kept[1].float()) and torch.equal(oi, kept[2]), (stride - n, first)
     ctx.check()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "bf16s"])
+@pytest.mark.parametrize("n,pad", [(1, 0), (255, 1), (257, 0), (12_345, 3), (200_001, 0)])
+def test_compact_units_of_every_count(env, dtype, n, pad):
+    """Units of 256 primitives that keep 0 to 12, 31 to 34 or all of theirs
+    (those of at most 8 are read element by element, those of at most 32 take
+    one store a row), the kept ones at random places, the unit's first and last
+    among them: equal to indexing the rows."""
+    torch, rb, ctx = env
+    dev = torch.device("cuda", 0)
+    rng = np.random.default_rng(n + pad)
+    keep = np.zeros(n, dtype=bool)
+    counts = list(range(13)) + [31, 32, 33, 34, 256]
+    for u in range(0, n, 256):
+        size = min(256, n - u)
+        k = min(size, counts[(u // 256) % len(counts)])
+        at = rng.permutation(size)[:k]
+        if k >= 2:
+            at = np.unique(np.concatenate([at[2:], [0, size - 1]]))
+        keep[u + at] = True
+    keep[n - 1] = True
+    words = np.packbits(np.pad(keep, (0, -n % 32)), bitorder="little").view(np.int32)
+    want = torch.from_numpy(np.nonzero(keep)[0]).to(dev)
+    g = torch.Generator(device=dev).manual_seed(n)
+    pos = torch.randn((3, n), generator=g, device=dev)
+    attr = torch.randn((56, n), generator=g, device=dev)
+    p, a = laid_out(torch, rb, pos, attr, dtype, n + pad, 0)
+    rows = a.float()[:, :n]
+    for with_idx in (True, False):
+        op, oa, oi, cnt = ctx.compact(p, a if dtype != "bf16s" else a[:, :n], torch.from_numpy(words).to(dev), want.numel(),
+                                      out_row_stride=want.numel() + pad, kept_idx=with_idx, return_count=True)
+        assert cnt == want.numel()
+        assert oi is None if not with_idx else torch.equal(oi, want.to(torch.int32))
+        assert torch.equal(op, p[:, want]) and torch.equal(oa.float(), rows[:, want])
