@@ -238,12 +238,15 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
             if (lane == 0) sum[warp] = t;
         }
         __syncthreads();
-        bool far = false;
+        // (a reciprocal that is a little off moves the line by as little; by
+        // division it took all threads a microsecond)
+        const float im = rcp_approx_ftz((float)m);
         float mean[4];
+        bool far = false;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            mean[q] = sum[q] / (float)m;
-            const float var = sum[4 + q] / (float)m - mean[q] * mean[q], d = (p[q] - base[q]) - mean[q];
+            mean[q] = sum[q] * im;
+            const float var = fmaf(-mean[q], mean[q], sum[4 + q] * im), d = (p[q] - base[q]) - mean[q];
             far |= use & (var > 0.f) & (d * d > kGridFar * kGridFar * var);
         }
         const int dropped = __syncthreads_count(far);  // (every thread has read the sums)
