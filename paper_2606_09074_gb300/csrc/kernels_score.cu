@@ -51,6 +51,9 @@ namespace refine {
 // Floor of PairIn::s3: with it, and E > 1e-3 and z > 1e-6 (classify), s3 K is
 // above every du whose (du z)^2 underflows, which the exact test would pass.
 constexpr float kMinS3 = 1e-12f;
+// From here on the square of du z may be infinite, which the exact test passes
+// when its other side is too: the footprint bound then excludes nothing.
+constexpr float kMaxDz = 1e18f;
 
 struct PairIn {
     float mx, my, mz;
@@ -147,7 +150,7 @@ __device__ __forceinline__ int classify(const CamRec &c, const TileBox &t, float
     const float dx = fmaxf(-U.lo, UW.hi), dy = fmaxf(-V.lo, VH.hi);  // largest du, dv of the box
     const float zs = z.lo - t.s3;
     const float iz = rcp_approx_ftz(z.lo), q = zs > 0.f ? z.lo * rcp_approx_ftz(zs) : INFINITY;
-    const bool safe = z.lo > 1e-6f && fminf(k.x, k.y) > 1e-3f && fmaxf(dx, dy) * z.hi < 1e18f;
+    const bool safe = z.lo > 1e-6f && fminf(k.x, k.y) > 1e-3f && fmaxf(dx, dy) * z.hi < kMaxDz;
     const float kx = safe ? fminf(k.x * q, fmaf(fmaxf(dx, 0.f), iz, k.x)) * 1.00390625f : INFINITY;
     const float ky = safe ? fminf(k.y * q, fmaf(fmaxf(dy, 0.f), iz, k.y)) * 1.00390625f : INFINITY;
     *reach = make_float2(kx, ky);
@@ -282,7 +285,8 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
         if (NZ) {
             const float4 k = c.k;
             const float zs = z[g] - p[g].s3, t = p[g].s3 * z[g] * 1.00390625f;
-            reaches &= (du[g] * zs <= k.x * t) & (dv[g] * zs <= k.y * t);
+            // (where a square of the exact test may overflow, that test decides, as with the depth range closed)
+            reaches &= ((du[g] * zs <= k.x * t) & (dv[g] * zs <= k.y * t)) | !(fmaxf(du[g], dv[g]) * z[g] < kMaxDz);
         }
         vis[g] = inside;
         nq[g] = !inside & reaches;

@@ -1,5 +1,6 @@
 """The plain calls away from ordinary scenes: more views under capture than in
-the calls before it; a few primitives far from all others."""
+the calls before it; a few primitives far from all others; overflowing pairs."""
+import numpy as np
 import pytest
 
 from paper_2606_09074_gb300 import synth
@@ -74,3 +75,28 @@ def test_outliers_leave_the_order_as_it_is(env, n, rows, value):
     ctx.close()
     own = len(far) * 64 * v  # each outlier's tile, all pairs
     assert got["mixed_pairs"] <= 1.02 * plain["mixed_pairs"] + own, (got["mixed_pairs"], plain["mixed_pairs"])
+
+
+def test_far_pair_does_not_depend_on_its_tile(env):
+    """A pair so far out that both sides of its footprint test overflow is
+    decided the same whether its tile leaves the depth range open or not (a
+    second primitive behind the camera opens it)."""
+    torch, rb, dev = env
+    cam = synth.random_scene(seed=1, n=1, v=1).cams.copy()
+    cam["R"], cam["t"] = np.eye(3, dtype=np.float32).reshape(cam["R"].shape), 0.0
+    cam["fx"] = cam["fy"] = 500.0
+    cam["cx"], cam["cy"], cam["width"], cam["height"] = 320.0, 240.0, 640, 480
+    cam["znear"], cam["zfar"] = 0.01, 1e13
+    cams = rb.cameras_to_device(cam, dev)
+    attr = np.zeros((56, 2), dtype=np.float32)
+    attr[0:3], attr[3] = 0.5, 1.0
+    pos = np.array([[-4e16, 0.0], [0.0, 0.0], [2e11, -1.0]], dtype=np.float32)
+    sums = []
+    for n in (1, 2):
+        ctx = rb.Context(0)
+        vs = torch.zeros(n, device=dev)
+        ctx.score(torch.from_numpy(pos[:, :n].copy()).to(dev), torch.from_numpy(attr[:, :n].copy()).to(dev), cams, view_sum=vs)
+        ctx.check()
+        sums.append(vs[0].item())
+        ctx.close()
+    assert sums[0] == sums[1] > 0.0
