@@ -122,9 +122,10 @@ __device__ __forceinline__ Range form_range(const float4 &a, const TileBox &t, f
 // distance of an edge from cx, so with E = sqrt(fx^2 + e^2)
 //   du <= 3 s_max (E + du / z),  i.e.  du (z - s3) <= s3 E z,  s3 = 3 s_max,
 // and over a box with z >= z_lo: du <= s3 K, K = min(E z_lo / (z_lo - max s3)
-// (if z_lo > max s3), E + max du / z_lo).  *reach (MIXED with the depth range
-// closed) is (Kx, Ky), infinite (nothing is excluded) where a square of the
-// exact test could overflow or underflow.
+// (if z_lo > max s3), E + max du / z_lo).  *reach (MIXED) is (Kx, Ky), infinite
+// (nothing is excluded) where a square of the exact test could overflow or
+// underflow; with the depth range open (Ex, Ey), infinite where one could
+// overflow.
 enum { kClsMixed = 0, kClsIn = 1, kClsOut = 2 };
 enum { kAxX = 4, kAxY = 8, kAxZ = 16 };
 
@@ -150,10 +151,12 @@ __device__ __forceinline__ int classify(const CamRec &c, const TileBox &t, float
     const float dx = fmaxf(-U.lo, UW.hi), dy = fmaxf(-V.lo, VH.hi);  // largest du, dv of the box
     const float zs = z.lo - t.s3;
     const float iz = rcp_approx_ftz(z.lo), q = zs > 0.f ? z.lo * rcp_approx_ftz(zs) : INFINITY;
-    const bool safe = z.lo > 1e-6f && fminf(k.x, k.y) > 1e-3f && fmaxf(dx, dy) * z.hi < kMaxDz;
+    const bool finite = fmaxf(dx, dy) * z.hi < kMaxDz;
+    const bool safe = z.lo > 1e-6f && fminf(k.x, k.y) > 1e-3f && finite;
     const float kx = safe ? fminf(k.x * q, fmaf(fmaxf(dx, 0.f), iz, k.x)) * 1.00390625f : INFINITY;
     const float ky = safe ? fminf(k.y * q, fmaf(fmaxf(dy, 0.f), iz, k.y)) * 1.00390625f : INFINITY;
-    *reach = make_float2(kx, ky);
+    const bool edge = !zin & finite;  // (kx and ky are infinite when not finite)
+    *reach = make_float2(edge ? k.x : kx, edge ? k.y : ky);
     // the whole box beyond an edge by more than the reach of its largest primitive
     if (fmaxf(-U.hi, UW.lo) > t.s3 * kx || fmaxf(-V.hi, VH.lo) > t.s3 * ky) return kClsOut;
     return mixed;
@@ -260,7 +263,7 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
                                            unsigned long long (&cnt)[kCountSlots])
 {
     const float4 c2 = c.r2, lim = c.lim;
-    const float2 K = NZ ? make_float2(0.f, 0.f) : reach;
+    const float2 K = reach;
     float z[GPT], U[GPT], V[GPT], du[GPT], dv[GPT];
     bool vis[GPT], nq[GPT];
 #pragma unroll
@@ -283,10 +286,8 @@ __device__ __forceinline__ void mixed_view(const CamRec &c, const CamExt *e, con
             if (!NZ) reaches &= dv[g] <= p[g].s3 * K.y;
         }
         if (NZ) {
-            const float4 k = c.k;
             const float zs = z[g] - p[g].s3, t = p[g].s3 * z[g] * 1.00390625f;
-            // (where a square of the exact test may overflow, that test decides, as with the depth range closed)
-            reaches &= ((du[g] * zs <= k.x * t) & (dv[g] * zs <= k.y * t)) | !(fmaxf(du[g], dv[g]) * z[g] < kMaxDz);
+            reaches &= (du[g] * zs <= K.x * t) & (dv[g] * zs <= K.y * t);
         }
         vis[g] = inside;
         nq[g] = !inside & reaches;
