@@ -201,7 +201,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
     // Sums of the offsets from primitive 0 and of their squares (a scene far
     // from the origin keeps its digits), and of ln s_max.  A sample beyond
     // kGridFar standard deviations (at most 1 in 36 can be, none in an ordinary
-    // scene) is left out and the sums are formed again about the mean found:
+    // scene) is left out and the sums are formed again about the mean found, as
+    // long as that halves some deviation (a round is 1 us):
     // one centre of 1M at 1,000 or 10,000 scene radii among the 1,024 made the
     // box, and with it all cells, so much wider that a pass over 60 views took
     // 306 or 761 us, against 155 without it and 157 so.
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
     __shared__ float red[8][kPrepThreads / 32];
     __shared__ float sum[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    bool again = false;
+    float before[4] = {0.f, 0.f, 0.f, 0.f};  // the variances found last
     for (int round = 0;; ++round) {
         float s[8];
 #pragma unroll
@@ -242,16 +243,18 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
         // division it took all threads a microsecond)
         const float im = rcp_approx_ftz((float)m);
         float mean[4];
-        bool far = false;
+        bool far = false, shrunk = round == 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             mean[q] = sum[q] * im;
             const float var = fmaf(-mean[q], mean[q], sum[4 + q] * im), d = (p[q] - base[q]) - mean[q];
             far |= use & (var > 0.f) & (d * d > kGridFar * kGridFar * var);
+            shrunk |= 4.f * var < before[q];
+            before[q] = var;
         }
+        if (!shrunk || round == kGridRounds) break;  // (the same in every thread)
         const int dropped = __syncthreads_count(far);  // (every thread has read the sums)
-        if ((dropped == 0 && !again) || round == kGridRounds) break;
-        again = dropped > 0;  // and once more when none is left out any longer: about the mean of those that stay
+        if (round == 0 && dropped == 0) break;
         use &= !far;
         m -= dropped;
 #pragma unroll
