@@ -58,6 +58,7 @@ struct OrderGrid {
     float lo[3];      // grid origin (mean - 3 sigma per axis)
     float qscale[3];  // cells per unit length per axis
     float big_ls;     // ln s_max above which a primitive is ordered with the large ones
+    int crowded;      // whether many primitives share few cells
 };
 
 // Scene statistics (host-visible copy of refine_scene_stats).

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
     __shared__ float red[8][kPrepThreads / 32];
     __shared__ float sum[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float before[4] = {0.f, 0.f, 0.f, 0.f};  // the variances found last
+    float before[4] = {0.f, 0.f, 0.f, 0.f}, im;  // the variances found last, 1 / m
     for (int round = 0;; ++round) {
         float s[8];
 #pragma unroll
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
         __syncthreads();
         // (a reciprocal that is a little off moves the line by as little; by
         // division it took all threads a microsecond)
-        const float im = rcp_approx_ftz((float)m);
+        im = rcp_approx_ftz((float)m);
         float mean[4];
         bool far = false, shrunk = round == 0;
 #pragma unroll
@@ -260,6 +260,24 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
 #pragma unroll
         for (int q = 0; q < 4; ++q) base[q] += mean[q];
     }
+    // Whether cells are crowded: in two of four warps three samples or more
+    // share one (by chance, every fifth of a scene whose fullest cell holds 5 %;
+    // cells of an ordinary scene hold less than 0.01 %).  All 32 warps would take
+    // 2 us: a match takes a step for each distinct value.
+    bool crowd = false;
+    if (warp % 8 == 0) {
+        uint32_t cell = 0u;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float cells = (float)(1 << a.cell_bits), var = before[q];
+            const float at = ((p[q] - base[q]) - sum[q] * im) * (var > 0.f ? rsqrtf(var) : 0.f);  // in sd
+            cell = cell << 8 | (uint32_t)fminf(fmaxf((at + 3.f) * cells / 6.f, 0.f), cells - 1.f);
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, threadIdx.x < n ? cell : 0xffffff00u + lane);
+        crowd = __any_sync(0xffffffffu, __popc(peers) >= 3);
+    }
+    const int crowds = __syncthreads_count(crowd);
+    if (threadIdx.x == 0) a.grid->crowded = crowds >= 2 * 32;
     if (threadIdx.x < 4) {
         const int q = threadIdx.x;  // x, y, z, ln s_max
         const float mean = sum[q] / (float)m, var = sum[4 + q] / (float)m - mean * mean;
@@ -386,6 +404,20 @@ __device__ __forceinline__ PrimRows read_rows(L &&ld)  // ld(r): row r of 59
     return p;
 }
 
+// The next slot of a primitive's cell.  Where the cells are crowded (k_prepare)
+// the lanes of a warp that share one take their slots in one add: adds to one
+// address are served one by one.  Elsewhere there is nothing to share, and the
+// search for it would take 1 us of 400k primitives.
+__device__ __forceinline__ unsigned take_slot(unsigned *counts, unsigned key, int crowded)
+{
+    if (!crowded) return atomicAdd(&counts[key], 1u);
+    const unsigned peers = __match_any_sync(__activemask(), key);
+    const int lead = __ffs(peers) - 1, lane = threadIdx.x & 31;
+    unsigned first = 0u;
+    if (lane == lead) first = atomicAdd(&counts[key], (unsigned)__popc(peers));
+    return __shfl_sync(peers, first, lead) + __popc(peers & ((1u << lane) - 1u));
+}
+
 template <int DT>
 __device__ __forceinline__ FeatTerms feature_one(const FeatureArgs<DT> &f, const uint16_t *hilbert, const OrderGrid &og,
                                                  int64_t i, const PrimRows &p, float &bad, bool &zero_q, uint2 &key_slot)
@@ -401,7 +433,7 @@ __device__ __forceinline__ FeatTerms feature_one(const FeatureArgs<DT> &f, const
     PrimRec *r = f.recs + i;
     r->a = ra; r->b = rb; r->c = rc; r->d = rd;
     key_slot.x = order_key(hilbert, og, f.cell_bits, p.x, p.y, p.z, fmaxf(p.ls0, fmaxf(p.ls1, p.ls2)));
-    key_slot.y = atomicAdd(&f.counts[key_slot.x], 1u);  // the slot in its cell
+    key_slot.y = take_slot(f.counts, key_slot.x, og.crowded);
     return t;
 }
 

@@ -1,9 +1,11 @@
 """The plain calls away from ordinary scenes: more views under capture than in
-the calls before it; a few primitives far from all others; overflowing pairs."""
+the calls before it; a few primitives far from all others; overflowing pairs; crowded cells."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2606_09074_gb300 import synth
+from parity_helpers import assert_score_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -100,3 +102,30 @@ def test_far_pair_does_not_depend_on_its_tile(env):
         sums.append(vs[0].item())
         ctx.close()
     assert sums[0] == sums[1] > 0.0
+
+
+@pytest.mark.parametrize("n,dtype", [(40, "f32"), (5_003, "bf16"), (330_001, "f32"), (330_001, "bf16"), (330_000, "bf16s")])
+@pytest.mark.parametrize("kind", ["two", "same", "sorted"])
+def test_crowded_cells(env, n, dtype, kind):
+    """Centres in a few cells of the processing order's grid (two dense clusters
+    far apart, in random and in spatial order, or all in one place): scores
+    against the oracle, for the small and the full-grid feature kernels."""
+    torch, rb, dev = env
+    rng = np.random.default_rng(n)
+    w = synth.random_scene(seed=n, n=n, v=3, means="core_shell")
+    pos = 0.2 * rng.standard_normal((3, n)) + np.where(rng.random(n) < 0.5, -6.0, 6.0)
+    if kind == "same":
+        pos[:] = np.array([[0.5], [0.25], [-0.125]])
+    elif kind == "sorted":
+        pos = pos[:, np.argsort(pos[0])]
+    w.scene.pos[:] = pos.astype(np.float32)
+    scene = {"f32": w.scene, "bf16": w.scene.to_bf16(), "bf16s": w.scene.to_bf16s()}[dtype]
+    pos_d, attr_d, cams = uploaded(torch, rb, dev, w)
+    attr_d = {"f32": lambda a: a, "bf16": lambda a: a.to(torch.bfloat16),
+              "bf16s": lambda a: rb.MixedRows.from_float(a, device=dev)}[dtype](attr_d)
+    ctx, vs = rb.Context(0), torch.empty(n, device=dev)
+    got = ctx.score(pos_d, attr_d, cams, view_sum=vs)
+    ctx.check()
+    ctx.close()
+    idx = np.unique(rng.integers(0, n, 2000))
+    assert_score_parity(got.cpu().numpy()[idx], vs.cpu().numpy()[idx], oracle.score_subset(scene.params_f64(), idx, w.cams))
