@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
+import test_gpu_parity as parity
 from paper_2606_09074_gb300 import synth
 from parity_helpers import assert_score_parity
 
@@ -129,3 +130,14 @@ def test_crowded_cells(env, n, dtype, kind):
     ctx.close()
     idx = np.unique(rng.integers(0, n, 2000))
     assert_score_parity(got.cpu().numpy()[idx], vs.cpu().numpy()[idx], oracle.score_subset(scene.params_f64(), idx, w.cams))
+
+
+@pytest.mark.parametrize("over,dtype", [(3, "f32"), (3, "bf16"), (8, "bf16"), (3, "bf16s")])
+def test_chained_large_scenes(env, over, dtype):
+    """The plain calls chained, as in test_chained_calls_same_bits, for scenes
+    past the small feature kernel's limit."""
+    torch, rb, dev = env
+    ctx = rb.Context(0)
+    n = 2048 * torch.cuda.get_device_properties(dev).multi_processor_count + 8 + over
+    parity.test_chained_calls_same_bits(torch, rb, ctx, n, 20, dtype)
+    ctx.close()
