@@ -261,8 +261,8 @@ refine_status refine_prune_host(refine_ctx *ctx, int64_t n, int32_t dtype,
 /* ------------------------------------------------------------ batches
  * Many scenes in one go: per-scene preparation (content features, lambda,
  * processing order) and per-scene selection and compaction run on parallel
- * streams, and all scenes are scored by persistent kernel launches over a
- * (scene, tile, camera block) work list: one launch per camera block level,
+ * streams, and all scenes are scored by persistent kernel launches whose
+ * warps draw the scenes' tiles: one launch per camera block level,
  * launch p scoring the p-th block of views of every scene that has one
  * (a single launch when every scene has at most camera_block views).  The
  * whole batch is captured into a CUDA graph on its first run and replayed
@@ -362,12 +362,13 @@ refine_status refine_ctx_set_shape(refine_ctx *ctx, const refine_shape *shape);
  *     through one input-copy stream, in admission order, so that each ends
  *     as early as the link allows), and its preparation follows on its
  *     slot stream;
- *   - the scorer batches continuously: as soon as the previous batched
- *     launch has ended, ONE persistent launch scores every request whose
- *     preparation has ended, or whose copy has ended if it is no larger
- *     than the oldest of them (those requests form a round; a request with
- *     more views than the camera block has its further blocks scored right
- *     after it, in order, on the same stream); selection and compaction
+ *   - the scorer batches continuously: when the previous batched launch
+ *     has ended, ONE persistent launch scores every request whose
+ *     preparation has ended, and every one of at most 1/64 of the oldest's
+ *     primitives whose copy has ended (one so small that is being issued is
+ *     waited for, 0.2 ms at most).  Those requests form a round; a request
+ *     with more views than the camera block has its further blocks scored
+ *     right after it, in order, on the same stream.  Selection and compaction
  *     then run on the requests' slot streams and the copies back on one
  *     output-copy stream.  Requests that arrive while others are on the GPU
  *     thus join the next launch, and their copies overlap the others'

@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kFeatCol, 4) k_features(FeatureArgs<DT> f)
 // SM).  The next tile is issued as soon as every thread has read the current
 // one, so it arrives while the records are formed.  ALIGNED: every row starts
 // on 16 bytes (the stride is a multiple of 8), so places are constants.  3.5M
-// bfloat16 primitives: 157 -> 142 us (4.6 TB/s; what is left is the latency of
+// bfloat16 primitives: 157 -> 139 us (4.9 TB/s; what is left is the latency of
 // a primitive's arithmetic at 32 warps an SM); the same with all copies issued
 // by one warp 160 us.
 template <int DT, bool ALIGNED>

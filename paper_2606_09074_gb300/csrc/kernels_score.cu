@@ -8,9 +8,10 @@ namespace refine {
 // ---------------------------------------------------------------------
 // The N x V importance kernel.
 //
-// One thread owns two primitives (the lanes of a warp hold 64 consecutive
-// primitives of the processing order, a "tile") and walks every camera of
-// the pass; the camera records are staged once per CTA into shared memory by
+// The lanes of a warp hold 64 consecutive primitives of the processing order,
+// two each, or 32 (a "tile"; score_plan), and walk the cameras of the pass, or
+// of an item of 64 views where the tile is split (TilePart); the camera records
+// are staged once per CTA into shared memory by
 // a TMA bulk copy.  For primitive i and view v (Eq. 13-14, Eq. 17, Eq. 20):
 //   (U, V, z) = P mu + p                  homogeneous pixel, u = U / z
 //   d_u z = max(-U, U - w z)              distance of the centre outside
@@ -29,19 +30,21 @@ namespace refine {
 //
 // Work is skipped only where the outcome is already implied, so every
 // decision equals the full test's, bit for bit:
-//  * per tile (the bounding box of its 64 centres) and view, a lane classifies
-//    one view (32 views at a time) with interval bounds of the linear forms
-//    U, V, z, U - w z, V - h z, fx x, fy y over the box, plus a 2^-14
-//    relative slack that covers float32 rounding:
+//  * per tile (the bounding box of its centres) and view, a lane classifies
+//    one view (32 views at a time) with interval bounds of the linear forms z,
+//    U, V, U - w z and V - h z over the box, widened by a slack that covers
+//    float32 rounding (2^-17 of the largest magnitude for z, 2^-16 for the
+//    others; classify):
 //      IN   every centre is in range and inside the image: vis = 1 for all
 //      OUT  every centre is out of range, or outside an image edge by more
-//           than the footprint bound below: vis = 0, the view is skipped
-//      MIXED otherwise: decided pair by pair;
-//  * pair by pair, in two warp-uniform stages entered only when some lane
-//    needs them: a centre inside the image is visible whatever Sigma2D; a
-//    centre outside is first tested against Qx <= 9 s_max^2 ((U - cx z)^2 +
-//    fx^2 z^2) (as |g0|^2 = fx^2 (x^2 + z^2); inflated by 2^-10), and only
-//    lanes passing that bound need Qx and Qy.
+//           than the footprint bound: vis = 0, the view is skipped
+//      MIXED otherwise: decided pair by pair, on the axes left open;
+//  * pair by pair (mixed_view) a centre inside the image is visible whatever
+//    Sigma2D, and one outside is tested against the footprint bound, d_u <=
+//    3 s_max K with the tile's K, or d_u (z - 3 s_max) <= 3 s_max E z with the
+//    depth range open (classify; s_max inflated by 2^-11, K and E by 2^-8).
+//    Only a pair within it needs Qx and Qy: a warp-uniform stage per axis,
+//    entered when some lane does.
 // Views are summed in blocks of 32, in view order (an invisible or skipped
 // view adds +0, which changes nothing), and the block sums are added to the
 // primitive's total with Kahan compensation, so a primitive's sum does not

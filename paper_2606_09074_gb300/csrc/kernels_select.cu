@@ -354,10 +354,11 @@ cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *s
 // What it saves is launches: six stream operations become one.  The cluster
 // has 1, 2, 4 or 8 CTAs, 6k keys each before the next size is taken (10k scores
 // take 8.0 us with 2 CTAs, 10.3 with 1, 11.4 with 8; 24k 10.1 with 4, 12.8 with
-// 2, 12.2 with 8).  Per selection 1k scores 5.1, 10k 8.0, 50k 14.3, 100k 18.0,
-// 150k 21.9, 200k 25.3 us, against the five kernels and a memset of the other
-// form, a chain of latencies that takes 20.5 us up to 200k scores when the
-// kernels are chained and 33 us when they are not: hence the limits,
+// 2, 12.2 with 8).  Per selection, chained: 1k scores 5.6, 10k 8.7, 50k 14.8,
+// 100k 19.0, 131k 21.2 us, against the five kernels and a memset of the other
+// form, a chain of latencies that takes 22.5-23 us from 131k to 400k scores.
+// Not chained, with a memset before: 100k 25, 200k 33, 262k 37 us, against 34 us
+// of the other form from 300k to 400k, in six nodes of a graph for one: hence the limits,
 // kSelClusterChained and kSelClusterMax.
 // ---------------------------------------------------------------------
 constexpr int kClThreads = 1024;

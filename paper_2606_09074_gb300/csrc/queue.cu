@@ -9,7 +9,8 @@
 //                preparation on the request's slot stream.
 //   scorer       continuous batching: as soon as the previous batched launch
 //                has ended, takes every request whose preparation has ended
-//                (or is about to) and scores them with ONE k_score_batch launch on the score
+//                (and much smaller ones whose copy has; kJoinFraction) and
+//                scores them with ONE k_score_batch launch on the score
 //                stream (its round); per request on its slot stream again the
 //                selection and the compaction, the copies back on the queue's
 //                one output-copy stream (asynchronous when the host buffers
