@@ -357,12 +357,14 @@ cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *s
 // 2, 12.2 with 8).  Per selection, chained: 1k scores 5.6, 10k 8.7, 50k 14.8,
 // 100k 19.0, 131k 21.2 us, against the five kernels and a memset of the other
 // form, a chain of latencies that takes 22.5-23 us from 131k to 400k scores.
-// Not chained, with a memset before: 100k 25, 200k 33, 262k 37 us, against 34 us
-// of the other form from 300k to 400k, in six nodes of a graph for one: hence the limits,
-// kSelClusterChained and kSelClusterMax.
+// Not chained, with a memset before: 100k 25, 200k 33, 262k 37 us, against 33 us.
+// In a batch's graph, which saves five nodes: alone, 150k as fast, 190k 4 and
+// 250k 8 us slower; 8 scenes of 150k or 190k 6 us of 180 faster, of 250k 2, 24 of
+// 250k 5 us of 740 slower.  Hence the limits, kSelClusterChained and
+// kSelClusterMax (batch and queue).
 // ---------------------------------------------------------------------
 constexpr int kClThreads = 1024;
-constexpr int kClKeys = 32 * 1024;  // keys of a CTA at most (128 KB)
+constexpr int kClKeys = 20 * 1024;  // keys of a CTA at most (80 KB)
 constexpr int kClMaxCtas = 8;
 constexpr int kClFill = 6 * 1024;  // keys per CTA at which a larger cluster is taken
 constexpr int kClLoads = 6;         // loads in flight per thread

@@ -1,5 +1,7 @@
 """The plain calls away from ordinary scenes: more views under capture than in
 the calls before it; a few primitives far from all others; overflowing pairs; crowded cells."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -140,4 +142,30 @@ def test_chained_large_scenes(env, over, dtype):
     ctx = rb.Context(0)
     n = 2048 * torch.cuda.get_device_properties(dev).multi_processor_count + 8 + over
     parity.test_chained_calls_same_bits(torch, rb, ctx, n, 20, dtype)
+    ctx.close()
+
+
+@pytest.mark.parametrize("n", [163_840, 163_841])
+def test_unchained_selection_limit(env, n):
+    """Sizes about the limit of the one-launch selection in a batch, whose
+    kernels are not chained, and the entry point that allocates nothing: the
+    masks of the plain call, which takes the passes there."""
+    torch, rb, dev = env
+    ctx = rb.Context(0)
+    pos, attr, cams = uploaded(torch, rb, dev, synth.random_scene(seed=n, n=n, v=2, means="core_shell"))
+    b = rb.Batch(ctx, [{"pos": pos, "attr": attr, "cams": cams, "ratio": 0.66}], compact=False)
+    for _ in range(2):
+        b.run()
+    b.results()
+    scores = b.outputs[0]["scores"]
+    want, thr, nk = ctx.select(scores, 0.66)
+    assert torch.equal(b.outputs[0]["mask"], want)
+    b.close()
+    for s in (scores, torch.floor(4.0 * torch.rand(n, generator=torch.Generator(dev).manual_seed(n), device=dev))):
+        want, thr, nk = ctx.select(s, 0.66)
+        got = torch.zeros_like(want)
+        c_thr, err = ctypes.c_float(), ctypes.create_string_buffer(64)
+        assert rb.refine_select_noalloc(s.data_ptr(), n, 0.66, got.data_ptr(), ctypes.byref(c_thr), None, err, 64,
+                                        torch.cuda.current_stream().cuda_stream) == rb.REFINE_OK
+        assert torch.equal(got, want) and c_thr.value == thr
     ctx.close()
