@@ -128,7 +128,10 @@ inline refine_status use_device(refine_ctx *c)
 inline bool capturing(cudaStream_t s)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {  // the legacy stream while another one captures
+        cudaGetLastError();
+        return false;
+    }
     return st == cudaStreamCaptureStatusActive;
 }
 
