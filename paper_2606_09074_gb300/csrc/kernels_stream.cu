@@ -14,13 +14,13 @@
 //
 // Measured (count and scatter, cold L2, kept at random; us at ratio 0 / 0.5 /
 // 0.9 / 0.98 / 0.995):
-//   3.5M float32   268 / 203 / 152 /  92 /  57   (units of 128, all copied whole:
+//   3.5M float32   272 / 201 / 149 /  92 /  55   (units of 128, all copied whole:
 //                  282 / 219 / 174 / 166 / 104; a warp for 256 primitives, rows
 //                  through registers: 272 / 222 / 187 / 178 / 173)
-//   3.5M bfloat16  156 / 115 /  90 /  76 /  47   (all units copied whole, 6 CTAs
+//   3.5M bfloat16  156 / 113 /  90 /  74 /  45   (all units copied whole, 6 CTAs
 //                  of 40 registers: 158 / 118 / 102 / 100 /  86; a warp for 32
 //                  primitives: 210 / 182 / 159 / 118 /  69)
-//   1M float32      84 /  66 /  55 /  37 /  23   (86 / 68 / 57 / 55 / 39 and
+//   1M float32      84 /  66 /  53 /  35 /  23   (86 / 68 / 57 / 55 / 39 and
 //                   92 /  82 /  69 /  51 /  36)
 // Units of at most 4 kept primitives instead of 8: 3.5M float32 133 us at 0.98;
 // at most 16: 164 us at 0.9.
@@ -44,9 +44,9 @@ using CmpRows = RowTile<DT, kCmpUnit>;
 
 // The rows of a unit's `kept` (at most kCmpFew) primitives by loads of their
 // own: every group of kCmpFew threads takes a row.  word: the unit's mask, a
-// word per lane.
+// word per lane from lane `at` on.
 template <int DT>
-__device__ __forceinline__ void copy_few(const CmpRows<DT> &in, int64_t i0, uint32_t word, int kept, int64_t dst,
+__device__ __forceinline__ void copy_few(const CmpRows<DT> &in, int64_t i0, uint32_t word, int at, int kept, int64_t dst,
                                          char *out_pos, char *out_attr, int64_t OS, int32_t *out_idx)
 {
     constexpr int kRows = kCmpThreads / kCmpFew, kTurns = (59 + kRows - 1) / kRows, NF = attr_f32_rows(DT);
@@ -57,7 +57,7 @@ __device__ __forceinline__ void copy_few(const CmpRows<DT> &in, int64_t i0, uint
     uint32_t mine = 0u;
 #pragma unroll
     for (int w = 0; w < kCmpUnit / 32; ++w) {
-        const uint32_t m = __shfl_sync(0xffffffffu, word, w);
+        const uint32_t m = __shfl_sync(0xffffffffu, word, at + w);
         const int c = __popc(m);
         if (left >= 0 && left < c) {
             mine = m;
@@ -234,14 +234,29 @@ __global__ void __launch_bounds__(kCmpThreads, cmp_ctas(DT)) k_compact(CmpRows<D
 
     // The units with few kept primitives, in a loop of their own: within the
     // other it took registers from it.  No barrier: the warps go through them
-    // on their own.
-    next_word = load_word(blockIdx.x);
-    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
-        const uint32_t word = next_word;
-        next_word = load_word(u + gridDim.x);
-        const int kept = __reduce_add_sync(0xffffffffu, (unsigned)__popc(word));
-        if (kept == 0 || kept > kCmpFew) continue;
-        copy_few<DT>(in, u * UNIT, word, kept, start_of(u), out_pos, out_attr, OS, out_idx);
+    // on their own, the words of four units at a time (lane l: word l % UW of the
+    // l / UW-th), so that a unit with nothing to copy costs a quarter of a load's
+    // latency: 30M bfloat16 at ratio 0.999 259 us with one unit at a time.  (In
+    // the main loop that cost the load of the next word ahead: 30M at 0.5 1,010
+    // against 1,168 us.)
+    const int64_t step = gridDim.x;
+    for (int64_t u0 = blockIdx.x; u0 < units; u0 += 32 / UW * step) {
+        const int64_t un = u0 + lane / UW * step, w = un * UW + lane % UW;
+        uint32_t word = 0u;
+        if (un < units && w < words) {
+            word = __ldg(mask + w);
+            const int64_t valid = n - w * 32;
+            if (valid < 32) word &= (1u << valid) - 1u;
+        }
+        int kept = __popc(word);
+#pragma unroll
+        for (int o = 1; o < UW; o <<= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
+        for (unsigned todo = __ballot_sync(0xffffffffu, lane % UW == 0 && kept > 0 && kept <= kCmpFew); todo; todo &= todo - 1u) {
+            const int at = __ffs(todo) - 1;
+            const int64_t u = u0 + at / UW * step;
+            copy_few<DT>(in, u * UNIT, word, at, __shfl_sync(0xffffffffu, kept, at), start_of(u), out_pos, out_attr, OS,
+                         out_idx);
+        }
     }
 }
 
