@@ -260,6 +260,19 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
 #pragma unroll
         for (int q = 0; q < 4; ++q) base[q] += mean[q];
     }
+    if (warp == 1 && lane < 4) {  // (beside the warps that look for crowds)
+        const int q = lane;  // x, y, z, ln s_max
+        const float mean = sum[q] / (float)m, var = sum[4 + q] / (float)m - mean * mean;
+        const float sd = var > 0.f ? sqrtf(var) : 0.f;
+        const float b = q == 0 ? base[0] : (q == 1 ? base[1] : (q == 2 ? base[2] : base[3]));
+        if (q < 3) {
+            a.grid->lo[q] = b + (mean - 3.f * sd);
+            a.grid->qscale[q] = sd > 0.f && isfinite(sd) ? (float)(1 << a.cell_bits) / (6.f * sd) : 0.f;
+        } else {
+            const float big = b + (mean + kSizeSplitSd * sd);
+            a.grid->big_ls = isfinite(big) ? big : INFINITY;
+        }
+    }
     // Whether cells are crowded: in two of four warps three samples or more
     // share one (by chance, every fifth of a scene whose fullest cell holds 5 %;
     // cells of an ordinary scene hold less than 0.01 %).  All 32 warps would take
@@ -278,19 +291,6 @@ __global__ void __launch_bounds__(kPrepThreads) k_prepare(const float *__restric
     }
     const int crowds = __syncthreads_count(crowd);
     if (threadIdx.x == 0) a.grid->crowded = crowds >= 2 * 32;
-    if (threadIdx.x < 4) {
-        const int q = threadIdx.x;  // x, y, z, ln s_max
-        const float mean = sum[q] / (float)m, var = sum[4 + q] / (float)m - mean * mean;
-        const float sd = var > 0.f ? sqrtf(var) : 0.f;
-        const float b = q == 0 ? base[0] : (q == 1 ? base[1] : (q == 2 ? base[2] : base[3]));
-        if (q < 3) {
-            a.grid->lo[q] = b + (mean - 3.f * sd);
-            a.grid->qscale[q] = sd > 0.f && isfinite(sd) ? (float)(1 << a.cell_bits) / (6.f * sd) : 0.f;
-        } else {
-            const float big = b + (mean + kSizeSplitSd * sd);
-            a.grid->big_ls = isfinite(big) ? big : INFINITY;
-        }
-    }
 }
 
 cudaError_t launch_prepare(const float *pos, const void *attr, int dtype, int64_t stride, int64_t n, const PrepLaunch &a,
