@@ -268,7 +268,7 @@ struct SelState {
 // (launch_select_cluster, which needs nothing cleared and only kstar of the
 // state); above it, the passes below, also where they are chained (then they
 // take 22.5-23 us instead of 34 up to 400k scores).
-constexpr int64_t kSelClusterMax = 8 * 20 * 1024;
+constexpr int64_t kSelClusterMax = 8 * 32 * 1024;
 constexpr int64_t kSelClusterChained = 128 * 1024;
 cudaError_t launch_select_cluster(const float *scores, int64_t n, uint32_t n_keep, SelState *st, uint32_t *mask,
                                   int *status, const Chain &s);

@@ -360,11 +360,13 @@ cudaError_t launch_select_mask(const float *scores, int64_t n, const SelState *s
 // Not chained, with a memset before: 100k 25, 200k 33, 262k 37 us, against 33 us.
 // In a batch's graph, which saves five nodes: alone, 150k as fast, 190k 4 and
 // 250k 8 us slower; 8 scenes of 150k or 190k 6 us of 180 faster, of 250k 2, 24 of
-// 250k 5 us of 740 slower.  Hence the limits, kSelClusterChained and
-// kSelClusterMax (batch and queue).
+// 250k 5 us of 740 slower.  In the queue, whose scorer issues every launch: three
+// jobs of 200k at once 785 against 862 us, eight 1,650 against 1,690, of 250k 2,130
+// against 2,180.  Hence the limits, kSelClusterChained and kSelClusterMax (batch
+// and queue).
 // ---------------------------------------------------------------------
 constexpr int kClThreads = 1024;
-constexpr int kClKeys = 20 * 1024;  // keys of a CTA at most (80 KB)
+constexpr int kClKeys = 32 * 1024;  // keys of a CTA at most (128 KB)
 constexpr int kClMaxCtas = 8;
 constexpr int kClFill = 6 * 1024;  // keys per CTA at which a larger cluster is taken
 constexpr int kClLoads = 6;         // loads in flight per thread

@@ -145,7 +145,7 @@ def test_chained_large_scenes(env, over, dtype):
     ctx.close()
 
 
-@pytest.mark.parametrize("n", [163_840, 163_841])
+@pytest.mark.parametrize("n", [196_609, 262_144, 262_145])
 def test_unchained_selection_limit(env, n):
     """Sizes about the limit of the one-launch selection in a batch, whose
     kernels are not chained, and the entry point that allocates nothing: the
